@@ -14,6 +14,7 @@
 //   (strongest unmatched strong neighbour, ties to the smaller index), pass
 //   k+1 on the aggregate graph with max-reduced weights; aggregates numbered
 //   by smallest fine index; nodes without any strong connection left out.
+#include <cooperative_groups.h>
 #include <cub/device/device_radix_sort.cuh>
 #include <cub/device/device_scan.cuh>
 
@@ -25,7 +26,7 @@
 
 namespace nbp {
 
-constexpr int kMatchRounds = 64;   // rounds per matching pass (extra rounds after convergence are no-ops)
+constexpr int kMatchRounds = 64;   // rounds per matching pass (rounds after one that makes no pair change nothing)
 
 // ------------------------------------------------------------- utilities
 void dmat_free(DMat &m, cudaStream_t s) {
@@ -102,11 +103,16 @@ __global__ void k_diag_norm(int n, int nb, const int *rp, const int *ci, const d
     dn[i] = (e >= 0) ? fnorm2_rn(v + (long long)e * nb, nb) : 0.0;
 }
 
-// w[e] = sigma_ij for off-diagonal entries, -1 on the diagonal
+// w[e] = sigma_ij for off-diagonal entries, -1 on the diagonal.  Eight lanes
+// per row: every entry is a chain of its own (the search for (j, i), then two
+// blocks), which one thread per row ran one after another (0.56M-unknown
+// tangent, all levels: 1.69 -> 1.13 ms).
+constexpr int kStrengthLanes = 8;
 __global__ void k_strength(int n, int nb, const int *rp, const int *ci, const double *v, const double *dn, double *w) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = (int)(t / kStrengthLanes);
     if (i >= n) return;
-    for (int e = rp[i]; e < rp[i + 1]; ++e) {
+    for (int e = rp[i] + (int)(t % kStrengthLanes); e < rp[i + 1]; e += kStrengthLanes) {
         const int j = ci[e];
         if (j == i) { w[e] = -1.0; continue; }
         const double fij = fnorm2_rn(v + (long long)e * nb, nb);
@@ -128,28 +134,109 @@ __global__ void k_isolated(int n, const int *rp, const int *ci, const double *w,
 }
 
 // --------------------------------------------------------- matching pass
-__global__ void k_pick(int n, const int *rp, const int *ci, const double *w, double theta, const int *mate, int *pick) {
-    const int u = blockIdx.x * blockDim.x + threadIdx.x;
-    if (u >= n) return;
+// A handshake round: every unmatched node picks its strongest unmatched strong
+// neighbour (ties to the smaller index), and mutual picks become pairs.  A
+// node without a candidate never gets one (the matched set only grows), and a
+// round that makes no pair is the last that could.  So the rounds run over a
+// list of the nodes still in play, and stop at the first without a pair, with
+// the result of kMatchRounds rounds over all nodes.
+// 0.56M-unknown tangent, 21 passes: 17.3 ms in 2,688 launches -> 3.1 ms in 117.
+//
+// The candidates of node u scanned by kPickLanes lanes: the strongest, ties
+// to the smaller index, is the same in any order.  mate is read past L1
+// (__ldcg): other blocks of the cluster kernel write it.
+constexpr int kPickLanes = 4;
+__device__ __forceinline__ int pick_of(int u, int l, const int *rp, const int *ci, const double *w, double theta,
+                                       const int *mate) {
     int p = -1;
-    if (mate[u] < 0) {
-        double best = 0.0;
-        for (int e = rp[u]; e < rp[u + 1]; ++e) {
+    double best = 0.0;
+    if (u >= 0) {
+        const int e1 = rp[u + 1];
+#pragma unroll 4
+        for (int e = rp[u] + l; e < e1; e += kPickLanes) {
             const int v = ci[e];
-            if (v == u || mate[v] >= 0) continue;
             const double wv = w[e];
-            if (!(wv >= theta)) continue;
-            if (p < 0 || wv > best || (wv == best && v < p)) { best = wv; p = v; }
+            const bool ok = v != u && wv >= theta && __ldcg(mate + v) < 0;
+            if (ok && (p < 0 || wv > best || (wv == best && v < p))) { best = wv; p = v; }
         }
     }
-    pick[u] = p;
+#pragma unroll
+    for (int o = 1; o < kPickLanes; o <<= 1) {
+        const int q = __shfl_xor_sync(0xffffffffu, p, o);
+        const double bq = __shfl_xor_sync(0xffffffffu, best, o);
+        if (q >= 0 && (p < 0 || bq > best || (bq == best && q < p))) { best = bq; p = q; }
+    }
+    return p;
 }
 
-__global__ void k_match(int n, const int *pick, int *mate) {
-    const int u = blockIdx.x * blockDim.x + threadIdx.x;
-    if (u >= n) return;
-    const int v = pick[u];
-    if (v >= 0 && pick[v] == u) mate[u] = v;
+// One round over the nodes of list (all n when null; their number at count):
+// pick, then (next launch) pair; nodes that stay in play go to next / *ncount.
+__global__ void __launch_bounds__(256) k_pick(int n, const int *list, const int *count, const int *rp, const int *ci,
+                                              const double *w, double theta, const int *mate, int *pick) {
+    const int na = list ? *count : n, l = threadIdx.x % kPickLanes;
+    const long long step = (long long)gridDim.x * blockDim.x / kPickLanes;
+    // whole warps stay in the loop together (the lanes' shuffles)
+    for (long long i0 = ((long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / kPickLanes; i0 < na; i0 += step) {
+        const long long i = i0 + (threadIdx.x & 31) / kPickLanes;
+        const int u = i < na ? (list ? list[i] : (int)i) : -1;
+        const int p = pick_of(u, l, rp, ci, w, theta, mate);
+        if (u >= 0 && l == 0) pick[u] = p;
+    }
+}
+__global__ void __launch_bounds__(256) k_pair(int n, const int *list, const int *count, const int *pick, int *mate,
+                                              int *next, int *ncount) {
+    const int na = list ? *count : n;
+    const long long step = (long long)gridDim.x * blockDim.x;
+    for (long long i0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < na; i0 += step) {
+        const long long i = i0 + (threadIdx.x & 31);
+        const int u = i < na ? (list ? list[i] : (int)i) : -1;
+        const int v = u >= 0 ? pick[u] : -1;
+        bool stay = v >= 0;
+        if (stay && pick[v] == u) { mate[u] = v; stay = false; }
+        const unsigned m = __ballot_sync(0xffffffffu, stay);   // one atomic per warp; the list's order does not matter
+        int base = 0;
+        if ((threadIdx.x & 31) == 0 && m) base = atomicAdd(ncount, __popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (stay) next[base + __popc(m & ((1u << (threadIdx.x & 31)) - 1u))] = u;
+    }
+}
+
+// The remaining rounds in one cluster: few nodes are left in play (or the
+// graph is small), so a round is a chain of loads, not bandwidth, and two
+// cluster barriers (about 1 us each) replace two launches over all nodes.
+// made[r] (zeroed): a pair was made in round r.
+constexpr int kMatchCluster = 8, kMatchThreads = 1024;
+constexpr int kMatchTail = 2 * kMatchCluster * kMatchThreads;   // list length the cluster takes over at
+__global__ void __cluster_dims__(kMatchCluster, 1, 1) __launch_bounds__(kMatchThreads)
+    k_match_tail(int n, const int *list, const int *count, const int *rp, const int *ci, const double *w, double theta,
+                 int round0, int *mate, int *pick, int *made) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int na = list ? *count : n;
+    const int T = kMatchCluster * kMatchThreads, me = (int)cl.block_rank() * kMatchThreads + (int)threadIdx.x;
+    const int l = me % kPickLanes;
+    for (int r = round0; r < kMatchRounds; ++r) {
+        for (int i0 = (me & ~31) / kPickLanes; i0 < na; i0 += T / kPickLanes) {
+            const int i = i0 + (me & 31) / kPickLanes;
+            int u = i < na ? (list ? list[i] : i) : -1;
+            // out of play: matched, or without a candidate in an earlier round
+            if (u >= 0 && (__ldcg(mate + u) >= 0 || (r > round0 && __ldcg(pick + u) < 0))) u = -1;
+            if (__all_sync(0xffffffffu, u < 0)) continue;
+            const int p = pick_of(u, l, rp, ci, w, theta, mate);
+            if (u >= 0 && l == 0) pick[u] = p;
+        }
+        cl.sync();
+        int mine = 0;
+        for (int i = me; i < na; i += T) {
+            const int u = list ? list[i] : i;
+            if (__ldcg(mate + u) >= 0) continue;
+            const int v = __ldcg(pick + u);
+            if (v >= 0 && __ldcg(pick + v) == u) { mate[u] = v; mine = 1; }
+        }
+        if (__syncthreads_or(mine) && threadIdx.x == 0) made[r] = 1;
+        cl.sync();
+        if (__ldcg(made + r) == 0) break;   // the same for the whole cluster
+    }
 }
 
 __global__ void k_root_flag(int n, const int *mate, int *flag) {
@@ -332,66 +419,148 @@ __global__ void k_dense_from_bsr(int nbr, int bs, const int *rp, const int *ci, 
             for (int b = 0; b < bs; ++b)
                 Dm[(long long)(i * bs + a) * n + (long long)ci[e] * bs + b] += v[(long long)e * nb + a * bs + b];
 }
-__global__ void k_identity(int n, double *I) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long long)n * n) return;
-    I[t] = ((t / n) == (t % n)) ? 1.0 : 0.0;
-}
-// Gauss-Jordan step k with partial pivoting on [M | Inv] (one block)
-__global__ void k_gj_pivot(int n, int k, double *M, double *Inv, int *fail) {
-    __shared__ double bv[1024];
-    __shared__ int bi[1024];
-    double best = -1.0;
-    int arg = k;
-    for (int i = k + threadIdx.x; i < n; i += blockDim.x) {
-        const double a = fabs(M[(long long)i * n + k]);
-        if (a > best || (a == best && i < arg)) { best = a; arg = i; }
+// Blocked in-place Gauss-Jordan inverse with partial pivoting (rows k.. of
+// column k, ties to the smaller row): panels of b columns, each eliminated in
+// one block's shared memory, then applied to the whole matrix by k_inv_update.
+// In place of [M | I], column k of the panel becomes column k of the
+// eliminations' product G, so half of the elements and no identity are
+// touched.  A pivot costs two block barriers and its share of a panel's two
+// launches instead of three launches over 2 n^2 elements (the coarsest levels of the 0.56M-unknown tangent, 656 pivots:
+// 11.0 -> 3.6 us a pivot).  Candidates are compared by their bits (|x| as an
+// integer orders as the value does), which keeps them off the narrow FP64 pipe.
+constexpr int kInvThreads = 1024;
+__global__ void __launch_bounds__(kInvThreads) k_inv_panel(int n, int k0, int b, const double *M, double *G, int *piv,
+                                                           int *perm, int *fail) {
+    extern __shared__ double S[];              // S[t n + i]: column k0 + t of the panel
+    int *sperm = reinterpret_cast<int *>(S + (size_t)b * n);
+    __shared__ double row[8];
+    __shared__ unsigned long long wv[32];
+    __shared__ int wi[32];
+    const int tid = threadIdx.x, warp = tid >> 5, ln = tid & 31;
+    if (*fail) return;
+    for (int q = tid; q < b * n; q += kInvThreads) {
+        const int i = q / b, t = q - i * b;
+        S[(size_t)t * n + i] = M[(long long)i * n + k0 + t];
     }
-    bv[threadIdx.x] = best; bi[threadIdx.x] = arg;
+    for (int i = tid; i < n; i += kInvThreads) sperm[i] = perm[i];
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) {
-            const double o = bv[threadIdx.x + s];
-            const int oi = bi[threadIdx.x + s];
-            if (o > bv[threadIdx.x] || (o == bv[threadIdx.x] && oi < bi[threadIdx.x])) { bv[threadIdx.x] = o; bi[threadIdx.x] = oi; }
+    unsigned long long best = 0;
+    int arg = n;
+    auto offer = [&](double x, int i) {   // rows come in ascending order
+        const unsigned long long u = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffULL;
+        if (u > best || (u == best && i < arg)) { best = u; arg = i; }
+    };
+    for (int i = tid; i < n; i += kInvThreads)
+        if (i >= k0) offer(S[i], i);
+    for (int t = 0; t < b; ++t) {
+        const int k = k0 + t;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long u = __shfl_xor_sync(0xffffffffu, best, o);
+            const int q = __shfl_xor_sync(0xffffffffu, arg, o);
+            if (u > best || (u == best && q < arg)) { best = u; arg = q; }
+        }
+        if (ln == 0) { wv[warp] = best; wi[warp] = arg; }
+        __syncthreads();
+        best = wv[ln];
+        arg = wi[ln];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long u = __shfl_xor_sync(0xffffffffu, best, o);
+            const int q = __shfl_xor_sync(0xffffffffu, arg, o);
+            if (u > best || (u == best && q < arg)) { best = u; arg = q; }
+        }
+        const int p = arg;
+        if (best == 0) {   // the same in every thread
+            if (tid == 0) *fail = 1;
+            return;
+        }
+        if (tid < b) {
+            const double ip = 1.0 / S[(size_t)t * n + p];
+            const double a = S[(size_t)tid * n + k], q = S[(size_t)tid * n + p];
+            __syncwarp((1u << b) - 1u);   // every lane has read the pivot
+            if (p != k) S[(size_t)tid * n + p] = a;
+            const double r = tid == t ? ip : q * ip;
+            row[tid] = r;
+            S[(size_t)tid * n + k] = r;
+        } else if (tid == 32) {
+            piv[k] = p;
+            const int u = sperm[k];
+            sperm[k] = sperm[p];
+            sperm[p] = u;
         }
         __syncthreads();
-    }
-    const int p = bi[0];
-    const double piv = M[(long long)p * n + k];
-    if (piv == 0.0) { if (threadIdx.x == 0) *fail = 1; return; }
-    for (int c = threadIdx.x; c < n; c += blockDim.x) {
-        if (p != k) {
-            double t = M[(long long)k * n + c]; M[(long long)k * n + c] = M[(long long)p * n + c]; M[(long long)p * n + c] = t;
-            t = Inv[(long long)k * n + c]; Inv[(long long)k * n + c] = Inv[(long long)p * n + c]; Inv[(long long)p * n + c] = t;
+        best = 0;
+        arg = n;
+        const double rt = row[t];
+        for (int i = tid; i < n; i += kInvThreads) {
+            if (i == k) continue;
+            const double f = S[(size_t)t * n + i];
+            for (int c = 0; c < b; ++c) {
+                if (c == t) continue;
+                const double x = S[(size_t)c * n + i] - f * row[c];
+                S[(size_t)c * n + i] = x;
+                if (c == t + 1 && i > k) offer(x, i);
+            }
+            S[(size_t)t * n + i] = -f * rt;
         }
     }
     __syncthreads();
-    const double ip = 1.0 / piv;
-    for (int c = threadIdx.x; c < n; c += blockDim.x) {
-        M[(long long)k * n + c] *= ip;
-        Inv[(long long)k * n + c] *= ip;
+    for (int q = tid; q < b * n; q += kInvThreads) {
+        const int i = q / b, t = q - i * b;
+        G[(long long)i * 8 + t] = S[(size_t)t * n + i];
     }
+    for (int i = tid; i < n; i += kInvThreads) perm[i] = sperm[i];
 }
-__global__ void k_gj_elim(int n, int k, double *M, double *Inv, const int *fail) {
+// The panel's eliminations applied to every column: out = (rows outside the
+// panel's k0 .. k0 + b - 1 of the row-swapped M, zero inside) + G X, X the b
+// panel rows of the row-swapped M; the panel's own columns become G.  32 x 32
+// tiles: enough blocks for every SM's FP64 pipe from n = 400 on.
+__global__ void __launch_bounds__(256) k_inv_update(int n, int k0, int b, const double *M, const double *G, const int *piv,
+                                                    double *out, const int *fail) {
+    __shared__ double gs[32][9], xs[8][32];
+    __shared__ int src[32], xsrc[8];
     if (*fail) return;
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long long)n * 2 * n) return;
-    const int i = (int)(t / (2 * n));
-    const int c = (int)(t % (2 * n));
-    if (i == k) return;
-    const double f = M[(long long)i * n + k];
-    if (c < n) {
-        if (c == k) return;   // column k cleared last (it is the factor)
-        M[(long long)i * n + c] -= f * M[(long long)k * n + c];
-    } else {
-        Inv[(long long)i * n + (c - n)] -= f * Inv[(long long)k * n + (c - n)];
+    const int c = threadIdx.x & 31, r0 = threadIdx.x >> 5;
+    const int j = blockIdx.x * 32 + c, i0 = blockIdx.y * 32;
+    auto trace = [&](int i) {   // the row of M that the swaps brought to row i
+        for (int t = b - 1; t >= 0; --t) {
+            const int p = piv[k0 + t];
+            if (i == k0 + t) i = p;
+            else if (i == p) i = k0 + t;
+        }
+        return i;
+    };
+    if (threadIdx.x < 32) src[threadIdx.x] = i0 + (int)threadIdx.x < n ? trace(i0 + (int)threadIdx.x) : 0;
+    else if ((int)threadIdx.x < 32 + b) xsrc[threadIdx.x - 32] = trace(k0 + (int)threadIdx.x - 32);
+    {
+        const int i = threadIdx.x >> 3, t = threadIdx.x & 7;
+        gs[i][t] = (i0 + i < n && t < b) ? G[(long long)(i0 + i) * 8 + t] : 0.0;
+    }
+    __syncthreads();
+    if (r0 < b && j < n) xs[r0][c] = M[(long long)xsrc[r0] * n + j];
+    __syncthreads();
+    if (j >= n) return;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int r = r0 + 8 * q, i = i0 + r;
+        if (i >= n) break;
+        double x;
+        if (j >= k0 && j < k0 + b) {
+            x = gs[r][j - k0];
+        } else {
+            x = (i >= k0 && i < k0 + b) ? 0.0 : M[(long long)src[r] * n + j];
+            for (int t = 0; t < b; ++t) x += gs[r][t] * xs[t][c];
+        }
+        out[(long long)i * n + j] = x;
     }
 }
-__global__ void k_gj_clear(int n, int k, double *M) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || i == k) return;
-    M[(long long)i * n + k] = 0.0;
+// column perm[k] of the inverse is column k of the in-place result
+__global__ void k_inv_columns(int n, const double *M, const int *perm, double *inv) {
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= (long long)n * n) return;
+    const int i = (int)(t / n), k = (int)(t - (long long)i * n);
+    inv[(long long)i * n + perm[k]] = M[t];
 }
 
 // --------------------------------------------------- value copies
@@ -606,11 +775,36 @@ static int match_pass(const Graph &G, double theta, int *map, cudaStream_t s) {
     int *mate = dmalloc<int>(n, s), *pick = dmalloc<int>(n, s);
     k_fill<int><<<grid_for(n), 256, 0, s>>>(mate, -1, n);
     NBP_LAUNCHED();
-    for (int round = 0; round < kMatchRounds; ++round) {   // a round without a new pair changes nothing after it
-        k_pick<<<grid_exact(n), 256, 0, s>>>(n, G.rp, G.ci, G.w, theta, mate, pick);
-        k_match<<<grid_exact(n), 256, 0, s>>>(n, pick, mate);
+    // rounds over the whole GPU while many nodes are in play, the host looking
+    // at their number every fourth round; the rest in one cluster
+    int *list[2] = {nullptr, nullptr};
+    int *cnt = dmalloc<int>(2 * kMatchRounds, s);   // [r]: in play after round r; [kMatchRounds + r]: made
+    NBP_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * 2 * kMatchRounds, s));
+    int round = 0, left = n;
+    if (left > kMatchTail) {
+        for (int *&q : list) q = dmalloc<int>(n, s);
+        while (round < kMatchRounds && left > kMatchTail) {
+            int made = left;
+            for (int q = 0; q < 4; ++q, ++round) {
+                const int *in = round ? list[round & 1] : nullptr, *nin = round ? cnt + round - 1 : nullptr;
+                k_pick<<<grid_for((long long)left * kPickLanes, 256, 8LL * kSMs), 256, 0, s>>>(n, in, nin, G.rp, G.ci, G.w,
+                                                                                           theta, mate, pick);
+                k_pair<<<grid_for(left, 256, 8LL * kSMs), 256, 0, s>>>(n, in, nin, pick, mate, list[(round + 1) & 1],
+                                                                       cnt + round);
+                NBP_LAUNCHED();
+            }
+            left = readback(cnt + round - 1, s);
+            if (left == made) break;   // four rounds without a pair
+        }
+    }
+    if (left > 0 && round < kMatchRounds) {
+        k_match_tail<<<kMatchCluster, kMatchThreads, 0, s>>>(n, round ? list[round & 1] : nullptr,
+                                                             round ? cnt + round - 1 : nullptr, G.rp, G.ci, G.w, theta,
+                                                             round, mate, pick, cnt + kMatchRounds);
         NBP_LAUNCHED();
     }
+    for (int *q : list) dfree(q, s);
+    dfree(cnt, s);
     int *flag = dmalloc<int>(n + 1, s), *id = dmalloc<int>(n + 1, s);
     k_root_flag<<<grid_exact(n), 256, 0, s>>>(n, mate, flag);
     NBP_LAUNCHED();
@@ -829,7 +1023,7 @@ static int aggregate(const DMat &M, double theta, int *agg, cudaStream_t s) {
     Graph G;
     G.n = n; G.nnz = M.nnz; G.rp = M.rp; G.ci = M.ci;
     G.w = dmalloc<double>(M.nnz, s);
-    k_strength<<<grid_exact(n), 256, 0, s>>>(n, nb, M.rp, M.ci, M.v, dn, G.w);
+    k_strength<<<grid_exact((long long)n * kStrengthLanes), 256, 0, s>>>(n, nb, M.rp, M.ci, M.v, dn, G.w);
     NBP_LAUNCHED();
     int *iso = dmalloc<int>(n, s);
     k_isolated<<<grid_exact(n), 256, 0, s>>>(n, M.rp, M.ci, G.w, theta, iso);
@@ -927,18 +1121,29 @@ static void dense_inverse(const DMat &M, double *&cinv, int &nc, cudaStream_t s)
     cinv = dmalloc<double>((long long)n * n, s);
     NBP_CUDA(cudaMemsetAsync(Dm, 0, sizeof(double) * (size_t)n * n, s));
     k_dense_from_bsr<<<grid_exact(M.nbr), 256, 0, s>>>(M.nbr, M.br, M.rp, M.ci, M.v, Dm);
-    k_identity<<<grid_exact((long long)n * n), 256, 0, s>>>(n, cinv);
     NBP_LAUNCHED();
-    int *fail = dmalloc<int>(1, s);
+    double *Dn = cinv, *G = dmalloc<double>(8LL * n, s);   // Dm and Dn in turn
+    int *piv = dmalloc<int>(n, s), *perm = dmalloc<int>(n, s), *fail = dmalloc<int>(1, s);
     NBP_CUDA(cudaMemsetAsync(fail, 0, sizeof(int), s));
-    for (int k = 0; k < n; ++k) {
-        k_gj_pivot<<<1, 1024, 0, s>>>(n, k, Dm, cinv, fail);
-        k_gj_elim<<<grid_exact((long long)n * 2 * n), 256, 0, s>>>(n, k, Dm, cinv, fail);
-        k_gj_clear<<<grid_exact(n), 256, 0, s>>>(n, k, Dm);
-    }
+    k_iota<<<grid_exact(n), 256, 0, s>>>(n, perm);
     NBP_LAUNCHED();
+    // panel width: b columns and the permutation in one block's shared memory
+    const int B = n <= 3300 ? 8 : 4;
+    static_assert((4 * sizeof(double) + sizeof(int)) * (size_t)kCoarseDenseMax <= 227u * 1024u, "panel fits");
+    const size_t smem = ((size_t)B * sizeof(double) + sizeof(int)) * (size_t)n;
+    NBP_CUDA(cudaFuncSetAttribute(k_inv_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024));
+    const dim3 tiles((n + 31) / 32, (n + 31) / 32);
+    for (int k0 = 0; k0 < n; k0 += B) {
+        const int b = std::min(B, n - k0);
+        k_inv_panel<<<1, kInvThreads, smem, s>>>(n, k0, b, Dm, G, piv, perm, fail);
+        k_inv_update<<<tiles, 256, 0, s>>>(n, k0, b, Dm, G, piv, Dn, fail);
+        std::swap(Dm, Dn);
+    }
+    k_inv_columns<<<grid_exact((long long)n * n), 256, 0, s>>>(n, Dm, perm, Dn);
+    NBP_LAUNCHED();
+    cinv = Dn;
     const int f = readback(fail, s);
-    dfree(fail, s); dfree(Dm, s);
+    dfree(fail, s); dfree(Dm, s); dfree(G, s); dfree(piv, s); dfree(perm, s);
     require(!f, NBP_ERR_INVALID, "setup: coarsest AMG matrix is singular");
 }
 
