@@ -39,7 +39,14 @@ struct SpmvArgs {
     int nslice;                       // sliced-ELL layout (k_sell): slices of C rows
     const long long *sl_ptr;
     const int *sl_ci;
+    bool d_read, d_write;             // EPI_CHEB: d is read (c1 != 0) / written (a later step reads it)
+    // device-driven loops: x, b and xout are column *jp of a basis where their
+    // column stride is set (0: the pointer itself)
+    const int *jp;
+    long long x_ld, b_ld, out_ld;
 };
+// a vector of the product, its basis column taken on the device
+__device__ __forceinline__ long long col_off(const SpmvArgs &a, long long ld) { return ld ? (long long)*a.jp * ld : 0; }
 
 template <int BR, int BC, int G, typename VT, typename XT, int EPI, bool LR>
 __global__ void __launch_bounds__(256) k_bspmv(SpmvArgs a) {
@@ -55,7 +62,7 @@ __global__ void __launch_bounds__(256) k_bspmv(SpmvArgs a) {
     const int cnt = (__ldg(a.rp + row + 1) - e0) * BB;
     const VT *__restrict__ val = (const VT *)a.val + (long long)e0 * BB;
     const int *__restrict__ ci = a.ci + e0;
-    const XT *__restrict__ x = (const XT *)a.x;
+    const XT *__restrict__ x = (const XT *)a.x + col_off(a, a.x_ld);
     AT acc0 = 0, acc1 = 0, acc2 = 0;
 #pragma unroll 4
     for (int v = lane; v < cnt; v += G) {
@@ -99,9 +106,9 @@ __global__ void __launch_bounds__(256) k_bspmv(SpmvArgs a) {
     } else if (EPI == EPI_SUB) {
         y[idx] -= s;
     } else if (EPI == EPI_RES) {
-        y[idx] = ((const XT *)a.b)[idx] - s;
+        y[idx] = ((const XT *)a.b + col_off(a, a.b_ld))[idx] - s;
     } else {   // EPI_CHEB, BR == BC
-        const XT *b = (const XT *)a.b;
+        const XT *b = (const XT *)a.b + col_off(a, a.b_ld);
         const XT *dinv = (const XT *)a.dinv + (long long)row * BR * BR + lane * BR;
         AT t;
         if (BR == 1) {
@@ -114,9 +121,9 @@ __global__ void __launch_bounds__(256) k_bspmv(SpmvArgs a) {
         }
         XT *d = (XT *)a.d;
         const AT c1 = sizeof(AT) == 4 ? (AT)a.c1f : (AT)a.c1, c2 = sizeof(AT) == 4 ? (AT)a.c2f : (AT)a.c2;
-        const AT dn = c1 * d[idx] + c2 * t;
-        d[idx] = dn;
-        ((XT *)a.xout)[idx] = x[idx] + dn;
+        const AT dn = (a.d_read ? c1 * d[idx] : AT(0)) + c2 * t;
+        if (a.d_write) d[idx] = dn;
+        ((XT *)a.xout + col_off(a, a.out_ld))[idx] = x[idx] + dn;
     }
 }
 
@@ -265,7 +272,7 @@ __global__ void __launch_bounds__(256) k_sell(SpmvArgs a) {
     const int w = (int)((a.sl_ptr[sl + 1] - base) / C);
     const VT *__restrict__ val = (const VT *)a.val;
     const int *__restrict__ ci = a.sl_ci;
-    const XT *__restrict__ x = (const XT *)a.x;
+    const XT *__restrict__ x = (const XT *)a.x + col_off(a, a.x_ld);
     AT acc0 = 0, acc1 = 0, acc2 = 0;
     if constexpr (std::is_same<VT, __nv_bfloat16>::value) {   // paired layout: w / 2 pairs, then one slot if w is odd
         sell_pairs<BS, C>(a, base / 2, w / 2, t, 0, 1, x, acc0, acc1, acc2);
@@ -292,10 +299,10 @@ __global__ void __launch_bounds__(256) k_sell(SpmvArgs a) {
     const bool lr = LR && EPI == EPI_SET;
     const int lr0 = lr ? a.lr_rp[row] : 0, lr1 = lr ? a.lr_rp[row + 1] : 0;
     if (EPI == EPI_CHEB) {
-        const XT *b = (const XT *)a.b;
+        const XT *b = (const XT *)a.b + col_off(a, a.b_ld);
         const XT *dinv = (const XT *)a.dinv + (long long)row * BB;
         XT *d = (XT *)a.d;
-        XT *xo = (XT *)a.xout;
+        XT *xo = (XT *)a.xout + col_off(a, a.out_ld);
         const AT c1 = sizeof(AT) == 4 ? (AT)a.c1f : (AT)a.c1, c2 = sizeof(AT) == 4 ? (AT)a.c2f : (AT)a.c2;
         AT r[3];
 #pragma unroll
@@ -306,8 +313,8 @@ __global__ void __launch_bounds__(256) k_sell(SpmvArgs a) {
 #pragma unroll
             for (int c = 0; c < BS; ++c) tq += dinv[q * BS + c] * r[c];
             const long long idx = (long long)row * BS + q;
-            const AT dn = c1 * d[idx] + c2 * tq;
-            d[idx] = dn;
+            const AT dn = (a.d_read ? c1 * d[idx] : AT(0)) + c2 * tq;
+            if (a.d_write) d[idx] = dn;
             xo[idx] = x[idx] + dn;
         }
         return;
@@ -332,7 +339,7 @@ __global__ void __launch_bounds__(256) k_sell(SpmvArgs a) {
         } else if (EPI == EPI_SUB) {
             y[idx] -= s;
         } else {
-            y[idx] = ((const XT *)a.b)[idx] - s;
+            y[idx] = ((const XT *)a.b + col_off(a, a.b_ld))[idx] - s;
         }
     }
 }
@@ -352,7 +359,7 @@ __global__ void __launch_bounds__(256) k_sellr(SpmvArgs a) {
     const int w = (int)((a.sl_ptr[sl + 1] - base) / C);
     const VT *__restrict__ val = (const VT *)a.val;
     const int *__restrict__ ci = a.sl_ci;
-    const XT *__restrict__ x = (const XT *)a.x;
+    const XT *__restrict__ x = (const XT *)a.x + col_off(a, a.x_ld);
     AT acc[BR];
 #pragma unroll
     for (int r = 0; r < BR; ++r) acc[r] = 0;
@@ -405,14 +412,14 @@ __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
     AT eb[3] = {0, 0, 0}, ed[3] = {0, 0, 0}, ex[3] = {0, 0, 0}, edi[BB];
     if (own && (EPI == EPI_RES || EPI == EPI_CHEB)) {
 #pragma unroll
-        for (int q = 0; q < BS; ++q) eb[q] = ((const XT *)a.b)[(long long)row * BS + q];
+        for (int q = 0; q < BS; ++q) eb[q] = ((const XT *)a.b + col_off(a, a.b_ld))[(long long)row * BS + q];
     }
     if (own && EPI == EPI_CHEB) {
         const XT *dv = (const XT *)a.dinv + (long long)row * BB;
 #pragma unroll
         for (int q = 0; q < BS; ++q) {
-            ed[q] = ((const XT *)a.d)[(long long)row * BS + q];
-            ex[q] = ((const XT *)a.x)[(long long)row * BS + q];
+            if (a.d_read) ed[q] = ((const XT *)a.d)[(long long)row * BS + q];
+            ex[q] = ((const XT *)a.x + col_off(a, a.x_ld))[(long long)row * BS + q];
         }
 #pragma unroll
         for (int q = 0; q < BB; ++q) edi[q] = dv[q];
@@ -421,7 +428,7 @@ __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
     const int w = live ? (int)((a.sl_ptr[sl + 1] - base) / C) : 0;
     const VT *__restrict__ val = (const VT *)a.val;
     const int *__restrict__ ci = a.sl_ci;
-    const XT *__restrict__ x = (const XT *)a.x;
+    const XT *__restrict__ x = (const XT *)a.x + col_off(a, a.x_ld);
     AT acc0 = 0, acc1 = 0, acc2 = 0;
     if constexpr (std::is_same<VT, __nv_bfloat16>::value) {   // paired layout: the T threads take alternate pairs
         sell_pairs<BS, C>(a, base / 2, w / 2, t, h, T, x, acc0, acc1, acc2);
@@ -455,7 +462,7 @@ __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
     XT *y = (XT *)a.y;
     if (EPI == EPI_CHEB) {
         XT *d = (XT *)a.d;
-        XT *xo = (XT *)a.xout;
+        XT *xo = (XT *)a.xout + col_off(a, a.out_ld);
         const AT c1 = sizeof(AT) == 4 ? (AT)a.c1f : (AT)a.c1, c2 = sizeof(AT) == 4 ? (AT)a.c2f : (AT)a.c2;
         AT r[3];
 #pragma unroll
@@ -466,8 +473,8 @@ __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
 #pragma unroll
             for (int c = 0; c < BS; ++c) tq += edi[q * BS + c] * r[c];
             const long long idx = (long long)row * BS + q;
-            const AT dn = c1 * ed[q] + c2 * tq;
-            d[idx] = dn;
+            const AT dn = (a.d_read ? c1 * ed[q] : AT(0)) + c2 * tq;
+            if (a.d_write) d[idx] = dn;
             xo[idx] = ex[q] + dn;
         }
         return;
@@ -556,21 +563,38 @@ __device__ __forceinline__ void block_reduce_partials(const double *partial, int
     }
 }
 
-// out[col] = sum_b of the float-float partials of column col: warp w takes
-// columns w, w + 8, ...; lane l adds partials b = l, l + 32, ... in ascending
-// order, then a fixed warp tree (one order whatever the scheduling).
+// out[col] = sum_b of the float-float partials of column col.  With 8, 4, 2
+// or 1 warps per column (few columns leave warps over), warp part p of a
+// column adds partials b = lane + 32 p, ... in ascending order, eight loads in
+// flight, then a fixed warp tree and the parts in order (one order whatever
+// the scheduling).  All threads of a 256-thread block.
 __device__ __forceinline__ void block_reduce_partials_ff(const double *partial, int nb, int ncols, double *out) {
-    const int warp = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int col = warp; col < ncols; col += nw) {
+    __shared__ FF red[8];
+    const int warp = threadIdx.x >> 5, ln = threadIdx.x & 31;
+    const int wpc = ncols <= 1 ? 8 : ncols <= 2 ? 4 : ncols <= 4 ? 2 : 1, step = 32 * wpc;
+    for (int col = warp / wpc; col < ncols; col += 8 / wpc) {
         const float2 *p = reinterpret_cast<const float2 *>(partial + (long long)col * nb);
         FF a{0.f, 0.f};
-#pragma unroll 4
-        for (int b = ln; b < nb; b += 32) {
-            const float2 v = __ldcg(p + b);
-            a = ff_add(a, FF{v.x, v.y});
+        for (int b0 = ln + 32 * (warp % wpc); b0 < nb; b0 += 8 * step) {
+            float2 v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = b0 + u * step < nb ? __ldcg(p + b0 + u * step) : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) a = ff_add(a, FF{v[u].x, v[u].y});
         }
         a = ff_warp_sum(a);
-        if (ln == 0) out[col] = ff_to_double(a);
+        if (ln == 0) {
+            if (wpc == 1) out[col] = ff_to_double(a);
+            else red[warp] = a;
+        }
+    }
+    if (wpc > 1) {   // uniform over the block; one column per group of warps then
+        __syncthreads();
+        if ((int)threadIdx.x < ncols) {
+            FF u = red[threadIdx.x * wpc];
+            for (int q = 1; q < wpc; ++q) u = ff_add(u, red[threadIdx.x * wpc + q]);
+            out[threadIdx.x] = ff_to_double(u);
+        }
     }
 }
 // the last block's reduction of a T kernel's partials
@@ -579,20 +603,59 @@ template <typename T> __device__ __forceinline__ void reduce_partials(const doub
     else block_reduce_partials(partial, nb, ncols, out);
 }
 
+// Warp sums of NQ values (a power of two up to 16) at once by folding: in
+// each of the first log2 NQ xor steps a lane keeps half of its values and
+// sends the other half, so NQ - 1 adds replace the NQ per step of NQ separate
+// trees (8 values: 9 adds a lane instead of 40).  On return every lane of
+// group g = lane / (32 / NQ) holds the sum of value g.
+template <typename V, int NQ, typename Add, typename Xor>
+__device__ __forceinline__ V fold_warp(V (&v)[NQ], int ln, Add add, Xor xr) {
+    int o = 16;
+#pragma unroll
+    for (int h = NQ / 2; h > 0; h >>= 1, o >>= 1) {
+        const bool up = (ln & o) != 0;
+#pragma unroll
+        for (int q = 0; q < h; ++q) {
+            const V keep = up ? v[q + h] : v[q], send = up ? v[q] : v[q + h];
+            v[q] = add(keep, xr(send, o));
+        }
+    }
+    V r = v[0];
+    for (; o > 0; o >>= 1) r = add(r, xr(r, o));
+    return r;
+}
+
 // Block stage of the grid reductions: for q < nq, the sum of acc[q] over the
 // block's threads into partial[(col0 + q) * gridDim.x + blockIdx.x].  FP64
 // kernels: FP64 warp trees, then the warps' sums in order; FP32 kernels: the
-// same in float-float (the partial stored as a float2).  256 threads.
+// same in float-float (the partial stored as a float2).  256 threads; columns
+// in folded groups of up to 8 (fold_warp).
 template <typename T, int NQ>
 __device__ __forceinline__ void block_partials(const T (&acc)[NQ], int nq, double *partial, int col0) {
     const int warp = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
+    constexpr int F = NQ < 8 ? NQ : 8;   // values folded together
+    static_assert(NQ % F == 0 && (F & (F - 1)) == 0, "fold size");
+    const int q_of = ln / (32 / F);      // fold_warp's value of this lane (its bits, top first)
+    const bool lead = ln % (32 / F) == 0;
     if constexpr (std::is_same<T, float>::value) {
         __shared__ FF redf[NQ][8];
+        auto add = [](FF a, FF b) { return ff_add(a, b); };
+        auto xr = [](FF a, int o) {
+            return FF{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+        };
 #pragma unroll
-        for (int q = 0; q < NQ; ++q)
-            if (q < nq) {   // uniform over the block
-                const FF v = ff_warp_sum(FF{acc[q], 0.f});
-                if (ln == 0) redf[q][warp] = v;
+        for (int q0 = 0; q0 < NQ; q0 += F)
+            if (q0 < nq) {   // uniform over the block
+                if (nq - q0 == 1) {   // one column left: a plain warp sum
+                    const FF v = ff_warp_sum(FF{acc[q0], 0.f});
+                    if (ln == 0) redf[q0][warp] = v;
+                } else {
+                    FF v[F];
+#pragma unroll
+                    for (int q = 0; q < F; ++q) v[q] = FF{acc[q0 + q], 0.f};
+                    const FF r = fold_warp<FF, F>(v, ln, add, xr);
+                    if (lead) redf[q0 + q_of][warp] = r;
+                }
             }
         __syncthreads();
         if ((int)threadIdx.x < nq) {
@@ -603,11 +666,21 @@ __device__ __forceinline__ void block_partials(const T (&acc)[NQ], int nq, doubl
         }
     } else {
         __shared__ double redd[NQ][8];
+        auto add = [](double a, double b) { return a + b; };
+        auto xr = [](double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); };
 #pragma unroll
-        for (int q = 0; q < NQ; ++q)
-            if (q < nq) {
-                const double v = warp_sum((double)acc[q]);
-                if (ln == 0) redd[q][warp] = v;
+        for (int q0 = 0; q0 < NQ; q0 += F)
+            if (q0 < nq) {
+                if (nq - q0 == 1) {
+                    const double v = warp_sum((double)acc[q0]);
+                    if (ln == 0) redd[q0][warp] = v;
+                } else {
+                    double v[F];
+#pragma unroll
+                    for (int q = 0; q < F; ++q) v[q] = (double)acc[q0 + q];
+                    const double r = fold_warp<double, F>(v, ln, add, xr);
+                    if (lead) redd[q0 + q_of][warp] = r;
+                }
             }
         __syncthreads();
         if ((int)threadIdx.x < nq) {
@@ -680,8 +753,26 @@ __global__ void __launch_bounds__(256) k_sell_dot(SpmvArgs a, DotArgs q) {
 struct GmState {
     double res;      // |g_{j+1}|
     double beta;     // h_{j+1,j}
+    double inv;      // 1 / beta (0 where beta is 0): the next basis vector is w inv
+    float invf;      // the same, rounded
     int nan;         // NaN/Inf met
-    int pad;
+};
+__device__ __forceinline__ void gm_set_beta(GmState *st, double beta) {
+    const double inv = beta == 0.0 ? 0.0 : 1.0 / beta;
+    st->beta = beta;
+    st->inv = inv;
+    st->invf = (float)inv;
+}
+template <typename T> __device__ __forceinline__ T gm_inv(const GmState *st) {
+    if constexpr (std::is_same<T, float>::value) return st->invf;
+    else return st->inv;
+}
+
+// Loop state of one device-driven GMRES level (graph WHILE nodes).
+struct GmDev {
+    int j, its, m, nmax;        // column of the current cycle, iterations, restart length, iteration limit
+    int conv, nan, pad0, pad1;  // pad0: restart cycles run (outer level)
+    double tol, bnorm, res, rel_true;
 };
 
 // What the fused Givens update of Hessenberg column j needs (H == nullptr:
@@ -689,41 +780,111 @@ struct GmState {
 struct GivensArgs {
     double *H = nullptr;
     int ldh = 0, j = 0;
-    const int *jp = nullptr;   // when set, the column index is read here (device-driven loops)
     const double *h1 = nullptr, *h2 = nullptr;
     double *cs = nullptr, *sn = nullptr, *g = nullptr;
     GmState *st = nullptr;
+    // device-driven loops: the column index is dl->j, and the update also ends
+    // the iteration (givens_step): it advances dl and sets the WHILE condition
+    GmDev *dl = nullptr;
+    cudaGraphConditionalHandle h = 0;
 };
+
+// Operands of the Givens update staged in shared memory by the block that
+// applies it (before it reduces the norm's partials, so that these loads and
+// the partials' are in flight together): as a chain of dependent global loads
+// in one thread they cost most of the norm pass's tail.  Bases longer than
+// kGivensCols read global memory instead.
+constexpr int kGivensCols = 64;
+struct GivensBuf {
+    double h[kGivensCols], cs[kGivensCols], sn[kGivensCols];
+    double g;
+    GmDev dl;
+    int j;
+};
+__device__ __forceinline__ void givens_stage(const GivensArgs &q, GivensBuf &B) {
+    const int j = q.dl ? q.dl->j : q.j;
+    if (threadIdx.x == 0) {
+        B.j = j;
+        B.g = q.g[j];
+        if (q.dl) B.dl = *q.dl;
+    }
+    if (j < kGivensCols)
+        for (int i = threadIdx.x; i <= j; i += blockDim.x) {
+            B.h[i] = q.h2 ? q.h1[i] + q.h2[i] : q.h1[i];
+            if (i < j) { B.cs[i] = q.cs[i]; B.sn[i] = q.sn[i]; }
+        }
+}
 
 // Column j of the Hessenberg matrix: H(i,j) = h1_i + h2_i (i <= j; h1_i
 // alone when h2 is null, a single Gram-Schmidt pass),
 // H(j+1,j) = ||w|| (from ||w||^2 = nrm2); the previous rotations applied, a
 // new rotation chosen to zero H(j+1,j), and the right-hand side g rotated
-// (Saad 1993, FGMRES with Givens rotations).  One thread.
-__device__ __forceinline__ void givens_step(const GivensArgs &q, double nrm2) {
+// (Saad 1993, FGMRES with Givens rotations).  In a device-driven loop then
+// the end of the iteration: the stopping rule of the host-driven loop --
+// continue while |g_{j+1}| > max(rtol ||b||, atol), h_{j+1,j} != 0, no NaN,
+// j < m and its < n_max -- as the WHILE node's condition (every block has
+// read j before it took its ticket, so dl may advance here).  One thread.
+__device__ __forceinline__ void givens_step(const GivensArgs &q, const GivensBuf &B, double nrm2) {
     double *H = q.H;
     const long long ldh = q.ldh;
-    const int j = q.jp ? *q.jp : q.j;
-    for (int i = 0; i <= j; ++i) H[i * ldh + j] = q.h2 ? q.h1[i] + q.h2[i] : q.h1[i];
+    const int j = B.j;
     const double beta = (nrm2 >= 0.0) ? sqrt(nrm2) : nrm2;   // NaN passes through
-    H[(j + 1) * ldh + j] = beta;
-    for (int i = 0; i < j; ++i) {
-        const double a = H[i * ldh + j], b = H[(i + 1) * ldh + j];
-        H[i * ldh + j] = q.cs[i] * a + q.sn[i] * b;
-        H[(i + 1) * ldh + j] = -q.sn[i] * a + q.cs[i] * b;
+    double a;   // H(j, j) after the previous rotations
+    if (j < kGivensCols) {
+        a = B.h[0];
+        for (int i = 0; i < j; ++i) {
+            const double b = B.h[i + 1], c = B.cs[i], s = B.sn[i];
+            H[i * ldh + j] = c * a + s * b;
+            a = -s * a + c * b;
+        }
+    } else {
+        for (int i = 0; i <= j; ++i) H[i * ldh + j] = q.h2 ? q.h1[i] + q.h2[i] : q.h1[i];
+        for (int i = 0; i < j; ++i) {
+            const double u = H[i * ldh + j], b = H[(i + 1) * ldh + j];
+            H[i * ldh + j] = q.cs[i] * u + q.sn[i] * b;
+            H[(i + 1) * ldh + j] = -q.sn[i] * u + q.cs[i] * b;
+        }
+        a = H[j * ldh + j];
     }
-    const double a = H[j * ldh + j], b = H[(j + 1) * ldh + j];
-    const double den = hypot(a, b);
-    if (den == 0.0) { q.cs[j] = 1.0; q.sn[j] = 0.0; }
-    else { q.cs[j] = a / den; q.sn[j] = b / den; }
+    const double den = hypot(a, beta);
+    double c = 1.0, s = 0.0;
+    if (den != 0.0) { c = a / den; s = beta / den; }
+    q.cs[j] = c;
+    q.sn[j] = s;
     H[j * ldh + j] = den;
     H[(j + 1) * ldh + j] = 0.0;
-    q.g[j + 1] = -q.sn[j] * q.g[j];
-    q.g[j] = q.cs[j] * q.g[j];
-    const double res = fabs(q.g[j + 1]);
+    const double g1 = -s * B.g;
+    q.g[j + 1] = g1;
+    q.g[j] = c * B.g;
+    const double res = fabs(g1);
+    const int nan = (isfinite(res) && isfinite(beta)) ? 0 : 1;
     q.st->res = res;
-    q.st->beta = beta;
-    q.st->nan = (isfinite(res) && isfinite(beta)) ? 0 : 1;
+    q.st->nan = nan;
+    gm_set_beta(q.st, beta);
+    if (q.dl) {
+        const int its = B.dl.its + 1, nan_any = B.dl.nan | nan;
+        q.dl->its = its;
+        q.dl->j = j + 1;
+        q.dl->res = res;
+        q.dl->nan = nan_any;
+        const bool go = !nan_any && res > B.dl.tol && beta != 0.0 && j + 1 < B.dl.m && its < B.dl.nmax;
+        cudaGraphSetConditional(q.h, go ? 1u : 0u);
+    }
+}
+
+// The last block's end of a reduction kernel: the partials of ncols columns
+// into out, then (gv.H set) the Givens update with out[0] = ||w||^2.
+template <typename T>
+__device__ __forceinline__ void finish_reduction(const double *partial, int ncols, double *out, unsigned *ticket,
+                                                 const GivensArgs &gv) {
+    __shared__ GivensBuf B;
+    if (gv.H) givens_stage(gv, B);
+    reduce_partials<T>(partial, gridDim.x, ncols, out);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (gv.H) givens_step(gv, B, out[0]);
+        *ticket = 0;
+    }
 }
 
 // out[c] = V(:, c)^T w for c < ncols (column c at V + c*ldv), over the fixed
@@ -773,12 +934,7 @@ __device__ __forceinline__ void mdot_body(const T *__restrict__ V, long long ldv
         __syncthreads();
     }
     if (!grid_last_block(ticket)) return;
-    reduce_partials<T>(partial, gridDim.x, ncols, out);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        if (gv.H) givens_step(gv, out[0]);
-        *ticket = 0;
-    }
+    finish_reduction<T>(partial, ncols, out, ticket, gv);
 }
 
 template <typename T, int CB, bool VEC>
@@ -894,12 +1050,7 @@ __device__ __forceinline__ void maxpy_dot_body(const T *__restrict__ V, long lon
     const int nout = norm_only ? 1 : ncols;
     block_partials<T, MAXC>(acc, nout, partial, 0);
     if (!grid_last_block(ticket)) return;
-    reduce_partials<T>(partial, gridDim.x, nout, out);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        if (gv.H) givens_step(gv, out[0]);
-        *ticket = 0;
-    }
+    finish_reduction<T>(partial, nout, out, ticket, gv);
 }
 
 template <typename T, int MAXC, bool VEC>
@@ -1011,8 +1162,11 @@ template <typename T, bool VEC> __global__ void k_scale_inv(T *v, const T *w, co
     scale_inv_body<T, VEC>(v, w, s, n);
 }
 
+// v = w / sqrt(*s2) (skips when *s2 is not positive)
+__global__ void k_scale_rsqrt(double *v, const double *w, const double *s2, long long n);
+
 // ============================================= least squares (GMRES end)
-// y = H(0:k,0:k)^{-1} g(0:k), upper triangular.  One thread.
+// y = H(0:k,0:k)^{-1} g(0:k), upper triangular.  One warp.
 __global__ void k_trisolve(const double *H, int ldh, const double *g, double *y, int k);
 // g = [beta, 0, ...]; st->res = beta
 __global__ void k_gm_init(double *g, int m1, const double *beta2, double *beta, GmState *st);
@@ -1020,12 +1174,6 @@ __global__ void k_gm_init(double *g, int m1, const double *beta2, double *beta, 
 __global__ void k_recip(long long n, const double *a, double *b);
 
 // ============================== device-driven Krylov loops (graph WHILE)
-// Loop state of one GMRES level on the device.
-struct GmDev {
-    int j, its, m, nmax;        // column of the current cycle, iterations, restart length, iteration limit
-    int conv, nan, pad0, pad1;  // pad0: restart cycles run (outer level)
-    double tol, bnorm, res, rel_true;
-};
 // Per-solve options of the device-driven solve (written before each launch).
 struct DlParams {
     double rtol, rtol_A, rtol_S, rtol_I, atol;
@@ -1038,55 +1186,50 @@ struct DlCounters {
 __global__ void k_dl_init(GmDev *st, double *g, int m1, const double *nrm2, double *beta, GmState *gs,
                           const double *rtol, const double *atol, const int *m, const int *nmax,
                           cudaGraphConditionalHandle h);
-// The end of one iteration of a device-driven GMRES loop (one thread):
-// counters, then the stopping rule of the host-driven loop -- continue while
-// |g_{j+1}| > max(rtol ||b||, atol), h_{j+1,j} != 0, no NaN, j < m and
-// its < n_max -- as the WHILE node's condition.
-__device__ __forceinline__ void dl_step(GmDev *st, const GmState *gs, cudaGraphConditionalHandle h) {
-    st->its += 1;
-    st->j += 1;
-    st->res = gs->res;
-    if (gs->nan) st->nan = 1;
-    const bool go = !st->nan && st->res > st->tol && gs->beta != 0.0 && st->j < st->m && st->its < st->nmax;
-    cudaGraphSetConditional(h, go ? 1u : 0u);
-}
-// The last kernel of an iteration: basis column j + 1 = w / h_{j+1,j}
-// (gs->beta, the reciprocal taken once per block as in k_scale_inv), then,
-// in the grid's last block -- every block has read j by then -- dl_step.
+// The first kernel of a device-driven iteration: basis column j = src / beta
+// (beta, and its reciprocal, from the norm pass before), src = w, or b where
+// the cycle starts (j = 0).  VEC: pointers and ld 16-byte aligned.
 template <typename T, bool VEC>
-__global__ void k_scale_step_dl(T *vbase, long long ld, GmDev *st, const T *w, const GmState *gs, long long n,
-                                unsigned *ticket, cudaGraphConditionalHandle h) {
+__global__ void k_start_col(T *vbase, long long ld, const int *jp, const T *b, const T *w, const GmState *gs, long long n) {
     constexpr int W = VEC ? Vec16<T>::W : 1;
-    __shared__ T inv_s;
-    __shared__ int zero;
-    if (threadIdx.x == 0) {
-        const double d = gs->beta;
-        zero = (d == 0.0);
-        inv_s = zero ? T(0) : (T)(1.0 / d);
-    }
-    __syncthreads();
-    T *v = vbase + (long long)(st->j + 1) * ld;
-    if (!zero) {
-        const T inv = inv_s;
-        const long long nv = n / W;
-        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += (long long)gridDim.x * blockDim.x) {
-            if constexpr (VEC) {
-                T u[W];
-                vld(w + i * W, u);
+    const int j = *jp;
+    const T *src = j == 0 ? b : w;
+    const T inv = gm_inv<T>(gs);
+    T *v = vbase + (long long)j * ld;
+    const long long nv = n / W;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += (long long)gridDim.x * blockDim.x) {
+        if constexpr (VEC) {
+            T u[W];
+            vld(src + i * W, u);
 #pragma unroll
-                for (int e = 0; e < W; ++e) u[e] *= inv;
-                vst(v + i * W, u);
-            } else {
-                v[i] = w[i] * inv;
-            }
+            for (int e = 0; e < W; ++e) u[e] *= inv;
+            vst(v + i * W, u);
+        } else {
+            v[i] = src[i] * inv;
         }
-        if (VEC && blockIdx.x == 0 && threadIdx.x < n - nv * W) v[nv * W + threadIdx.x] = w[nv * W + threadIdx.x] * inv;
     }
-    if (!grid_last_block(ticket)) return;
-    if (threadIdx.x == 0) {
-        dl_step(st, gs, h);
-        *ticket = 0;
-    }
+    if (VEC && blockIdx.x == 0 && threadIdx.x < n - nv * W) v[nv * W + threadIdx.x] = src[nv * W + threadIdx.x] * inv;
+}
+// k_start_col fused with the AMG cycle's first smoothing step from zero on
+// that column (k_cheb_first): x = c2 Dinv v, and d = x where a later step of
+// the same smoothing reads it (d may be null).  Saves a launch and a pass
+// over v per iteration; 0.56M unknowns (421k components): 4.8 + 3.7 -> 4.0 us.
+template <typename T>
+__global__ void k_start_cheb(int nbr, int bs, const T *__restrict__ dinv, T *__restrict__ vbase, long long ld,
+                             const int *jp, const T *b, const T *w, const GmState *gs, T c2, T *__restrict__ d,
+                             T *__restrict__ x) {
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= (long long)nbr * bs) return;
+    const int j = *jp;
+    const T *src = j == 0 ? b : w;
+    const T inv = gm_inv<T>(gs);
+    vbase[(long long)j * ld + t] = src[t] * inv;
+    const int i = (int)(t / bs), a = (int)(t - (long long)i * bs);
+    T s = 0;
+    for (int c = 0; c < bs; ++c) s += dinv[(long long)i * bs * bs + a * bs + c] * (src[(long long)i * bs + c] * inv);
+    const T dn = c2 * s;
+    if (d) d[t] = dn;
+    x[t] = dn;
 }
 __global__ void k_dl_cycle_start(GmDev *st, cudaGraphConditionalHandle h);
 __global__ void k_dl_end(GmDev *st, const double *H, int ldh, const double *g, double *y, long long *its_total,
@@ -1177,7 +1320,7 @@ __global__ void k_restrict_first(const int *__restrict__ mptr, const int *__rest
     for (int c = 0; c < 3; ++c)
         if (c < bs) s += dinv[(long long)I * bs * bs + l * bs + c] * v[c];
     const T dn = c2 * s;
-    d[t] = dn;
+    if (d) d[t] = dn;   // read by a second pre-smoothing step only
     x[t] = dn;
 }
 // x[i] += e_c[agg[i]]
@@ -1229,21 +1372,6 @@ __global__ void k_cheb_first(int nbr, int bs, const T *__restrict__ dinv, const 
                              T *__restrict__ x, T *__restrict__ bcopy) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (long long)nbr * bs) return;
-    if (bcopy) bcopy[t] = b[t];
-    const int i = (int)(t / bs), a = (int)(t - (long long)i * bs);
-    T s = 0;
-    for (int c = 0; c < bs; ++c) s += dinv[(long long)i * bs * bs + a * bs + c] * b[(long long)i * bs + c];
-    const T dn = c2 * s;
-    d[t] = dn;
-    x[t] = dn;
-}
-// k_cheb_first with b = basis column *jp (stride ld)
-template <typename T>
-__global__ void k_cheb_first_col(int nbr, int bs, const T *__restrict__ dinv, const T *__restrict__ vbase, long long ld,
-                                 const int *jp, T c2, T *__restrict__ d, T *__restrict__ x, T *__restrict__ bcopy) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long long)nbr * bs) return;
-    const T *b = vbase + (long long)(*jp) * ld;
     if (bcopy) bcopy[t] = b[t];
     const int i = (int)(t / bs), a = (int)(t - (long long)i * bs);
     T s = 0;
@@ -1477,9 +1605,11 @@ template <typename T> __global__ void k_kupd3(T *x, const T *z1, const T *z2, co
 // f[k] = r_k * (a^k . x), one block per outlet (fixed-order tree reduction)
 template <typename T>
 __global__ void k_lowrank_dots(const int *__restrict__ optr, const int *__restrict__ oidx, const double *__restrict__ oval,
-                               const double *__restrict__ r, const T *__restrict__ x, double *__restrict__ f) {
+                               const double *__restrict__ r, const T *__restrict__ x, double *__restrict__ f,
+                               const int *jp = nullptr, long long x_ld = 0) {
     __shared__ double red[8];
     const int k = blockIdx.x;
+    if (jp) x += (long long)*jp * x_ld;   // x is basis column *jp
     double s = 0.0;
     for (int q = optr[k] + threadIdx.x; q < optr[k + 1]; q += blockDim.x) s += oval[q] * (double)x[oidx[q]];
     s = warp_sum(s);

@@ -163,6 +163,16 @@ struct nbp_ctx {
     // inside an inner A-solve of Algorithm 2 with gs_passes_I = 1: one
     // classical Gram-Schmidt pass per Arnoldi step instead of two
     bool gs_one_pass = false;
+    // while capturing the AMG cycle of a device-driven loop: level 0's
+    // right-hand side is column *jp of V and the cycle's result goes straight
+    // into column *jp of Z (null: plain buffers)
+    struct ColIO {
+        const nbp::Level *level = nullptr;
+        const void *V = nullptr;
+        void *Z = nullptr;
+        long long ld = 0;
+        const int *jp = nullptr;
+    } col;
     CycleGraph graphs[2][3][kMaxChebDegree + 1];
     cudaStream_t cap = nullptr;   // private stream used only while capturing
     bool use_graphs = true;
@@ -296,12 +306,16 @@ template <class F> static void as_inner_solve(nbp_ctx *c, F f) {
 }
 
 // y = A x (+ sum_k r_k a^k (a^k . x)); the rank-one factors f_k are FP64
-template <typename T> static void apply_A(nbp_ctx *c, int vsel, const T *x, T *y) {
+// (x: basis column *jp of stride x_ld when jp is set)
+template <typename T>
+static void apply_A(nbp_ctx *c, int vsel, const T *x, T *y, const int *jp = nullptr, long long x_ld = 0) {
     LowRank &lr = c->lr;
     SpmvArgs a = sargs(x, y);
+    a.jp = jp;
+    a.x_ld = x_ld;
     if (lr.n_out > 0) {
         c->prof.launches++;
-        k_lowrank_dots<T><<<lr.n_out, 256, 0, c->s>>>(lr.optr, lr.oidx, lr.oval, lr.r, x, lr.f);
+        k_lowrank_dots<T><<<lr.n_out, 256, 0, c->s>>>(lr.optr, lr.oidx, lr.oval, lr.r, x, lr.f, jp, x_ld);
         NBP_LAUNCHED();
         a.lr_rp = lr.lr_rp; a.lr_k = lr.lr_k; a.lr_c = lr.lr_c; a.lr_val = lr.lr_val; a.lr_f = lr.f;
     }
@@ -567,7 +581,7 @@ static GmResult gmres(nbp_ctx *c, Krylov<T> &K, long long n, Op op, Pc pc, const
             if (res <= tol || c->hst->beta == 0.0) break;
         }
         c->prof.launches += 1;
-        k_trisolve<<<1, 1, 0, s>>>(K.H, K.m, K.g, K.y, jend);   // H is laid out with the allocated restart length
+        k_trisolve<<<1, 32, 0, s>>>(K.H, K.m, K.g, K.y, jend);   // H is laid out with the allocated restart length
         NBP_LAUNCHED();
         maxpy<T>(c, n, K.Z, K.ld, jend, K.y, 1.0, x);
         const bool est_conv = res <= tol;
@@ -613,22 +627,44 @@ static Cheb cheb_of(const Level &L) {
     return ch;
 }
 
+// right-hand side of level L for a fused epilogue (basis column *jp where the
+// cycle of a device-driven loop has set one, else b)
+static void set_rhs(nbp_ctx *c, const Level &L, SpmvArgs &a, const void *b) {
+    a.b = b;
+    if (c->col.level == &L) {
+        a.b = c->col.V;
+        a.b_ld = c->col.ld;
+        a.jp = c->col.jp;
+    }
+}
+
 // One Chebyshev step on level L: r = b - A x; d = c1 d + c2 Dinv r; xout = x + d
+// (d read only when c1 != 0, written only when a later step reads it: more;
+// last: the cycle's last step on this level, see ColIO)
 template <typename T>
-static void cheb_step(nbp_ctx *c, Level &L, int vsel, const T *b, const T *x, T *xout, T *d, double c1, double c2) {
+static void cheb_step(nbp_ctx *c, Level &L, int vsel, const T *b, const T *x, T *xout, T *d, double c1, double c2,
+                      bool more, bool last) {
     SpmvArgs a = sargs(x, nullptr);
-    a.b = b; a.dinv = dinv_of<T>(L); a.d = d; a.xout = xout; a.c1 = c1; a.c2 = c2;
+    set_rhs(c, L, a, b);
+    a.dinv = dinv_of<T>(L); a.d = d; a.xout = xout; a.c1 = c1; a.c2 = c2;
     a.c1f = (float)c1; a.c2f = (float)c2;
+    a.d_read = c1 != 0.0;
+    a.d_write = more;
+    if (last && c->col.level == &L) {
+        a.xout = c->col.Z;
+        a.out_ld = c->col.ld;
+    }
     do_spmv<T>(c, L.M, vsel, a, EPI_CHEB, false, (&L == &c->HA.L[0]) ? CAT_CHEB_A0 : CAT_SPMV);
 }
 
 // Chebyshev smoothing of degree k on level L; from x = 0 when zero_start.
 // Returns the buffer holding the result (x or alt).
 // first_done: the first step from zero (d = x = Dinv b / theta) was already
-// made by the restriction that produced b.
+// made by the restriction that produced b.  post: the cycle's last smoothing
+// on this level.
 template <typename T>
 static T *chebyshev(nbp_ctx *c, Level &L, int vsel, int k, const T *b, T *x, T *alt, bool zero_start,
-                    bool first_done = false) {
+                    bool first_done = false, bool post = false) {
     const int bs = L.M.br;
     const Cheb ch = cheb_of(L);
     T *d = wvec<T>(L, 4);
@@ -643,12 +679,13 @@ static T *chebyshev(nbp_ctx *c, Level &L, int vsel, int k, const T *b, T *x, T *
                                                                                    (T)(1.0 / ch.theta), d, cur, nullptr);
         });
     } else {
-        cheb_step<T>(c, L, vsel, b, cur, nxt, d, 0.0, 1.0 / ch.theta);
+        cheb_step<T>(c, L, vsel, b, cur, nxt, d, 0.0, 1.0 / ch.theta, k > 1, post && k == 1);
         std::swap(cur, nxt);
     }
     for (int it = 1; it < k; ++it) {
         const double rho_new = 1.0 / (2.0 * ch.sigma - rho_old);
-        cheb_step<T>(c, L, vsel, b, cur, nxt, d, rho_new * rho_old, 2.0 * rho_new / ch.delta);
+        cheb_step<T>(c, L, vsel, b, cur, nxt, d, rho_new * rho_old, 2.0 * rho_new / ch.delta, it + 1 < k,
+                     post && it + 1 == k);
         std::swap(cur, nxt);
         rho_old = rho_new;
     }
@@ -750,7 +787,7 @@ static void vcycle_level(nbp_ctx *c, Hier &H, int l, int vsel, const T *b, T *ou
     T *oth = (cur == out) ? alt : out;
     // residual and restriction
     T *r = wvec<T>(L, 3);
-    do_spmv<T>(c, L.M, vsel, [&] { SpmvArgs a = sargs(cur, r); a.b = b; return a; }(), EPI_RES, false);
+    do_spmv<T>(c, L.M, vsel, [&] { SpmvArgs a = sargs(cur, r); set_rhs(c, L, a, b); return a; }(), EPI_RES, false);
     Level &Lc = H.L[l + 1];
     T *bc = wvec<T>(Lc, 0), *xc = wvec<T>(Lc, 1);
     const bool kc = H.kcycle && l + 1 < H.nlev - 1 && l + 1 <= H.kdepth;
@@ -764,11 +801,12 @@ static void vcycle_level(nbp_ctx *c, Hier &H, int l, int vsel, const T *b, T *ou
     const double rbytes = (double)(Lc.M.nbr + 1) * 4.0 + (double)L.M.nbr * 4.0 + (double)n * sizeof(T) + ncv;
     if (fuse) {
         const Cheb chc = cheb_of(Lc);
-        // + the coarse block-diagonal inverse read, d and x written (+ the copy)
-        const double fbytes = rbytes + (double)Lc.M.nbr * bs * bs * sizeof(T) + 2.0 * ncv + (kc ? ncv : 0.0);
+        // + the coarse block-diagonal inverse read, d (degree > 1) and x written (+ the copy)
+        const double fbytes = rbytes + (double)Lc.M.nbr * bs * bs * sizeof(T) + (k > 1 ? 2.0 : 1.0) * ncv + (kc ? ncv : 0.0);
         timed(c, "amg/restrict+first", fbytes, [&] {
             k_restrict_first<T><<<grid_exact((long long)Lc.M.nbr * 8), 256, 0, c->s>>>(
-                L.mptr, L.mem, Lc.M.nbr, bs, r, bc, dinv_of<T>(Lc), (T)(1.0 / chc.theta), wvec<T>(Lc, 4), wvec<T>(Lc, 2),
+                L.mptr, L.mem, Lc.M.nbr, bs, r, bc, dinv_of<T>(Lc), (T)(1.0 / chc.theta), k > 1 ? wvec<T>(Lc, 4) : (T *)nullptr,
+                wvec<T>(Lc, 2),
                 kc ? wvec<T>(Lc, 5) : (T *)nullptr);
         });
     } else {
@@ -791,7 +829,7 @@ static void vcycle_level(nbp_ctx *c, Hier &H, int l, int vsel, const T *b, T *ou
             k_prolong<T><<<grid_exact(n), 256, 0, c->s>>>(L.agg, L.M.nbr, bs, xc, cur);
         }
     });
-    T *fin = chebyshev<T>(c, L, vsel, k, b, cur, oth, false);
+    T *fin = chebyshev<T>(c, L, vsel, k, b, cur, oth, false, false, true);
     if (fin != out) copy<T>(out, fin, n, c->s);
 }
 
@@ -1199,13 +1237,16 @@ template <class F> static long long emit_while(nbp_ctx *c, cudaGraphConditionalH
 // The Arnoldi step of iteration st->j (the host loop's kernels, index read
 // on the device): h1 = V^T w; w -= V h1, h2 = V^T w; w -= V h2, ||w|| and the
 // Givens update of column j; V(:, j+1) = w / ||w||.
-// One Arnoldi step of a device-driven loop, ending the iteration (its last
-// kernel advances the loop state and sets the WHILE condition h)
+// One Arnoldi step of a device-driven loop; its last kernel (the norm pass)
+// applies the Givens update, advances the loop state and sets the WHILE
+// condition h.  The new basis vector w / ||w|| is made by the first kernel of
+// the next iteration (k_start_col, k_start_cheb).
 template <typename T> static void arnoldi_dl(nbp_ctx *c, Krylov<T> &K, GmDev *st, cudaGraphConditionalHandle h) {
     const bool vec = al16(K.V) && al16(K.w) && (K.ld * (long long)sizeof(T)) % 16 == 0;
     const int *jp = &st->j;
     GivensArgs gv = K.givens(0);
-    gv.jp = jp;
+    gv.dl = st;
+    gv.h = h;
     if (c->gs_one_pass) gv.h2 = nullptr;
     // one pass: the multi-dot, then subtract + norm + Givens update
     const double *coef = c->gs_one_pass ? K.h1 : K.h2;
@@ -1218,8 +1259,6 @@ template <typename T> static void arnoldi_dl(nbp_ctx *c, Krylov<T> &K, GmDev *st
                                                                       K.h2, K.ticket, GivensArgs());
         k_maxpy_dot_dl<T, kFusedCols, true><<<g2, 256, 0, c->s>>>(K.V, K.ld, jp, 1, coef, K.w, K.n, 1, K.partial, K.nrm,
                                                                   K.ticket, gv);
-        k_scale_step_dl<T, true><<<grid_for(K.n / Vec16<T>::W + 1), 256, 0, c->s>>>(K.V, K.ld, st, K.w, K.st, K.n,
-                                                                                   K.ticket, h);
     } else {
         const unsigned g1 = K.grid_md ? K.grid_md : arnoldi_grids<T>().mdot_dl_s;
         const unsigned g2 = K.grid ? K.grid : arnoldi_grids<T>().mpd_dl_s;
@@ -1229,8 +1268,16 @@ template <typename T> static void arnoldi_dl(nbp_ctx *c, Krylov<T> &K, GmDev *st
                                                                        K.h2, K.ticket, GivensArgs());
         k_maxpy_dot_dl<T, kFusedCols, false><<<g2, 256, 0, c->s>>>(K.V, K.ld, jp, 1, coef, K.w, K.n, 1, K.partial,
                                                                    K.nrm, K.ticket, gv);
-        k_scale_step_dl<T, false><<<grid_for(K.n + 1), 256, 0, c->s>>>(K.V, K.ld, st, K.w, K.st, K.n, K.ticket, h);
     }
+    NBP_LAUNCHED();
+}
+
+// Basis column j = (j == 0 ? b : w) / beta, the first kernel of an iteration
+template <typename T> static void start_col(nbp_ctx *c, Krylov<T> &K, GmDev *st, const T *b) {
+    const bool vec = al16(K.V) && al16(K.w) && al16(b) && (K.ld * (long long)sizeof(T)) % 16 == 0;
+    const unsigned grid = grid_for(K.n / (vec ? Vec16<T>::W : 1) + 1);
+    if (vec) k_start_col<T, true><<<grid, 256, 0, c->s>>>(K.V, K.ld, &st->j, b, K.w, K.st, K.n);
+    else k_start_col<T, false><<<grid, 256, 0, c->s>>>(K.V, K.ld, &st->j, b, K.w, K.st, K.n);
     NBP_LAUNCHED();
 }
 
@@ -1243,8 +1290,10 @@ template <typename T> static void update_dl(nbp_ctx *c, Krylov<T> &K, GmDev *st,
     NBP_LAUNCHED();
 }
 
-// One single-cycle GMRES level (inner A- and S-solves): pc(vbase, ld, jp)
-// preconditions basis column j into a fixed buffer it returns; op(z, w).
+// One single-cycle GMRES level (inner A- and S-solves): pc(K, st, b) makes
+// basis column j and preconditions it, returning a fixed buffer or, where it
+// wrote column j of K.Z itself, null; op(z, jp, ld, w) applies the operator
+// to z (basis column *jp when jp is set).
 template <typename T, typename Op, typename Pc>
 static long long gmres_dl(nbp_ctx *c, Krylov<T> &K, long long n, GmDev *st, const double *rtol, const int *m,
                           const int *nmax, long long *its_total, long long *solves, const T *b, T *x, Pc pc, Op op,
@@ -1254,39 +1303,53 @@ static long long gmres_dl(nbp_ctx *c, Krylov<T> &K, long long n, GmDev *st, cons
     const cudaGraphConditionalHandle h = new_handle(c);
     k_dl_init<<<1, 256, 0, c->s>>>(st, K.g, K.m + 1, K.nrm, K.beta, K.st, rtol, &c->dl_par->atol, m, nmax, h);
     NBP_LAUNCHED();
-    scale_inv<T>(c, K.V, b, K.beta, n);
-    NBP_LAUNCHED();
     const long long kb = emit_while(c, h, depth, [&] {
-        T *z = pc(K.V, K.ld, &st->j);
-        op(z, K.w);
-        k_col_put<T, T><<<grid_for(n), 256, 0, c->s>>>(K.Z, K.ld, &st->j, 0, 0, z, n);
-        NBP_LAUNCHED();
+        const T *z = pc(K, st, b);
+        if (z) {
+            op(z, (const int *)nullptr, 0LL, K.w);
+            k_col_put<T, T><<<grid_for(n), 256, 0, c->s>>>(K.Z, K.ld, &st->j, 0, 0, z, n);
+            NBP_LAUNCHED();
+        } else {
+            op((const T *)K.Z, &st->j, K.ld, K.w);
+        }
         arnoldi_dl<T>(c, K, st, h);
     });
-    k_dl_end<<<1, 1, 0, c->s>>>(st, K.H, K.m, K.g, K.y, its_total, solves);
+    k_dl_end<<<1, 32, 0, c->s>>>(st, K.H, K.m, K.g, K.y, its_total, solves);
     NBP_LAUNCHED();
     update_dl<T>(c, K, st, x);
     return kb;
 }
 
-// An AMG cycle on hierarchy H from basis column *jp into the hierarchy's
-// level-0 output buffer (the copy-in fused with the first smoothing step, as
-// the replayed cycle does); returns that buffer.
-template <typename T> static T *cycle_from_col(nbp_ctx *c, Hier &H, const T *vbase, long long ld, const int *jp) {
+// An AMG cycle on hierarchy H from basis column j, which it makes first (the
+// scaling fused with the cycle's first smoothing step), into column j of K.Z:
+// level 0 reads its right-hand side from the column and its last smoothing
+// step writes there (null).  Without smoothing, or with one level, through
+// the hierarchy's level-0 buffers: returns the output one.
+template <typename T> static const T *cycle_from_col(nbp_ctx *c, Hier &H, Krylov<T> &K, GmDev *st, const T *b) {
     const int avsel = amg_vsel_of(c->opt.precision);
     Level &L0 = H.L[0];
     const long long n = (long long)L0.M.nbr * H.bs;
     T *gb = wvec<T>(L0, 0), *gx = wvec<T>(L0, 1);
-    const bool first_in = H.cheb > 0 && H.nlev > 1;
-    if (first_in) {
+    if (H.cheb > 0 && H.nlev > 1) {
         const Cheb ch = cheb_of(L0);
-        k_cheb_first_col<T><<<grid_exact(n), 256, 0, c->s>>>(L0.M.nbr, H.bs, dinv_of<T>(L0), vbase, ld, jp,
-                                                             (T)(1.0 / ch.theta), wvec<T>(L0, 4), wvec<T>(L0, 2), gb);
-    } else {
-        k_col_get<T, T><<<grid_for(n), 256, 0, c->s>>>(gb, vbase, ld, jp, 0, 0, n);
+        k_start_cheb<T><<<grid_exact(n), 256, 0, c->s>>>(L0.M.nbr, H.bs, dinv_of<T>(L0), K.V, K.ld, &st->j, b, K.w, K.st,
+                                                         (T)(1.0 / ch.theta), H.cheb > 1 ? wvec<T>(L0, 4) : (T *)nullptr,
+                                                         wvec<T>(L0, 2));
+        NBP_LAUNCHED();
+        c->col = nbp_ctx::ColIO{&L0, K.V, K.Z, K.ld, &st->j};
+        try {
+            vcycle_level<T>(c, H, 0, avsel, gb, gx, true);
+        } catch (...) {
+            c->col = nbp_ctx::ColIO{};
+            throw;
+        }
+        c->col = nbp_ctx::ColIO{};
+        return nullptr;
     }
+    start_col<T>(c, K, st, b);
+    k_col_get<T, T><<<grid_for(n), 256, 0, c->s>>>(gb, K.V, K.ld, &st->j, 0, 0, n);
     NBP_LAUNCHED();
-    vcycle_level<T>(c, H, 0, avsel, gb, gx, first_in);
+    vcycle_level<T>(c, H, 0, avsel, gb, gx, false);
     return gx;
 }
 
@@ -1295,15 +1358,16 @@ template <typename T>
 static void solve_A_dl(nbp_ctx *c, int vsel, const T *s, T *y, const double *rtol, long long *its, long long *solves,
                        int depth) {
     const long long n = 3LL * c->N;
-    auto op = [&](const T *x, T *out) { apply_A<T>(c, vsel, x, out); };
-    auto pc = [&](T *vbase, long long ld, const int *jp) -> T * {
+    auto op = [&](const T *x, const int *jp, long long ld, T *out) { apply_A<T>(c, vsel, x, out, jp, ld); };
+    auto pc = [&](Krylov<T> &K, GmDev *st, const T *b) -> const T * {
         if (c->opt.pc_A == 1) {
             T *z = (T *)c->dl_zA;
-            k_mul_col<T><<<grid_for(n), 256, 0, c->s>>>(z, vbase, ld, jp, BUF<T>(c).dinvA, n);
+            start_col<T>(c, K, st, b);
+            k_mul_col<T><<<grid_for(n), 256, 0, c->s>>>(z, K.V, K.ld, &st->j, BUF<T>(c).dinvA, n);
             NBP_LAUNCHED();
             return z;
         }
-        return cycle_from_col<T>(c, c->HA, vbase, ld, jp);
+        return cycle_from_col<T>(c, c->HA, K, st, b);
     };
     c->dl_k_A = gmres_dl<T>(c, KA<T>(c), n, &c->dl_st[2], rtol, &c->dl_par->m_A, &c->dl_par->nmax_A, its, solves, s, y, pc,
                             op, depth);
@@ -1323,22 +1387,29 @@ template <typename T> static double *pscr_dl(nbp_ctx *c, const double *vbase, lo
         solve_A_dl<T>(c, vsel, Bf.sv, Bf.yvh, &par->rtol_A, &cnt->A, &cnt->nA, depth);            // step 1
         do_spmv<T>(c, c->C, vsel, sargs(Bf.yvh, Bf.sp), EPI_SUB, false);                          // step 2
     }
-    auto opS = [&](const T *x, T *out) {                                                          // Algorithm 2
-        do_spmv<T>(c, c->D, vsel, sargs(x, out), EPI_SET, false);
-        do_spmv<T>(c, c->B, vsel, sargs(x, Bf.xbar), EPI_SET, false);
+    auto opS = [&](const T *x, const int *jp, long long ld, T *out) {                             // Algorithm 2
+        auto from_x = [&](T *y) {
+            SpmvArgs a = sargs(x, y);
+            a.jp = jp;
+            a.x_ld = ld;
+            return a;
+        };
+        do_spmv<T>(c, c->D, vsel, from_x(out), EPI_SET, false);
+        do_spmv<T>(c, c->B, vsel, from_x(Bf.xbar), EPI_SET, false);
         as_inner_solve(c, [&] {
             solve_A_dl<T>(c, vsel_I_of(c->opt.precision), Bf.xbar, Bf.xtil, &par->rtol_I, &cnt->I, &cnt->nI, depth + 1);
         });
         do_spmv<T>(c, c->C, vsel, sargs(Bf.xtil, out), EPI_SUB, false);
     };
-    auto pcS = [&](T *vb, long long l, const int *j) -> T * {
+    auto pcS = [&](Krylov<T> &K, GmDev *st, const T *b) -> const T * {
         if (c->opt.pc_S == 1) {
             T *z = (T *)c->dl_zS;
-            k_col_get<T, T><<<grid_for(N), 256, 0, c->s>>>(z, vb, l, j, 0, 0, N);
+            start_col<T>(c, K, st, b);
+            k_col_get<T, T><<<grid_for(N), 256, 0, c->s>>>(z, K.V, K.ld, &st->j, 0, 0, N);
             NBP_LAUNCHED();
             return z;
         }
-        return cycle_from_col<T>(c, c->HS, vb, l, j);
+        return cycle_from_col<T>(c, c->HS, K, st, b);
     };
     c->dl_k_S = gmres_dl<T>(c, KS<T>(c), N, &c->dl_st[1], &par->rtol_S, &par->m_S, &par->nmax_S, &cnt->S, &cnt->nS,
                             Bf.sp, Bf.yp, pcS, opS, depth);                                         // step 3
@@ -1367,9 +1438,8 @@ static void outer_dl(nbp_ctx *c) {
         const cudaGraphConditionalHandle hi = new_handle(c);
         k_dl_cycle_start<<<1, 1, 0, c->s>>>(st, hi);
         NBP_LAUNCHED();
-        scale_inv<double>(c, K.V, K.r, K.beta, n);
-        NBP_LAUNCHED();
         c->dl_k_outer = emit_while(c, hi, 1, [&] {   // iterations
+            start_col<double>(c, K, st, K.r);
             double *z = c->opt.precision == 0 ? pscr_dl<double>(c, K.V, K.ld, &st->j, 2)
                                               : pscr_dl<float>(c, K.V, K.ld, &st->j, 2);
             apply_full(c, z, K.w);
@@ -1377,7 +1447,7 @@ static void outer_dl(nbp_ctx *c) {
             NBP_LAUNCHED();
             arnoldi_dl<double>(c, K, st, hi);
         });
-        k_dl_end<<<1, 1, 0, c->s>>>(st, K.H, K.m, K.g, K.y, nullptr, nullptr);
+        k_dl_end<<<1, 32, 0, c->s>>>(st, K.H, K.m, K.g, K.y, nullptr, nullptr);
         NBP_LAUNCHED();
         update_dl<double>(c, K, st, x);
         apply_full(c, x, K.w);                       // true residual: the next restart vector or the check
@@ -1692,54 +1762,91 @@ static double gelfand_radius(int k, const std::vector<double> &H) {
 // on AMG(S_hat), smoothed with degree 1 (damped Jacobi with weight 1/theta),
 // the tighter bound over-relaxes the top of the nonsymmetric spectrum and
 // costs S-iterations (measured), so that hierarchy keeps Gershgorin.
+// The steps of every level are queued without a host round trip (the
+// Hessenberg entries stay on the device, one slot per step); the host reads
+// them back and takes the spectral radius later, while the GPU works on the
+// rest of the setup.
 constexpr int kRhoSteps = 20;
-static void refine_rho(nbp_ctx *c, Hier &H, int l) {
+constexpr int kRhoSlot = 2 * kRhoSteps + 1;   // h1 (j + 1), h2 (j + 1), ||w||^2 of one step
+struct RhoEstimate {
+    Hier *H = nullptr;
+    std::vector<int> levels;
+    std::vector<double *> dev;   // kRhoSteps slots per level
+};
+static void queue_rho(nbp_ctx *c, Hier &H, int l, Krylov<double> &K, double *out) {
     Level &L = H.L[l];
-    if (!L.dinv) return;
     const long long n = (long long)L.M.nbr * H.bs;
     cudaStream_t s = c->s;
-    Krylov<double> K;
-    K.ensure(n, kRhoSteps, s);
+    K.n = n;                      // the space is sized for the finest level
+    K.ld = (n + 31) / 32 * 32;
+    // about 2,000 elements per block: the FP64 block stages cost microseconds
+    // of the narrow pipe each, so short vectors take fewer blocks
+    K.grid = K.grid_md = (unsigned)std::max<long long>(1, std::min<long long>(2 * kSMs, n / 2048));
     fill<double>(K.V, 1.0 / std::sqrt((double)n), n, s);
-    std::vector<double> Hk((size_t)kRhoSteps * kRhoSteps, 0.0), h1(kRhoSteps + 1), h2(kRhoSteps + 1);
-    int k = kRhoSteps;
     for (int j = 0; j < kRhoSteps; ++j) {
+        double *h1 = out + (size_t)j * kRhoSlot, *h2 = h1 + kRhoSteps, *nrm2 = h2 + kRhoSteps;
         do_spmv<double>(c, L.M, 0, sargs(K.V + (size_t)j * K.ld, K.w), EPI_SET, false);   // w = A v_j
         c->prof.launches++;
         k_cheb_first<double><<<grid_exact(n), 256, 0, s>>>(L.M.nbr, H.bs, L.dinv, K.w, 1.0, K.r, K.r, nullptr);
         NBP_LAUNCHED();                                                                   // r = D_b^{-1} w
-        mdot<double>(c, K, K.V, K.ld, j + 1, K.r, K.h1);
-        maxpy<double>(c, n, K.V, K.ld, j + 1, K.h1, -1.0, K.r);
-        mdot<double>(c, K, K.V, K.ld, j + 1, K.r, K.h2);
-        maxpy<double>(c, n, K.V, K.ld, j + 1, K.h2, -1.0, K.r);
-        mdot<double>(c, K, K.r, K.ld, 1, K.r, K.nrm);
-        double nrm2 = 0.0;
-        NBP_CUDA(cudaMemcpyAsync(h1.data(), K.h1, sizeof(double) * (j + 1), cudaMemcpyDeviceToHost, s));
-        NBP_CUDA(cudaMemcpyAsync(h2.data(), K.h2, sizeof(double) * (j + 1), cudaMemcpyDeviceToHost, s));
-        NBP_CUDA(cudaMemcpyAsync(&nrm2, K.nrm, sizeof(double), cudaMemcpyDeviceToHost, s));
-        NBP_CUDA(cudaStreamSynchronize(s));
-        for (int i = 0; i <= j; ++i) Hk[(size_t)i * kRhoSteps + j] = h1[i] + h2[i];
-        const double nrm = std::sqrt(std::max(nrm2, 0.0));
-        if (j + 1 < kRhoSteps) Hk[(size_t)(j + 1) * kRhoSteps + j] = nrm;
-        if (!(nrm > 0.0)) { k = j + 1; break; }
+        mdot<double>(c, K, K.V, K.ld, j + 1, K.r, h1);
+        if (j + 1 <= kFusedCols) {
+            maxpy_dot<double>(c, K, K.V, K.ld, j + 1, h1, K.r, 0, h2);
+            maxpy_dot<double>(c, K, K.V, K.ld, j + 1, h2, K.r, 1, nrm2);
+        } else {
+            maxpy<double>(c, n, K.V, K.ld, j + 1, h1, -1.0, K.r);
+            mdot<double>(c, K, K.V, K.ld, j + 1, K.r, h2);
+            maxpy<double>(c, n, K.V, K.ld, j + 1, h2, -1.0, K.r);
+            mdot<double>(c, K, K.r, K.ld, 1, K.r, nrm2);
+        }
         if (j + 1 < kRhoSteps) {
-            NBP_CUDA(cudaMemcpyAsync(K.beta, &nrm, sizeof(double), cudaMemcpyHostToDevice, s));
-            scale_inv<double>(c, K.V + (size_t)(j + 1) * K.ld, K.r, K.beta, n);
+            c->prof.launches++;
+            k_scale_rsqrt<<<grid_for(n), 256, 0, s>>>(K.V + (size_t)(j + 1) * K.ld, K.r, nrm2, n);
             NBP_LAUNCHED();
         }
     }
-    std::vector<double> Hs((size_t)k * k);
-    for (int i = 0; i < k; ++i)
-        for (int j = 0; j < k; ++j) Hs[(size_t)i * k + j] = Hk[(size_t)i * kRhoSteps + j];
-    const double est = 1.1 * gelfand_radius(k, Hs);
-    NBP_CUDA(cudaStreamSynchronize(s));
-    K.release(s);
-    if (std::isfinite(est) && est < L.rho) L.rho = est;
 }
 
-static void refine_rhos(nbp_ctx *c, Hier &H) {
+static RhoEstimate queue_rhos(nbp_ctx *c, Hier &H) {
+    RhoEstimate R;
+    R.H = &H;
     for (int l = 0; l < H.nlev; ++l)
-        if (l < H.nlev - 1 || !H.cinv) refine_rho(c, H, l);
+        if ((l < H.nlev - 1 || !H.cinv) && H.L[l].dinv) R.levels.push_back(l);
+    if (R.levels.empty()) return R;
+    Krylov<double> K;
+    K.ensure((long long)H.L[0].M.nbr * H.bs, kRhoSteps, c->s);
+    for (int l : R.levels) {
+        R.dev.push_back(dmalloc<double>((size_t)kRhoSteps * kRhoSlot, c->s));
+        queue_rho(c, H, l, K, R.dev.back());
+    }
+    K.release(c->s);
+    return R;
+}
+
+static void take_rhos(nbp_ctx *c, RhoEstimate &R) {
+    std::vector<double> buf((size_t)kRhoSteps * kRhoSlot);
+    for (size_t q = 0; q < R.levels.size(); ++q) {
+        NBP_CUDA(cudaMemcpyAsync(buf.data(), R.dev[q], sizeof(double) * buf.size(), cudaMemcpyDeviceToHost, c->s));
+        NBP_CUDA(cudaStreamSynchronize(c->s));
+        dfree(R.dev[q], c->s);
+        std::vector<double> Hk((size_t)kRhoSteps * kRhoSteps, 0.0);
+        int k = kRhoSteps;
+        for (int j = 0; j < kRhoSteps; ++j) {
+            const double *h1 = buf.data() + (size_t)j * kRhoSlot, *h2 = h1 + kRhoSteps;
+            for (int i = 0; i <= j; ++i) Hk[(size_t)i * kRhoSteps + j] = h1[i] + h2[i];
+            const double nrm = std::sqrt(std::max(h2[kRhoSteps], 0.0));
+            if (j + 1 < kRhoSteps) Hk[(size_t)(j + 1) * kRhoSteps + j] = nrm;
+            if (!(nrm > 0.0)) { k = j + 1; break; }   // breakdown: the later steps ran on nothing
+        }
+        std::vector<double> Hs((size_t)k * k);
+        for (int i = 0; i < k; ++i)
+            for (int j = 0; j < k; ++j) Hs[(size_t)i * k + j] = Hk[(size_t)i * kRhoSteps + j];
+        const double est = 1.1 * gelfand_radius(k, Hs);
+        Level &L = R.H->L[R.levels[q]];
+        if (std::isfinite(est) && est < L.rho) L.rho = est;
+    }
+    R.levels.clear();
+    R.dev.clear();
 }
 
 // numeric: rebuild both hierarchies on the aggregates of the last full
@@ -1751,9 +1858,10 @@ static void do_setup(nbp_ctx *c, bool numeric = false) {
     const int prec = build_level(c->opt.precision);
     if (!c->diagA) c->diagA = dmalloc<double>(3LL * c->N, s);
     amg_build(c->HA, c->A, c->opt, prec, s, numeric);
-    refine_rhos(c, c->HA);
+    RhoEstimate rhos = queue_rhos(c, c->HA);
     build_shat(c->A, c->B, c->C, c->D, c->lr, c->N, c->Shat, c->diagA, s);
-    amg_build(c->HS, c->Shat, c->opt, prec, s, numeric);   // AMG(S_hat) keeps the Gershgorin bound (see refine_rho)
+    amg_build(c->HS, c->Shat, c->opt, prec, s, numeric);   // AMG(S_hat) keeps the Gershgorin bound (see kRhoSteps)
+    take_rhos(c, rhos);
     // Chebyshev intervals [rho/10, rho] on AMG(A) and [rho/3, rho] on AMG(S_hat):
     // for the degree-1 smoothing of S_hat the lower end only sets the Jacobi
     // weight (1.5 / rho); rho/3 there cut S-iterations 97 -> 91 on the 4.34M
