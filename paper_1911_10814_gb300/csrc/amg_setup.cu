@@ -40,6 +40,7 @@ void hier_free(Hier &H, cudaStream_t s) {
     for (int l = 0; l < H.nlev; ++l) {
         Level &L = H.L[l];
         dmat_free(L.M, s);
+        dmat_free(L.AP, s);
         dfree(L.agg, s); dfree(L.mptr, s); dfree(L.mem, s); dfree(L.dinv, s); dfree(L.dinv32, s);
         for (int q = 0; q < Level::kWork; ++q) { dfree(L.w64[q], s); dfree(L.w32[q], s); }
         dfree(L.kdots, s); dfree(L.kpart, s);
@@ -1114,6 +1115,122 @@ static void members_of(const int *map, int n, int nc, int *&mptr, int *&mem, cud
 
 static void member_lists(Level &L, int n, int nc, cudaStream_t s) { members_of(L.agg, n, nc, L.mptr, L.mem, s); }
 
+// ---- A P, one row per warp: the row's entries in chunks of 32, each chunk's
+// coarse columns looked up in the row's list (first occurrence order), new ones
+// appended, and the blocks summed per column in entry order.  Rows with more
+// than kApCap coarse columns have no A P (the level keeps the prolongation and
+// the full product).
+constexpr int kApCap = 64, kApWarps = 8;
+
+// list position of this lane's coarse column J (-1: dropped), the list and its
+// length updated; *over is set when the list is full
+__device__ __forceinline__ int ap_position(int J, int lane, int *list, int &len, bool *over) {
+    int pos = -1;
+    for (int t = 0; t < len; ++t)
+        if (list[t] == J) pos = t;
+    if (J < 0) pos = -1;
+    const bool fresh = J >= 0 && pos < 0;
+    const unsigned same = __match_any_sync(0xffffffffu, fresh ? J : -1 - lane);
+    const bool lead = fresh && (__ffs(same) - 1) == lane;
+    const unsigned leads = __ballot_sync(0xffffffffu, lead);
+    int at = len + __popc(leads & ((1u << lane) - 1u));
+    at = __shfl_sync(0xffffffffu, at, __ffs(same) - 1);
+    len += __popc(leads);
+    if (len > kApCap) { *over = true; len = kApCap; }
+    if (lead && at < kApCap) list[at] = J;
+    __syncwarp();
+    if (fresh) pos = at < kApCap ? at : -1;
+    return pos;
+}
+__global__ void __launch_bounds__(32 * kApWarps) k_ap_count(int n, const int *rp, const int *ci, const int *agg, int *cnt,
+                                                           int *over) {
+    __shared__ int lists[kApWarps][kApCap];
+    const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i = blockIdx.x * kApWarps + wp;
+    if (i >= n) return;
+    int len = 0;
+    bool full = false;
+    const int e1 = rp[i + 1];
+    for (int e0 = rp[i]; e0 < e1; e0 += 32) {
+        const int e = e0 + lane;
+        ap_position(e < e1 ? agg[ci[e]] : -1, lane, lists[wp], len, &full);
+    }
+    if (lane == 0) {
+        cnt[i] = len;
+        if (full) *over = 1;
+    }
+}
+template <int NB>
+__global__ void __launch_bounds__(32 * kApWarps) k_ap_fill(int n, const int *rp, const int *ci, const double *v,
+                                                          const int *agg, const int *rp_out, int *ci_out, double *v_out) {
+    __shared__ int lists[kApWarps][kApCap];
+    __shared__ double sums[kApWarps][kApCap * NB];
+    const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i = blockIdx.x * kApWarps + wp;
+    if (i >= n) return;
+    double *acc = sums[wp];
+    for (int q = lane; q < kApCap * NB; q += 32) acc[q] = 0.0;
+    __syncwarp();
+    int len = 0;
+    bool full = false;
+    const int e1 = rp[i + 1];
+    for (int e0 = rp[i]; e0 < e1; e0 += 32) {
+        const int e = e0 + lane;
+        const int pos = ap_position(e < e1 ? agg[ci[e]] : -1, lane, lists[wp], len, &full);
+        unsigned same = __match_any_sync(0xffffffffu, pos >= 0 ? pos : -1 - lane);
+        if (pos >= 0 && (__ffs(same) - 1) == lane) {   // the column's first lane adds its blocks in entry order
+            double a[NB];
+#pragma unroll
+            for (int q = 0; q < NB; ++q) a[q] = acc[pos * NB + q];
+            while (same) {
+                const double *src = v + (long long)(e0 + __ffs(same) - 1) * NB;
+                same &= same - 1;
+#pragma unroll
+                for (int q = 0; q < NB; ++q) a[q] += src[q];
+            }
+#pragma unroll
+            for (int q = 0; q < NB; ++q) acc[pos * NB + q] = a[q];
+        }
+        __syncwarp();
+    }
+    const int o = rp_out[i];
+    for (int t = lane; t < len; t += 32) ci_out[o + t] = lists[wp][t];
+    for (int q = lane; q < len * NB; q += 32) v_out[(long long)o * NB + q] = acc[q];
+}
+
+// A P of a level with an aggregate map, in the sliced copies that the solves
+// use (the CSR arrays are dropped)
+static void make_ap(Level &L, int nc, int precision, cudaStream_t s) {
+    const DMat &M = L.M;
+    const int n = M.nbr;
+    if (n == 0 || nc == 0 || (M.bb() != 9 && M.bb() != 1)) return;
+    const unsigned blocks = (unsigned)((n + kApWarps - 1) / kApWarps);
+    int *cnt = dmalloc<int>(n + 2, s);   // rows, 0, overflow flag
+    NBP_CUDA(cudaMemsetAsync(cnt + n, 0, 2 * sizeof(int), s));
+    k_ap_count<<<blocks, 32 * kApWarps, 0, s>>>(n, M.rp, M.ci, L.agg, cnt, cnt + n + 1);
+    NBP_LAUNCHED();
+    DMat P;
+    P.nbr = n; P.nbc = nc; P.br = M.br; P.bc = M.bc;
+    P.rp = dmalloc<int>(n + 2, s);
+    exclusive_scan(cnt, P.rp, n + 1, s);
+    NBP_CUDA(cudaMemcpyAsync(P.rp + n + 1, cnt + n + 1, sizeof(int), cudaMemcpyDeviceToDevice, s));
+    int end[2];
+    NBP_CUDA(cudaMemcpyAsync(end, P.rp + n, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    NBP_CUDA(cudaStreamSynchronize(s));
+    dfree(cnt, s);
+    P.nnz = end[0];
+    if (end[1] || P.nnz == 0) { dmat_free(P, s); return; }
+    P.ci = dmalloc<int>(P.nnz, s);
+    P.v = dmalloc<double>(P.nnz * P.bb(), s);
+    if (P.bb() == 9) k_ap_fill<9><<<blocks, 32 * kApWarps, 0, s>>>(n, M.rp, M.ci, M.v, L.agg, P.rp, P.ci, P.v);
+    else k_ap_fill<1><<<blocks, 32 * kApWarps, 0, s>>>(n, M.rp, M.ci, M.v, L.agg, P.rp, P.ci, P.v);
+    NBP_LAUNCHED();
+    make_sell(P, precision, s);
+    dfree(P.rp, s); dfree(P.ci, s); dfree(P.v, s);
+    P.rp = nullptr; P.ci = nullptr; P.v = nullptr;
+    L.AP = P;
+}
+
 static void dense_inverse(const DMat &M, double *&cinv, int &nc, cudaStream_t s) {
     const int n = M.nbr * M.br;
     nc = n;
@@ -1229,6 +1346,7 @@ void amg_build(Hier &H, const DMat &fine, const nbp_options &o, int precision, c
             }
             make_lowcopies(L.M, precision, s);
             make_sell(L.M, precision, s);
+            if (k + 1 < H.nlev) make_ap(L, H.L[k + 1].M.nbr, precision, s);
             if (L.M.sl_ci) {   // grids of the sliced kernels, up to 8 threads per row
                 L.kpart_blocks = ((long long)L.M.nslice * L.M.sl_c * 8 + 255) / 256;
                 L.kpart = dmalloc<double>(2 * L.kpart_blocks, s);

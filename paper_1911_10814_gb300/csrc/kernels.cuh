@@ -20,7 +20,11 @@ namespace nbp {
 //   EPI_SET  y = Mx (+ rank-one term, LR)      EPI_ADD  y += Mx
 //   EPI_SUB  y -= Mx                           EPI_RES  y = b - Mx
 //   EPI_CHEB r = b - Mx; d = c1 d + c2 Dinv r; xout = x + d   (Chebyshev step)
-enum Epi { EPI_SET = 0, EPI_ADD = 1, EPI_SUB = 2, EPI_RES = 3, EPI_CHEB = 4 };
+//   EPI_POST M = A P, x = e the coarse correction, b the residual before the
+//            restriction: d = c2 Dinv (b - M e); xout = xin + P e + d, i.e. the
+//            prolongation and the first post-smoothing step (c1 = 0) in one
+//            (sliced kernel k_sellm only)
+enum Epi { EPI_SET = 0, EPI_ADD = 1, EPI_SUB = 2, EPI_RES = 3, EPI_CHEB = 4, EPI_POST = 5 };
 
 struct SpmvArgs {
     int nbr;
@@ -32,6 +36,8 @@ struct SpmvArgs {
     const void *dinv;       // EPI_CHEB: BR x BR per row (same type as vectors)
     void *d;                // EPI_CHEB: Chebyshev direction (in/out)
     void *xout;             // EPI_CHEB: x + d
+    const void *xin;        // EPI_POST: the iterate before the correction
+    const int *agg;         // EPI_POST: aggregate of each row (-1: none)
     double c1, c2;          // EPI_CHEB coefficients (FP64 vectors)
     float c1f, c2f;         // the same, pre-rounded for FP32 vectors (no FP64 work per element)
     const int *lr_rp, *lr_k, *lr_c;   // rank-one epilogue (EPI_SET only)
@@ -410,7 +416,7 @@ __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
     // latency-bound: fewer rows than the GPU has threads in flight)
     const bool own = h == 0 && live && row < a.nbr;
     AT eb[3] = {0, 0, 0}, ed[3] = {0, 0, 0}, ex[3] = {0, 0, 0}, edi[BB];
-    if (own && (EPI == EPI_RES || EPI == EPI_CHEB)) {
+    if (own && (EPI == EPI_RES || EPI == EPI_CHEB || EPI == EPI_POST)) {
 #pragma unroll
         for (int q = 0; q < BS; ++q) eb[q] = ((const XT *)a.b + col_off(a, a.b_ld))[(long long)row * BS + q];
     }
@@ -420,6 +426,17 @@ __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
         for (int q = 0; q < BS; ++q) {
             if (a.d_read) ed[q] = ((const XT *)a.d)[(long long)row * BS + q];
             ex[q] = ((const XT *)a.x + col_off(a, a.x_ld))[(long long)row * BS + q];
+        }
+#pragma unroll
+        for (int q = 0; q < BB; ++q) edi[q] = dv[q];
+    }
+    if (own && EPI == EPI_POST) {
+        const XT *dv = (const XT *)a.dinv + (long long)row * BB;
+        const int g = a.agg[row];
+#pragma unroll
+        for (int q = 0; q < BS; ++q) {
+            ex[q] = ((const XT *)a.xin)[(long long)row * BS + q];
+            if (g >= 0) ex[q] += ((const XT *)a.x)[(long long)g * BS + q];
         }
 #pragma unroll
         for (int q = 0; q < BB; ++q) edi[q] = dv[q];
@@ -460,7 +477,7 @@ __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
     if (!own) return;
     const AT accs[3] = {acc0, acc1, acc2};
     XT *y = (XT *)a.y;
-    if (EPI == EPI_CHEB) {
+    if (EPI == EPI_CHEB || EPI == EPI_POST) {
         XT *d = (XT *)a.d;
         XT *xo = (XT *)a.xout + col_off(a, a.out_ld);
         const AT c1 = sizeof(AT) == 4 ? (AT)a.c1f : (AT)a.c1, c2 = sizeof(AT) == 4 ? (AT)a.c2f : (AT)a.c2;
@@ -473,7 +490,7 @@ __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
 #pragma unroll
             for (int c = 0; c < BS; ++c) tq += edi[q * BS + c] * r[c];
             const long long idx = (long long)row * BS + q;
-            const AT dn = (a.d_read ? c1 * ed[q] : AT(0)) + c2 * tq;
+            const AT dn = (EPI == EPI_CHEB && a.d_read ? c1 * ed[q] : AT(0)) + c2 * tq;
             if (a.d_write) d[idx] = dn;
             xo[idx] = ex[q] + dn;
         }

@@ -151,6 +151,10 @@ struct Level {
     DMat M;
     int *agg = nullptr;                      // map to next level (-1 = left out)
     int *mptr = nullptr, *mem = nullptr;     // members of each next-level aggregate
+    // A P (rows of this level, columns of the next): the post-smoothing's first
+    // residual is r - (A P) e, with r that of before the restriction.  Sliced
+    // copies only; empty (no sl_ci) where it was not built
+    DMat AP;
     double *dinv = nullptr;                  // bs*bs per row
     float *dinv32 = nullptr;
     double rho = 0.0;

@@ -248,7 +248,7 @@ template <class F> static void timed(nbp_ctx *c, const char *tag, double bytes, 
 }
 
 static std::string mat_tag(nbp_ctx *c, const DMat &M, int epi) {
-    static const char *en[] = {"set", "add", "sub", "res", "cheb"};
+    static const char *en[] = {"set", "add", "sub", "res", "cheb", "post"};
     std::string t;
     if (&M == &c->A) t = "A";
     else if (&M == &c->B) t = "B";
@@ -817,6 +817,26 @@ static void vcycle_level(nbp_ctx *c, Hier &H, int l, int vsel, const T *b, T *ou
     // over each aggregate's members, was slower: uncoalesced fine updates)
     if (kc) kcycle_level<T>(c, H, l + 1, vsel, bc, xc, fuse);
     else vcycle_level<T>(c, H, l + 1, vsel, bc, xc, fuse);
+    if (k > 0 && L.AP.sl_ci) {   // prolongation and first post-smoothing step in one
+        const Cheb ch = cheb_of(L);
+        SpmvArgs a = sargs(xc, nullptr);
+        a.b = r; a.xin = cur; a.agg = L.agg; a.dinv = dinv_of<T>(L); a.d = wvec<T>(L, 4); a.xout = oth;
+        a.c2 = 1.0 / ch.theta;
+        a.c2f = (float)a.c2;
+        a.d_write = k > 1;
+        if (k == 1 && c->col.level == &L) {
+            a.xout = c->col.Z;
+            a.out_ld = c->col.ld;
+            a.jp = c->col.jp;
+        }
+        cudaEvent_t e0;
+        prof_begin(c, e0);
+        const double bytes = spmv_post<T>(L.AP, vsel, a, c->s);
+        prof_end(c, CAT_SPMV, bytes, c->prof.on ? mat_tag(c, L.M, EPI_POST) : std::string());
+        T *fin = chebyshev<T>(c, L, vsel, k, b, oth, cur, true, true, true);
+        if (fin != out) copy<T>(out, fin, n, c->s);
+        return;
+    }
     // prolongation bytes: the aggregate map, the coarse correction, x read and written
     const double pbytes = (double)L.M.nbr * 4.0 + ncv + 2.0 * n * sizeof(T);
     timed(c, "amg/prolong", pbytes, [&] {

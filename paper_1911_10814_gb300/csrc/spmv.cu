@@ -279,6 +279,55 @@ double spmv(const DMat &M, int vsel, SpmvArgs a, int epi, bool lr, cudaStream_t 
     return product_bytes(M, vsel, xs, epi, false);
 }
 
+// threads per row of the post-smoothing product (rows of A P hold 6-7 blocks,
+// those of S_hat P 10-20 scalars)
+static int post_threads(const DMat &AP) { return AP.nbr < 40000 ? 4 : AP.nbr < 400000 ? 2 : 1; }
+
+template <int BS, typename VT, typename XT>
+static void launch_post(const DMat &AP, const SpmvArgs &a, cudaStream_t s) {
+    const int T = post_threads(AP);
+    const unsigned grid = grid_exact((long long)AP.nslice * AP.sl_c * T);
+    auto go = [&](auto c, auto t) { k_sellm<BS, VT, XT, EPI_POST, decltype(c)::value, decltype(t)::value><<<grid, 256, 0, s>>>(a); };
+    auto with_t = [&](auto c) {
+        if (T == 4) go(c, std::integral_constant<int, 4>());
+        else if (T == 2) go(c, std::integral_constant<int, 2>());
+        else go(c, std::integral_constant<int, 1>());
+    };
+    if (AP.sl_c == 8) with_t(std::integral_constant<int, 8>());
+    else with_t(std::integral_constant<int, 32>());
+    NBP_LAUNCHED();
+}
+template <int BS, typename XT> static void launch_post_v(const DMat &AP, int vsel, SpmvArgs a, cudaStream_t s) {
+    if constexpr (sizeof(XT) == 8) {
+        a.val = AP.sl_v;
+        launch_post<BS, double, double>(AP, a, s);
+    } else if (vsel == 2) {
+        require(AP.sl_v16 != nullptr, NBP_ERR_STATE, "spmv: BF16 sliced values not built");
+        a.sl_ptr = AP.sl2_ptr;   // paired layout
+        a.sl_ci = AP.sl2_ci;
+        a.val = AP.sl_v16;
+        launch_post<BS, __nv_bfloat16, float>(AP, a, s);
+    } else {
+        require(AP.sl_v32 != nullptr, NBP_ERR_STATE, "spmv: FP32 sliced values not built");
+        a.val = AP.sl_v32;
+        launch_post<BS, float, float>(AP, a, s);
+    }
+}
+template <typename XT> double spmv_post(const DMat &AP, int vsel, SpmvArgs a, cudaStream_t s) {
+    a.nbr = AP.nbr;
+    a.nslice = AP.nslice;
+    a.sl_ptr = AP.sl_ptr;
+    a.sl_ci = AP.sl_ci;
+    if (AP.br == 3) launch_post_v<3, XT>(AP, vsel, a, s);
+    else launch_post_v<1, XT>(AP, vsel, a, s);
+    constexpr int xs = (int)sizeof(XT);
+    const double ny = (double)AP.nbr * AP.br * xs;
+    // the product's bytes (with b read and xout written), xin and the
+    // aggregates read, the block-diagonal inverse, d where it is written
+    return product_bytes(AP, vsel, xs, EPI_RES, true) + ny + (double)AP.nbr * 4.0 + ny * AP.br + (a.d_write ? ny : 0.0);
+}
+template double spmv_post<double>(const DMat &, int, SpmvArgs, cudaStream_t);
+template double spmv_post<float>(const DMat &, int, SpmvArgs, cudaStream_t);
 template double spmv<double>(const DMat &, int, SpmvArgs, int, bool, cudaStream_t, int);
 template double spmv<float>(const DMat &, int, SpmvArgs, int, bool, cudaStream_t, int);
 template double spmv_dot<double>(const DMat &, int, SpmvArgs, const DotArgs &, cudaStream_t);

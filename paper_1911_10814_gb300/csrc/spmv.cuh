@@ -26,5 +26,9 @@ bool spmv_dot_ok(const DMat &M, int vsel, int xbytes, long long max_blocks);
 template <typename XT>
 double spmv_dot(const DMat &M, int vsel, SpmvArgs a, const DotArgs &q, cudaStream_t s);
 
+// The prolongation and the first post-smoothing step (EPI_POST) with AP's
+// sliced copy; returns the algorithmic bytes.
+template <typename XT> double spmv_post(const DMat &AP, int vsel, SpmvArgs a, cudaStream_t s);
+
 
 }  // namespace nbp
