@@ -351,18 +351,20 @@ __global__ void __launch_bounds__(256) k_sell(SpmvArgs a) {
 }
 
 // Sliced-ELL product for the rectangular coupling blocks (B: 3x1, C: 1x3):
-// one thread per block row, slot values component-major as in k_sell (value
-// q = r BC + c of the C slots at (slot base) * BR BC + C q + t).  Epilogues
-// SET / ADD / SUB; FP64 or FP32 values.
-template <int BR, int BC, typename VT, typename XT, int EPI, int C>
+// T threads per block row as in k_sellm (T = 1: one), slot values
+// component-major as in k_sell (value q = r BC + c of the C slots at (slot
+// base) * BR BC + C q + t).  Epilogues SET / ADD / SUB; FP64 or FP32 values.
+template <int BR, int BC, typename VT, typename XT, int EPI, int C, int T>
 __global__ void __launch_bounds__(256) k_sellr(SpmvArgs a) {
     using AT = XT;
     constexpr int BB = BR * BC;
-    const int row = blockIdx.x * blockDim.x + threadIdx.x;
+    const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int row = (int)(gid / T), h = (int)(gid % T);
     const int sl = row / C, t = row % C;
-    if (sl >= a.nslice) return;
-    const long long base = a.sl_ptr[sl];
-    const int w = (int)((a.sl_ptr[sl + 1] - base) / C);
+    if (T == 1 && sl >= a.nslice) return;
+    const bool live = sl < a.nslice;   // T > 1: whole warps stay for the shuffles
+    const long long base = live ? a.sl_ptr[sl] : 0;
+    const int w = live ? (int)((a.sl_ptr[sl + 1] - base) / C) : 0;
     const VT *__restrict__ val = (const VT *)a.val;
     const int *__restrict__ ci = a.sl_ci;
     const XT *__restrict__ x = (const XT *)a.x + col_off(a, a.x_ld);
@@ -370,7 +372,7 @@ __global__ void __launch_bounds__(256) k_sellr(SpmvArgs a) {
 #pragma unroll
     for (int r = 0; r < BR; ++r) acc[r] = 0;
 #pragma unroll 2
-    for (int k = 0; k < w; ++k) {
+    for (int k = h; k < w; k += T) {
         const long long g = base + (long long)C * k;
         const int c = ldm<C == 32>(ci + g + t);
         const VT *v = val + g * BB + t;
@@ -385,7 +387,11 @@ __global__ void __launch_bounds__(256) k_sellr(SpmvArgs a) {
             acc[r] += u;
         }
     }
-    if (row >= a.nbr) return;
+#pragma unroll
+    for (int o = T / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int r = 0; r < BR; ++r) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
+    if (row >= a.nbr || h != 0) return;
     XT *y = (XT *)a.y;
 #pragma unroll
     for (int r = 0; r < BR; ++r) {
@@ -398,12 +404,11 @@ __global__ void __launch_bounds__(256) k_sellr(SpmvArgs a) {
 
 // Sliced-ELL product with T threads per block row (T = 2, 4, 8: thread h
 // takes slots h, h + T, ..., then an xor-shuffle tree over the T lanes), for
-// coarse levels whose rows are few, so that one thread per row leaves the
-// SMs with little memory parallelism.  No rank-one epilogue (coarse levels
-// need none).
+// levels whose rows are few, so that one thread per row leaves the SMs with
+// little memory parallelism.
 constexpr int kSellMT = 1000;   // DMat::tuned code kSellMT + T selects this kernel with T threads per row
 __host__ __device__ inline bool is_sellm(int g) { return g == kSellMT + 2 || g == kSellMT + 4 || g == kSellMT + 8; }
-template <int BS, typename VT, typename XT, int EPI, int C, int T>
+template <int BS, typename VT, typename XT, int EPI, int C, int T, bool LR = false>
 __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
     using AT = XT;
     constexpr int BB = BS * BS;
@@ -416,6 +421,7 @@ __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
     // latency-bound: fewer rows than the GPU has threads in flight)
     const bool own = h == 0 && live && row < a.nbr;
     AT eb[3] = {0, 0, 0}, ed[3] = {0, 0, 0}, ex[3] = {0, 0, 0}, edi[BB];
+    const int lr0 = LR && own ? a.lr_rp[row] : 0, lr1 = LR && own ? a.lr_rp[row + 1] : 0;
     if (own && (EPI == EPI_RES || EPI == EPI_CHEB || EPI == EPI_POST)) {
 #pragma unroll
         for (int q = 0; q < BS; ++q) eb[q] = ((const XT *)a.b + col_off(a, a.b_ld))[(long long)row * BS + q];
@@ -499,7 +505,16 @@ __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
 #pragma unroll
     for (int q = 0; q < BS; ++q) {
         const long long idx = (long long)row * BS + q;
-        if (EPI == EPI_SET) y[idx] = accs[q];
+        if (EPI == EPI_SET) {
+            AT s = accs[q];
+            if (LR && lr1 > lr0) {   // the rank-one term in FP64, on the rows that carry its entries (see k_sell)
+                double tt = 0.0;
+                for (int e = lr0; e < lr1; ++e)
+                    if (a.lr_c[e] == q) tt += a.lr_f[a.lr_k[e]] * a.lr_val[e];
+                s = (AT)((double)s + tt);
+            }
+            y[idx] = s;
+        }
         else if (EPI == EPI_ADD) y[idx] += accs[q];
         else if (EPI == EPI_SUB) y[idx] -= accs[q];
         else y[idx] = eb[q] - accs[q];
@@ -580,7 +595,7 @@ __device__ __forceinline__ void block_reduce_partials(const double *partial, int
     }
 }
 
-// out[col] = sum_b of the float-float partials of column col.  With 8, 4, 2
+// out[col] = sum_b of the float-float partials of column col.  With 4, 2
 // or 1 warps per column (few columns leave warps over), warp part p of a
 // column adds partials b = lane + 32 p, ... in ascending order, eight loads in
 // flight, then a fixed warp tree and the parts in order (one order whatever
@@ -588,7 +603,7 @@ __device__ __forceinline__ void block_reduce_partials(const double *partial, int
 __device__ __forceinline__ void block_reduce_partials_ff(const double *partial, int nb, int ncols, double *out) {
     __shared__ FF red[8];
     const int warp = threadIdx.x >> 5, ln = threadIdx.x & 31;
-    const int wpc = ncols <= 1 ? 8 : ncols <= 2 ? 4 : ncols <= 4 ? 2 : 1, step = 32 * wpc;
+    const int wpc = ncols <= 2 ? 4 : ncols <= 4 ? 2 : 1, step = 32 * wpc;
     for (int col = warp / wpc; col < ncols; col += 8 / wpc) {
         const float2 *p = reinterpret_cast<const float2 *>(partial + (long long)col * nb);
         FF a{0.f, 0.f};
@@ -814,22 +829,33 @@ struct GivensArgs {
 constexpr int kGivensCols = 64;
 struct GivensBuf {
     double h[kGivensCols], cs[kGivensCols], sn[kGivensCols];
-    double g;
+    double g, a;   // a: H(j, j) after the previous rotations (j < kGivensCols)
     GmDev dl;
     int j;
 };
+// by one warp, which also applies the previous rotations to the column: they
+// do not wait for the norm
 __device__ __forceinline__ void givens_stage(const GivensArgs &q, GivensBuf &B) {
-    const int j = q.dl ? q.dl->j : q.j;
-    if (threadIdx.x == 0) {
+    const int ln = threadIdx.x & 31, j = q.dl ? q.dl->j : q.j;
+    if (ln == 0) {
         B.j = j;
         B.g = q.g[j];
         if (q.dl) B.dl = *q.dl;
     }
-    if (j < kGivensCols)
-        for (int i = threadIdx.x; i <= j; i += blockDim.x) {
-            B.h[i] = q.h2 ? q.h1[i] + q.h2[i] : q.h1[i];
-            if (i < j) { B.cs[i] = q.cs[i]; B.sn[i] = q.sn[i]; }
-        }
+    if (j >= kGivensCols) return;
+    for (int i = ln; i <= j; i += 32) {
+        B.h[i] = q.h2 ? q.h1[i] + q.h2[i] : q.h1[i];
+        if (i < j) { B.cs[i] = q.cs[i]; B.sn[i] = q.sn[i]; }
+    }
+    __syncwarp();
+    if (ln != 0) return;
+    double a = B.h[0];
+    for (int i = 0; i < j; ++i) {
+        const double b = B.h[i + 1], c = B.cs[i], s = B.sn[i];
+        q.H[(long long)i * q.ldh + j] = c * a + s * b;
+        a = -s * a + c * b;
+    }
+    B.a = a;
 }
 
 // Column j of the Hessenberg matrix: H(i,j) = h1_i + h2_i (i <= j; h1_i
@@ -845,15 +871,9 @@ __device__ __forceinline__ void givens_step(const GivensArgs &q, const GivensBuf
     double *H = q.H;
     const long long ldh = q.ldh;
     const int j = B.j;
-    const double beta = (nrm2 >= 0.0) ? sqrt(nrm2) : nrm2;   // NaN passes through
     double a;   // H(j, j) after the previous rotations
     if (j < kGivensCols) {
-        a = B.h[0];
-        for (int i = 0; i < j; ++i) {
-            const double b = B.h[i + 1], c = B.cs[i], s = B.sn[i];
-            H[i * ldh + j] = c * a + s * b;
-            a = -s * a + c * b;
-        }
+        a = B.a;
     } else {
         for (int i = 0; i <= j; ++i) H[i * ldh + j] = q.h2 ? q.h1[i] + q.h2[i] : q.h1[i];
         for (int i = 0; i < j; ++i) {
@@ -863,9 +883,24 @@ __device__ __forceinline__ void givens_step(const GivensArgs &q, const GivensBuf
         }
         a = H[j * ldh + j];
     }
-    const double den = hypot(a, beta);
-    double c = 1.0, s = 0.0;
-    if (den != 0.0) { c = a / den; s = beta / den; }
+    // Away from under- and overflow from two independent reciprocal square
+    // roots: the square root, hypot and three divisions one after another took
+    // about 2 us of the pass (an FP64 operation waits tens of clocks here).
+    double beta, inv, den, c = 1.0, s = 0.0;
+    const double sq = a * a + nrm2;
+    if (nrm2 > 1e-280 && sq < 1e280) {
+        inv = rsqrt(nrm2);
+        const double r = rsqrt(sq);
+        beta = nrm2 * inv;
+        den = sq * r;
+        c = a * r;
+        s = beta * r;
+    } else {
+        beta = (nrm2 >= 0.0) ? sqrt(nrm2) : nrm2;   // NaN passes through
+        inv = beta == 0.0 ? 0.0 : 1.0 / beta;
+        den = hypot(a, beta);
+        if (den != 0.0) { c = a / den; s = beta / den; }
+    }
     q.cs[j] = c;
     q.sn[j] = s;
     H[j * ldh + j] = den;
@@ -877,7 +912,9 @@ __device__ __forceinline__ void givens_step(const GivensArgs &q, const GivensBuf
     const int nan = (isfinite(res) && isfinite(beta)) ? 0 : 1;
     q.st->res = res;
     q.st->nan = nan;
-    gm_set_beta(q.st, beta);
+    q.st->beta = beta;
+    q.st->inv = inv;
+    q.st->invf = (float)inv;
     if (q.dl) {
         const int its = B.dl.its + 1, nan_any = B.dl.nan | nan;
         q.dl->its = its;
@@ -895,7 +932,7 @@ template <typename T>
 __device__ __forceinline__ void finish_reduction(const double *partial, int ncols, double *out, unsigned *ticket,
                                                  const GivensArgs &gv) {
     __shared__ GivensBuf B;
-    if (gv.H) givens_stage(gv, B);
+    if (gv.H && threadIdx.x >> 5 == 7) givens_stage(gv, B);   // a warp that a norm's reduction leaves idle
     reduce_partials<T>(partial, gridDim.x, ncols, out);
     __syncthreads();
     if (threadIdx.x == 0) {

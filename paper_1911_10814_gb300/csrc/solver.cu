@@ -1901,11 +1901,13 @@ static void do_setup(nbp_ctx *c, bool numeric = false) {
         make_lowcopies(c->C, prec, s);
         make_lowcopies(c->D, prec, s);
     }
-    // kernel choice per matrix: the fine levels use the sliced-ELL kernel;
-    // coarse levels are tuned in place by timing whole AMG cycles
-    c->A.tuned = c->A.sl_ci ? 0 : -1;
-    for (DMat *M : {&c->B, &c->C, &c->D}) M->tuned = M->sl_ci ? 0 : -1;
-    for (Hier *H : {&c->HA, &c->HS}) H->L[0].M.tuned = H->L[0].M.sl_ci ? 0 : -1;
+    // kernel choice per matrix: the fine levels use the sliced-ELL kernels,
+    // threads per row by their size; coarse levels are tuned in place by timing
+    // whole AMG cycles
+    const int ft = fine_threads(c->N), fine = ft > 1 ? kSellMT + ft : 0;
+    c->A.tuned = c->A.sl_ci ? fine : -1;
+    for (DMat *M : {&c->B, &c->C, &c->D}) M->tuned = M->sl_ci ? fine : -1;
+    for (Hier *H : {&c->HA, &c->HS}) H->L[0].M.tuned = H->L[0].M.sl_ci ? fine : -1;
     if (prec >= 1) autotune_cycles<float>(c);
     else autotune_cycles<double>(c);
     NBP_CUDA(cudaStreamSynchronize(s));

@@ -68,6 +68,8 @@ static void launch_vt(const DMat &M, int vsel, SpmvArgs a, int G, int epi, bool 
     }
 }
 
+int fine_threads(int rows) { return rows < 10000 ? 8 : rows < 32000 ? 4 : rows < 80000 ? 2 : 1; }
+
 int choose_group(const DMat &M) {
     const double per_row = M.nbr ? (double)M.nnz * M.bb() / M.nbr : 0.0;
     if (per_row <= 10) return 4;
@@ -96,10 +98,15 @@ static void launch_sell_epi(const SpmvArgs &a, int epi, bool lr, cudaStream_t s)
 }
 
 template <int BS, typename VT, typename XT, int C, int T>
-static void launch_sellm_epi(const SpmvArgs &a, int epi, cudaStream_t s) {
+static void launch_sellm_epi(const SpmvArgs &a, int epi, bool lr, cudaStream_t s) {
     const unsigned grid = grid_exact((long long)a.nslice * C * T);
     switch (epi) {
-    case EPI_SET: k_sellm<BS, VT, XT, EPI_SET, C, T><<<grid, 256, 0, s>>>(a); break;
+    case EPI_SET:
+        if constexpr (BS == 3) {
+            if (lr) { k_sellm<BS, VT, XT, EPI_SET, C, T, true><<<grid, 256, 0, s>>>(a); break; }
+        }
+        k_sellm<BS, VT, XT, EPI_SET, C, T><<<grid, 256, 0, s>>>(a);
+        break;
     case EPI_ADD: k_sellm<BS, VT, XT, EPI_ADD, C, T><<<grid, 256, 0, s>>>(a); break;
     case EPI_SUB: k_sellm<BS, VT, XT, EPI_SUB, C, T><<<grid, 256, 0, s>>>(a); break;
     case EPI_RES: k_sellm<BS, VT, XT, EPI_RES, C, T><<<grid, 256, 0, s>>>(a); break;
@@ -110,19 +117,18 @@ static void launch_sellm_epi(const SpmvArgs &a, int epi, cudaStream_t s) {
 }
 
 template <int BS, typename VT, typename XT, int C>
-static void launch_sellm_t(const SpmvArgs &a, int epi, cudaStream_t s, int T) {
-    if (T == 8) launch_sellm_epi<BS, VT, XT, C, 8>(a, epi, s);
-    else if (T == 4) launch_sellm_epi<BS, VT, XT, C, 4>(a, epi, s);
-    else launch_sellm_epi<BS, VT, XT, C, 2>(a, epi, s);
+static void launch_sellm_t(const SpmvArgs &a, int epi, bool lr, cudaStream_t s, int T) {
+    if (T == 8) launch_sellm_epi<BS, VT, XT, C, 8>(a, epi, lr, s);
+    else if (T == 4) launch_sellm_epi<BS, VT, XT, C, 4>(a, epi, lr, s);
+    else launch_sellm_epi<BS, VT, XT, C, 2>(a, epi, lr, s);
 }
 
-// T threads per row (T = 1: the one-thread kernel, which also has the
-// rank-one epilogue)
+// T threads per row (T = 1: the one-thread kernel)
 template <int BS, typename VT, typename XT>
 static void launch_sell_c(const DMat &M, const SpmvArgs &a, int epi, bool lr, cudaStream_t s, int T) {
-    if (T > 1 && !lr) {
-        if (M.sl_c == 8) launch_sellm_t<BS, VT, XT, 8>(a, epi, s, T);
-        else launch_sellm_t<BS, VT, XT, 32>(a, epi, s, T);
+    if (T > 1) {
+        if (M.sl_c == 8) launch_sellm_t<BS, VT, XT, 8>(a, epi, lr, s, T);
+        else launch_sellm_t<BS, VT, XT, 32>(a, epi, lr, s, T);
         return;
     }
     if (M.sl_c == 8) launch_sell_epi<BS, VT, XT, 8>(a, epi, lr, s);
@@ -150,16 +156,25 @@ static void launch_sell(const DMat &M, int vsel, SpmvArgs a, int epi, bool lr, c
     }
 }
 
-template <int BR, int BC, typename VT, typename XT, int C>
-static void launch_sellr_epi(const SpmvArgs &a, int epi, cudaStream_t s) {
-    const unsigned grid = grid_exact((long long)a.nslice * C);
+template <int BR, int BC, typename VT, typename XT, int C, int T>
+static void launch_sellr_t(const SpmvArgs &a, int epi, cudaStream_t s) {
+    const unsigned grid = grid_exact((long long)a.nslice * C * T);
     switch (epi) {
-    case EPI_SET: k_sellr<BR, BC, VT, XT, EPI_SET, C><<<grid, 256, 0, s>>>(a); break;
-    case EPI_ADD: k_sellr<BR, BC, VT, XT, EPI_ADD, C><<<grid, 256, 0, s>>>(a); break;
-    case EPI_SUB: k_sellr<BR, BC, VT, XT, EPI_SUB, C><<<grid, 256, 0, s>>>(a); break;
+    case EPI_SET: k_sellr<BR, BC, VT, XT, EPI_SET, C, T><<<grid, 256, 0, s>>>(a); break;
+    case EPI_ADD: k_sellr<BR, BC, VT, XT, EPI_ADD, C, T><<<grid, 256, 0, s>>>(a); break;
+    case EPI_SUB: k_sellr<BR, BC, VT, XT, EPI_SUB, C, T><<<grid, 256, 0, s>>>(a); break;
     default: throw Error{NBP_ERR_INVALID, "spmv: rectangular blocks take SET, ADD or SUB"};
     }
     NBP_LAUNCHED();
+}
+template <int BR, int BC, typename VT, typename XT, int C>
+static void launch_sellr_epi(const SpmvArgs &a, int epi, cudaStream_t s) {
+    switch (fine_threads(a.nbr)) {
+    case 8: launch_sellr_t<BR, BC, VT, XT, C, 8>(a, epi, s); break;
+    case 4: launch_sellr_t<BR, BC, VT, XT, C, 4>(a, epi, s); break;
+    case 2: launch_sellr_t<BR, BC, VT, XT, C, 2>(a, epi, s); break;
+    default: launch_sellr_t<BR, BC, VT, XT, C, 1>(a, epi, s);
+    }
 }
 
 // rectangular blocks (3x1, 1x3) on their sliced-ELL copy, FP64 or FP32 values

@@ -16,6 +16,12 @@ double spmv(const DMat &M, int vsel, SpmvArgs a, int epi, bool lr, cudaStream_t 
 
 int choose_group(const DMat &M);
 
+// Threads per row of the finest level's products (A, its AMG level and the
+// coupling blocks, about 15 entries a row): one where the rows alone fill the
+// GPU (152 SMs x 2048 threads), up to eight where they do not and a row's
+// chain of loads is what a product takes.
+int fine_threads(int rows);
+
 // Whether y = M x with the K-cycle's inner products fused (k_sell_dot) runs
 // for this matrix: scalar blocks, the sliced kernel (1-8 threads per row) as
 // the tuned choice, the value copy of vsel built, and a grid of at most
