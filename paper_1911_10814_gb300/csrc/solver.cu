@@ -1268,6 +1268,11 @@ template <typename T> static void arnoldi_dl(nbp_ctx *c, Krylov<T> &K, GmDev *st
     gv.dl = st;
     gv.h = h;
     if (c->gs_one_pass) gv.h2 = nullptr;
+    if (vec && K.n <= gs_cluster_max<T>() && K.m <= kGsCols) {   // a short vector: the whole step in one cluster
+        k_gs_cluster<T><<<kGsCluster, kGsThreads, 0, c->s>>>(K.V, K.ld, jp, K.w, K.n, c->gs_one_pass ? 1 : 2, K.h1, K.h2, gv);
+        NBP_LAUNCHED();
+        return;
+    }
     // one pass: the multi-dot, then subtract + norm + Givens update
     const double *coef = c->gs_one_pass ? K.h1 : K.h2;
     if (vec) {

@@ -55,3 +55,14 @@ def test_odd_lengths(nx, ny, nz, precision, passes):
     s.setup()
     _check(d, s, torch.as_tensor(d["b"], device="cuda:0"))
     s.close()
+
+
+@pytest.mark.parametrize("nx,ny,nz,precision", [(21, 21, 21, 0), (22, 21, 21, 0), (26, 27, 27, 1), (27, 27, 27, 4)])
+def test_cluster_length(nx, ny, nz, precision):
+    """Either side of the longest vector (32,768 doubles, 65,536 floats) whose
+    step runs in one cluster: A-vectors of 31,944 / 33,396 and 63,504 / 65,856."""
+    d = synth.generate(synth.MeshSpec(nx, ny, nz, Re=400.0, seed=nx, R=(1e3,)))
+    s = Solver(d, precision=precision)
+    s.setup()
+    _check(d, s, torch.as_tensor(d["b"], device="cuda:0"))
+    s.close()
