@@ -1329,8 +1329,8 @@ void amg_build(Hier &H, const DMat &fine, const nbp_options &o, int precision, c
             L.w64[q] = dmalloc<double>(nv, s);
             L.w32[q] = dmalloc<float>(nv, s);
         }
-        L.kdots = dmalloc<double>(8 + 2 * kKdotBlocks, s);
-        NBP_CUDA(cudaMemsetAsync(L.kdots, 0, sizeof(double) * (8 + 2 * kKdotBlocks), s));
+        L.kdots = dmalloc<double>(8 + 3 * kKdotBlocks, s);
+        NBP_CUDA(cudaMemsetAsync(L.kdots, 0, sizeof(double) * (8 + 3 * kKdotBlocks), s));
         {   // every level, the coarsest included (it is smoothed when too large for a dense solve)
             L.dinv = dmalloc<double>(nv * bs, s);
             k_block_dinv<<<grid_exact(n), 256, 0, s>>>(n, bs, L.M.rp, L.M.ci, L.M.v, L.dinv, singular);
@@ -1349,7 +1349,7 @@ void amg_build(Hier &H, const DMat &fine, const nbp_options &o, int precision, c
             if (k + 1 < H.nlev) make_ap(L, H.L[k + 1].M.nbr, precision, s);
             if (L.M.sl_ci) {   // grids of the sliced kernels, up to 8 threads per row
                 L.kpart_blocks = ((long long)L.M.nslice * L.M.sl_c * 8 + 255) / 256;
-                L.kpart = dmalloc<double>(2 * L.kpart_blocks, s);
+                L.kpart = dmalloc<double>(3 * L.kpart_blocks, s);
             }
         }
     }

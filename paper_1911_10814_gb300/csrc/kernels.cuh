@@ -26,7 +26,7 @@ namespace nbp {
 //   EPI_POST M = A P, x = e the coarse correction, b the residual before the
 //            restriction: d = c2 Dinv (b - M e); xout = xin + P e + d, i.e. the
 //            prolongation and the first post-smoothing step (c1 = 0) in one
-//            (sliced kernel k_sellm only)
+//            (sliced kernels k_sell and k_sellm)
 enum Epi { EPI_SET = 0, EPI_ADD = 1, EPI_SUB = 2, EPI_RES = 3, EPI_CHEB = 4, EPI_POST = 5 };
 
 struct SpmvArgs {
@@ -71,7 +71,11 @@ __global__ void __launch_bounds__(256) k_bspmv(SpmvArgs a) {
     const int cnt = (__ldg(a.rp + row + 1) - e0) * BB;
     const VT *__restrict__ val = (const VT *)a.val + (long long)e0 * BB;
     const int *__restrict__ ci = a.ci + e0;
-    const XT *__restrict__ x = (const XT *)a.x + col_off(a, a.x_ld);
+    // the first entry's value and column before the wait
+    const VT v0 = lane < cnt ? __ldg(val + lane) : VT(0.f);
+    const int c0 = lane < cnt ? __ldg(ci + lane / BB) : 0;
+    pdl_wait();
+    const XT *x = (const XT *)a.x + col_off(a, a.x_ld);
     AT acc0 = 0, acc1 = 0, acc2 = 0;
 #pragma unroll 4
     for (int v = lane; v < cnt; v += G) {
@@ -79,7 +83,8 @@ __global__ void __launch_bounds__(256) k_bspmv(SpmvArgs a) {
         const int rc = v - e * BB;
         const int r = rc / BC;
         const int c = rc - r * BC;
-        const AT p = cvt<AT>(__ldg(val + v)) * __ldg(x + (long long)__ldg(ci + e) * BC + c);
+        const bool first = v == lane;
+        const AT p = cvt<AT>(first ? v0 : __ldg(val + v)) * x[(long long)(first ? c0 : __ldg(ci + e)) * BC + c];
         if (BR == 1) acc0 += p;
         else {
             acc0 += (r == 0) ? p : AT(0);
@@ -136,6 +141,10 @@ __global__ void __launch_bounds__(256) k_bspmv(SpmvArgs a) {
     }
 }
 
+// What a solve writes (x, b, d, bases, ...) is read with plain loads, never
+// through the read-only path: in a device-driven loop a kernel may have started
+// before its predecessor wrote it (see pdl_wait).
+//
 // Streamed loads of matrix values and columns: each is read once per
 // product, so they can bypass L1 allocation (ld.global.nc.L1::no_allocate)
 // and leave L1 to the x gathers, which neighbouring rows share.
@@ -186,15 +195,15 @@ template <bool STREAM, typename P> __device__ __forceinline__ P ldm(const P *p) 
 // One pair of slots of the paired BF16 layout: columns c, values m, added in
 // slot order (the first slot of the pair, then the second).
 template <int BS>
-__device__ __forceinline__ void pair_fma(const int2 c, const __nv_bfloat162 (&m)[BS * BS], const float *__restrict__ x,
+__device__ __forceinline__ void pair_fma(const int2 c, const __nv_bfloat162 (&m)[BS * BS], const float *x,
                                          float &acc0, float &acc1, float &acc2) {
     if (BS == 1) {
         const float2 mm = __bfloat1622float2(m[0]);
-        acc0 += mm.x * __ldg(x + c.x);
-        acc0 += mm.y * __ldg(x + c.y);
+        acc0 += mm.x * x[c.x];
+        acc0 += mm.y * x[c.y];
     } else {
-        const float xa0 = __ldg(x + 3LL * c.x), xa1 = __ldg(x + 3LL * c.x + 1), xa2 = __ldg(x + 3LL * c.x + 2);
-        const float xb0 = __ldg(x + 3LL * c.y), xb1 = __ldg(x + 3LL * c.y + 1), xb2 = __ldg(x + 3LL * c.y + 2);
+        const float xa0 = x[3LL * c.x], xa1 = x[3LL * c.x + 1], xa2 = x[3LL * c.x + 2];
+        const float xb0 = x[3LL * c.y], xb1 = x[3LL * c.y + 1], xb2 = x[3LL * c.y + 2];
         float2 mm[9];
 #pragma unroll
         for (int q = 0; q < 9; ++q) mm[q] = __bfloat1622float2(m[q]);
@@ -209,38 +218,39 @@ __device__ __forceinline__ void pair_fma(const int2 c, const __nv_bfloat162 (&m)
 
 // Slots p0, p0 + step, ... of the paired BF16 layout (DMat::sl2_ptr) of one
 // row: per pair, one int2 of columns and one bf16x2 per component; the two
-// slots are added in slot order, as the unpaired loop adds them.  Two pairs
-// are loaded before either is used (more loads in flight per thread); the
-// pairs are still added in ascending order.
-template <int BS, int C>
-__device__ __forceinline__ void sell_pairs(const SpmvArgs &a, long long base2, int np, int t, int p0, int step,
-                                           const float *__restrict__ x, float &acc0, float &acc1, float &acc2) {
+// slots are added in slot order, as the unpaired loop adds them.  Several pairs
+// (PairBatch) are loaded before any is used (more loads in flight per thread);
+// the pairs are still added in ascending order.  The first batch is loaded
+// by sell_pairs_load, before the kernel waits for its predecessor.
+// 32-row slices (the fine level, HBM-bound): two pairs per step; 8-row slices
+// (coarse levels) measured faster one pair at a time.
+template <int BS, int C, int K = C == 32 ? 2 : 1> struct PairBatch {
+    int2 c[K];
+    __nv_bfloat162 m[K][BS * BS];
+};
+template <int BS, int C, int K>
+__device__ __forceinline__ void sell_pairs_load(PairBatch<BS, C, K> &B, const SpmvArgs &a, long long base2, int np, int t, int p,
+                                                int step) {
     constexpr int BB = BS * BS;
     const __nv_bfloat162 *__restrict__ val = (const __nv_bfloat162 *)a.val;
     const int2 *__restrict__ ci = (const int2 *)a.sl_ci;
-    int p = p0;
-    // 32-row slices (the fine level, HBM-bound): two pairs per step; 8-row
-    // slices (coarse levels) measured faster one pair at a time
-    if (C == 32) {
-        for (; p + step < np; p += 2 * step) {
-            const long long g0 = base2 + (long long)C * p, g1 = g0 + (long long)C * step;
-            const int2 c0 = ldm<C == 32>(ci + g0 + t), c1 = ldm<C == 32>(ci + g1 + t);
-            __nv_bfloat162 m0[BB], m1[BB];
 #pragma unroll
-            for (int q = 0; q < BB; ++q) m0[q] = ldm<C == 32>(val + g0 * BB + t + q * C);
+    for (int u = 0; u < K; ++u) {
+        if (p + u * step >= np) break;
+        const long long g = base2 + (long long)C * (p + u * step);
+        B.c[u] = ldm<C == 32>(ci + g + t);
 #pragma unroll
-            for (int q = 0; q < BB; ++q) m1[q] = ldm<C == 32>(val + g1 * BB + t + q * C);
-            pair_fma<BS>(c0, m0, x, acc0, acc1, acc2);
-            pair_fma<BS>(c1, m1, x, acc0, acc1, acc2);
-        }
+        for (int q = 0; q < BB; ++q) B.m[u][q] = ldm<C == 32>(val + g * BB + t + q * C);
     }
-    for (; p < np; p += step) {
-        const long long g0 = base2 + (long long)C * p;
-        const int2 c0 = ldm<C == 32>(ci + g0 + t);
-        __nv_bfloat162 m0[BB];
+}
+template <int BS, int C, int K>
+__device__ __forceinline__ void sell_pairs(PairBatch<BS, C, K> &B, const SpmvArgs &a, long long base2, int np, int t, int p0,
+                                           int step, const float *x, float &acc0, float &acc1, float &acc2) {
+    for (int p = p0; p < np; p += K * step) {
+        if (p != p0) sell_pairs_load(B, a, base2, np, t, p, step);
 #pragma unroll
-        for (int q = 0; q < BB; ++q) m0[q] = ldm<C == 32>(val + g0 * BB + t + q * C);
-        pair_fma<BS>(c0, m0, x, acc0, acc1, acc2);
+        for (int u = 0; u < K; ++u)
+            if (p + u * step < np) pair_fma<BS>(B.c[u], B.m[u], x, acc0, acc1, acc2);
     }
 }
 
@@ -248,14 +258,14 @@ __device__ __forceinline__ void sell_pairs(const SpmvArgs &a, long long base2, i
 // columns at sl_ci[g + t] and value q at val[g bb + C q + t] (int and bf16
 // units), g = the slice's slot offset + C (width - 1).
 template <int BS, int C>
-__device__ __forceinline__ void sell_single(const SpmvArgs &a, long long g, int t, const float *__restrict__ x,
+__device__ __forceinline__ void sell_single(const SpmvArgs &a, long long g, int t, const float *x,
                                             float &acc0, float &acc1, float &acc2) {
     const __nv_bfloat16 *__restrict__ val = (const __nv_bfloat16 *)a.val + g * (BS * BS) + t;
     const int c = ldm<C == 32>(a.sl_ci + g + t);
     if (BS == 1) {
-        acc0 += __bfloat162float(ldm<C == 32>(val)) * __ldg(x + c);
+        acc0 += __bfloat162float(ldm<C == 32>(val)) * x[c];
     } else {
-        const float x0 = __ldg(x + 3LL * c), x1 = __ldg(x + 3LL * c + 1), x2 = __ldg(x + 3LL * c + 2);
+        const float x0 = x[3LL * c], x1 = x[3LL * c + 1], x2 = x[3LL * c + 2];
         float m[9];
 #pragma unroll
         for (int q = 0; q < 9; ++q) m[q] = __bfloat162float(ldm<C == 32>(val + q * C));
@@ -265,12 +275,38 @@ __device__ __forceinline__ void sell_single(const SpmvArgs &a, long long g, int 
     }
 }
 
+// One slot of the unpaired layouts: its column and the block's values
+template <int BB, typename VT> struct SlotBatch {
+    int c;
+    VT m[BB];
+};
+template <int BB, int C, typename VT>
+__device__ __forceinline__ void slot_load(SlotBatch<BB, VT> &B, const VT *__restrict__ val, const int *__restrict__ ci,
+                                          long long base, int t, int k) {
+    const long long g = base + (long long)C * k;
+    B.c = ldm<C == 32>(ci + g + t);
+#pragma unroll
+    for (int q = 0; q < BB; ++q) B.m[q] = ldm<C == 32>(val + g * BB + t + q * C);
+}
+template <int BS, typename VT, typename AT>
+__device__ __forceinline__ void slot_fma(const SlotBatch<BS * BS, VT> &B, const AT *x, AT &acc0, AT &acc1,
+                                         AT &acc2) {
+    if constexpr (BS == 1) {
+        acc0 += cvt<AT>(B.m[0]) * x[B.c];
+    } else {
+        const AT x0 = x[3LL * B.c], x1 = x[3LL * B.c + 1], x2 = x[3LL * B.c + 2];
+        acc0 += cvt<AT>(B.m[0]) * x0 + cvt<AT>(B.m[1]) * x1 + cvt<AT>(B.m[2]) * x2;
+        acc1 += cvt<AT>(B.m[3]) * x0 + cvt<AT>(B.m[4]) * x1 + cvt<AT>(B.m[5]) * x2;
+        acc2 += cvt<AT>(B.m[6]) * x0 + cvt<AT>(B.m[7]) * x1 + cvt<AT>(B.m[8]) * x2;
+    }
+}
+
 // Sliced-ELL product for square BS x BS blocks: one thread per block row, C
 // rows per slice (C = 32: a warp per slice; C = 8 for matrices whose row
 // lengths vary, to cut padding).  Every load of values and columns by the C
 // threads of a slice is one contiguous segment (C x value bytes).  Same
 // epilogues as k_bspmv (a.rp unused; a.sl_* describe the slices).
-template <int BS, typename VT, typename XT, int EPI, bool LR, int C>
+template <int BS, typename VT, typename XT, int EPI, bool LR, int C, int K = C == 32 ? 2 : 1>
 __global__ void __launch_bounds__(256) k_sell(SpmvArgs a) {
     using AT = XT;
     constexpr int BB = BS * BS;
@@ -281,30 +317,57 @@ __global__ void __launch_bounds__(256) k_sell(SpmvArgs a) {
     const int w = (int)((a.sl_ptr[sl + 1] - base) / C);
     const VT *__restrict__ val = (const VT *)a.val;
     const int *__restrict__ ci = a.sl_ci;
-    const XT *__restrict__ x = (const XT *)a.x + col_off(a, a.x_ld);
     AT acc0 = 0, acc1 = 0, acc2 = 0;
     if constexpr (std::is_same<VT, __nv_bfloat16>::value) {   // paired layout: w / 2 pairs, then one slot if w is odd
-        sell_pairs<BS, C>(a, base / 2, w / 2, t, 0, 1, x, acc0, acc1, acc2);
+        PairBatch<BS, C, K> pb;
+        sell_pairs_load(pb, a, base / 2, w / 2, t, 0, 1);
+        pdl_wait();
+        const XT *x = (const XT *)a.x + col_off(a, a.x_ld);
+        sell_pairs(pb, a, base / 2, w / 2, t, 0, 1, x, acc0, acc1, acc2);
         if (w & 1) sell_single<BS, C>(a, base + (long long)C * (w - 1), t, x, acc0, acc1, acc2);
     } else {
+        SlotBatch<BB, VT> sb;
+        if (w > 0) slot_load<BB, C>(sb, val, ci, base, t, 0);
+        pdl_wait();
+        const XT *x = (const XT *)a.x + col_off(a, a.x_ld);
+        if (w > 0) slot_fma<BS, VT, AT>(sb, x, acc0, acc1, acc2);
 #pragma unroll 2
-        for (int k = 0; k < w; ++k) {
-            const long long g = base + (long long)C * k;
-            const int c = ldm<C == 32>(ci + g + t);
-            const VT *v = val + g * BB + t;
-            if (BS == 1) {
-                acc0 += cvt<AT>(ldm<C == 32>(v)) * __ldg(x + c);
-            } else {
-                const AT x0 = __ldg(x + 3LL * c), x1 = __ldg(x + 3LL * c + 1), x2 = __ldg(x + 3LL * c + 2);
-                acc0 += cvt<AT>(ldm<C == 32>(v)) * x0 + cvt<AT>(ldm<C == 32>(v + C)) * x1 + cvt<AT>(ldm<C == 32>(v + 2 * C)) * x2;
-                acc1 += cvt<AT>(ldm<C == 32>(v + 3 * C)) * x0 + cvt<AT>(ldm<C == 32>(v + 4 * C)) * x1 + cvt<AT>(ldm<C == 32>(v + 5 * C)) * x2;
-                acc2 += cvt<AT>(ldm<C == 32>(v + 6 * C)) * x0 + cvt<AT>(ldm<C == 32>(v + 7 * C)) * x1 + cvt<AT>(ldm<C == 32>(v + 8 * C)) * x2;
-            }
+        for (int k = 1; k < w; ++k) {
+            SlotBatch<BB, VT> u;
+            slot_load<BB, C>(u, val, ci, base, t, k);
+            slot_fma<BS, VT, AT>(u, x, acc0, acc1, acc2);
         }
     }
+    const XT *x = (const XT *)a.x + col_off(a, a.x_ld);
     if (row >= a.nbr) return;
     AT accs[3] = {acc0, acc1, acc2};
     XT *y = (XT *)a.y;
+    if (EPI == EPI_POST) {
+        const XT *b = (const XT *)a.b;
+        const XT *dinv = (const XT *)a.dinv + (long long)row * BB;
+        const XT *xi = (const XT *)a.xin;
+        XT *xo = (XT *)a.xout + col_off(a, a.out_ld);
+        const int g = a.agg[row];
+        const AT c2 = sizeof(AT) == 4 ? (AT)a.c2f : (AT)a.c2;
+        AT r[3], e[3];
+#pragma unroll
+        for (int q = 0; q < BS; ++q) {
+            r[q] = b[(long long)row * BS + q] - accs[q];
+            e[q] = xi[(long long)row * BS + q];
+            if (g >= 0) e[q] += x[(long long)g * BS + q];
+        }
+#pragma unroll
+        for (int q = 0; q < BS; ++q) {
+            AT tq = 0;
+#pragma unroll
+            for (int c = 0; c < BS; ++c) tq += dinv[q * BS + c] * r[c];
+            const long long idx = (long long)row * BS + q;
+            const AT dn = c2 * tq;
+            if (a.d_write) ((XT *)a.d)[idx] = dn;
+            xo[idx] = e[q] + dn;
+        }
+        return;
+    }
     const bool lr = LR && EPI == EPI_SET;
     const int lr0 = lr ? a.lr_rp[row] : 0, lr1 = lr ? a.lr_rp[row + 1] : 0;
     if (EPI == EPI_CHEB) {
@@ -370,25 +433,31 @@ __global__ void __launch_bounds__(256) k_sellr(SpmvArgs a) {
     const int w = live ? (int)((a.sl_ptr[sl + 1] - base) / C) : 0;
     const VT *__restrict__ val = (const VT *)a.val;
     const int *__restrict__ ci = a.sl_ci;
-    const XT *__restrict__ x = (const XT *)a.x + col_off(a, a.x_ld);
+    SlotBatch<BB, VT> sb;
+    if (h < w) slot_load<BB, C>(sb, val, ci, base, t, h);
+    pdl_wait();
+    const XT *x = (const XT *)a.x + col_off(a, a.x_ld);
     AT acc[BR];
 #pragma unroll
     for (int r = 0; r < BR; ++r) acc[r] = 0;
-#pragma unroll 2
-    for (int k = h; k < w; k += T) {
-        const long long g = base + (long long)C * k;
-        const int c = ldm<C == 32>(ci + g + t);
-        const VT *v = val + g * BB + t;
+    auto add = [&](const SlotBatch<BB, VT> &s) {
         AT xs[BC];
 #pragma unroll
-        for (int cc = 0; cc < BC; ++cc) xs[cc] = __ldg(x + (long long)BC * c + cc);
+        for (int cc = 0; cc < BC; ++cc) xs[cc] = x[(long long)BC * s.c + cc];
 #pragma unroll
         for (int r = 0; r < BR; ++r) {
             AT u = 0;
 #pragma unroll
-            for (int cc = 0; cc < BC; ++cc) u += cvt<AT>(ldm<C == 32>(v + (r * BC + cc) * C)) * xs[cc];
+            for (int cc = 0; cc < BC; ++cc) u += cvt<AT>(s.m[r * BC + cc]) * xs[cc];
             acc[r] += u;
         }
+    };
+    if (h < w) add(sb);
+#pragma unroll 2
+    for (int k = h + T; k < w; k += T) {
+        SlotBatch<BB, VT> u;
+        slot_load<BB, C>(u, val, ci, base, t, k);
+        add(u);
     }
 #pragma unroll
     for (int o = T / 2; o > 0; o >>= 1)
@@ -411,7 +480,7 @@ __global__ void __launch_bounds__(256) k_sellr(SpmvArgs a) {
 // little memory parallelism.
 constexpr int kSellMT = 1000;   // DMat::tuned code kSellMT + T selects this kernel with T threads per row
 __host__ __device__ inline bool is_sellm(int g) { return g == kSellMT + 2 || g == kSellMT + 4 || g == kSellMT + 8; }
-template <int BS, typename VT, typename XT, int EPI, int C, int T, bool LR = false>
+template <int BS, typename VT, typename XT, int EPI, int C, int T, bool LR = false, int K = C == 32 ? 2 : 1>
 __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
     using AT = XT;
     constexpr int BB = BS * BS;
@@ -419,60 +488,62 @@ __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
     const int row = (int)(gid / T), h = (int)(gid % T);
     const int sl = row / C, t = row % C;
     const bool live = sl < a.nslice;
+    // everything that the solve does not write first (see pdl_wait): the slice,
+    // the first slots, the block-diagonal inverse, the row's aggregate
+    const bool own = h == 0 && live && row < a.nbr;
+    const long long base = live ? a.sl_ptr[sl] : 0;
+    const int w = live ? (int)((a.sl_ptr[sl + 1] - base) / C) : 0;
+    const VT *__restrict__ val = (const VT *)a.val;
+    const int *__restrict__ ci = a.sl_ci;
+    constexpr bool PAIRED = std::is_same<VT, __nv_bfloat16>::value;
+    PairBatch<BS, C, K> pb;
+    SlotBatch<BB, VT> sb;
+    if constexpr (PAIRED) sell_pairs_load(pb, a, base / 2, w / 2, t, h, T);   // the T threads take alternate pairs
+    else if (h < w) slot_load<BB, C>(sb, val, ci, base, t, h);
+    AT edi[BB];
+    int agg = -1;
+    if (own && (EPI == EPI_CHEB || EPI == EPI_POST)) {
+        const XT *dv = (const XT *)a.dinv + (long long)row * BB;
+#pragma unroll
+        for (int q = 0; q < BB; ++q) edi[q] = dv[q];
+        if (EPI == EPI_POST) agg = a.agg[row];
+    }
+    const int lr0 = LR && own ? a.lr_rp[row] : 0, lr1 = LR && own ? a.lr_rp[row + 1] : 0;
+    pdl_wait();
     // the row's own epilogue operands are loaded before the slot loop, so that
     // their latency overlaps the gather chain (these small levels are
     // latency-bound: fewer rows than the GPU has threads in flight)
-    const bool own = h == 0 && live && row < a.nbr;
-    AT eb[3] = {0, 0, 0}, ed[3] = {0, 0, 0}, ex[3] = {0, 0, 0}, edi[BB];
-    const int lr0 = LR && own ? a.lr_rp[row] : 0, lr1 = LR && own ? a.lr_rp[row + 1] : 0;
+    const XT *x = (const XT *)a.x + col_off(a, a.x_ld);
+    AT eb[3] = {0, 0, 0}, ed[3] = {0, 0, 0}, ex[3] = {0, 0, 0};
     if (own && (EPI == EPI_RES || EPI == EPI_CHEB || EPI == EPI_POST)) {
 #pragma unroll
         for (int q = 0; q < BS; ++q) eb[q] = ((const XT *)a.b + col_off(a, a.b_ld))[(long long)row * BS + q];
     }
     if (own && EPI == EPI_CHEB) {
-        const XT *dv = (const XT *)a.dinv + (long long)row * BB;
 #pragma unroll
         for (int q = 0; q < BS; ++q) {
             if (a.d_read) ed[q] = ((const XT *)a.d)[(long long)row * BS + q];
-            ex[q] = ((const XT *)a.x + col_off(a, a.x_ld))[(long long)row * BS + q];
+            ex[q] = x[(long long)row * BS + q];
         }
-#pragma unroll
-        for (int q = 0; q < BB; ++q) edi[q] = dv[q];
     }
     if (own && EPI == EPI_POST) {
-        const XT *dv = (const XT *)a.dinv + (long long)row * BB;
-        const int g = a.agg[row];
 #pragma unroll
         for (int q = 0; q < BS; ++q) {
             ex[q] = ((const XT *)a.xin)[(long long)row * BS + q];
-            if (g >= 0) ex[q] += ((const XT *)a.x)[(long long)g * BS + q];
+            if (agg >= 0) ex[q] += x[(long long)agg * BS + q];
         }
-#pragma unroll
-        for (int q = 0; q < BB; ++q) edi[q] = dv[q];
     }
-    const long long base = live ? a.sl_ptr[sl] : 0;
-    const int w = live ? (int)((a.sl_ptr[sl + 1] - base) / C) : 0;
-    const VT *__restrict__ val = (const VT *)a.val;
-    const int *__restrict__ ci = a.sl_ci;
-    const XT *__restrict__ x = (const XT *)a.x + col_off(a, a.x_ld);
     AT acc0 = 0, acc1 = 0, acc2 = 0;
-    if constexpr (std::is_same<VT, __nv_bfloat16>::value) {   // paired layout: the T threads take alternate pairs
-        sell_pairs<BS, C>(a, base / 2, w / 2, t, h, T, x, acc0, acc1, acc2);
+    if constexpr (PAIRED) {
+        sell_pairs(pb, a, base / 2, w / 2, t, h, T, x, acc0, acc1, acc2);
         // an odd width's last slot goes to the thread whose turn comes next
         if ((w & 1) && h == (w / 2) % T) sell_single<BS, C>(a, base + (long long)C * (w - 1), t, x, acc0, acc1, acc2);
     } else {
-        for (int k = h; k < w; k += T) {
-            const long long g = base + (long long)C * k;
-            const int c = ldm<C == 32>(ci + g + t);
-            const VT *v = val + g * BB + t;
-            if (BS == 1) {
-                acc0 += cvt<AT>(ldm<C == 32>(v)) * __ldg(x + c);
-            } else {
-                const AT x0 = __ldg(x + 3LL * c), x1 = __ldg(x + 3LL * c + 1), x2 = __ldg(x + 3LL * c + 2);
-                acc0 += cvt<AT>(ldm<C == 32>(v)) * x0 + cvt<AT>(ldm<C == 32>(v + C)) * x1 + cvt<AT>(ldm<C == 32>(v + 2 * C)) * x2;
-                acc1 += cvt<AT>(ldm<C == 32>(v + 3 * C)) * x0 + cvt<AT>(ldm<C == 32>(v + 4 * C)) * x1 + cvt<AT>(ldm<C == 32>(v + 5 * C)) * x2;
-                acc2 += cvt<AT>(ldm<C == 32>(v + 6 * C)) * x0 + cvt<AT>(ldm<C == 32>(v + 7 * C)) * x1 + cvt<AT>(ldm<C == 32>(v + 8 * C)) * x2;
-            }
+        if (h < w) slot_fma<BS, VT, AT>(sb, x, acc0, acc1, acc2);
+        for (int k = h + T; k < w; k += T) {
+            SlotBatch<BB, VT> u;
+            slot_load<BB, C>(u, val, ci, base, t, k);
+            slot_fma<BS, VT, AT>(u, x, acc0, acc1, acc2);
         }
     }
 #pragma unroll
@@ -727,19 +798,17 @@ __device__ __forceinline__ void block_partials(const T (&acc)[NQ], int nq, doubl
 }
 
 // Scalar-block (Ŝ level) sliced-ELL product y = M x fused with the inner
-// products the K-cycle takes of it: kd[o0] = y . da and, when db is set,
-// kd[o1] = y . db (da may be y itself).  T threads per row as in k_sellm
-// (T = 1: one thread per row); each row's sum is the same as the unfused
-// kernels'.  The row products are summed per warp in FP64, per block in a
-// fixed order into part[b] and part[nb + b], and the last block to finish
-// (ticket kd[7]) adds the block partials in a fixed order -- one launch
-// instead of a product and a reduction, the same result whatever the order
-// the blocks run in.
+// products the K-cycle takes of it: y . y, y . da and, when db is set, y . db.
+// T threads per row as in k_sellm (T = 1: one thread per row); each row's sum
+// is the same as the unfused kernels'.  The row products are summed per block
+// (block_partials) into part, and the last block to finish (ticket kd[7])
+// adds the block partials in a fixed order -- one launch instead of a product
+// and a reduction, the same result whatever the order the blocks run in.
 struct DotArgs {
     const void *da, *db;   // vectors the product is dotted with (same type as y); db may be null
-    double *part;          // 2 x gridDim.x block partials
-    double *kd;            // results kd[o0], kd[o1]; kd[7] is the ticket
-    int o0, o1;
+    double *part;          // 3 x gridDim.x block partials
+    double *kd;            // results; kd[7] is the ticket
+    int oy, oa, ob;        // kd[oy] = y . y, kd[oa] = y . da, kd[ob] = y . db
 };
 template <typename VT, typename XT, int C, int T>
 __global__ void __launch_bounds__(256) k_sell_dot(SpmvArgs a, DotArgs q) {
@@ -751,35 +820,45 @@ __global__ void __launch_bounds__(256) k_sell_dot(SpmvArgs a, DotArgs q) {
     const long long base = live ? a.sl_ptr[sl] : 0;
     const int w = live ? (int)((a.sl_ptr[sl + 1] - base) / C) : 0;
     const VT *__restrict__ val = (const VT *)a.val;
-    const XT *__restrict__ x = (const XT *)a.x;
+    const XT *x = (const XT *)a.x;
     AT acc0 = 0, acc1 = 0, acc2 = 0;
     if constexpr (std::is_same<VT, __nv_bfloat16>::value) {
-        sell_pairs<1, C>(a, base / 2, w / 2, t, h, T, x, acc0, acc1, acc2);
+        PairBatch<1, C> pb;
+        sell_pairs_load(pb, a, base / 2, w / 2, t, h, T);
+        pdl_wait();
+        sell_pairs(pb, a, base / 2, w / 2, t, h, T, x, acc0, acc1, acc2);
         if ((w & 1) && h == (w / 2) % T) sell_single<1, C>(a, base + (long long)C * (w - 1), t, x, acc0, acc1, acc2);
     } else {
-        for (int k = h; k < w; k += T) {
-            const long long g = base + (long long)C * k;
-            acc0 += cvt<AT>(ldm<C == 32>(val + g + t)) * __ldg(x + ldm<C == 32>(a.sl_ci + g + t));
+        SlotBatch<1, VT> sb;
+        if (h < w) slot_load<1, C>(sb, val, a.sl_ci, base, t, h);
+        pdl_wait();
+        if (h < w) slot_fma<1, VT, AT>(sb, x, acc0, acc1, acc2);
+        for (int k = h + T; k < w; k += T) {
+            SlotBatch<1, VT> u;
+            slot_load<1, C>(u, val, a.sl_ci, base, t, k);
+            slot_fma<1, VT, AT>(u, x, acc0, acc1, acc2);
         }
     }
 #pragma unroll
     for (int o = T / 2; o > 0; o >>= 1) acc0 += __shfl_xor_sync(0xffffffffu, acc0, o);
-    AT p0 = 0, p1 = 0;
+    AT pp[4] = {0, 0, 0, 0};
     if (h == 0 && live && row < a.nbr) {
         ((XT *)a.y)[row] = acc0;
-        p0 = acc0 * (q.da == a.y ? acc0 : ((const XT *)q.da)[row]);
-        if (q.db) p1 = acc0 * ((const XT *)q.db)[row];
+        pp[0] = acc0 * acc0;
+        pp[1] = acc0 * ((const XT *)q.da)[row];
+        if (q.db) pp[2] = acc0 * ((const XT *)q.db)[row];
     }
-    const AT pp[2] = {p0, p1};
-    block_partials<AT, 2>(pp, 2, q.part, 0);
+    const int nq = q.db ? 3 : 2;
+    block_partials<AT, 4>(pp, nq, q.part, 0);
     unsigned *ticket = (unsigned *)(q.kd + 7);
     if (!grid_last_block(ticket)) return;
-    __shared__ double out[2];
-    reduce_partials<AT>(q.part, gridDim.x, q.db ? 2 : 1, out);
+    __shared__ double out[3];
+    reduce_partials<AT>(q.part, gridDim.x, nq, out);
     __syncthreads();
     if (threadIdx.x == 0) {
-        q.kd[q.o0] = out[0];
-        if (q.db) q.kd[q.o1] = out[1];
+        q.kd[q.oy] = out[0];
+        q.kd[q.oa] = out[1];
+        if (q.db) q.kd[q.ob] = out[2];
         *ticket = 0;
     }
 }
@@ -949,8 +1028,8 @@ __device__ __forceinline__ void finish_reduction(const double *partial, int ncol
 // (ncols == 1, w the new Arnoldi vector) the last block also applies the
 // Givens update with out[0] = ||w||^2.
 template <typename T, int CB, bool VEC>
-__device__ __forceinline__ void mdot_body(const T *__restrict__ V, long long ldv, int ncols, const T *__restrict__ w,
-                                          long long n, double *__restrict__ partial, double *__restrict__ out,
+__device__ __forceinline__ void mdot_body(const T *V, long long ldv, int ncols, const T *w,
+                                          long long n, double *partial, double *out,
                                           unsigned *ticket, const GivensArgs &gv) {
     constexpr int W = VEC ? Vec16<T>::W : 1;
     long long lo, hi;
@@ -995,27 +1074,29 @@ __device__ __forceinline__ void mdot_body(const T *__restrict__ V, long long ldv
 }
 
 template <typename T, int CB, bool VEC>
-__global__ void __launch_bounds__(256) k_mdot(const T *__restrict__ V, long long ldv, int ncols, const T *__restrict__ w,
-                                              long long n, double *__restrict__ partial, double *__restrict__ out,
+__global__ void __launch_bounds__(256) k_mdot(const T *V, long long ldv, int ncols, const T *w,
+                                              long long n, double *partial, double *out,
                                               unsigned *ticket, GivensArgs gv) {
     mdot_body<T, CB, VEC>(V, ldv, ncols, w, n, partial, out, ticket, gv);
 }
 // the same with ncols = *jp + off read on the device (device-driven loops)
 template <typename T, int CB, bool VEC>
-__global__ void __launch_bounds__(256) k_mdot_dl(const T *__restrict__ V, long long ldv, const int *jp, int off,
-                                                 const T *__restrict__ w, long long n, double *__restrict__ partial,
-                                                 double *__restrict__ out, unsigned *ticket, GivensArgs gv) {
+__global__ void __launch_bounds__(256) k_mdot_dl(const T *V, long long ldv, const int *jp, int off,
+                                                 const T *w, long long n, double *partial,
+                                                 double *out, unsigned *ticket, GivensArgs gv) {
+    pdl_wait();
     mdot_body<T, CB, VEC>(V, ldv, *jp + off, w, n, partial, out, ticket, gv);
 }
 
 // w[t] += alpha * sum_j coef[j] V[j][t]  (coef on the device, FP64)
-template <typename T, bool VEC>
-__device__ __forceinline__ void maxpy_body(const T *__restrict__ V, long long ldv, int ncols, const double *__restrict__ coef,
-                                           double alpha, T *__restrict__ w, long long n) {
+// (set: w = alpha * the sum instead)
+template <typename T, bool VEC, bool SET = false>
+__device__ __forceinline__ void maxpy_body(const T *V, long long ldv, int ncols, const double *coef, double alpha, T *w,
+                                           long long n) {
     constexpr int W = VEC ? Vec16<T>::W : 1;
     __shared__ T cs[256];
     const long long nv = n / W;
-    for (int c0 = 0; c0 < ncols; c0 += 256) {
+    for (int c0 = 0; c0 < ncols || (SET && c0 == 0); c0 += 256) {
         const int cn = min(256, ncols - c0);
         __syncthreads();
         if ((int)threadIdx.x < cn) cs[threadIdx.x] = (T)(alpha * coef[c0 + threadIdx.x]);
@@ -1023,8 +1104,14 @@ __device__ __forceinline__ void maxpy_body(const T *__restrict__ V, long long ld
         for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += (long long)gridDim.x * blockDim.x) {
             const long long t = i * W;
             T acc[W];
-            if constexpr (VEC) vld(w + t, acc);
-            else acc[0] = w[t];
+            if (SET && c0 == 0) {
+#pragma unroll
+                for (int e = 0; e < W; ++e) acc[e] = T(0);
+            } else {
+                if constexpr (VEC) vld(w + t, acc);
+                else acc[0] = w[t];
+            }
+#pragma unroll 4
             for (int j = 0; j < cn; ++j) {
                 T v[W];
                 if constexpr (VEC) vld(V + (long long)(c0 + j) * ldv + t, v);
@@ -1037,7 +1124,7 @@ __device__ __forceinline__ void maxpy_body(const T *__restrict__ V, long long ld
         }
         if (VEC && blockIdx.x == 0 && threadIdx.x < n - nv * W) {   // ragged end
             const long long t = nv * W + threadIdx.x;
-            T acc = w[t];
+            T acc = SET && c0 == 0 ? T(0) : w[t];
             for (int j = 0; j < cn; ++j) acc += cs[j] * V[(long long)(c0 + j) * ldv + t];
             w[t] = acc;
         }
@@ -1045,15 +1132,16 @@ __device__ __forceinline__ void maxpy_body(const T *__restrict__ V, long long ld
 }
 
 template <typename T, bool VEC>
-__global__ void __launch_bounds__(256) k_maxpy(const T *__restrict__ V, long long ldv, int ncols, const double *__restrict__ coef,
-                                               double alpha, T *__restrict__ w, long long n) {
+__global__ void __launch_bounds__(256) k_maxpy(const T *V, long long ldv, int ncols, const double *coef, double alpha, T *w,
+                                               long long n) {
     maxpy_body<T, VEC>(V, ldv, ncols, coef, alpha, w, n);
 }
-template <typename T, bool VEC>
-__global__ void __launch_bounds__(256) k_maxpy_dl(const T *__restrict__ V, long long ldv, const int *jp, int off,
-                                                  const double *__restrict__ coef, double alpha, T *__restrict__ w,
+// w = sum_j coef[j] V[j] (set) or w += it, *jp columns
+template <typename T, bool VEC, bool SET>
+__global__ void __launch_bounds__(256) k_maxpy_dl(const T *V, long long ldv, const int *jp, const double *coef, T *w,
                                                   long long n) {
-    maxpy_body<T, VEC>(V, ldv, *jp + off, coef, alpha, w, n);
+    pdl_wait();
+    maxpy_body<T, VEC, SET>(V, ldv, *jp, coef, 1.0, w, n);
 }
 
 // Fused CGS pass for up to MAXC columns: w_new = w - sum_j coef[j] V[j], then
@@ -1061,9 +1149,9 @@ __global__ void __launch_bounds__(256) k_maxpy_dl(const T *__restrict__ V, long 
 // of w_new (norm_only = 1), V read once; partials reduced by the last block
 // into out (and, with gv.H set, the Givens update with out[0] = ||w_new||^2).
 template <typename T, int MAXC, bool VEC>
-__device__ __forceinline__ void maxpy_dot_body(const T *__restrict__ V, long long ldv, int ncols,
-                                               const double *__restrict__ coef, T *__restrict__ w, long long n,
-                                               int norm_only, double *__restrict__ partial, double *__restrict__ out,
+__device__ __forceinline__ void maxpy_dot_body(const T *V, long long ldv, int ncols,
+                                               const double *coef, T *w, long long n,
+                                               int norm_only, double *partial, double *out,
                                                unsigned *ticket, const GivensArgs &gv) {
     constexpr int W = VEC ? Vec16<T>::W : 1;
     __shared__ T cs[MAXC];
@@ -1111,26 +1199,27 @@ __device__ __forceinline__ void maxpy_dot_body(const T *__restrict__ V, long lon
 }
 
 template <typename T, int MAXC, bool VEC>
-__global__ void __launch_bounds__(256) k_maxpy_dot(const T *__restrict__ V, long long ldv, int ncols,
-                                                   const double *__restrict__ coef, T *__restrict__ w, long long n,
-                                                   int norm_only, double *__restrict__ partial, double *__restrict__ out,
+__global__ void __launch_bounds__(256) k_maxpy_dot(const T *V, long long ldv, int ncols,
+                                                   const double *coef, T *w, long long n,
+                                                   int norm_only, double *partial, double *out,
                                                    unsigned *ticket, GivensArgs gv) {
     maxpy_dot_body<T, MAXC, VEC>(V, ldv, ncols, coef, w, n, norm_only, partial, out, ticket, gv);
 }
 
-// The device-driven form of the fused pass, ncols = *jp + off read on the
-// device.  A basis longer than MAXC takes two sweeps over the block's own
-// chunk: the subtraction w -= V coef (columns in ascending order, each
-// thread on the elements it owns), then mdot_body's products (or norm and
-// Givens update) on the same elements, so no element crosses threads.
+// The device-driven form of the fused pass with products, ncols = *jp + off
+// read on the device.  A basis longer than MAXC takes two sweeps over the
+// block's own chunk: the subtraction w -= V coef (columns in ascending order,
+// each thread on the elements it owns), then mdot_body's products on the same
+// elements, so no element crosses threads.
 template <typename T, int MAXC, bool VEC>
-__global__ void __launch_bounds__(256) k_maxpy_dot_dl(const T *__restrict__ V, long long ldv, const int *jp, int off,
-                                                      const double *__restrict__ coef, T *__restrict__ w, long long n,
-                                                      int norm_only, double *__restrict__ partial,
-                                                      double *__restrict__ out, unsigned *ticket, GivensArgs gv) {
+__global__ void __launch_bounds__(256) k_maxpy_dot_dl(const T *V, long long ldv, const int *jp, int off,
+                                                      const double *coef, T *w, long long n,
+                                                      double *partial,
+                                                      double *out, unsigned *ticket) {
+    pdl_wait();
     const int ncols = *jp + off;
     if (ncols <= MAXC) {
-        maxpy_dot_body<T, MAXC, VEC>(V, ldv, ncols, coef, w, n, norm_only, partial, out, ticket, gv);
+        maxpy_dot_body<T, MAXC, VEC>(V, ldv, ncols, coef, w, n, 0, partial, out, ticket, GivensArgs());
         return;
     }
     constexpr int W = VEC ? Vec16<T>::W : 1;
@@ -1166,8 +1255,62 @@ __global__ void __launch_bounds__(256) k_maxpy_dot_dl(const T *__restrict__ V, l
         }
     }
     __syncthreads();
-    if (norm_only) mdot_body<T, 8, VEC>(w, ldv, 1, w, n, partial, out, ticket, gv);
-    else mdot_body<T, 8, VEC>(V, ldv, ncols, w, n, partial, out, ticket, gv);
+    mdot_body<T, 8, VEC>(V, ldv, ncols, w, n, partial, out, ticket, GivensArgs());
+}
+
+// The last pass of a device-driven step: w -= V coef (ncols = *jp + 1 columns),
+// ||w||^2, and in the last block the Givens update and the end of the
+// iteration.  Columns in groups of eight: the products' kernel above keeps
+// its 16 columns in registers for the dots, which this pass does not need, and
+// two blocks of it fill an SM against five of this.  cap: entries of coef.
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(256) k_maxpy_norm_dl(const T *V, long long ldv, const int *jp, const double *coef, int cap,
+                                                       T *w, long long n, double *partial, double *out, unsigned *ticket,
+                                                       GivensArgs gv) {
+    pdl_wait();
+    constexpr int W = VEC ? Vec16<T>::W : 1;
+    __shared__ T cs[256];
+    const int tid = threadIdx.x;
+    // the first 256 coefficients without waiting for the column count
+    const double c0 = tid < cap ? coef[tid] : 0.0;
+    const int ncols = *jp + 1;
+    cs[tid] = (T)c0;
+    __syncthreads();
+    long long lo, hi;
+    block_chunk(n, Vec16<T>::W, lo, hi);
+    const long long nv = (hi - lo) / W;
+    T nn[1] = {0};
+    auto body = [&](long long t, auto wtag) {
+        constexpr int L = decltype(wtag)::value;
+        T s[L];
+        if constexpr (L > 1) vld(w + t, s);
+        else s[0] = w[t];
+        for (int q0 = 0; q0 < ncols; q0 += 8) {
+            T v[8][L];
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (q0 + q < ncols) {
+                    if constexpr (L > 1) vld(V + (long long)(q0 + q) * ldv + t, v[q]);
+                    else v[q][0] = V[(long long)(q0 + q) * ldv + t];
+                }
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (q0 + q < ncols) {
+                    const T k = q0 + q < 256 ? cs[q0 + q] : (T)coef[q0 + q];
+#pragma unroll
+                    for (int e = 0; e < L; ++e) s[e] -= k * v[q][e];
+                }
+        }
+        if constexpr (L > 1) vst(w + t, s);
+        else w[t] = s[0];
+#pragma unroll
+        for (int e = 0; e < L; ++e) nn[0] += s[e] * s[e];
+    };
+    for (long long i = tid; i < nv; i += blockDim.x) body(lo + i * W, std::integral_constant<int, W>());
+    if (VEC && tid < hi - lo - nv * W) body(lo + nv * W + tid, std::integral_constant<int, 1>());
+    block_partials<T, 1>(nn, 1, partial, 0);
+    if (!grid_last_block(ticket)) return;
+    finish_reduction<T>(partial, 1, out, ticket, gv);
 }
 
 // ------------------------------------------- Gram-Schmidt in one cluster
@@ -1198,7 +1341,7 @@ __device__ __forceinline__ double gs_double(FF a) { return ff_to_double(a); }
 __device__ __forceinline__ double gs_double(double a) { return a; }
 template <typename T>
 __global__ void __cluster_dims__(kGsCluster, 1, 1) __launch_bounds__(kGsThreads)
-    k_gs_cluster(const T *__restrict__ V, long long ld, const int *jp, T *__restrict__ w, long long n, int passes, double *h1,
+    k_gs_cluster(const T *V, long long ld, const int *jp, T *w, long long n, int passes, double *h1,
                  double *h2, GivensArgs gv) {
     namespace cg = cooperative_groups;
     using S = typename GsSum<T>::type;
@@ -1214,6 +1357,7 @@ __global__ void __cluster_dims__(kGsCluster, 1, 1) __launch_bounds__(kGsThreads)
     // memory: arrive here, wait before the first such write
     auto started = cl.barrier_arrive();
     bool waited = false;
+    pdl_wait();
     const int ncols = *jp + 1;
     long long at[P];   // first element of each piece
 #pragma unroll
@@ -1401,12 +1545,77 @@ struct DlCounters {
 __global__ void k_dl_init(GmDev *st, double *g, int m1, const double *nrm2, double *beta, GmState *gs,
                           const double *rtol, const double *atol, const int *m, const int *nmax,
                           cudaGraphConditionalHandle h);
+// The start of an inner solve of a device-driven loop in one kernel: ||b||
+// and, in the last block, the loop's state (k_dl_init's, which the outer level
+// keeps) and the WHILE condition.
+struct DlStart {
+    GmDev *st;
+    double *g, *beta;
+    GmState *gs;
+    const double *rtol, *atol;
+    const int *m, *nmax;
+    cudaGraphConditionalHandle h;
+};
+__device__ __forceinline__ void dl_start(const DlStart &q, double nrm2) {
+    const double b = (nrm2 >= 0.0) ? sqrt(nrm2) : nrm2;   // NaN passes through
+    q.g[0] = b;
+    *q.beta = b;
+    q.gs->res = b;
+    gm_set_beta(q.gs, b);
+    const int nan = isfinite(b) ? 0 : 1, nmax = *q.nmax;
+    const double tol = fmax(*q.rtol * b, *q.atol);
+    const int conv = (b <= tol) ? 1 : 0;
+    q.gs->nan = nan;
+    q.st->j = 0;
+    q.st->its = 0;
+    q.st->pad0 = 0;
+    q.st->m = *q.m;
+    q.st->nmax = nmax;
+    q.st->bnorm = b;
+    q.st->res = b;
+    q.st->tol = tol;
+    q.st->nan = nan;
+    q.st->conv = conv;
+    q.st->rel_true = b > 0.0 ? 1.0 : 0.0;
+    cudaGraphSetConditional(q.h, (!conv && !nan && nmax > 0) ? 1u : 0u);
+}
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(256) k_norm_start(const T *b, long long n, double *partial, double *out, unsigned *ticket,
+                                                    DlStart q) {
+    pdl_wait();
+    constexpr int W = VEC ? Vec16<T>::W : 1;
+    long long lo, hi;
+    block_chunk(n, Vec16<T>::W, lo, hi);
+    const long long nv = (hi - lo) / W;
+    T nn[1] = {0};
+    for (long long i = threadIdx.x; i < nv; i += blockDim.x) {
+        T v[W];
+        if constexpr (VEC) vld(b + lo + i * W, v);
+        else v[0] = b[lo + i];
+#pragma unroll
+        for (int e = 0; e < W; ++e) nn[0] += v[e] * v[e];
+    }
+    if (VEC && threadIdx.x < hi - lo - nv * W) {
+        const T v = b[lo + nv * W + threadIdx.x];
+        nn[0] += v * v;
+    }
+    block_partials<T, 1>(nn, 1, partial, 0);
+    if (!grid_last_block(ticket)) return;
+    reduce_partials<T>(partial, gridDim.x, 1, out);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        dl_start(q, out[0]);
+        *ticket = 0;
+    }
+}
+
 // The first kernel of a device-driven iteration: basis column j = src / beta
 // (beta, and its reciprocal, from the norm pass before), src = w, or b where
 // the cycle starts (j = 0).  VEC: pointers and ld 16-byte aligned.
 template <typename T, bool VEC>
 __global__ void k_start_col(T *vbase, long long ld, const int *jp, const T *b, const T *w, const GmState *gs, long long n) {
     constexpr int W = VEC ? Vec16<T>::W : 1;
+    pdl_wait();
     const int j = *jp;
     const T *src = j == 0 ? b : w;
     const T inv = gm_inv<T>(gs);
@@ -1430,18 +1639,25 @@ __global__ void k_start_col(T *vbase, long long ld, const int *jp, const T *b, c
 // the same smoothing reads it (d may be null).  Saves a launch and a pass
 // over v per iteration; 0.56M unknowns (421k components): 4.8 + 3.7 -> 4.0 us.
 template <typename T>
-__global__ void k_start_cheb(int nbr, int bs, const T *__restrict__ dinv, T *__restrict__ vbase, long long ld,
-                             const int *jp, const T *b, const T *w, const GmState *gs, T c2, T *__restrict__ d,
-                             T *__restrict__ x) {
+__global__ void k_start_cheb(int nbr, int bs, const T *__restrict__ dinv, T *vbase, long long ld,
+                             const int *jp, const T *b, const T *w, const GmState *gs, T c2, T *d,
+                             T *x) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (long long)nbr * bs) return;
+    const int i = (int)(t / bs), a = (int)(t - (long long)i * bs);
+    T di[3] = {T(0), T(0), T(0)};
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        if (c < bs) di[c] = dinv[(long long)i * bs * bs + a * bs + c];
+    pdl_wait();
     const int j = *jp;
     const T *src = j == 0 ? b : w;
     const T inv = gm_inv<T>(gs);
     vbase[(long long)j * ld + t] = src[t] * inv;
-    const int i = (int)(t / bs), a = (int)(t - (long long)i * bs);
     T s = 0;
-    for (int c = 0; c < bs; ++c) s += dinv[(long long)i * bs * bs + a * bs + c] * (src[(long long)i * bs + c] * inv);
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        if (c < bs) s += di[c] * (src[(long long)i * bs + c] * inv);
     const T dn = c2 * s;
     if (d) d[t] = dn;
     x[t] = dn;
@@ -1479,16 +1695,17 @@ __global__ void k_mul_col(T *out, const T *vbase, long long ld, const int *jp, c
 // (aggregates have at most 8 members), member loads in parallel, then a
 // fixed xor-shuffle tree inside the 8 lanes
 template <typename T>
-__global__ void k_restrict(const int *__restrict__ mptr, const int *__restrict__ mem, int nc, int bs, const T *__restrict__ r,
-                           T *__restrict__ rc) {
+__global__ void k_restrict(const int *__restrict__ mptr, const int *__restrict__ mem, int nc, int bs, const T *r,
+                           T *rc) {
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int I = (int)(g >> 3), l = (int)(g & 7);
     const bool live = I < nc;
     const unsigned mask = 0xffu << (threadIdx.x & 24u);
-    if (__all_sync(0xffffffffu, !live)) return;   // whole warp past the end
     int q = 0, beg = 0;
     if (live) { beg = mptr[I]; q = mptr[I + 1] - beg; }
     const int m = (live && l < q) ? mem[beg + l] : -1;
+    pdl_wait();
+    if (__all_sync(0xffffffffu, !live)) return;   // whole warp past the end
     for (int a = 0; a < bs; ++a) {
         T s = (m >= 0) ? r[(long long)m * bs + a] : T(0);
         s += __shfl_xor_sync(mask, s, 4);
@@ -1503,16 +1720,23 @@ __global__ void k_restrict(const int *__restrict__ mptr, const int *__restrict__
 // them (same operations, same order); rcopy (optional) gets a copy of rc.
 template <typename T>
 __global__ void k_restrict_first(const int *__restrict__ mptr, const int *__restrict__ mem, int nc, int bs,
-                                 const T *__restrict__ r, T *__restrict__ rc, const T *__restrict__ dinv, T c2,
-                                 T *__restrict__ d, T *__restrict__ x, T *__restrict__ rcopy) {
+                                 const T *r, T *rc, const T *__restrict__ dinv, T c2,
+                                 T *d, T *x, T *rcopy) {
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int I = (int)(g >> 3), l = (int)(g & 7);
     const bool live = I < nc;
     const unsigned mask = 0xffu << (threadIdx.x & 24u);
-    if (__all_sync(0xffffffffu, !live)) return;
     int q = 0, beg = 0;
     if (live) { beg = mptr[I]; q = mptr[I + 1] - beg; }
     const int m = (live && l < q) ? mem[beg + l] : -1;
+    T di[3] = {T(0), T(0), T(0)};   // row l of the coarse block-diagonal inverse
+    if (live && l < bs) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            if (c < bs) di[c] = dinv[(long long)I * bs * bs + l * bs + c];
+    }
+    pdl_wait();
+    if (__all_sync(0xffffffffu, !live)) return;
     T v[3] = {T(0), T(0), T(0)};   // bs <= 3; every lane of the group ends with the sums
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -1533,14 +1757,14 @@ __global__ void k_restrict_first(const int *__restrict__ mptr, const int *__rest
     T s = 0;
 #pragma unroll
     for (int c = 0; c < 3; ++c)
-        if (c < bs) s += dinv[(long long)I * bs * bs + l * bs + c] * v[c];
+        if (c < bs) s += di[c] * v[c];
     const T dn = c2 * s;
     if (d) d[t] = dn;   // read by a second pre-smoothing step only
     x[t] = dn;
 }
 // x[i] += e_c[agg[i]]
 template <typename T>
-__global__ void k_prolong(const int *__restrict__ agg, int n, int bs, const T *__restrict__ ec, T *__restrict__ x) {
+__global__ void k_prolong(const int *__restrict__ agg, int n, int bs, const T *ec, T *x) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (long long)n * bs) return;
     const int i = (int)(t / bs), a = (int)(t - (long long)i * bs);
@@ -1553,10 +1777,11 @@ __global__ void k_prolong(const int *__restrict__ agg, int n, int bs, const T *_
 // same per-element adds; the last n % W nodes one per thread.  x and agg
 // 16-byte aligned.
 template <typename T, int BS>
-__global__ void k_prolong_v(const int *__restrict__ agg, int n, const T *__restrict__ ec, T *__restrict__ x) {
+__global__ void k_prolong_v(const int *__restrict__ agg, int n, const T *ec, T *x) {
     constexpr int W = Vec16<T>::W;
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long ng = n / W;
+    pdl_wait();
     if (g < ng) {
         int I[W];
 #pragma unroll
@@ -1583,14 +1808,21 @@ __global__ void k_prolong_v(const int *__restrict__ agg, int n, const T *__restr
 // Chebyshev first step from x = 0: d = c2 Dinv b; x = d
 // (bcopy != nullptr: b is also copied there, for a cycle replayed on fixed buffers)
 template <typename T>
-__global__ void k_cheb_first(int nbr, int bs, const T *__restrict__ dinv, const T *__restrict__ b, T c2, T *__restrict__ d,
-                             T *__restrict__ x, T *__restrict__ bcopy) {
+__global__ void k_cheb_first(int nbr, int bs, const T *__restrict__ dinv, const T *b, T c2, T *d,
+                             T *x, T *bcopy) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (long long)nbr * bs) return;
-    if (bcopy) bcopy[t] = b[t];
     const int i = (int)(t / bs), a = (int)(t - (long long)i * bs);
+    T di[3] = {T(0), T(0), T(0)};
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        if (c < bs) di[c] = dinv[(long long)i * bs * bs + a * bs + c];
+    pdl_wait();
+    if (bcopy) bcopy[t] = b[t];
     T s = 0;
-    for (int c = 0; c < bs; ++c) s += dinv[(long long)i * bs * bs + a * bs + c] * b[(long long)i * bs + c];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        if (c < bs) s += di[c] * b[(long long)i * bs + c];
     const T dn = c2 * s;
     d[t] = dn;
     x[t] = dn;
@@ -1601,11 +1833,12 @@ __global__ void k_cheb_first(int nbr, int bs, const T *__restrict__ dinv, const 
 // at a time, so a lane has several loads in flight instead of one long
 // chain of dependent adds; the partials are added in a fixed order.
 template <typename T>
-__global__ void k_dense_gemv(const T *__restrict__ Cinv, int n, const T *__restrict__ b, T *__restrict__ x) {
+__global__ void k_dense_gemv(const T *__restrict__ Cinv, int n, const T *b, T *x) {
     constexpr int W = Vec16<T>::W;
     const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int ln = threadIdx.x & 31;
     if (row >= n) return;
+    pdl_wait();
     const T *r = Cinv + (long long)row * n;
     T s[4] = {0, 0, 0, 0};
     if (n % W == 0 && ((uintptr_t)Cinv & 15u) == 0 && ((uintptr_t)b & 15u) == 0) {
@@ -1642,7 +1875,7 @@ __global__ void k_dense_gemv(const T *__restrict__ Cinv, int n, const T *__restr
 constexpr int kGemvThreads = 128;
 template <typename T, bool VEC>   // float
 __global__ void __launch_bounds__(kGemvThreads) k_dense_gemv_rows(const T *__restrict__ Cinv, int n,
-                                                                  const T *__restrict__ b, T *__restrict__ x) {
+                                                                  const T *b, T *x) {
     static_assert(std::is_same<T, float>::value, "FP32 form");
     __shared__ float ws[kGemvThreads / 32];
     const int row = blockIdx.x;
@@ -1650,15 +1883,27 @@ __global__ void __launch_bounds__(kGemvThreads) k_dense_gemv_rows(const T *__res
     float s[4] = {0.f, 0.f, 0.f, 0.f};
     if constexpr (VEC) {
         const int nv = n / 4;
+        float a[4] = {0.f, 0.f, 0.f, 0.f}, v[4];
+        if ((int)threadIdx.x < nv) vld(r + (long long)threadIdx.x * 4, a);
+        pdl_wait();
         for (int c = threadIdx.x; c < nv; c += kGemvThreads) {
-            float a[4], v[4];
-            vld(r + (long long)c * 4, a);
+            if (c != (int)threadIdx.x) vld(r + (long long)c * 4, a);
             vld(b + (long long)c * 4, v);
 #pragma unroll
             for (int e = 0; e < 4; ++e) s[e] += a[e] * v[e];
         }
     } else {
         int c = threadIdx.x;
+        float a[4];   // the row's first four values of this thread
+#pragma unroll
+        for (int e = 0; e < 4; ++e) a[e] = c + e * kGemvThreads < n ? r[c + e * kGemvThreads] : 0.f;
+        pdl_wait();
+        if (n <= 4 * kGemvThreads) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (c + e * kGemvThreads < n) s[e] += a[e] * b[c + e * kGemvThreads];
+            c = n;
+        }
         for (; c + 3 * kGemvThreads < n; c += 4 * kGemvThreads) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) s[e] += r[c + e * kGemvThreads] * b[c + e * kGemvThreads];
@@ -1678,97 +1923,47 @@ __global__ void __launch_bounds__(kGemvThreads) k_dense_gemv_rows(const T *__res
 }
 
 // ============================================================== K-cycle
-// kd[o0] = a.b and, when c != nullptr, kd[o1] = c.d.  Each block reduces a
-// fixed contiguous chunk into kd[8 + 2 blk], and the last block to finish
-// (ticket in kd[7]) sums the block partials in a fixed order (one warp,
-// lanes over blocks): one launch, same result whatever order the blocks run in.
+// The inner products of a K-cycle step where the level's product is the flat
+// kernel or its blocks are 3x3: kd[oy] = y . y, kd[oa] = y . a and, when b is
+// set, kd[ob] = y . b.  Each block reduces a fixed contiguous chunk into
+// kd[8 + blk], kd[8 + nb + blk], ..., and the last block to finish (ticket in
+// kd[7]) sums the block partials in a fixed order: one launch, same result
+// whatever order the blocks run in.
 constexpr int kKdotBlocks = 96;
-
-// The two sums p0, p1 of every thread reduced over the grid: per block into
-// kd[8 + 2 blk], kd[9 + 2 blk], then by warp 0 of the last block to finish
-// (ticket kd[7]; lanes over the blocks in steps of 32, a warp tree) into
-// kd[o0] and, when two, kd[o1].  FP64 for FP64 vectors; float-float (float2
-// in the slots) for FP32 ones.
 template <typename T>
-__device__ __forceinline__ void kdot_reduce(T p0, T p1, double *kd, int o0, int o1, bool two) {
-    __shared__ bool last;
-    if constexpr (std::is_same<T, float>::value) {
-        __shared__ FF s0[8], s1[8];
-        const FF t0 = ff_warp_sum(FF{p0, 0.f}), t1 = ff_warp_sum(FF{p1, 0.f});
-        if ((threadIdx.x & 31) == 0) { s0[threadIdx.x >> 5] = t0; s1[threadIdx.x >> 5] = t1; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            FF u0 = s0[0], u1 = s1[0];
-            for (int w = 1; w < (int)(blockDim.x >> 5); ++w) { u0 = ff_add(u0, s0[w]); u1 = ff_add(u1, s1[w]); }
-            *reinterpret_cast<float2 *>(kd + 8 + 2 * blockIdx.x) = make_float2(u0.hi, u0.lo);
-            *reinterpret_cast<float2 *>(kd + 9 + 2 * blockIdx.x) = make_float2(u1.hi, u1.lo);
-            __threadfence();
-            last = (atomicAdd((unsigned int *)(kd + 7), 1u) == gridDim.x - 1);
-        }
-        __syncthreads();
-        if (last && threadIdx.x < 32) {
-            __threadfence();
-            FF u0{0.f, 0.f}, u1{0.f, 0.f};
-            for (unsigned qb = threadIdx.x; qb < gridDim.x; qb += 32) {
-                const float2 a0 = __ldcg(reinterpret_cast<const float2 *>(kd + 8 + 2 * qb));
-                const float2 a1 = __ldcg(reinterpret_cast<const float2 *>(kd + 9 + 2 * qb));
-                u0 = ff_add(u0, FF{a0.x, a0.y});
-                u1 = ff_add(u1, FF{a1.x, a1.y});
-            }
-            u0 = ff_warp_sum(u0);
-            u1 = ff_warp_sum(u1);
-            if (threadIdx.x == 0) {
-                kd[o0] = ff_to_double(u0);
-                if (two) kd[o1] = ff_to_double(u1);
-                *(unsigned int *)(kd + 7) = 0u;   // ready for the next call
-            }
-        }
-    } else {
-        __shared__ double s0[8], s1[8];
-        const double t0 = warp_sum((double)p0), t1 = warp_sum((double)p1);
-        if ((threadIdx.x & 31) == 0) { s0[threadIdx.x >> 5] = t0; s1[threadIdx.x >> 5] = t1; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double u0 = 0.0, u1 = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { u0 += s0[w]; u1 += s1[w]; }
-            kd[8 + 2 * blockIdx.x] = u0;
-            kd[9 + 2 * blockIdx.x] = u1;
-            __threadfence();
-            last = (atomicAdd((unsigned int *)(kd + 7), 1u) == gridDim.x - 1);
-        }
-        __syncthreads();
-        if (last && threadIdx.x < 32) {
-            __threadfence();
-            double u0 = 0.0, u1 = 0.0;
-            for (unsigned qb = threadIdx.x; qb < gridDim.x; qb += 32) {
-                u0 += __ldcg(kd + 8 + 2 * qb);
-                u1 += __ldcg(kd + 9 + 2 * qb);
-            }
-            u0 = warp_sum(u0);
-            u1 = warp_sum(u1);
-            if (threadIdx.x == 0) {
-                kd[o0] = u0;
-                if (two) kd[o1] = u1;
-                *(unsigned int *)(kd + 7) = 0u;
-            }
-        }
-    }
-}
-template <typename T>
-__global__ void __launch_bounds__(256) k_kdots(const T *__restrict__ a, const T *__restrict__ b, const T *__restrict__ c,
-                                               const T *__restrict__ d, long long n, double *kd, int o0, int o1) {
+__global__ void __launch_bounds__(256) k_kdots(const T *y, const T *a, const T *b, long long n, double *kd, int oy, int oa,
+                                               int ob) {
+    pdl_wait();
     const long long chunk = (n + gridDim.x - 1) / gridDim.x;
     const long long lo = (long long)blockIdx.x * chunk, hi = min(n, lo + chunk);
-    T p0 = 0, p1 = 0;   // per-thread sums in the vector type
+    T pp[4] = {0, 0, 0, 0};   // per-thread sums in the vector type
     for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        p0 += a[i] * b[i];
-        if (c) p1 += c[i] * d[i];
+        const T u = y[i];
+        pp[0] += u * u;
+        pp[1] += u * a[i];
+        if (b) pp[2] += u * b[i];
     }
-    kdot_reduce<T>(p0, p1, kd, o0, o1, c != nullptr);
+    const int nq = b ? 3 : 2;
+    block_partials<T, 4>(pp, nq, kd + 8, 0);
+    unsigned *ticket = (unsigned *)(kd + 7);
+    if (!grid_last_block(ticket)) return;
+    __shared__ double out[3];
+    reduce_partials<T>(kd + 8, gridDim.x, nq, out);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        kd[oy] = out[0];
+        kd[oa] = out[1];
+        if (b) kd[ob] = out[2];
+        *ticket = 0;
+    }
 }
-// r -= a1 w1 with a1 = (w1.r)/(w1.w1) = kd[1]/kd[0]; a1 saved in kd[2]
-template <typename T> __global__ void k_kupd1(T *r, const T *w1, double *kd, long long n) {
+// r -= a1 w1 with a1 = (w1.r)/(w1.w1) = kd[1]/kd[0], saved in kd[2]; then, where
+// the second cycle starts with a smoothing step from zero (dinv set), that
+// step: x = c2 Dinv r, and d = x when d is set.  One thread per block row.
+template <typename T>
+__global__ void k_kupd1(T *r, const T *w1, double *kd, int nbr, int bs, const T *__restrict__ dinv, T c2, T *d, T *x) {
     __shared__ T a1s;
+    pdl_wait();
     if (threadIdx.x == 0) {
         const double a1 = kd[0] > 0.0 ? kd[1] / kd[0] : 0.0;
         a1s = (T)a1;
@@ -1776,57 +1971,68 @@ template <typename T> __global__ void k_kupd1(T *r, const T *w1, double *kd, lon
     }
     __syncthreads();
     const T a1 = a1s;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        r[i] = r[i] - a1 * w1[i];
-}
-// w2 -= beta w1 and z2 -= beta z1 with beta = (w2.w1)/(w1.w1) = kd[3]/kd[0],
-// followed by kd[4] = w2.w2, kd[5] = w2.r on the updated w2, in one
-// launch: the chunks, per-thread sums and fixed-order block and grid
-// reductions of k_kdots (grid kKdotBlocks, ticket kd[7])
-template <typename T>
-__global__ void __launch_bounds__(256) k_kupd2_dots(T *__restrict__ w2, T *__restrict__ z2, const T *__restrict__ w1,
-                                                    const T *__restrict__ z1, const T *__restrict__ r, double *kd,
-                                                    long long n) {
-    __shared__ T bs_;
-    if (threadIdx.x == 0) bs_ = (T)(kd[0] > 0.0 ? kd[3] / kd[0] : 0.0);
-    __syncthreads();
-    const T beta = bs_;
-    const long long chunk = (n + gridDim.x - 1) / gridDim.x;
-    const long long lo = (long long)blockIdx.x * chunk, hi = min(n, lo + chunk);
-    T p0 = 0, p1 = 0;
-    for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        const T wn = w2[i] - beta * w1[i];
-        w2[i] = wn;
-        z2[i] = z2[i] - beta * z1[i];
-        p0 += wn * wn;
-        p1 += wn * r[i];
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nbr; i += gridDim.x * blockDim.x) {
+        T v[3] = {T(0), T(0), T(0)};
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            if (c < bs) {
+                const long long t = (long long)i * bs + c;
+                v[c] = r[t] - a1 * w1[t];
+                r[t] = v[c];
+            }
+        if (!dinv) continue;
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            if (a < bs) {
+                T s = 0;
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    if (c < bs) s += dinv[(long long)i * bs * bs + a * bs + c] * v[c];
+                const T dn = c2 * s;
+                const long long t = (long long)i * bs + a;
+                if (d) d[t] = dn;
+                x[t] = dn;
+            }
     }
-    kdot_reduce<T>(p0, p1, kd, 4, 5, true);
 }
-// x = a1 z1 + a2 z2 with a2 = (w2.r)/(w2.w2) = kd[5]/kd[4]
-template <typename T> __global__ void k_kupd3(T *x, const T *z1, const T *z2, const double *kd, long long n) {
-    __shared__ T a1s, a2s;
+// x = a1 z1 + a2 (z2 - beta z1), the second search direction made orthogonal
+// to the first: beta = (w2.w1)/(w1.w1) = kd[3]/kd[0], w2' = w2 - beta w1, and
+// a2 = (w2'.r)/(w2'.w2') = kd[5] / (kd[4] - beta kd[3]) since w1.r = 0 after
+// the first step: the inner products of w2 itself give it, without a pass
+// that forms w2' and z2' (2 launches and 10 vector passes fewer per K-cycle
+// than updating, reducing and then combining).  Where w2 is parallel to w1 to
+// rounding the second direction is dropped.
+template <typename T> __global__ void k_kupd2(T *x, const T *z1, const T *z2, const double *kd, long long n) {
+    __shared__ T c1s, c2s;
+    pdl_wait();
     if (threadIdx.x == 0) {
-        a1s = (T)kd[2];
-        a2s = (T)(kd[4] > 0.0 ? kd[5] / kd[4] : 0.0);
+        const double beta = kd[0] > 0.0 ? kd[3] / kd[0] : 0.0;
+        const double ww = kd[4] - beta * kd[3];
+        const double a2 = ww > (sizeof(T) == 4 ? 1e-6 : 1e-12) * kd[4] ? kd[5] / ww : 0.0;
+        c1s = (T)(kd[2] - a2 * beta);
+        c2s = (T)a2;
     }
     __syncthreads();
-    const T a1 = a1s, a2 = a2s;
+    const T c1 = c1s, c2 = c2s;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        x[i] = a1 * z1[i] + a2 * z2[i];
+        x[i] = c1 * z1[i] + c2 * z2[i];
 }
 
 // =============================================================== rank one
 // f[k] = r_k * (a^k . x), one block per outlet (fixed-order tree reduction)
 template <typename T>
 __global__ void k_lowrank_dots(const int *__restrict__ optr, const int *__restrict__ oidx, const double *__restrict__ oval,
-                               const double *__restrict__ r, const T *__restrict__ x, double *__restrict__ f,
+                               const double *__restrict__ r, const T *x, double *f,
                                const int *jp = nullptr, long long x_ld = 0) {
     __shared__ double red[8];
     const int k = blockIdx.x;
+    const int q0 = optr[k] + threadIdx.x, q1 = optr[k + 1];
+    const int i0 = q0 < q1 ? oidx[q0] : 0;
+    const double v0 = q0 < q1 ? oval[q0] : 0.0;
+    pdl_wait();
     if (jp) x += (long long)*jp * x_ld;   // x is basis column *jp
-    double s = 0.0;
-    for (int q = optr[k] + threadIdx.x; q < optr[k + 1]; q += blockDim.x) s += oval[q] * (double)x[oidx[q]];
+    double s = q0 < q1 ? v0 * (double)x[i0] : 0.0;
+    for (int q = q0 + blockDim.x; q < q1; q += blockDim.x) s += oval[q] * (double)x[oidx[q]];
     s = warp_sum(s);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();

@@ -115,6 +115,7 @@ __global__ void k_dl_cycle_start(GmDev *st, cudaGraphConditionalHandle h) {
 
 __global__ void k_dl_end(GmDev *st, const double *H, int ldh, const double *g, double *y, long long *its_total,
                          long long *solves) {
+    pdl_wait();
     trisolve(H, ldh, g, y, st->j);
     if (threadIdx.x != 0) return;
     st->conv = st->res <= st->tol ? 1 : 0;

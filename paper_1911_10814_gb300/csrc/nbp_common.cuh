@@ -44,6 +44,48 @@ inline void require(bool ok, nbp_status st, const std::string &msg) {
     if (!ok) throw Error{st, msg};
 }
 
+// ------------------------------------------- programmatic dependent launch
+// Inside the device-driven loops a kernel boundary and the first dependent
+// loads of the next kernel are a good part of every small kernel's time.
+// There consecutive kernels are launched with programmatic stream
+// serialization: the next one starts while its predecessor still runs, loads
+// what no kernel of a solve writes (matrices, block-diagonal inverses,
+// aggregate maps, outlet vectors) and waits (pdl_wait) for the predecessor's
+// end before anything else.  Every thread that reads or writes a solve's
+// vectors or states waits first; since each kernel waits, the end of one
+// implies the end of all before it.  A kernel lets its successor start only
+// after its own wait, so that no more than one kernel waits per chain (the
+// branches of a batch share the SMs).  Without the attribute both
+// instructions are no-ops.
+__device__ __forceinline__ void pdl_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// on: this thread is capturing a device-driven solve; prev: the last captured
+// node is a kernel (a conditional or copy node cannot be overlapped)
+struct PdlState {
+    bool on = false, prev = false;
+};
+inline thread_local PdlState g_pdl;
+
+// kernel<<<grid, block, 0, s>>>(args...), overlapped with its predecessor where
+// g_pdl allows; for kernels that call pdl_wait only
+template <typename... P, typename... A>
+inline void klaunch(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t s, A &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = g_pdl.on && g_pdl.prev ? 1 : 0;
+    NBP_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
+    g_pdl.prev = g_pdl.on;
+}
+
 // --------------------------------------------------------------- numerics
 template <typename T> struct Acc { using type = T; };
 template <> struct Acc<__nv_bfloat16> { using type = float; };

@@ -27,7 +27,9 @@
 #include <numeric>
 #include <map>
 #include <memory>
+#include <exception>
 #include <mutex>
+#include <thread>
 #include <tuple>
 
 #include "kernels.cuh"
@@ -223,6 +225,7 @@ template <typename D_, typename S_> static void convert(D_ *d, const S_ *src, lo
 }
 template <typename T> static void copy(T *d, const T *src, long long n, cudaStream_t s) {
     NBP_CUDA(cudaMemcpyAsync(d, src, sizeof(T) * n, cudaMemcpyDeviceToDevice, s));
+    g_pdl.prev = false;
 }
 
 static void prof_begin(nbp_ctx *c, cudaEvent_t &e) {
@@ -315,7 +318,7 @@ static void apply_A(nbp_ctx *c, int vsel, const T *x, T *y, const int *jp = null
     a.x_ld = x_ld;
     if (lr.n_out > 0) {
         c->prof.launches++;
-        k_lowrank_dots<T><<<lr.n_out, 256, 0, c->s>>>(lr.optr, lr.oidx, lr.oval, lr.r, x, lr.f, jp, x_ld);
+        klaunch(k_lowrank_dots<T>, lr.n_out, (unsigned)256, c->s, lr.optr, lr.oidx, lr.oval, lr.r, x, lr.f, jp, x_ld);
         NBP_LAUNCHED();
         a.lr_rp = lr.lr_rp; a.lr_k = lr.lr_k; a.lr_c = lr.lr_c; a.lr_val = lr.lr_val; a.lr_f = lr.f;
     }
@@ -675,8 +678,8 @@ static T *chebyshev(nbp_ctx *c, Level &L, int vsel, int k, const T *b, T *x, T *
         // d and x already hold the first step
     } else if (zero_start) {
         timed(c, "amg/cheb_first", (double)L.M.nbr * bs * (bs + 3) * sizeof(T), [&] {
-            k_cheb_first<T><<<grid_exact((long long)L.M.nbr * bs), 256, 0, c->s>>>(L.M.nbr, bs, dinv_of<T>(L), b,
-                                                                                   (T)(1.0 / ch.theta), d, cur, nullptr);
+            klaunch(k_cheb_first<T>, grid_exact((long long)L.M.nbr * bs), 256u, c->s, L.M.nbr, bs, dinv_of<T>(L), b,
+                    (T)(1.0 / ch.theta), d, cur, (T *)nullptr);
         });
     } else {
         cheb_step<T>(c, L, vsel, b, cur, nxt, d, 0.0, 1.0 / ch.theta, k > 1, post && k == 1);
@@ -698,18 +701,19 @@ static void vcycle_level(nbp_ctx *c, Hier &H, int l, int vsel, const T *b, T *ou
 // K-cycle on coarse level cl (Notay's Krylov-accelerated multigrid): two GCR
 // steps on L_cl e = b, each preconditioned by one cycle on level cl; every
 // coefficient stays on the device, so the whole cycle can be replayed from a
-// CUDA graph.  x = a1 z1 + a2 z2 with a1 = (w1.b)/(w1.w1), r = b - a1 w1,
-// beta = (w2.w1)/(w1.w1), w2 -= beta w1, z2 -= beta z1, a2 = (w2.r)/(w2.w2).
-// w = L.M z with kd[o0] = w . da and (db set) kd[o1] = w . db: one fused
-// launch (k_sell_dot) where the level's tuned kernel is a scalar sliced one,
-// else the product and k_kdots
+// CUDA graph.  x = a1 z1 + a2 (z2 - beta z1) with a1 = (w1.b)/(w1.w1), r = b -
+// a1 w1, beta = (w2.w1)/(w1.w1), a2 = (w2'.r)/(w2'.w2'), w2' = w2 - beta w1.
+// w = L.M z with kd[oy] = w . w, kd[oa] = w . da and (db set) kd[ob] = w . db:
+// one fused launch (k_sell_dot) where the level's tuned kernel is a scalar
+// sliced one, else the product and k_kdots
 template <typename T>
-static void kc_product_dots(nbp_ctx *c, Level &L, int vsel, const T *z, T *w, const T *da, const T *db, int o0, int o1) {
+static void kc_product_dots(nbp_ctx *c, Level &L, int vsel, const T *z, T *w, const T *da, const T *db, int oy, int oa,
+                            int ob) {
     const long long n = (long long)L.M.nbr * L.M.br;
     if (L.kpart && spmv_dot_ok(L.M, vsel, (int)sizeof(T), L.kpart_blocks)) {
         cudaEvent_t e0;
         prof_begin(c, e0);
-        DotArgs q{da, db, L.kpart, L.kdots, o0, o1};
+        DotArgs q{da, db, L.kpart, L.kdots, oy, oa, ob};
         const double bytes = spmv_dot<T>(L.M, vsel, sargs(z, w), q, c->s);
         std::string tag;
         if (c->prof.on) {
@@ -720,12 +724,8 @@ static void kc_product_dots(nbp_ctx *c, Level &L, int vsel, const T *z, T *w, co
         return;
     }
     do_spmv<T>(c, L.M, vsel, sargs(z, w), EPI_SET, false);
-    // algorithmic bytes: each distinct vector the dots read, once
-    const double vn = (double)n * sizeof(T);
-    const double nvec = 1.0 + (da != w ? 1.0 : 0.0) + (db && db != w && db != da ? 1.0 : 0.0);
-    timed(c, "kcycle/dots", nvec * vn, [&] {
-        k_kdots<T><<<kKdotBlocks, 256, 0, c->s>>>(w, da, db ? w : (const T *)nullptr, db, n, L.kdots, o0, o1);
-    });
+    timed(c, "kcycle/dots", (db ? 3.0 : 2.0) * (double)n * sizeof(T),
+          [&] { klaunch(k_kdots<T>, (unsigned)kKdotBlocks, 256u, c->s, w, da, db, n, L.kdots, oy, oa, ob); });
 }
 
 template <typename T>
@@ -733,19 +733,22 @@ static void kcycle_level(nbp_ctx *c, Hier &H, int cl, int vsel, const T *b, T *x
     Level &L = H.L[cl];
     const long long n = (long long)L.M.nbr * H.bs;
     T *r = wvec<T>(L, 5), *z1 = wvec<T>(L, 6), *w1 = wvec<T>(L, 7), *z2 = wvec<T>(L, 8), *w2 = wvec<T>(L, 9);
-    const unsigned g = grid_for(n);
     const double vn = (double)n * sizeof(T);   // bytes of one level vector
     if (!first_done) copy<T>(r, b, n, c->s);   // else the restriction wrote r
     vcycle_level<T>(c, H, cl, vsel, b, z1, first_done);
-    kc_product_dots<T>(c, L, vsel, z1, w1, w1, r, 0, 1);   // kd[0] = w1.w1, kd[1] = w1.r
-    // algorithmic bytes: each distinct vector an update reads or writes, once
-    timed(c, "kcycle/update", 3.0 * vn, [&] { k_kupd1<T><<<g, 256, 0, c->s>>>(r, w1, L.kdots, n); });
-    vcycle_level<T>(c, H, cl, vsel, r, z2);
-    kc_product_dots<T>(c, L, vsel, z2, w2, w1, (const T *)nullptr, 3, 3);   // kd[3] = w2.w1
-    // w2 -= beta w1, z2 -= beta z1, then kd[4] = w2.w2, kd[5] = w2.r
-    timed(c, "kcycle/update+dots", 7.0 * vn,
-          [&] { k_kupd2_dots<T><<<kKdotBlocks, 256, 0, c->s>>>(w2, z2, w1, z1, r, L.kdots, n); });
-    timed(c, "kcycle/update", 3.0 * vn, [&] { k_kupd3<T><<<g, 256, 0, c->s>>>(x, z1, z2, L.kdots, n); });
+    kc_product_dots<T>(c, L, vsel, z1, w1, r, (const T *)nullptr, 0, 1, 1);   // kd[0] = w1.w1, kd[1] = w1.r
+    // r -= a1 w1 and, with smoothing on this level, the second cycle's first
+    // step; algorithmic bytes: each distinct vector read or written, once
+    const bool first = H.cheb > 0 && cl < H.nlev - 1;
+    const double fb = first ? (double)L.M.nbr * H.bs * H.bs * sizeof(T) + (H.cheb > 1 ? 2.0 : 1.0) * vn : 0.0;
+    timed(c, "kcycle/update", 3.0 * vn + fb, [&] {
+        klaunch(k_kupd1<T>, grid_for(L.M.nbr), 256u, c->s, r, w1, L.kdots, L.M.nbr, H.bs,
+                first ? dinv_of<T>(L) : (const T *)nullptr, first ? (T)(1.0 / cheb_of(L).theta) : T(0),
+                first && H.cheb > 1 ? wvec<T>(L, 4) : (T *)nullptr, wvec<T>(L, 2));
+    });
+    vcycle_level<T>(c, H, cl, vsel, r, z2, first);
+    kc_product_dots<T>(c, L, vsel, z2, w2, w1, r, 4, 3, 5);   // kd[4] = w2.w2, kd[3] = w2.w1, kd[5] = w2.r
+    timed(c, "kcycle/update", 3.0 * vn, [&] { klaunch(k_kupd2<T>, grid_for(n), 256u, c->s, x, z1, z2, L.kdots, n); });
 }
 
 // V(1,1)-cycle from level l with right-hand side b; result written to out.
@@ -764,11 +767,11 @@ static void vcycle_level(nbp_ctx *c, Hier &H, int l, int vsel, const T *b, T *ou
                       const T *ci = cinv_of<T>(H);
                       if constexpr (std::is_same<T, float>::value) {
                           if (H.nc % 4 == 0 && al16(ci) && al16(b))
-                              k_dense_gemv_rows<float, true><<<(unsigned)H.nc, kGemvThreads, 0, c->s>>>(ci, H.nc, b, out);
+                              klaunch(k_dense_gemv_rows<float, true>, (unsigned)H.nc, (unsigned)kGemvThreads, c->s, ci, H.nc, b, out);
                           else
-                              k_dense_gemv_rows<float, false><<<(unsigned)H.nc, kGemvThreads, 0, c->s>>>(ci, H.nc, b, out);
+                              klaunch(k_dense_gemv_rows<float, false>, (unsigned)H.nc, (unsigned)kGemvThreads, c->s, ci, H.nc, b, out);
                       } else {
-                          k_dense_gemv<T><<<grid_exact((long long)H.nc * 32), 256, 0, c->s>>>(ci, H.nc, b, out);
+                          klaunch(k_dense_gemv<T>, grid_exact((long long)H.nc * 32), (unsigned)256, c->s, ci, H.nc, b, out);
                       }
                   });
         } else {
@@ -804,14 +807,14 @@ static void vcycle_level(nbp_ctx *c, Hier &H, int l, int vsel, const T *b, T *ou
         // + the coarse block-diagonal inverse read, d (degree > 1) and x written (+ the copy)
         const double fbytes = rbytes + (double)Lc.M.nbr * bs * bs * sizeof(T) + (k > 1 ? 2.0 : 1.0) * ncv + (kc ? ncv : 0.0);
         timed(c, "amg/restrict+first", fbytes, [&] {
-            k_restrict_first<T><<<grid_exact((long long)Lc.M.nbr * 8), 256, 0, c->s>>>(
+            klaunch(k_restrict_first<T>, grid_exact((long long)Lc.M.nbr * 8), (unsigned)256, c->s, 
                 L.mptr, L.mem, Lc.M.nbr, bs, r, bc, dinv_of<T>(Lc), (T)(1.0 / chc.theta), k > 1 ? wvec<T>(Lc, 4) : (T *)nullptr,
                 wvec<T>(Lc, 2),
                 kc ? wvec<T>(Lc, 5) : (T *)nullptr);
         });
     } else {
         timed(c, "amg/restrict", rbytes,
-              [&] { k_restrict<T><<<grid_exact((long long)Lc.M.nbr * 8), 256, 0, c->s>>>(L.mptr, L.mem, Lc.M.nbr, bs, r, bc); });
+              [&] { klaunch(k_restrict<T>, grid_exact((long long)Lc.M.nbr * 8), (unsigned)256, c->s, L.mptr, L.mem, Lc.M.nbr, bs, r, bc); });
     }
     // (a prolongation fused into the coarse level's last kernel, as a scatter
     // over each aggregate's members, was slower: uncoalesced fine updates)
@@ -843,8 +846,8 @@ static void vcycle_level(nbp_ctx *c, Hier &H, int l, int vsel, const T *b, T *ou
         constexpr int W = Vec16<T>::W;
         const long long threads = L.M.nbr / W + L.M.nbr % W;
         if ((bs == 3 || bs == 1) && al16(cur) && al16(L.agg)) {
-            if (bs == 3) k_prolong_v<T, 3><<<grid_exact(threads), 256, 0, c->s>>>(L.agg, L.M.nbr, xc, cur);
-            else k_prolong_v<T, 1><<<grid_exact(threads), 256, 0, c->s>>>(L.agg, L.M.nbr, xc, cur);
+            if (bs == 3) klaunch(k_prolong_v<T, 3>, grid_exact(threads), (unsigned)256, c->s, L.agg, L.M.nbr, xc, cur);
+            else klaunch(k_prolong_v<T, 1>, grid_exact(threads), (unsigned)256, c->s, L.agg, L.M.nbr, xc, cur);
         } else {
             k_prolong<T><<<grid_exact(n), 256, 0, c->s>>>(L.agg, L.M.nbr, bs, xc, cur);
         }
@@ -1240,6 +1243,7 @@ template <class F> static long long emit_while(nbp_ctx *c, cudaGraphConditionalH
     cudaStream_t saved = c->s;
     NBP_CUDA(cudaStreamBeginCaptureToGraph(c->dl_cap[depth], bg, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     c->s = c->dl_cap[depth];
+    g_pdl.prev = false;
     try {
         body();
     } catch (...) {
@@ -1251,6 +1255,7 @@ template <class F> static long long emit_while(nbp_ctx *c, cudaGraphConditionalH
     cudaGraph_t out = nullptr;
     NBP_CUDA(cudaStreamEndCapture(c->dl_cap[depth], &out));
     c->s = saved;
+    g_pdl.prev = false;
     return kernel_nodes(bg);
 }
 
@@ -1269,30 +1274,33 @@ template <typename T> static void arnoldi_dl(nbp_ctx *c, Krylov<T> &K, GmDev *st
     gv.h = h;
     if (c->gs_one_pass) gv.h2 = nullptr;
     if (vec && K.n <= gs_cluster_max<T>() && K.m <= kGsCols) {   // a short vector: the whole step in one cluster
-        k_gs_cluster<T><<<kGsCluster, kGsThreads, 0, c->s>>>(K.V, K.ld, jp, K.w, K.n, c->gs_one_pass ? 1 : 2, K.h1, K.h2, gv);
+        klaunch(k_gs_cluster<T>, kGsCluster, (unsigned)kGsThreads, c->s, K.V, K.ld, jp, K.w, K.n, c->gs_one_pass ? 1 : 2, K.h1, K.h2, gv);
         NBP_LAUNCHED();
         return;
     }
     // one pass: the multi-dot, then subtract + norm + Givens update
     const double *coef = c->gs_one_pass ? K.h1 : K.h2;
+    // the norm pass: a block per 256 pieces up to the partials' kReduceBlocks
+    const long long pieces = (K.n + Vec16<T>::W - 1) / Vec16<T>::W;
+    const unsigned gn = (unsigned)std::max<long long>(1, std::min<long long>(kReduceBlocks, (pieces + 255) / 256));
     if (vec) {
         const unsigned g1 = K.grid_md ? K.grid_md : arnoldi_grids<T>().mdot_dl_v;
         const unsigned g2 = K.grid ? K.grid : arnoldi_grids<T>().mpd_dl_v;
-        k_mdot_dl<T, 8, true><<<g1, 256, 0, c->s>>>(K.V, K.ld, jp, 1, K.w, K.n, K.partial, K.h1, K.ticket, GivensArgs());
+        klaunch(k_mdot_dl<T, 8, true>, g1, (unsigned)256, c->s, K.V, K.ld, jp, 1, K.w, K.n, K.partial, K.h1, K.ticket, GivensArgs());
         if (!c->gs_one_pass)
-            k_maxpy_dot_dl<T, kFusedCols, true><<<g2, 256, 0, c->s>>>(K.V, K.ld, jp, 1, K.h1, K.w, K.n, 0, K.partial,
-                                                                      K.h2, K.ticket, GivensArgs());
-        k_maxpy_dot_dl<T, kFusedCols, true><<<g2, 256, 0, c->s>>>(K.V, K.ld, jp, 1, coef, K.w, K.n, 1, K.partial, K.nrm,
-                                                                  K.ticket, gv);
+            klaunch(k_maxpy_dot_dl<T, kFusedCols, true>, g2, (unsigned)256, c->s, K.V, K.ld, jp, 1, K.h1, K.w, K.n, K.partial,
+                    K.h2, K.ticket);
+        klaunch(k_maxpy_norm_dl<T, true>, gn, 256u, c->s, K.V, K.ld, jp, coef, K.m + 1, K.w, K.n, K.partial, K.nrm, K.ticket,
+                gv);
     } else {
         const unsigned g1 = K.grid_md ? K.grid_md : arnoldi_grids<T>().mdot_dl_s;
         const unsigned g2 = K.grid ? K.grid : arnoldi_grids<T>().mpd_dl_s;
-        k_mdot_dl<T, 8, false><<<g1, 256, 0, c->s>>>(K.V, K.ld, jp, 1, K.w, K.n, K.partial, K.h1, K.ticket, GivensArgs());
+        klaunch(k_mdot_dl<T, 8, false>, g1, (unsigned)256, c->s, K.V, K.ld, jp, 1, K.w, K.n, K.partial, K.h1, K.ticket, GivensArgs());
         if (!c->gs_one_pass)
-            k_maxpy_dot_dl<T, kFusedCols, false><<<g2, 256, 0, c->s>>>(K.V, K.ld, jp, 1, K.h1, K.w, K.n, 0, K.partial,
-                                                                       K.h2, K.ticket, GivensArgs());
-        k_maxpy_dot_dl<T, kFusedCols, false><<<g2, 256, 0, c->s>>>(K.V, K.ld, jp, 1, coef, K.w, K.n, 1, K.partial,
-                                                                   K.nrm, K.ticket, gv);
+            klaunch(k_maxpy_dot_dl<T, kFusedCols, false>, g2, (unsigned)256, c->s, K.V, K.ld, jp, 1, K.h1, K.w, K.n, K.partial,
+                    K.h2, K.ticket);
+        klaunch(k_maxpy_norm_dl<T, false>, gn, 256u, c->s, K.V, K.ld, jp, coef, K.m + 1, K.w, K.n, K.partial, K.nrm, K.ticket,
+                gv);
     }
     NBP_LAUNCHED();
 }
@@ -1301,17 +1309,18 @@ template <typename T> static void arnoldi_dl(nbp_ctx *c, Krylov<T> &K, GmDev *st
 template <typename T> static void start_col(nbp_ctx *c, Krylov<T> &K, GmDev *st, const T *b) {
     const bool vec = al16(K.V) && al16(K.w) && al16(b) && (K.ld * (long long)sizeof(T)) % 16 == 0;
     const unsigned grid = grid_for(K.n / (vec ? Vec16<T>::W : 1) + 1);
-    if (vec) k_start_col<T, true><<<grid, 256, 0, c->s>>>(K.V, K.ld, &st->j, b, K.w, K.st, K.n);
-    else k_start_col<T, false><<<grid, 256, 0, c->s>>>(K.V, K.ld, &st->j, b, K.w, K.st, K.n);
+    if (vec) klaunch(k_start_col<T, true>, grid, (unsigned)256, c->s, K.V, K.ld, &st->j, b, K.w, K.st, K.n);
+    else klaunch(k_start_col<T, false>, grid, (unsigned)256, c->s, K.V, K.ld, &st->j, b, K.w, K.st, K.n);
     NBP_LAUNCHED();
 }
 
-// x += Z(:, 0..j-1) y after the cycle (j read on the device)
-template <typename T> static void update_dl(nbp_ctx *c, Krylov<T> &K, GmDev *st, T *x) {
+// x = Z(:, 0..j-1) y after the cycle (j read on the device); add: x += it
+template <typename T> static void update_dl(nbp_ctx *c, Krylov<T> &K, GmDev *st, T *x, bool add) {
     const bool vec = al16(K.Z) && al16(x) && (K.ld * (long long)sizeof(T)) % 16 == 0;
     const unsigned grid = grid_for(K.n / (vec ? Vec16<T>::W : 1) + 1, 256, 8LL * kSMs * 4);
-    if (vec) k_maxpy_dl<T, true><<<grid, 256, 0, c->s>>>(K.Z, K.ld, &st->j, 0, K.y, 1.0, x, K.n);
-    else k_maxpy_dl<T, false><<<grid, 256, 0, c->s>>>(K.Z, K.ld, &st->j, 0, K.y, 1.0, x, K.n);
+    auto go = [&](auto kernel) { klaunch(kernel, grid, 256u, c->s, K.Z, K.ld, &st->j, K.y, x, K.n); };
+    if (vec) add ? go(k_maxpy_dl<T, true, false>) : go(k_maxpy_dl<T, true, true>);
+    else add ? go(k_maxpy_dl<T, false, false>) : go(k_maxpy_dl<T, false, true>);
     NBP_LAUNCHED();
 }
 
@@ -1323,11 +1332,15 @@ template <typename T, typename Op, typename Pc>
 static long long gmres_dl(nbp_ctx *c, Krylov<T> &K, long long n, GmDev *st, const double *rtol, const int *m,
                           const int *nmax, long long *its_total, long long *solves, const T *b, T *x, Pc pc, Op op,
                           int depth) {
-    fill<T>(x, T(0), n, c->s);
-    mdot<T>(c, K, b, n, 1, b, K.nrm);
     const cudaGraphConditionalHandle h = new_handle(c);
-    k_dl_init<<<1, 256, 0, c->s>>>(st, K.g, K.m + 1, K.nrm, K.beta, K.st, rtol, &c->dl_par->atol, m, nmax, h);
-    NBP_LAUNCHED();
+    {
+        const DlStart q{st, K.g, K.beta, K.st, rtol, &c->dl_par->atol, m, nmax, h};
+        const long long pieces = (n + Vec16<T>::W - 1) / Vec16<T>::W;
+        const unsigned g = (unsigned)std::max<long long>(1, std::min<long long>(2 * kSMs, pieces / 1024));
+        if (al16(b)) klaunch(k_norm_start<T, true>, g, 256u, c->s, b, n, K.partial, K.nrm, K.ticket, q);
+        else klaunch(k_norm_start<T, false>, g, 256u, c->s, b, n, K.partial, K.nrm, K.ticket, q);
+        NBP_LAUNCHED();
+    }
     const long long kb = emit_while(c, h, depth, [&] {
         const T *z = pc(K, st, b);
         if (z) {
@@ -1339,9 +1352,9 @@ static long long gmres_dl(nbp_ctx *c, Krylov<T> &K, long long n, GmDev *st, cons
         }
         arnoldi_dl<T>(c, K, st, h);
     });
-    k_dl_end<<<1, 32, 0, c->s>>>(st, K.H, K.m, K.g, K.y, its_total, solves);
+    klaunch(k_dl_end, 1u, 32u, c->s, st, K.H, K.m, K.g, K.y, its_total, solves);
     NBP_LAUNCHED();
-    update_dl<T>(c, K, st, x);
+    update_dl<T>(c, K, st, x, false);
     return kb;
 }
 
@@ -1357,7 +1370,7 @@ template <typename T> static const T *cycle_from_col(nbp_ctx *c, Hier &H, Krylov
     T *gb = wvec<T>(L0, 0), *gx = wvec<T>(L0, 1);
     if (H.cheb > 0 && H.nlev > 1) {
         const Cheb ch = cheb_of(L0);
-        k_start_cheb<T><<<grid_exact(n), 256, 0, c->s>>>(L0.M.nbr, H.bs, dinv_of<T>(L0), K.V, K.ld, &st->j, b, K.w, K.st,
+        klaunch(k_start_cheb<T>, grid_exact(n), (unsigned)256, c->s, L0.M.nbr, H.bs, dinv_of<T>(L0), K.V, K.ld, &st->j, b, K.w, K.st,
                                                          (T)(1.0 / ch.theta), H.cheb > 1 ? wvec<T>(L0, 4) : (T *)nullptr,
                                                          wvec<T>(L0, 2));
         NBP_LAUNCHED();
@@ -1472,9 +1485,9 @@ static void outer_dl(nbp_ctx *c) {
             NBP_LAUNCHED();
             arnoldi_dl<double>(c, K, st, hi);
         });
-        k_dl_end<<<1, 32, 0, c->s>>>(st, K.H, K.m, K.g, K.y, nullptr, nullptr);
+        klaunch(k_dl_end, 1u, 32u, c->s, st, K.H, K.m, K.g, K.y, (long long *)nullptr, (long long *)nullptr);
         NBP_LAUNCHED();
-        update_dl<double>(c, K, st, x);
+        update_dl<double>(c, K, st, x, true);
         apply_full(c, x, K.w);                       // true residual: the next restart vector or the check
         k_sub<double><<<grid_for(n), 256, 0, c->s>>>(K.r, b, K.w, n);
         NBP_LAUNCHED();
@@ -1565,15 +1578,18 @@ static void dl_prepare(nbp_ctx *c) {
 static void capture_solve(nbp_ctx *c) {
     const bool prof = c->prof.on;
     c->prof.on = false;
+    g_pdl = PdlState{true, false};
     try {
         const long long k0 = kernel_nodes(capture_graph_of(c->s));
         outer_dl(c);
         c->dl_k_top = kernel_nodes(capture_graph_of(c->s)) - k0;
     } catch (...) {
         c->prof.on = prof;
+        g_pdl = PdlState{};
         throw;
     }
     c->prof.on = prof;
+    g_pdl = PdlState{};
 }
 
 static void dl_build(nbp_ctx *c) {
@@ -2457,7 +2473,6 @@ const char *nbp_profile_report(const nbp_ctx *c) { return c ? c->report.c_str() 
 // stream per instance, a pool of host threads driving the instances' nested
 // solves so that their kernels (and graph replays) overlap on the GPU.
 #include <atomic>
-#include <thread>
 
 struct nbp_batch {
     std::vector<nbp_ctx *> ctx;

@@ -18,17 +18,17 @@ static void launch_epi(const SpmvArgs &a, int epi, bool lr, cudaStream_t s) {
     switch (epi) {
     case EPI_SET:
         if constexpr (BR == 3 && BC == 3) {
-            if (lr) { k_bspmv<BR, BC, G, VT, XT, EPI_SET, true><<<grid, 256, 0, s>>>(a); break; }
+            if (lr) { klaunch(k_bspmv<BR, BC, G, VT, XT, EPI_SET, true>, grid, 256u, s, a); break; }
         }
-        k_bspmv<BR, BC, G, VT, XT, EPI_SET, false><<<grid, 256, 0, s>>>(a);
+        klaunch(k_bspmv<BR, BC, G, VT, XT, EPI_SET, false>, grid, 256u, s, a);
         break;
-    case EPI_ADD: k_bspmv<BR, BC, G, VT, XT, EPI_ADD, false><<<grid, 256, 0, s>>>(a); break;
-    case EPI_SUB: k_bspmv<BR, BC, G, VT, XT, EPI_SUB, false><<<grid, 256, 0, s>>>(a); break;
+    case EPI_ADD: klaunch(k_bspmv<BR, BC, G, VT, XT, EPI_ADD, false>, grid, 256u, s, a); break;
+    case EPI_SUB: klaunch(k_bspmv<BR, BC, G, VT, XT, EPI_SUB, false>, grid, 256u, s, a); break;
     case EPI_RES:
-        if constexpr (BR == BC) { k_bspmv<BR, BC, G, VT, XT, EPI_RES, false><<<grid, 256, 0, s>>>(a); break; }
+        if constexpr (BR == BC) { klaunch(k_bspmv<BR, BC, G, VT, XT, EPI_RES, false>, grid, 256u, s, a); break; }
         throw Error{NBP_ERR_INVALID, "spmv: residual epilogue needs square blocks"};
     case EPI_CHEB:
-        if constexpr (BR == BC) { k_bspmv<BR, BC, G, VT, XT, EPI_CHEB, false><<<grid, 256, 0, s>>>(a); break; }
+        if constexpr (BR == BC) { klaunch(k_bspmv<BR, BC, G, VT, XT, EPI_CHEB, false>, grid, 256u, s, a); break; }
         throw Error{NBP_ERR_INVALID, "spmv: Chebyshev epilogue needs square blocks"};
     default: throw Error{NBP_ERR_INVALID, "spmv: unknown epilogue"};
     }
@@ -68,7 +68,7 @@ static void launch_vt(const DMat &M, int vsel, SpmvArgs a, int G, int epi, bool 
     }
 }
 
-int fine_threads(int rows) { return rows < 10000 ? 8 : rows < 32000 ? 4 : rows < 80000 ? 2 : 1; }
+int fine_threads(int rows) { return rows < 12000 ? 8 : rows < 45000 ? 4 : rows < 200000 ? 2 : 1; }
 
 int choose_group(const DMat &M) {
     const double per_row = M.nbr ? (double)M.nnz * M.bb() / M.nbr : 0.0;
@@ -78,20 +78,26 @@ int choose_group(const DMat &M) {
     return 32;
 }
 
+// threads per row of the sliced kernel that M is tuned to (0: a flat kernel)
+static int sell_threads(const DMat &M) {
+    const int G = M.tuned >= 0 ? M.tuned : 0;
+    return G == 0 ? 1 : (is_sellm(G) ? G - kSellMT : 0);
+}
+
 template <int BS, typename VT, typename XT, int C>
 static void launch_sell_epi(const SpmvArgs &a, int epi, bool lr, cudaStream_t s) {
     const unsigned grid = grid_exact((long long)a.nslice * C);
     switch (epi) {
     case EPI_SET:
         if constexpr (BS == 3) {
-            if (lr) { k_sell<BS, VT, XT, EPI_SET, true, C><<<grid, 256, 0, s>>>(a); break; }
+            if (lr) { klaunch(k_sell<BS, VT, XT, EPI_SET, true, C>, grid, 256u, s, a); break; }
         }
-        k_sell<BS, VT, XT, EPI_SET, false, C><<<grid, 256, 0, s>>>(a);
+        klaunch(k_sell<BS, VT, XT, EPI_SET, false, C>, grid, 256u, s, a);
         break;
-    case EPI_ADD: k_sell<BS, VT, XT, EPI_ADD, false, C><<<grid, 256, 0, s>>>(a); break;
-    case EPI_SUB: k_sell<BS, VT, XT, EPI_SUB, false, C><<<grid, 256, 0, s>>>(a); break;
-    case EPI_RES: k_sell<BS, VT, XT, EPI_RES, false, C><<<grid, 256, 0, s>>>(a); break;
-    case EPI_CHEB: k_sell<BS, VT, XT, EPI_CHEB, false, C><<<grid, 256, 0, s>>>(a); break;
+    case EPI_ADD: klaunch(k_sell<BS, VT, XT, EPI_ADD, false, C>, grid, 256u, s, a); break;
+    case EPI_SUB: klaunch(k_sell<BS, VT, XT, EPI_SUB, false, C>, grid, 256u, s, a); break;
+    case EPI_RES: klaunch(k_sell<BS, VT, XT, EPI_RES, false, C>, grid, 256u, s, a); break;
+    case EPI_CHEB: klaunch(k_sell<BS, VT, XT, EPI_CHEB, false, C>, grid, 256u, s, a); break;
     default: throw Error{NBP_ERR_INVALID, "spmv: unknown epilogue"};
     }
     NBP_LAUNCHED();
@@ -103,14 +109,14 @@ static void launch_sellm_epi(const SpmvArgs &a, int epi, bool lr, cudaStream_t s
     switch (epi) {
     case EPI_SET:
         if constexpr (BS == 3) {
-            if (lr) { k_sellm<BS, VT, XT, EPI_SET, C, T, true><<<grid, 256, 0, s>>>(a); break; }
+            if (lr) { klaunch(k_sellm<BS, VT, XT, EPI_SET, C, T, true>, grid, 256u, s, a); break; }
         }
-        k_sellm<BS, VT, XT, EPI_SET, C, T><<<grid, 256, 0, s>>>(a);
+        klaunch(k_sellm<BS, VT, XT, EPI_SET, C, T>, grid, 256u, s, a);
         break;
-    case EPI_ADD: k_sellm<BS, VT, XT, EPI_ADD, C, T><<<grid, 256, 0, s>>>(a); break;
-    case EPI_SUB: k_sellm<BS, VT, XT, EPI_SUB, C, T><<<grid, 256, 0, s>>>(a); break;
-    case EPI_RES: k_sellm<BS, VT, XT, EPI_RES, C, T><<<grid, 256, 0, s>>>(a); break;
-    case EPI_CHEB: k_sellm<BS, VT, XT, EPI_CHEB, C, T><<<grid, 256, 0, s>>>(a); break;
+    case EPI_ADD: klaunch(k_sellm<BS, VT, XT, EPI_ADD, C, T>, grid, 256u, s, a); break;
+    case EPI_SUB: klaunch(k_sellm<BS, VT, XT, EPI_SUB, C, T>, grid, 256u, s, a); break;
+    case EPI_RES: klaunch(k_sellm<BS, VT, XT, EPI_RES, C, T>, grid, 256u, s, a); break;
+    case EPI_CHEB: klaunch(k_sellm<BS, VT, XT, EPI_CHEB, C, T>, grid, 256u, s, a); break;
     default: throw Error{NBP_ERR_INVALID, "spmv: unknown epilogue"};
     }
     NBP_LAUNCHED();
@@ -160,16 +166,16 @@ template <int BR, int BC, typename VT, typename XT, int C, int T>
 static void launch_sellr_t(const SpmvArgs &a, int epi, cudaStream_t s) {
     const unsigned grid = grid_exact((long long)a.nslice * C * T);
     switch (epi) {
-    case EPI_SET: k_sellr<BR, BC, VT, XT, EPI_SET, C, T><<<grid, 256, 0, s>>>(a); break;
-    case EPI_ADD: k_sellr<BR, BC, VT, XT, EPI_ADD, C, T><<<grid, 256, 0, s>>>(a); break;
-    case EPI_SUB: k_sellr<BR, BC, VT, XT, EPI_SUB, C, T><<<grid, 256, 0, s>>>(a); break;
+    case EPI_SET: klaunch(k_sellr<BR, BC, VT, XT, EPI_SET, C, T>, grid, 256u, s, a); break;
+    case EPI_ADD: klaunch(k_sellr<BR, BC, VT, XT, EPI_ADD, C, T>, grid, 256u, s, a); break;
+    case EPI_SUB: klaunch(k_sellr<BR, BC, VT, XT, EPI_SUB, C, T>, grid, 256u, s, a); break;
     default: throw Error{NBP_ERR_INVALID, "spmv: rectangular blocks take SET, ADD or SUB"};
     }
     NBP_LAUNCHED();
 }
 template <int BR, int BC, typename VT, typename XT, int C>
-static void launch_sellr_epi(const SpmvArgs &a, int epi, cudaStream_t s) {
-    switch (fine_threads(a.nbr)) {
+static void launch_sellr_epi(const SpmvArgs &a, int T, int epi, cudaStream_t s) {
+    switch (T) {
     case 8: launch_sellr_t<BR, BC, VT, XT, C, 8>(a, epi, s); break;
     case 4: launch_sellr_t<BR, BC, VT, XT, C, 4>(a, epi, s); break;
     case 2: launch_sellr_t<BR, BC, VT, XT, C, 2>(a, epi, s); break;
@@ -183,14 +189,15 @@ static void launch_sellr(const DMat &M, int vsel, SpmvArgs a, int epi, cudaStrea
     a.nslice = M.nslice;
     a.sl_ptr = M.sl_ptr;
     a.sl_ci = M.sl_ci;
+    const int T = std::max(1, sell_threads(M));
     if constexpr (sizeof(XT) == 8) {
         a.val = M.sl_v;
-        if (M.sl_c == 8) launch_sellr_epi<BR, BC, double, double, 8>(a, epi, s);
-        else launch_sellr_epi<BR, BC, double, double, 32>(a, epi, s);
+        if (M.sl_c == 8) launch_sellr_epi<BR, BC, double, double, 8>(a, T, epi, s);
+        else launch_sellr_epi<BR, BC, double, double, 32>(a, T, epi, s);
     } else {
         a.val = M.sl_v32;
-        if (M.sl_c == 8) launch_sellr_epi<BR, BC, float, float, 8>(a, epi, s);
-        else launch_sellr_epi<BR, BC, float, float, 32>(a, epi, s);
+        if (M.sl_c == 8) launch_sellr_epi<BR, BC, float, float, 8>(a, T, epi, s);
+        else launch_sellr_epi<BR, BC, float, float, 32>(a, T, epi, s);
     }
 }
 
@@ -212,11 +219,6 @@ static double product_bytes(const DMat &M, int vsel, int xs, int epi, bool slice
     return b;
 }
 
-static int sell_threads(const DMat &M) {
-    const int G = M.tuned >= 0 ? M.tuned : 0;
-    return G == 0 ? 1 : (is_sellm(G) ? G - kSellMT : 0);
-}
-
 bool spmv_dot_ok(const DMat &M, int vsel, int xbytes, long long max_blocks) {
     if (M.br != 1 || M.bc != 1 || !M.sl_ci || M.nbr == 0) return false;
     const int T = sell_threads(M);
@@ -229,10 +231,10 @@ bool spmv_dot_ok(const DMat &M, int vsel, int xbytes, long long max_blocks) {
 template <typename VT, typename XT, int C>
 static void launch_sell_dot(const SpmvArgs &a, const DotArgs &q, int T, cudaStream_t s) {
     const unsigned grid = grid_exact((long long)a.nslice * C * T);
-    if (T == 8) k_sell_dot<VT, XT, C, 8><<<grid, 256, 0, s>>>(a, q);
-    else if (T == 4) k_sell_dot<VT, XT, C, 4><<<grid, 256, 0, s>>>(a, q);
-    else if (T == 2) k_sell_dot<VT, XT, C, 2><<<grid, 256, 0, s>>>(a, q);
-    else k_sell_dot<VT, XT, C, 1><<<grid, 256, 0, s>>>(a, q);
+    if (T == 8) klaunch(k_sell_dot<VT, XT, C, 8>, grid, 256u, s, a, q);
+    else if (T == 4) klaunch(k_sell_dot<VT, XT, C, 4>, grid, 256u, s, a, q);
+    else if (T == 2) klaunch(k_sell_dot<VT, XT, C, 2>, grid, 256u, s, a, q);
+    else klaunch(k_sell_dot<VT, XT, C, 1>, grid, 256u, s, a, q);
     NBP_LAUNCHED();
 }
 template <typename VT, typename XT>
@@ -261,7 +263,7 @@ double spmv_dot(const DMat &M, int vsel, SpmvArgs a, const DotArgs &q, cudaStrea
         launch_sell_dot_c<float, float>(M, a, q, T, s);
     }
     const double ny = (double)M.nbr * sizeof(XT);
-    return product_bytes(M, vsel, (int)sizeof(XT), EPI_SET, true) + (q.da != a.y ? ny : 0.0) + (q.db ? ny : 0.0);
+    return product_bytes(M, vsel, (int)sizeof(XT), EPI_SET, true) + ny + (q.db ? ny : 0.0);
 }
 
 template <typename XT>
@@ -294,19 +296,28 @@ double spmv(const DMat &M, int vsel, SpmvArgs a, int epi, bool lr, cudaStream_t 
     return product_bytes(M, vsel, xs, epi, false);
 }
 
-// threads per row of the post-smoothing product (rows of A P hold 6-7 blocks,
-// those of S_hat P 10-20 scalars)
-static int post_threads(const DMat &AP) { return AP.nbr < 40000 ? 4 : AP.nbr < 400000 ? 2 : 1; }
+// Threads per row and pairs loaded at once of the post-smoothing product (rows
+// of A P hold 6-8 blocks, those of S_hat P 10-20 scalars): one thread streams
+// long levels, its epilogue's operands loaded after the products (4.34M unknowns:
+// 745 ms a solve; 752 with them loaded first; 806 against 780 with two threads), two with two pairs fill the GPU on shorter ones (0.56M: 171.8 ms
+// against 178.0 with one pair each and 174.9 with one thread and four; 171.0
+// against 176.6 with four threads on its 20,000-row level), four where a row's
+// chain of loads is all there is (cube of 16: 20.6 ms against 21.2; unpaired
+// values, 29,760 rows: 40.1 against 41.0).
+static int post_threads(const DMat &AP, bool paired) {
+    if (AP.nbr < (paired ? 8000 : 40000)) return 4;
+    return AP.nbr < 400000 ? 2 : 1;
+}
 
 template <int BS, typename VT, typename XT>
 static void launch_post(const DMat &AP, const SpmvArgs &a, cudaStream_t s) {
-    const int T = post_threads(AP);
+    const int T = post_threads(AP, std::is_same<VT, __nv_bfloat16>::value);
     const unsigned grid = grid_exact((long long)AP.nslice * AP.sl_c * T);
-    auto go = [&](auto c, auto t) { k_sellm<BS, VT, XT, EPI_POST, decltype(c)::value, decltype(t)::value><<<grid, 256, 0, s>>>(a); };
     auto with_t = [&](auto c) {
-        if (T == 4) go(c, std::integral_constant<int, 4>());
-        else if (T == 2) go(c, std::integral_constant<int, 2>());
-        else go(c, std::integral_constant<int, 1>());
+        constexpr int C = decltype(c)::value;
+        if (T == 4) klaunch(k_sellm<BS, VT, XT, EPI_POST, C, 4, false, 1>, grid, 256u, s, a);
+        else if (T == 2) klaunch(k_sellm<BS, VT, XT, EPI_POST, C, 2, false, 2>, grid, 256u, s, a);
+        else klaunch(k_sell<BS, VT, XT, EPI_POST, false, C, 2>, grid, 256u, s, a);
     };
     if (AP.sl_c == 8) with_t(std::integral_constant<int, 8>());
     else with_t(std::integral_constant<int, 32>());

@@ -19,7 +19,10 @@ int choose_group(const DMat &M);
 // Threads per row of the finest level's products (A, its AMG level and the
 // coupling blocks, about 15 entries a row): one where the rows alone fill the
 // GPU (152 SMs x 2048 threads), up to eight where they do not and a row's
-// chain of loads is what a product takes.
+// chain of loads is what a product takes.  Solves with 1 / 2 / 4 / 8 threads:
+// 29,760 rows 52.1 / 42.4 / 41.4 / 42.9 ms, 60,625 rows 51.3 / 47.8 / 48.3 /
+// 54.0 ms, 68,921 rows 66.7 / 61.9 / 64.1 / 71.5 ms; 140,481 rows 176.6 / 169.8;
+// 452,393 and 1,085,825 rows are faster with one.
 int fine_threads(int rows);
 
 // Whether y = M x with the K-cycle's inner products fused (k_sell_dot) runs
@@ -28,7 +31,7 @@ int fine_threads(int rows);
 // max_blocks blocks (the partials buffer).
 bool spmv_dot_ok(const DMat &M, int vsel, int xbytes, long long max_blocks);
 // Launch it (spmv_dot_ok must hold); returns the algorithmic bytes: the
-// product's, plus da and db when they are not y.
+// product's, plus da and db.
 template <typename XT>
 double spmv_dot(const DMat &M, int vsel, SpmvArgs a, const DotArgs &q, cudaStream_t s);
 
