@@ -42,7 +42,7 @@ void hier_free(Hier &H, cudaStream_t s) {
         dmat_free(L.M, s);
         dmat_free(L.AP, s);
         dfree(L.agg, s); dfree(L.mptr, s); dfree(L.mem, s); dfree(L.dinv, s); dfree(L.dinv32, s);
-        for (int q = 0; q < Level::kWork; ++q) { dfree(L.w64[q], s); dfree(L.w32[q], s); }
+        dfree(L.work, s);
         dfree(L.kdots, s); dfree(L.kpart, s);
         L = Level();
     }
@@ -240,24 +240,28 @@ __global__ void __cluster_dims__(kMatchCluster, 1, 1) __launch_bounds__(kMatchTh
     }
 }
 
-__global__ void k_root_flag(int n, const int *mate, int *flag) {
+// Numbering of a pass's aggregates by smallest node, and their member lists:
+// the root of a pair is its smaller node, so one scan over the nodes of
+// (1, members) of every root, packed in 64 bits, gives a root's aggregate and
+// where its members start (ascending).  No sort.
+__global__ void k_root_size(int n, const int *mate, unsigned long long *v) {
     const int u = blockIdx.x * blockDim.x + threadIdx.x;
-    if (u >= n) return;
-    const int m = mate[u];
-    flag[u] = (m < 0 || m > u) ? 1 : 0;
+    if (u > n) return;
+    const int m = u < n ? mate[u] : -1;
+    const bool root = u < n && (m < 0 || m > u);
+    v[u] = root ? (1ULL << 32) | (m >= 0 ? 2ULL : 1ULL) : 0ULL;
 }
-
-__global__ void k_map_from_roots(int n, const int *mate, const int *id, int *map) {
+__global__ void k_pair_members(int n, const int *mate, const unsigned long long *at, int *map, int *mptr, int *mem) {
     const int u = blockIdx.x * blockDim.x + threadIdx.x;
-    if (u >= n) return;
+    if (u > n) return;
+    if (u == n) { mptr[at[n] >> 32] = n; return; }   // the end of the last list
     const int m = mate[u];
-    map[u] = (m >= 0 && m < u) ? id[m] : id[u];
-}
-
-__global__ void k_compose(int n, const int *map, int *agg) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    agg[i] = map[agg[i]];
+    const int root = (m >= 0 && m < u) ? m : u;
+    const unsigned long long v = at[root];
+    const int I = (int)(v >> 32), p = (int)(v & 0xffffffffULL);
+    map[u] = I;
+    mem[root == u ? p : p + 1] = u;
+    if (root == u) mptr[I] = p;
 }
 
 __global__ void k_iota(int n, int *a) {
@@ -347,18 +351,6 @@ __global__ void k_count_valid(long long n, const unsigned long long *key, unsign
     const bool valid = key[t] != ~0ULL;
     const bool next_invalid = (t + 1 == n) || key[t + 1] == ~0ULL;
     if (valid && next_invalid) *cnt = (unsigned long long)(t + 1);
-}
-
-// keep flags of aggregates holding at least one non-isolated node
-__global__ void k_mark_keep(int n, const int *agg, const int *iso, int *keep) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (!iso[i]) keep[agg[i]] = 1;
-}
-__global__ void k_drop_isolated(int n, const int *iso, const int *newid, int *agg) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    agg[i] = iso[i] ? -1 : newid[agg[i]];
 }
 
 // ---------------------------------------------------- diagonal inverses
@@ -770,9 +762,17 @@ static int *rowptr_from_segments(const Segments &sg, int ncl, cudaStream_t s) {
     return rp;
 }
 
-// One matching pass on G; map (n) gets aggregate ids; returns the count.
-static int match_pass(const Graph &G, double theta, int *map, cudaStream_t s) {
+// Aggregates of one matching pass: their number and member lists
+struct Pairs {
+    int n = 0;
+    int *mptr = nullptr, *mem = nullptr;
+};
+static void pairs_free(Pairs &P, cudaStream_t s) { dfree(P.mptr, s); dfree(P.mem, s); P = Pairs(); }
+
+// One matching pass on G; map (n) gets aggregate ids.
+static Pairs match_pass(const Graph &G, double theta, int *map, cudaStream_t s) {
     const int n = G.n;
+    Pairs P;
     int *mate = dmalloc<int>(n, s), *pick = dmalloc<int>(n, s);
     k_fill<int><<<grid_for(n), 256, 0, s>>>(mate, -1, n);
     NBP_LAUNCHED();
@@ -806,16 +806,18 @@ static int match_pass(const Graph &G, double theta, int *map, cudaStream_t s) {
     }
     for (int *q : list) dfree(q, s);
     dfree(cnt, s);
-    int *flag = dmalloc<int>(n + 1, s), *id = dmalloc<int>(n + 1, s);
-    k_root_flag<<<grid_exact(n), 256, 0, s>>>(n, mate, flag);
+    unsigned long long *size = dmalloc<unsigned long long>(n + 1, s), *at = dmalloc<unsigned long long>(n + 1, s);
+    k_root_size<<<grid_exact(n + 1), 256, 0, s>>>(n, mate, size);
     NBP_LAUNCHED();
-    NBP_CUDA(cudaMemsetAsync(flag + n, 0, sizeof(int), s));
-    exclusive_scan(flag, id, n + 1, s);
-    const int nc = readback(id + n, s);
-    k_map_from_roots<<<grid_exact(n), 256, 0, s>>>(n, mate, id, map);
+    exclusive_scan(size, at, n + 1, s);
+    const int nc = (int)(readback(at + n, s) >> 32);
+    P.n = nc;
+    P.mptr = dmalloc<int>(nc + 1, s);
+    P.mem = dmalloc<int>(n, s);
+    k_pair_members<<<grid_exact(n + 1), 256, 0, s>>>(n, mate, at, map, P.mptr, P.mem);
     NBP_LAUNCHED();
-    dfree(mate, s); dfree(pick, s); dfree(flag, s); dfree(id, s);
-    return nc;
+    dfree(mate, s); dfree(pick, s); dfree(size, s); dfree(at, s);
+    return P;
 }
 
 // ---- coarse rows one per warp: coarse row I gathers its members' entries
@@ -846,15 +848,27 @@ __device__ __forceinline__ int group_row_entries(int I, int lane, const int *mpt
             const int v = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += v;
         }
-        const int start = off + incl - len;
-        for (int f = 0; f < len; ++f) {
-            const int e = rp[i] + f, q = start + f;
-            const int J = map[ci[e]];
-            const bool keep = J >= 0 && !(drop_diag && J == I);
-            sk[q] = keep ? (((unsigned)J * (unsigned)kGroupCap) | (unsigned)q) : ~0u;
-            se[q] = e;
+        // the entries of these members, a lane each: entry q belongs to the last
+        // member starting at or before it (its start and first entry by shuffle)
+        const int total = __shfl_sync(0xffffffffu, incl, 31), begin = incl - len, e0 = a < nm ? rp[i] : 0;
+        for (int p0 = 0; p0 < total; p0 += 32) {
+            const int p = p0 + lane;
+            int m = 0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const int b = __shfl_sync(0xffffffffu, begin, m + o);
+                if (b <= p) m += o;
+            }
+            const int e = __shfl_sync(0xffffffffu, e0, m) + p - __shfl_sync(0xffffffffu, begin, m);
+            if (p < total) {
+                const int q = off + p;
+                const int J = map[ci[e]];
+                const bool keep = J >= 0 && !(drop_diag && J == I);
+                sk[q] = keep ? (((unsigned)J * (unsigned)kGroupCap) | (unsigned)q) : ~0u;
+                se[q] = e;
+            }
         }
-        off += __shfl_sync(0xffffffffu, incl, 31);
+        off += total;
     }
     int L = 32;
     while (L < off) L <<= 1;
@@ -879,14 +893,24 @@ __device__ __forceinline__ int group_row_entries(int I, int lane, const int *mpt
     return L;
 }
 
+// entries of each coarse row; a row whose members hold more than kGroupCap
+// entries sets *over and is skipped
 __global__ void __launch_bounds__(32 * kGroupWarps) k_group_count(int nc, const int *mptr, const int *mem, const int *rp,
-                                                                 const int *ci, const int *map, int drop_diag, int *cnt) {
+                                                                 const int *ci, const int *map, int drop_diag, int *cnt,
+                                                                 int *over) {
     __shared__ unsigned keys[kGroupWarps][kGroupCap];
     __shared__ int ents[kGroupWarps][kGroupCap];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int I = blockIdx.x * kGroupWarps + w;
     if (I >= nc) return;
     unsigned *sk = keys[w];
+    int all = 0;
+    for (int a = mptr[I] + lane; a < mptr[I + 1]; a += 32) all += rp[mem[a] + 1] - rp[mem[a]];
+    for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
+    if (all > kGroupCap) {
+        if (lane == 0) { *over = 1; cnt[I] = 0; }
+        return;
+    }
     int n;
     group_row_entries(I, lane, mptr, mem, rp, ci, map, drop_diag, sk, ents[w], &n);
     int c = 0;
@@ -896,8 +920,10 @@ __global__ void __launch_bounds__(32 * kGroupWarps) k_group_count(int nc, const 
 }
 
 // MAX: the graph's edge weight, fmax over the coarse column's entries (one
-// value per entry); otherwise the Galerkin block, the sum of nb values per
-// entry in order q
+// value per entry); otherwise the Galerkin block, the sum of nb (1 or 9) values
+// per entry in order q.  3x3 blocks are summed by nine lanes, a component each,
+// three coarse columns at a time, so that a block is read as one 72-byte
+// segment.
 template <bool MAX>
 __global__ void __launch_bounds__(32 * kGroupWarps) k_group_fill(int nc, const int *mptr, const int *mem, const int *rp,
                                                                 const int *ci, const int *map, int drop_diag, int nb,
@@ -905,11 +931,13 @@ __global__ void __launch_bounds__(32 * kGroupWarps) k_group_fill(int nc, const i
                                                                 double *v_out) {
     __shared__ unsigned keys[kGroupWarps][kGroupCap];
     __shared__ int ents[kGroupWarps][kGroupCap];
+    __shared__ unsigned short starts[MAX ? 1 : kGroupWarps][MAX ? 1 : kGroupCap];   // first position of each coarse column
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int I = blockIdx.x * kGroupWarps + w;
     if (I >= nc) return;
     unsigned *sk = keys[w];
     const int *se = ents[w];
+    unsigned short *first = starts[MAX ? 0 : w];
     int n;
     const int P = group_row_entries(I, lane, mptr, mem, rp, ci, map, drop_diag, sk, ents[w], &n) / 32;
     const int p0 = lane * P;   // P contiguous positions per lane
@@ -924,36 +952,57 @@ __global__ void __launch_bounds__(32 * kGroupWarps) k_group_fill(int nc, const i
         if (lane >= o) incl += x;
     }
     long long slot = (long long)rp_out[I] + incl - mine;
+    auto in_run = [&](int r, unsigned J) { return r < n && sk[r] / kGroupCap == J; };
     for (int u = 0; u < P; ++u) {
         const int p = p0 + u;
         if (!(p < n && (p == 0 || sk[p] / kGroupCap != sk[p - 1] / kGroupCap))) continue;
         const unsigned J = sk[p] / kGroupCap;
         ci_out[slot] = (int)J;
-        if (MAX) {
+        if (!MAX && nb == 9) {
+            first[slot - rp_out[I]] = (unsigned short)p;
+        } else if (MAX) {
             double m = v[se[sk[p] % kGroupCap]];
-            for (int r = p + 1; r < n && sk[r] / kGroupCap == J; ++r) m = fmax(m, v[se[sk[r] % kGroupCap]]);
+            for (int r = p + 1; r < n && sk[r] / kGroupCap == J; r += 4) {   // four loads in flight
+                double x[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) x[t] = in_run(r + t, J) ? v[se[sk[r + t] % kGroupCap]] : m;
+#pragma unroll
+                for (int t = 0; t < 4; ++t) m = fmax(m, x[t]);
+            }
             v_out[slot] = m;
         } else {
-            double acc[9];
-            const double *src = v + (long long)se[sk[p] % kGroupCap] * nb;
-            for (int q = 0; q < nb; ++q) acc[q] = src[q];
-            for (int r = p + 1; r < n && sk[r] / kGroupCap == J; ++r) {
-                src = v + (long long)se[sk[r] % kGroupCap] * nb;
-                for (int q = 0; q < nb; ++q) acc[q] = __dadd_rn(acc[q], src[q]);
+            double acc = v[se[sk[p] % kGroupCap]];
+            for (int r = p + 1; r < n && sk[r] / kGroupCap == J; r += 8) {   // eight loads in flight, added in order
+                double x[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) x[t] = in_run(r + t, J) ? v[se[sk[r + t] % kGroupCap]] : 0.0;
+#pragma unroll
+                for (int t = 0; t < 8; ++t)
+                    if (in_run(r + t, J)) acc = __dadd_rn(acc, x[t]);
             }
-            for (int q = 0; q < nb; ++q) v_out[slot * nb + q] = acc[q];
+            v_out[slot] = acc;
         }
         ++slot;
     }
-}
-
-// entries of each coarse row before any drop (members' row lengths summed)
-__global__ void k_group_size(int nc, const int *mptr, const int *mem, const int *rp, unsigned long long *mx) {
-    const int I = blockIdx.x * blockDim.x + threadIdx.x;
-    if (I >= nc) return;
-    long long t = 0;
-    for (int a = mptr[I]; a < mptr[I + 1]; ++a) t += rp[mem[a] + 1] - rp[mem[a]];
-    atomicMax(mx, (unsigned long long)t);
+    if (MAX || nb != 9) return;
+    __syncwarp();
+    const long long o = rp_out[I];
+    const int runs = rp_out[I + 1] - rp_out[I], q = lane % 9;
+    if (lane >= 27) return;
+    for (int r = lane / 9; r < runs; r += 3) {
+        const int a = first[r], b = r + 1 < runs ? first[r + 1] : n;
+        auto at = [&](int u) { return v[(long long)se[sk[u] % kGroupCap] * 9 + q]; };
+        double acc = at(a);
+        for (int u = a + 1; u < b; u += 4) {   // four loads in flight, added in order
+            double x[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) x[t] = u + t < b ? at(u + t) : 0.0;
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                if (u + t < b) acc = __dadd_rn(acc, x[t]);
+        }
+        v_out[(o + r) * 9 + q] = acc;
+    }
 }
 
 // Coarse CSR (rp, ci, values) from the per-row grouping; false, with nothing
@@ -964,22 +1013,24 @@ static bool group_rows_local(int nc, const int *mptr, const int *mem, const int 
                              int drop_diag, int nb, const double *v, int *&rp_out, int *&ci_out, double *&v_out,
                              long long &nnz_out, cudaStream_t s) {
     if (nc <= 0 || (unsigned long long)nc * kGroupCap >= (1ULL << 32)) return false;
-    unsigned long long *mx = dmalloc<unsigned long long>(1, s);
-    NBP_CUDA(cudaMemsetAsync(mx, 0, sizeof(unsigned long long), s));
-    k_group_size<<<grid_exact(nc), 256, 0, s>>>(nc, mptr, mem, rp, mx);
-    NBP_LAUNCHED();
-    const unsigned long long most = readback(mx, s);
-    dfree(mx, s);
-    if (most > (unsigned long long)kGroupCap) return false;
     const unsigned blocks = (unsigned)((nc + kGroupWarps - 1) / kGroupWarps);
     int *cnt = dmalloc<int>(nc + 1, s);
-    k_group_count<<<blocks, 32 * kGroupWarps, 0, s>>>(nc, mptr, mem, rp, ci, map, drop_diag, cnt);
-    NBP_LAUNCHED();
+    rp_out = dmalloc<int>(nc + 2, s);   // row pointers, then the overflow flag: read back together
     NBP_CUDA(cudaMemsetAsync(cnt + nc, 0, sizeof(int), s));
-    rp_out = dmalloc<int>(nc + 1, s);
+    NBP_CUDA(cudaMemsetAsync(rp_out + nc + 1, 0, sizeof(int), s));
+    k_group_count<<<blocks, 32 * kGroupWarps, 0, s>>>(nc, mptr, mem, rp, ci, map, drop_diag, cnt, rp_out + nc + 1);
+    NBP_LAUNCHED();
     exclusive_scan(cnt, rp_out, nc + 1, s);
     dfree(cnt, s);
-    nnz_out = readback(rp_out + nc, s);
+    int end[2];
+    NBP_CUDA(cudaMemcpyAsync(end, rp_out + nc, sizeof(end), cudaMemcpyDeviceToHost, s));
+    NBP_CUDA(cudaStreamSynchronize(s));
+    if (end[1]) {
+        dfree(rp_out, s);
+        rp_out = nullptr;
+        return false;
+    }
+    nnz_out = end[0];
     ci_out = dmalloc<int>(nnz_out > 0 ? nnz_out : 1, s);
     v_out = dmalloc<double>((nnz_out > 0 ? nnz_out : 1) * nb, s);
     k_group_fill<MAX><<<blocks, 32 * kGroupWarps, 0, s>>>(nc, mptr, mem, rp, ci, map, drop_diag, nb, v, rp_out, ci_out,
@@ -988,19 +1039,11 @@ static bool group_rows_local(int nc, const int *mptr, const int *mem, const int 
     return true;
 }
 
-static void members_of(const int *map, int n, int nc, int *&mptr, int *&mem, cudaStream_t s);
-
-static Graph coarse_graph(const Graph &G, const int *map, int nc, cudaStream_t s) {
+static Graph coarse_graph(const Graph &G, const int *map, const Pairs &P, cudaStream_t s) {
+    const int nc = P.n;
     Graph Gc;
     Gc.n = nc;
-    {
-        int *mptr = nullptr, *mem = nullptr;
-        members_of(map, G.n, nc, mptr, mem, s);
-        const bool local = group_rows_local<true>(nc, mptr, mem, G.rp, G.ci, map, 1, 1, G.w, Gc.rp, Gc.ci, Gc.w,
-                                                  Gc.nnz, s);
-        dfree(mptr, s); dfree(mem, s);
-        if (local) return Gc;
-    }
+    if (group_rows_local<true>(nc, P.mptr, P.mem, G.rp, G.ci, map, 1, 1, G.w, Gc.rp, Gc.ci, Gc.w, Gc.nnz, s)) return Gc;
     Segments sg = group_by_coarse(G.n, G.nnz, G.rp, G.ci, map, nc, 1, s);
     Gc.nnz = sg.nseg;
     Gc.rp = rowptr_from_segments(sg, nc, s);
@@ -1015,8 +1058,52 @@ static Graph coarse_graph(const Graph &G, const int *map, int nc, cudaStream_t s
     return Gc;
 }
 
-// 3 passes; agg (n) gets the final map (-1 = isolated); returns the aggregate count
-static int aggregate(const DMat &M, double theta, int *agg, cudaStream_t s) {
+// The members of every final aggregate, from the passes' pair lists: up to two
+// nodes a pass, so up to eight, sorted; isolated nodes left out.  cnt: their
+// number per kept aggregate (fill: at mptr[newid], and the map of the nodes)
+__device__ __forceinline__ int expand_members(int I, const Pairs &a, const Pairs &b, const Pairs &c, const int *iso,
+                                              int (&out)[8]) {
+    int k = 0;
+    for (int p = c.mptr[I]; p < c.mptr[I + 1]; ++p)
+        for (int q = b.mptr[c.mem[p]]; q < b.mptr[c.mem[p] + 1]; ++q)
+            for (int r = a.mptr[b.mem[q]]; r < a.mptr[b.mem[q] + 1]; ++r)
+                if (!iso[a.mem[r]] && k < 8) out[k++] = a.mem[r];
+    return k;
+}
+// v[I] = (1 if the aggregate holds a node, members), packed for one scan
+__global__ void k_final_size(int nc, Pairs a, Pairs b, Pairs c, const int *iso, unsigned long long *v) {
+    const int I = blockIdx.x * blockDim.x + threadIdx.x;
+    if (I > nc) return;
+    int m[8];
+    const int k = I < nc ? expand_members(I, a, b, c, iso, m) : 0;
+    v[I] = k > 0 ? (1ULL << 32) | (unsigned long long)k : 0ULL;
+}
+__global__ void k_final_members(int nc, Pairs a, Pairs b, Pairs c, const int *iso, const unsigned long long *at, int *agg,
+                                int *mptr, int *mem) {
+    const int I = blockIdx.x * blockDim.x + threadIdx.x;
+    if (I > nc) return;
+    const unsigned long long v = at[I];
+    const int J = (int)(v >> 32), p = (int)(v & 0xffffffffULL);
+    if (I == nc) { mptr[J] = p; return; }
+    int m[8];
+    const int k = expand_members(I, a, b, c, iso, m);
+    if (k == 0) return;
+    for (int i = 1; i < k; ++i)   // ascending
+        for (int j = i; j > 0 && m[j - 1] > m[j]; --j) {
+            const int t = m[j];
+            m[j] = m[j - 1];
+            m[j - 1] = t;
+        }
+    mptr[J] = p;
+    for (int i = 0; i < k; ++i) {
+        mem[p + i] = m[i];
+        agg[m[i]] = J;
+    }
+}
+
+// 3 passes; agg (n) gets the final map (-1 = isolated) and mptr / mem the
+// aggregates' member lists (ascending fine index); returns the aggregate count
+static int aggregate(const DMat &M, double theta, int *agg, int *&mptr, int *&mem, cudaStream_t s) {
     const int n = M.nbr, nb = M.bb();
     double *dn = dmalloc<double>(n, s);
     k_diag_norm<<<grid_exact(n), 256, 0, s>>>(n, nb, M.rp, M.ci, M.v, dn);
@@ -1030,33 +1117,34 @@ static int aggregate(const DMat &M, double theta, int *agg, cudaStream_t s) {
     k_isolated<<<grid_exact(n), 256, 0, s>>>(n, M.rp, M.ci, G.w, theta, iso);
     NBP_LAUNCHED();
     dfree(dn, s);
-    k_iota<<<grid_exact(n), 256, 0, s>>>(n, agg);
-    NBP_LAUNCHED();
     int *map = dmalloc<int>(n, s);
-    int nc = n;
     bool own = false;   // the first graph borrows the matrix pattern
+    Pairs P[3];
     for (int pass = 0; pass < 3; ++pass) {
-        const int nn = match_pass(G, theta, map, s);
-        k_compose<<<grid_exact(n), 256, 0, s>>>(n, map, agg);
-        NBP_LAUNCHED();
-        Graph Gc = coarse_graph(G, map, nn, s);
-        if (own) graph_free(G, s);
-        else dfree(G.w, s);
-        G = Gc;
-        own = true;
-        nc = nn;
+        P[pass] = match_pass(G, theta, map, s);
+        if (pass < 2) {   // the last pass needs no graph of its aggregates
+            Graph Gc = coarse_graph(G, map, P[pass], s);
+            if (own) graph_free(G, s);
+            else dfree(G.w, s);
+            G = Gc;
+            own = true;
+        }
     }
     graph_free(G, s);
     dfree(map, s);
-    int *keep = dmalloc<int>(nc + 1, s), *newid = dmalloc<int>(nc + 1, s);
-    NBP_CUDA(cudaMemsetAsync(keep, 0, sizeof(int) * (nc + 1), s));
-    k_mark_keep<<<grid_exact(n), 256, 0, s>>>(n, agg, iso, keep);
+    const int nc = P[2].n;
+    unsigned long long *size = dmalloc<unsigned long long>(nc + 1, s), *at = dmalloc<unsigned long long>(nc + 1, s);
+    k_final_size<<<grid_exact(nc + 1), 256, 0, s>>>(nc, P[0], P[1], P[2], iso, size);
     NBP_LAUNCHED();
-    exclusive_scan(keep, newid, nc + 1, s);
-    const int m = readback(newid + nc, s);
-    k_drop_isolated<<<grid_exact(n), 256, 0, s>>>(n, iso, newid, agg);
+    exclusive_scan(size, at, nc + 1, s);
+    k_fill<int><<<grid_for(n), 256, 0, s>>>(agg, -1, n);
+    mptr = dmalloc<int>(nc + 1, s);   // nc is at least the number of kept aggregates
+    mem = dmalloc<int>(n, s);
+    k_final_members<<<grid_exact(nc + 1), 256, 0, s>>>(nc, P[0], P[1], P[2], iso, at, agg, mptr, mem);
     NBP_LAUNCHED();
-    dfree(keep, s); dfree(newid, s); dfree(iso, s);
+    const int m = (int)(readback(at + nc, s) >> 32);
+    for (Pairs &p : P) pairs_free(p, s);
+    dfree(size, s); dfree(at, s); dfree(iso, s);
     return m;
 }
 
@@ -1081,39 +1169,6 @@ static void galerkin(const DMat &M, const int *agg, const int *mptr, const int *
     }
     free_segments(sg, s);
 }
-
-// aggregate member lists (ascending fine index) for the restriction
-__global__ void k_member_keys(int n, const int *agg, int nc, unsigned int *key, int *val) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    key[i] = agg[i] < 0 ? (unsigned)nc : (unsigned)agg[i];
-    val[i] = i;
-}
-__global__ void k_member_count(int n, const int *agg, int *cnt) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (agg[i] >= 0) atomicAdd(cnt + agg[i], 1);
-}
-
-// members of coarse node I (map[i] == I) at mem[mptr[I] .. mptr[I+1]-1],
-// ascending; nodes with map < 0 trail
-static void members_of(const int *map, int n, int nc, int *&mptr, int *&mem, cudaStream_t s) {
-    unsigned int *key = dmalloc<unsigned int>(n, s);
-    int *val = dmalloc<int>(n, s);
-    k_member_keys<<<grid_exact(n), 256, 0, s>>>(n, map, nc, key, val);
-    NBP_LAUNCHED();
-    sort_pairs(key, val, n, bits_for((unsigned long long)nc), s);
-    int *cnt = dmalloc<int>(nc + 1, s);
-    NBP_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * (nc + 1), s));
-    k_member_count<<<grid_exact(n), 256, 0, s>>>(n, map, cnt);
-    NBP_LAUNCHED();
-    mptr = dmalloc<int>(nc + 1, s);
-    exclusive_scan(cnt, mptr, nc + 1, s);
-    mem = val;
-    dfree(cnt, s); dfree(key, s);
-}
-
-static void member_lists(Level &L, int n, int nc, cudaStream_t s) { members_of(L.agg, n, nc, L.mptr, L.mem, s); }
 
 // ---- A P, one row per warp: the row's entries in chunks of 32, each chunk's
 // coarse columns looked up in the row's list (first occurrence order), new ones
@@ -1306,9 +1361,12 @@ void amg_build(Hier &H, const DMat &fine, const nbp_options &o, int precision, c
                 nc = knc[l];
             } else {
                 L.agg = dmalloc<int>(n, s);
-                nc = aggregate(L.M, o.theta, L.agg, s);
-                if (nc >= n || nc == 0) { dfree(L.agg, s); L.agg = nullptr; break; }
-                member_lists(L, n, nc, s);
+                nc = aggregate(L.M, o.theta, L.agg, L.mptr, L.mem, s);
+                if (nc >= n || nc == 0) {
+                    dfree(L.agg, s); dfree(L.mptr, s); dfree(L.mem, s);
+                    L.agg = nullptr; L.mptr = nullptr; L.mem = nullptr;
+                    break;
+                }
             }
             galerkin(L.M, L.agg, L.mptr, L.mem, nc, H.L[l + 1].M, s);
             ++l;
@@ -1325,9 +1383,11 @@ void amg_build(Hier &H, const DMat &fine, const nbp_options &o, int precision, c
         Level &L = H.L[k];
         const int n = L.M.nbr, bs = H.bs;
         const long long nv = (long long)n * bs;
+        const size_t v64 = ((size_t)nv * 8 + 255) / 256 * 256, v32 = ((size_t)nv * 4 + 255) / 256 * 256;
+        L.work = dmalloc<char>(Level::kWork * (v64 + v32), s);
         for (int q = 0; q < Level::kWork; ++q) {
-            L.w64[q] = dmalloc<double>(nv, s);
-            L.w32[q] = dmalloc<float>(nv, s);
+            L.w64[q] = reinterpret_cast<double *>(L.work + q * v64);
+            L.w32[q] = reinterpret_cast<float *>(L.work + Level::kWork * v64 + q * v32);
         }
         L.kdots = dmalloc<double>(8 + 3 * kKdotBlocks, s);
         NBP_CUDA(cudaMemsetAsync(L.kdots, 0, sizeof(double) * (8 + 3 * kKdotBlocks), s));
@@ -1444,134 +1504,154 @@ __global__ void k_shat_reduce(int nseg, long long ntup, const unsigned long long
     atomicAdd(rowcnt + i, 1);
 }
 
-// ---- S_hat one row per warp: the row's tuples (the same as k_shat_fill
-// makes, in the same order q) sorted in shared memory by (column, q), so that
-// every entry is D_ij minus its terms in order q, as k_shat_reduce sums them;
-// for rows of at most kShatRowTuples tuples.
+// ---- S_hat one row per warp, for rows of at most kShatRowTuples tuples: the
+// row's distinct columns (D's and those of the B rows that C's row meets) are
+// collected in a hash table in shared memory and sorted; then the terms
+// C_ik B_kj are subtracted from D_ij entry by entry of C's row (k ascending),
+// a lane per entry of B's row k, which are distinct columns: every entry of
+// S_hat takes its terms in the order that k_shat_fill numbers them and
+// k_shat_reduce sums them, without sorting the terms themselves (0.56M
+// unknowns, count + fill: 1.93 -> 1.00 ms).
 constexpr int kShatRowTuples = 256;
-constexpr int kShatWarps = 8;   // warps per block
+constexpr int kShatTable = 512;   // hash slots: at most half full
+constexpr int kShatWarps = 8;     // warps per block
 
-// Tuples of row i into sk (key = column * 256 + q, padded with ~0u) and, when
-// t is set, their terms into t[q].  Returns the tuple count.
-__device__ __forceinline__ int shat_row_tuples(int i, int lane, const int *drp, const int *dci, const int *crp,
-                                               const int *cci, const double *cv, const int *brp, const int *bci,
-                                               const double *bv, const double *dinv, unsigned *sk, double *t) {
-    const int d0 = drp[i], dlen = drp[i + 1] - d0;
-    const int c0 = crp[i], clen = crp[i + 1] - c0;
-    for (int q = lane; q < kShatRowTuples; q += 32) sk[q] = ~0u;
+// this lane's column j (< 0: none) into the table; true where it is new
+__device__ __forceinline__ bool shat_insert(int *table, int j) {
+    if (j < 0) return false;
+    unsigned h = ((unsigned)j * 2654435761u) >> 23;   // 9 bits
+    for (int t = 0; t < kShatTable; ++t, h = (h + 1) & (kShatTable - 1)) {
+        const int old = atomicCAS(table + h, -1, j);
+        if (old == -1) return true;
+        if (old == j) return false;
+    }
+    return false;
+}
+// the distinct columns of row i into the table (cleared first); their number
+__device__ __forceinline__ int shat_columns(int i, int lane, const int *drp, const int *dci, const int *crp, const int *cci,
+                                            const int *brp, const int *bci, int *table) {
+    for (int q = lane; q < kShatTable; q += 32) table[q] = -1;
     __syncwarp();
-    for (int q = lane; q < dlen; q += 32) {   // the D pattern first, placeholder terms 0
-        sk[q] = ((unsigned)dci[d0 + q] << 8) | (unsigned)q;
-        if (t) t[q] = 0.0;
+    int c = 0;
+    for (int q = drp[i] + lane; q < drp[i + 1]; q += 32) c += shat_insert(table, dci[q]) ? 1 : 0;
+    for (int e = crp[i]; e < crp[i + 1]; ++e) {
+        const int k = cci[e], b1 = brp[k + 1];
+        for (int f = brp[k] + lane; f < b1; f += 32) c += shat_insert(table, bci[f]) ? 1 : 0;
     }
-    // then C_ik B_kj for k ascending (C's row order), j in B's row order; the
-    // start of entry e's tuples is dlen + the B row lengths before it
-    int off = dlen;
-    for (int e0 = 0; e0 < clen; e0 += 32) {
-        const int e = e0 + lane;
-        const int k = e < clen ? cci[c0 + e] : 0;
-        const int len = e < clen ? brp[k + 1] - brp[k] : 0;
-        int incl = len;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        const int start = off + incl - len;
-        if (e < clen) {
-            const long long ce = c0 + e;
-            double w0 = 0.0, w1 = 0.0, w2 = 0.0;
-            if (t) {
-                w0 = __dmul_rn(cv[3LL * ce], dinv[3LL * k]);
-                w1 = __dmul_rn(cv[3LL * ce + 1], dinv[3LL * k + 1]);
-                w2 = __dmul_rn(cv[3LL * ce + 2], dinv[3LL * k + 2]);
-            }
-            for (int f = 0; f < len; ++f) {
-                const int fe = brp[k] + f, q = start + f;
-                sk[q] = ((unsigned)bci[fe] << 8) | (unsigned)q;
-                if (t) {
-                    double tt = __dmul_rn(w0, bv[3LL * fe]);
-                    tt = __dadd_rn(tt, __dmul_rn(w1, bv[3LL * fe + 1]));
-                    tt = __dadd_rn(tt, __dmul_rn(w2, bv[3LL * fe + 2]));
-                    t[q] = tt;
-                }
-            }
-        }
-        off += __shfl_sync(0xffffffffu, incl, 31);
-    }
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     __syncwarp();
-    // bitonic sort of the 256 keys (unique: q differs), ascending
-    for (int k = 2; k <= kShatRowTuples; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int p = lane; p < kShatRowTuples; p += 32) {
-                const int x = p ^ j;
-                if (x > p) {
-                    const unsigned a = sk[p], b = sk[x];
-                    if ((a > b) == ((p & k) == 0)) { sk[p] = b; sk[x] = a; }
-                }
-            }
-            __syncwarp();
-        }
-    }
-    return off;
+    return c;
 }
 
 // entries per row (distinct columns)
 __global__ void __launch_bounds__(32 * kShatWarps) k_shat_row_count(int N, const int *drp, const int *dci, const int *crp,
                                                                    const int *cci, const int *brp, const int *bci, int *cnt) {
-    __shared__ unsigned keys[kShatWarps][kShatRowTuples];
+    __shared__ int tables[kShatWarps][kShatTable];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int i = blockIdx.x * kShatWarps + w;
     if (i >= N) return;
-    unsigned *sk = keys[w];
-    const int n = shat_row_tuples(i, lane, drp, dci, crp, cci, nullptr, brp, bci, nullptr, nullptr, sk, nullptr);
-    int c = 0;
-    for (int p = lane; p < n; p += 32) c += (p == 0 || (sk[p] >> 8) != (sk[p - 1] >> 8)) ? 1 : 0;
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if (lane == 0) cnt[i] = c;
+    const int n = shat_columns(i, lane, drp, dci, crp, cci, brp, bci, tables[w]);
+    if (lane == 0) cnt[i] = n;
 }
 
 // the row's entries at rp_out[i]..: columns ascending, each D_ij (or 0)
-// minus its terms in order q (as k_shat_reduce)
+// minus its terms in order
 __global__ void __launch_bounds__(32 * kShatWarps) k_shat_row_fill(int N, const int *drp, const int *dci, const double *dv,
                                                                   const int *crp, const int *cci, const double *cv,
                                                                   const int *brp, const int *bci, const double *bv,
                                                                   const double *dinv, const int *rp_out, int *ci_out,
                                                                   double *v_out) {
-    __shared__ unsigned keys[kShatWarps][kShatRowTuples];
-    __shared__ double terms[kShatWarps][kShatRowTuples];
+    __shared__ int tables[kShatWarps][kShatTable];
+    __shared__ int cols[kShatWarps][kShatRowTuples];
+    __shared__ double sums[kShatWarps][kShatRowTuples];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int i = blockIdx.x * kShatWarps + w;
     if (i >= N) return;
-    unsigned *sk = keys[w];
-    double *tv = terms[w];
-    const int n = shat_row_tuples(i, lane, drp, dci, crp, cci, cv, brp, bci, bv, dinv, sk, tv);
-    constexpr int P = kShatRowTuples / 32;   // positions per lane, contiguous
-    const int p0 = lane * P;
-    bool head[P];
-    int mine = 0;
-#pragma unroll
-    for (int u = 0; u < P; ++u) {
-        const int p = p0 + u;
-        head[u] = p < n && (p == 0 || (sk[p] >> 8) != (sk[p - 1] >> 8));
-        mine += head[u] ? 1 : 0;
+    int *table = tables[w], *col = cols[w];
+    double *sum = sums[w];
+    const int n = shat_columns(i, lane, drp, dci, crp, cci, brp, bci, table);
+    int at = 0;   // the table's columns packed, then sorted (bitonic, padded to a power of two)
+    for (int q = lane; q < kShatTable; q += 32) {
+        const int j = table[q];
+        const unsigned m = __ballot_sync(0xffffffffu, j >= 0);
+        if (j >= 0) col[at + __popc(m & ((1u << lane) - 1u))] = j;
+        at += __popc(m);
     }
-    int incl = mine;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
+    int L = 32;
+    while (L < n) L <<= 1;
+    for (int q = n + lane; q < L; q += 32) col[q] = 0x7fffffff;
+    __syncwarp();
+    for (int k = 2; k <= L; k <<= 1)
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int p = lane; p < L; p += 32) {
+                const int x = p ^ j;
+                if (x > p) {
+                    const int a = col[p], b = col[x];
+                    if ((a > b) == ((p & k) == 0)) { col[p] = b; col[x] = a; }
+                }
+            }
+            __syncwarp();
+        }
+    auto find = [&](int j) {   // j is in the list
+        int lo = 0, hi = n - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (col[mid] < j) lo = mid + 1; else hi = mid;
+        }
+        return lo;
+    };
+    for (int q = lane; q < n; q += 32) sum[q] = 0.0;
+    __syncwarp();
+    for (int q = drp[i] + lane; q < drp[i + 1]; q += 32) {
+        const int u = find(dci[q]);
+        sum[u] = __dsub_rn(dv[q], 0.0);   // D_ij minus its placeholder term
     }
-    int slot = rp_out[i] + incl - mine;
-#pragma unroll
-    for (int u = 0; u < P; ++u) {
-        if (!head[u]) continue;
-        const int p = p0 + u;
-        const unsigned j = sk[p] >> 8;
-        const int e = find_entry(drp, dci, i, (int)j);
-        double sum = (e >= 0) ? dv[e] : 0.0;
-        for (int r = p; r < n && (sk[r] >> 8) == j; ++r) sum = __dsub_rn(sum, tv[sk[r] & 255u]);
-        ci_out[slot] = (int)j;
-        v_out[slot] = sum;
-        ++slot;
+    __syncwarp();
+    // two entries of C's row at a time, half a warp each, where B's rows fit (an
+    // FP64 operation holds the pipe for a warp whatever lanes it has): the
+    // terms together, then the first entry's subtracted before the second's
+    const int c1 = crp[i + 1], half = lane >> 4;
+    auto term = [&](int e, int k, int f) {
+        const double w0 = __dmul_rn(cv[3LL * e], dinv[3LL * k]);
+        const double w1 = __dmul_rn(cv[3LL * e + 1], dinv[3LL * k + 1]);
+        const double w2 = __dmul_rn(cv[3LL * e + 2], dinv[3LL * k + 2]);
+        double tt = __dmul_rn(w0, bv[3LL * f]);
+        tt = __dadd_rn(tt, __dmul_rn(w1, bv[3LL * f + 1]));
+        return __dadd_rn(tt, __dmul_rn(w2, bv[3LL * f + 2]));
+    };
+    for (int e0 = crp[i]; e0 < c1; e0 += 2) {
+        const int e = e0 + half;
+        const int k = e < c1 ? cci[e] : 0;
+        const int b0 = e < c1 ? brp[k] : 0, len = e < c1 ? brp[k + 1] - b0 : 0;
+        if (__all_sync(0xffffffffu, len <= 16)) {
+            const bool on = (lane & 15) < len;
+            const int f = b0 + (lane & 15);
+            int u = 0;
+            double tt = 0.0;
+            if (on) {
+                tt = term(e, k, f);
+                u = find(bci[f]);
+            }
+            if (on && half == 0) sum[u] = __dsub_rn(sum[u], tt);
+            __syncwarp();
+            if (on && half == 1) sum[u] = __dsub_rn(sum[u], tt);
+            __syncwarp();
+            continue;
+        }
+        for (int e2 = e0; e2 < min(c1, e0 + 2); ++e2) {
+            const int k2 = cci[e2], b1 = brp[k2 + 1];
+            for (int f = brp[k2] + lane; f < b1; f += 32) {
+                const double tt = term(e2, k2, f);
+                const int u = find(bci[f]);
+                sum[u] = __dsub_rn(sum[u], tt);
+            }
+            __syncwarp();
+        }
+    }
+    const int o = rp_out[i];
+    for (int q = lane; q < n; q += 32) {
+        ci_out[o + q] = col[q];
+        v_out[o + q] = sum[q];
     }
 }
 

@@ -206,6 +206,7 @@ struct Level {
     static constexpr int kWork = 10;
     double *w64[kWork] = {};
     float *w32[kWork] = {};
+    char *work = nullptr;                    // the allocation they lie in
     double *kdots = nullptr;                 // K-cycle inner products (device)
     double *kpart = nullptr;                 // block partials of the K-cycle's product + inner products kernel
     long long kpart_blocks = 0;              // ... for grids up to this many blocks
@@ -228,9 +229,14 @@ struct Hier {
 namespace nbp {
 
 // ------------------------------------------------------ device memory helpers
+// The memory pool of the context this thread works for (set at the start of
+// every call on it; null: the device's default pool)
+inline thread_local cudaMemPool_t g_pool = nullptr;
 template <typename T> inline T *dmalloc(size_t n, cudaStream_t s) {
     void *p = nullptr;
-    NBP_CUDA(cudaMallocAsync(&p, (n ? n : 1) * sizeof(T), s));
+    const size_t bytes = (n ? n : 1) * sizeof(T);
+    if (g_pool) NBP_CUDA(cudaMallocFromPoolAsync(&p, bytes, g_pool, s));
+    else NBP_CUDA(cudaMallocAsync(&p, bytes, s));
     return (T *)p;
 }
 inline void dfree(void *p, cudaStream_t s) {
