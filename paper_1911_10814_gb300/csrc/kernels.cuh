@@ -45,6 +45,12 @@ struct SpmvArgs {
     float c1f, c2f;         // the same, pre-rounded for FP32 vectors (no FP64 work per element)
     const int *lr_rp, *lr_k, *lr_c;   // rank-one epilogue (EPI_SET only)
     const double *lr_val, *lr_f;
+    // the factors r_k (a^k . x) taken by the product's own blocks where lr_rev is
+    // 0 or 1 (see lr_factors; -1: read from lr_f): the outlets' vectors and
+    // weights, and whether the blocks run from the last rows (1)
+    const int *lr_optr, *lr_oidx;
+    const double *lr_oval, *lr_r;
+    int lr_n, lr_rev;
     int nslice;                       // sliced-ELL layout (k_sell): slices of C rows
     const long long *sl_ptr;
     const int *sl_ci;
@@ -301,6 +307,53 @@ __device__ __forceinline__ void slot_fma(const SlotBatch<BS * BS, VT> &B, const 
     }
 }
 
+// Rank-one factors f_k = r_k (a^k . x) inside the product: a block whose rows
+// [r0, r1) carry outlet entries takes the inner products of their outlets
+// itself (at most kLrInline in any 256 rows, a rule the host has checked), in
+// the order of k_lowrank_dots, instead of a launch before every product that
+// does nothing else.  The few blocks that do run first where the outlets' rows
+// are last (lr_rev), so that the others hide them.  Returns the first outlet of
+// fs.  All 256 threads of the block.  Not inlined: its registers would cost
+// every block's occupancy.
+constexpr int kLrInline = 4;
+template <typename XT>
+__device__ __noinline__ int lr_factors(const SpmvArgs &a, int r0, int r1, const XT *x, double (&fs)[kLrInline]) {
+    __shared__ int kfirst;
+    __shared__ double red[kLrInline][8];
+    r0 = min(r0, a.nbr);
+    r1 = min(r1, a.nbr);
+    const int e0 = a.lr_rp[r0], e1 = a.lr_rp[r1];
+    if (e1 <= e0) return 0;   // uniform over the block
+    const int tid = threadIdx.x;
+    if (tid == 0) kfirst = a.lr_n;
+    __syncthreads();
+    for (int e = e0 + tid; e < e1; e += 256) atomicMin(&kfirst, a.lr_k[e]);
+    __syncthreads();
+    const int k0 = kfirst, nk = min(kLrInline, a.lr_n - k0);
+    for (int q = 0; q < nk; ++q) {
+        double s = 0.0;
+        for (int e = a.lr_optr[k0 + q] + tid; e < a.lr_optr[k0 + q + 1]; e += 256)
+            s += a.lr_oval[e] * (double)x[a.lr_oidx[e]];
+        s = warp_sum(s);
+        if ((tid & 31) == 0) red[q][tid >> 5] = s;
+    }
+    __syncthreads();
+    if (tid < nk) {
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += red[tid][w];
+        fs[tid] = a.lr_r[k0 + tid] * t;
+    }
+    __syncthreads();
+    return k0;
+}
+// the rank-one terms of component q of a row with entries [e0, e1)
+__device__ __forceinline__ double lr_term(const SpmvArgs &a, int e0, int e1, int q, const double *fs, int k0) {
+    double t = 0.0;
+    for (int e = e0; e < e1; ++e)
+        if (a.lr_c[e] == q) t += (a.lr_rev >= 0 ? fs[a.lr_k[e] - k0] : a.lr_f[a.lr_k[e]]) * a.lr_val[e];
+    return t;
+}
+
 // Sliced-ELL product for square BS x BS blocks: one thread per block row, C
 // rows per slice (C = 32: a warp per slice; C = 8 for matrices whose row
 // lengths vary, to cut padding).  Every load of values and columns by the C
@@ -310,11 +363,13 @@ template <int BS, typename VT, typename XT, int EPI, bool LR, int C, int K = C =
 __global__ void __launch_bounds__(256) k_sell(SpmvArgs a) {
     using AT = XT;
     constexpr int BB = BS * BS;
-    const int row = blockIdx.x * blockDim.x + threadIdx.x;
+    const int bx = LR && a.lr_rev == 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    const int row = bx * blockDim.x + threadIdx.x;
     const int sl = row / C, t = row % C;
-    if (sl >= a.nslice) return;
-    const long long base = a.sl_ptr[sl];
-    const int w = (int)((a.sl_ptr[sl + 1] - base) / C);
+    const bool live = sl < a.nslice;
+    if (!LR && !live) return;   // LR: whole blocks stay for lr_factors
+    const long long base = live ? a.sl_ptr[sl] : 0;
+    const int w = live ? (int)((a.sl_ptr[sl + 1] - base) / C) : 0;
     const VT *__restrict__ val = (const VT *)a.val;
     const int *__restrict__ ci = a.sl_ci;
     AT acc0 = 0, acc1 = 0, acc2 = 0;
@@ -339,6 +394,9 @@ __global__ void __launch_bounds__(256) k_sell(SpmvArgs a) {
         }
     }
     const XT *x = (const XT *)a.x + col_off(a, a.x_ld);
+    __shared__ double fs[kLrInline];
+    int k0 = 0;
+    if (LR && a.lr_rev >= 0) k0 = lr_factors(a, bx * 256, bx * 256 + 256, x, fs);
     if (row >= a.nbr) return;
     AT accs[3] = {acc0, acc1, acc2};
     XT *y = (XT *)a.y;
@@ -399,12 +457,7 @@ __global__ void __launch_bounds__(256) k_sell(SpmvArgs a) {
             // the rank-one term in FP64, only on the rows that carry its
             // entries (outlet rows): GB300's FP64 pipe would otherwise hold
             // every warp for the conversions of every row
-            if (lr && lr1 > lr0) {
-                double tt = 0.0;
-                for (int e = lr0; e < lr1; ++e)
-                    if (a.lr_c[e] == q) tt += a.lr_f[a.lr_k[e]] * a.lr_val[e];
-                s = (AT)((double)s + tt);
-            }
+            if (lr && lr1 > lr0) s = (AT)((double)s + lr_term(a, lr0, lr1, q, fs, k0));
             y[idx] = s;
         } else if (EPI == EPI_ADD) {
             y[idx] += s;
@@ -484,7 +537,8 @@ template <int BS, typename VT, typename XT, int EPI, int C, int T, bool LR = fal
 __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
     using AT = XT;
     constexpr int BB = BS * BS;
-    const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int bx = LR && a.lr_rev == 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    const long long gid = (long long)bx * blockDim.x + threadIdx.x;
     const int row = (int)(gid / T), h = (int)(gid % T);
     const int sl = row / C, t = row % C;
     const bool live = sl < a.nslice;
@@ -554,6 +608,9 @@ __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
             acc2 += __shfl_xor_sync(0xffffffffu, acc2, o);
         }
     }
+    __shared__ double fs[kLrInline];
+    int k0 = 0;
+    if (LR && a.lr_rev >= 0) k0 = lr_factors(a, bx * (256 / T), (bx + 1) * (256 / T), x, fs);
     if (!own) return;
     const AT accs[3] = {acc0, acc1, acc2};
     XT *y = (XT *)a.y;
@@ -581,12 +638,8 @@ __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
         const long long idx = (long long)row * BS + q;
         if (EPI == EPI_SET) {
             AT s = accs[q];
-            if (LR && lr1 > lr0) {   // the rank-one term in FP64, on the rows that carry its entries (see k_sell)
-                double tt = 0.0;
-                for (int e = lr0; e < lr1; ++e)
-                    if (a.lr_c[e] == q) tt += a.lr_f[a.lr_k[e]] * a.lr_val[e];
-                s = (AT)((double)s + tt);
-            }
+            // the rank-one term in FP64, on the rows that carry its entries (see k_sell)
+            if (LR && lr1 > lr0) s = (AT)((double)s + lr_term(a, lr0, lr1, q, fs, k0));
             y[idx] = s;
         }
         else if (EPI == EPI_ADD) y[idx] += accs[q];

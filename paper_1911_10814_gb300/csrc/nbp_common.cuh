@@ -187,6 +187,7 @@ struct LowRank {
     int *lr_k = nullptr, *lr_c = nullptr;
     double *lr_val = nullptr;
     double *f = nullptr;                     // r_k (a^k . x), device, n_out
+    int in_product = -1;                     // the product's blocks take f themselves (SpmvArgs::lr_rev); -1: k_lowrank_dots
 };
 
 struct Level {

@@ -323,9 +323,19 @@ static void apply_A(nbp_ctx *c, int vsel, const T *x, T *y, const int *jp = null
     a.jp = jp;
     a.x_ld = x_ld;
     if (lr.n_out > 0) {
-        c->prof.launches++;
-        klaunch(k_lowrank_dots<T>, lr.n_out, (unsigned)256, c->s, lr.optr, lr.oidx, lr.oval, lr.r, x, lr.f, jp, x_ld);
-        NBP_LAUNCHED();
+        // in the product's blocks on long vectors only: on short ones most of the
+        // GPU waits for the few blocks that take the inner products (solves,
+        // k_lowrank_dots / in the product: 140,481 rows 162.0 / 157.8 ms, 1.09M
+        // 744.7 / 735.5; 60,625 rows FP64 73.6 / 74.5, 29,760 rows 37.2 / 37.8)
+        const bool inside = lr.in_product >= 0 && c->N >= 100000 && c->A.sl_ci &&
+                            (c->A.tuned <= 0 || is_sellm(c->A.tuned));
+        a.lr_rev = inside ? lr.in_product : -1;
+        a.lr_optr = lr.optr; a.lr_oidx = lr.oidx; a.lr_oval = lr.oval; a.lr_r = lr.r; a.lr_n = lr.n_out;
+        if (!inside) {
+            c->prof.launches++;
+            klaunch(k_lowrank_dots<T>, (unsigned)lr.n_out, 256u, c->s, lr.optr, lr.oidx, lr.oval, lr.r, x, lr.f, jp, x_ld);
+            NBP_LAUNCHED();
+        }
         a.lr_rp = lr.lr_rp; a.lr_k = lr.lr_k; a.lr_c = lr.lr_c; a.lr_val = lr.lr_val; a.lr_f = lr.f;
     }
     // rank-one epilogue: the per-row list pointers, each (outlet, component,
@@ -1753,6 +1763,24 @@ static void load_lowrank(nbp_ctx *c, const nbp_system *sys) {
             const int p = fillp[oidx[q] / 3]++;
             lk[p] = k; lc[p] = oidx[q] % 3; lv[p] = oval[q];
         }
+    // the product's blocks (256 to 32 rows each) may take the outlets' inner
+    // products themselves: few outlets in any 256 rows, and no more than 400,000
+    // entries read again over all 32-row blocks (outlet nodes numbered close
+    // together; scattered ones would make every block sum whole outlets)
+    {
+        bool few = true;
+        long long again = 0, mean = 0;
+        for (int g : {256, 32})
+            for (int r0 = 0; r0 < N; r0 += g) {
+                const int e0 = cnt[r0], e1 = cnt[std::min(N, r0 + g)];
+                if (e0 == e1) continue;
+                const auto mm = std::minmax_element(lk.begin() + e0, lk.begin() + e1);
+                if (g == 256) few = few && *mm.second - *mm.first < kLrInline;
+                else again += optr[*mm.second + 1] - optr[*mm.first];
+            }
+        for (int q = 0; q < no; ++q) mean += oidx[q] / 3;
+        if (no > 0 && few && again <= 400000) lr.in_product = mean / no > N / 2 ? 1 : 0;
+    }
     lr.optr = dmalloc<int>(lr.n_out + 1, s);
     lr.oidx = dmalloc<int>(no, s);
     lr.oval = dmalloc<double>(no, s);
@@ -2042,6 +2070,7 @@ static nbp_ctx *make_transposed(nbp_ctx *c) {
         // same outlets and weights (the rank-one term is symmetric)
         LowRank &a = c->lr, &b = t->lr;
         b.n_out = a.n_out;
+        b.in_product = a.in_product;
         b.r_host = a.r_host;
         const int N = c->N;
         b.lr_rp = dmalloc<int>(N + 1, c->s);
