@@ -29,10 +29,31 @@ namespace nbp {
 constexpr int kMatchRounds = 64;   // rounds per matching pass (rounds after one that makes no pair change nothing)
 
 // ------------------------------------------------------------- utilities
+// the sliced copies of m, freed unless they are another matrix's
+void drop_sell(DMat &m, cudaStream_t s) {
+    if (!m.sl_lent) {
+        dfree(m.sl_ptr, s); dfree(m.sl_ci, s); dfree(m.sl_v, s); dfree(m.sl_v32, s); dfree(m.sl_v16, s);
+        dfree(m.sl2_ptr, s); dfree(m.sl2_ci, s);
+    }
+    m.sl_ptr = nullptr; m.sl_ci = nullptr; m.sl_v = nullptr; m.sl_v32 = nullptr; m.sl_v16 = nullptr;
+    m.sl2_ptr = nullptr; m.sl2_ci = nullptr;
+    m.sl_lent = false;
+}
+
+// `to`, of the same pattern and values, uses the sliced copies of `from`
+// until its own are dropped, which has to be before those of `from`
+void lend_sell(const DMat &from, DMat &to, cudaStream_t s) {
+    drop_sell(to, s);
+    to.nslice = from.nslice; to.sl_c = from.sl_c;
+    to.sl_ptr = from.sl_ptr; to.sl_ci = from.sl_ci;
+    to.sl_v = from.sl_v; to.sl_v32 = from.sl_v32; to.sl_v16 = from.sl_v16;
+    to.sl2_ptr = from.sl2_ptr; to.sl2_ci = from.sl2_ci;
+    to.sl_lent = true;
+}
+
 void dmat_free(DMat &m, cudaStream_t s) {
     dfree(m.rp, s); dfree(m.ci, s); dfree(m.v, s); dfree(m.v32, s); dfree(m.v16, s);
-    dfree(m.sl_ptr, s); dfree(m.sl_ci, s); dfree(m.sl_v, s); dfree(m.sl_v32, s); dfree(m.sl_v16, s);
-    dfree(m.sl2_ptr, s); dfree(m.sl2_ci, s);
+    drop_sell(m, s);
     m = DMat();
 }
 
@@ -651,10 +672,7 @@ static long long sell_layout(const DMat &m, int C, long long *&sp, cudaStream_t 
 void make_sell(DMat &m, int precision, cudaStream_t s) {
     if (m.nbr == 0) return;
     if (m.sl_ci && (precision < 1 || m.sl_v32) && (precision < 2 || m.sl_v16)) return;   // 2, 3: FP32 and BF16
-    dfree(m.sl_ptr, s); dfree(m.sl_ci, s); dfree(m.sl_v, s); dfree(m.sl_v32, s); dfree(m.sl_v16, s);
-    dfree(m.sl2_ptr, s); dfree(m.sl2_ci, s);
-    m.sl_ptr = nullptr; m.sl_ci = nullptr; m.sl_v = nullptr; m.sl_v32 = nullptr; m.sl_v16 = nullptr;
-    m.sl2_ptr = nullptr; m.sl2_ci = nullptr;
+    drop_sell(m, s);
     int C = 32;
     long long total = sell_layout(m, 32, m.sl_ptr, s);
     if (total > m.nnz + m.nnz / 10) {

@@ -170,6 +170,7 @@ struct DMat {
     long long *sl2_ptr = nullptr;
     int *sl2_ci = nullptr;
     __nv_bfloat16 *sl_v16 = nullptr;
+    bool sl_lent = false;            // the sl_* arrays belong to another matrix (lend_sell)
     int tuned = -1;                  // autotuned kernel: -1 untuned, 0 sliced ELL, 1000 + T sliced ELL with T threads per row, other > 0 flat with that many lanes per row
     int bb() const { return br * bc; }
 };
@@ -261,6 +262,8 @@ inline unsigned grid_exact(long long n, int block = 256) {
 }
 
 void dmat_free(DMat &m, cudaStream_t s);
+void drop_sell(DMat &m, cudaStream_t s);
+void lend_sell(const DMat &from, DMat &to, cudaStream_t s);
 void hier_free(Hier &H, cudaStream_t s);
 
 // Setup entry points (amg_setup.cu)
