@@ -1337,7 +1337,8 @@ static void dense_inverse(const DMat &M, double *&cinv, int &nc, cudaStream_t s)
     require(!f, NBP_ERR_INVALID, "setup: coarsest AMG matrix is singular");
 }
 
-void amg_build(Hier &H, const DMat &fine, const nbp_options &o, int precision, cudaStream_t s, bool keep_aggregates) {
+void amg_build(Hier &H, const DMat &fine, const nbp_options &o, int precision, cudaStream_t s, bool keep_aggregates,
+               const std::function<void()> &levels_ready) {
     // numeric re-setup: the aggregate maps and member lists of the hierarchy
     // H holds are taken over (same pattern); every operator is rebuilt
     int knlev = 0, knc[kMaxLevels] = {};
@@ -1435,6 +1436,7 @@ void amg_build(Hier &H, const DMat &fine, const nbp_options &o, int precision, c
     const int sing = readback(singular, s);
     dfree(singular, s);
     require(sing == 0, NBP_ERR_INVALID, "setup: singular diagonal block in an AMG level");
+    if (levels_ready) levels_ready();   // everything but the coarsest inverse is there
     const Level &C = H.L[H.nlev - 1];
     if ((long long)C.M.nbr * H.bs <= kCoarseDenseMax) {
         dense_inverse(C.M, H.cinv, H.nc, s);
