@@ -1304,41 +1304,69 @@ static void make_ap(Level &L, int nc, int precision, cudaStream_t s) {
     L.AP = P;
 }
 
-static void dense_inverse(const DMat &M, double *&cinv, int &nc, cudaStream_t s) {
-    const int n = M.nbr * M.br;
-    nc = n;
-    double *Dm = dmalloc<double>((long long)n * n, s);
-    cinv = dmalloc<double>((long long)n * n, s);
-    NBP_CUDA(cudaMemsetAsync(Dm, 0, sizeof(double) * (size_t)n * n, s));
-    k_dense_from_bsr<<<grid_exact(M.nbr), 256, 0, s>>>(M.nbr, M.br, M.rp, M.ci, M.v, Dm);
-    NBP_LAUNCHED();
-    double *Dn = cinv, *G = dmalloc<double>(8LL * n, s);   // Dm and Dn in turn
-    int *piv = dmalloc<int>(n, s), *perm = dmalloc<int>(n, s), *fail = dmalloc<int>(1, s);
-    NBP_CUDA(cudaMemsetAsync(fail, 0, sizeof(int), s));
-    k_iota<<<grid_exact(n), 256, 0, s>>>(n, perm);
-    NBP_LAUNCHED();
-    // panel width: b columns and the permutation in one block's shared memory
-    const int B = n <= 3300 ? 8 : 4;
-    static_assert((4 * sizeof(double) + sizeof(int)) * (size_t)kCoarseDenseMax <= 227u * 1024u, "panel fits");
-    const size_t smem = ((size_t)B * sizeof(double) + sizeof(int)) * (size_t)n;
-    NBP_CUDA(cudaFuncSetAttribute(k_inv_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024));
-    const dim3 tiles((n + 31) / 32, (n + 31) / 32);
-    for (int k0 = 0; k0 < n; k0 += B) {
-        const int b = std::min(B, n - k0);
-        k_inv_panel<<<1, kInvThreads, smem, s>>>(n, k0, b, Dm, G, piv, perm, fail);
-        k_inv_update<<<tiles, 256, 0, s>>>(n, k0, b, Dm, G, piv, Dn, fail);
-        std::swap(Dm, Dn);
+// The inverse of the coarsest matrix, a chain of small kernels: queued on a
+// stream of its own (side), beside the levels' smoothing data and sliced
+// copies that s makes, and taken up by finish().  Setups, with the spectral
+// estimates queued level by level: cube of 16 7.4 -> 7.0 ms, 0.56M unknowns
+// numeric 13.2 -> 12.1, 1.85M 46.0 -> 44.2.
+struct DenseInverse {
+    cudaStream_t s = nullptr, side = nullptr;
+    cudaEvent_t ev = nullptr;
+    double *Dm = nullptr, *Dn = nullptr, *G = nullptr;   // Dn: the inverse
+    int *piv = nullptr, *perm = nullptr, *fail = nullptr;
+    DenseInverse(cudaStream_t s_, cudaStream_t side_) : s(s_), side(side_) {}
+    void queue(const DMat &M) {
+        NBP_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        NBP_CUDA(cudaEventRecord(ev, s));
+        NBP_CUDA(cudaStreamWaitEvent(side, ev, 0));
+        const int n = M.nbr * M.br;
+        Dm = dmalloc<double>((long long)n * n, side);
+        Dn = dmalloc<double>((long long)n * n, side);
+        NBP_CUDA(cudaMemsetAsync(Dm, 0, sizeof(double) * (size_t)n * n, side));
+        k_dense_from_bsr<<<grid_exact(M.nbr), 256, 0, side>>>(M.nbr, M.br, M.rp, M.ci, M.v, Dm);
+        NBP_LAUNCHED();
+        G = dmalloc<double>(8LL * n, side);
+        piv = dmalloc<int>(n, side);
+        perm = dmalloc<int>(n, side);
+        fail = dmalloc<int>(1, side);
+        NBP_CUDA(cudaMemsetAsync(fail, 0, sizeof(int), side));
+        k_iota<<<grid_exact(n), 256, 0, side>>>(n, perm);
+        NBP_LAUNCHED();
+        // panel width: b columns and the permutation in one block's shared memory
+        const int B = n <= 3300 ? 8 : 4;
+        static_assert((4 * sizeof(double) + sizeof(int)) * (size_t)kCoarseDenseMax <= 227u * 1024u, "panel fits");
+        const size_t smem = ((size_t)B * sizeof(double) + sizeof(int)) * (size_t)n;
+        NBP_CUDA(cudaFuncSetAttribute(k_inv_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024));
+        const dim3 tiles((n + 31) / 32, (n + 31) / 32);
+        for (int k0 = 0; k0 < n; k0 += B) {   // Dm and Dn in turn
+            const int b = std::min(B, n - k0);
+            k_inv_panel<<<1, kInvThreads, smem, side>>>(n, k0, b, Dm, G, piv, perm, fail);
+            k_inv_update<<<tiles, 256, 0, side>>>(n, k0, b, Dm, G, piv, Dn, fail);
+            std::swap(Dm, Dn);
+        }
+        k_inv_columns<<<grid_exact((long long)n * n), 256, 0, side>>>(n, Dm, perm, Dn);
+        NBP_LAUNCHED();
     }
-    k_inv_columns<<<grid_exact((long long)n * n), 256, 0, s>>>(n, Dm, perm, Dn);
-    NBP_LAUNCHED();
-    cinv = Dn;
-    const int f = readback(fail, s);
-    dfree(fail, s); dfree(Dm, s); dfree(G, s); dfree(piv, s); dfree(perm, s);
-    require(!f, NBP_ERR_INVALID, "setup: coarsest AMG matrix is singular");
-}
+    bool join() {   // s goes on after side
+        return cudaEventRecord(ev, side) == cudaSuccess && cudaStreamWaitEvent(s, ev, 0) == cudaSuccess;
+    }
+    double *finish() {
+        require(join(), NBP_ERR_CUDA, "setup: the coarsest inverse's stream could not be joined");
+        require(readback(fail, s) == 0, NBP_ERR_INVALID, "setup: coarsest AMG matrix is singular");
+        double *inv = Dn;
+        Dn = nullptr;
+        return inv;
+    }
+    ~DenseInverse() {   // also where a setup ends with an error: side reads the hierarchy
+        if (!ev) return;
+        if (!join()) cudaStreamSynchronize(side);
+        cudaEventDestroy(ev);
+        dfree(fail, s); dfree(Dm, s); dfree(Dn, s); dfree(G, s); dfree(piv, s); dfree(perm, s);
+    }
+};
 
 void amg_build(Hier &H, const DMat &fine, const nbp_options &o, int precision, cudaStream_t s, bool keep_aggregates,
-               const std::function<void()> &levels_ready) {
+               cudaStream_t side, const std::function<void(int)> &level_ready) {
     // numeric re-setup: the aggregate maps and member lists of the hierarchy
     // H holds are taken over (same pattern); every operator is rebuilt
     int knlev = 0, knc[kMaxLevels] = {};
@@ -1395,6 +1423,10 @@ void amg_build(Hier &H, const DMat &fine, const nbp_options &o, int precision, c
         throw;
     }
     H.nlev = l + 1;
+    const Level &C = H.L[H.nlev - 1];
+    const bool dense = (long long)C.M.nbr * H.bs <= kCoarseDenseMax;
+    DenseInverse inverse(s, side);
+    if (dense) inverse.queue(C.M);
     int *singular = dmalloc<int>(1, s);
     NBP_CUDA(cudaMemsetAsync(singular, 0, sizeof(int), s));
     unsigned long long *rb = dmalloc<unsigned long long>(1, s);
@@ -1430,16 +1462,16 @@ void amg_build(Hier &H, const DMat &fine, const nbp_options &o, int precision, c
                 L.kpart_blocks = ((long long)L.M.nslice * L.M.sl_c * 8 + 255) / 256;
                 L.kpart = dmalloc<double>(3 * L.kpart_blocks, s);
             }
+            if (level_ready) level_ready(k);
         }
     }
     dfree(rb, s);
     const int sing = readback(singular, s);
     dfree(singular, s);
     require(sing == 0, NBP_ERR_INVALID, "setup: singular diagonal block in an AMG level");
-    if (levels_ready) levels_ready();   // everything but the coarsest inverse is there
-    const Level &C = H.L[H.nlev - 1];
-    if ((long long)C.M.nbr * H.bs <= kCoarseDenseMax) {
-        dense_inverse(C.M, H.cinv, H.nc, s);
+    if (dense) {
+        H.cinv = inverse.finish();
+        H.nc = C.M.nbr * H.bs;
         const long long nn = (long long)H.nc * H.nc;
         H.cinv32 = dmalloc<float>(nn, s);
         k_to_f32<<<grid_for(nn), 256, 0, s>>>(H.cinv, H.cinv32, nn);

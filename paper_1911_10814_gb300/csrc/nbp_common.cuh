@@ -272,7 +272,7 @@ void hier_free(Hier &H, cudaStream_t s);
 // operator of the hierarchy H already holds (same pattern) from the new
 // values on its aggregate maps instead of aggregating again.
 void amg_build(Hier &H, const DMat &fine, const nbp_options &o, int precision, cudaStream_t s,
-               bool keep_aggregates = false, const std::function<void()> &levels_ready = nullptr);
+               bool keep_aggregates, cudaStream_t side, const std::function<void(int)> &level_ready = nullptr);
 void build_shat(const DMat &A, const DMat &B, const DMat &C, const DMat &D, const LowRank &lr, int N, DMat &Shat,
                 double *diagA_out, cudaStream_t s);
 void make_lowcopies(DMat &m, int precision, cudaStream_t s);

@@ -183,6 +183,7 @@ struct nbp_ctx {
     cudaStream_t cap = nullptr;   // private stream used only while capturing
     cudaStream_t s2 = nullptr;    // S_hat and its hierarchy are built here, beside AMG(A) on s
     cudaEvent_t ev2 = nullptr;    // orders s2 after s and s after s2
+    cudaStream_t s_inv[2] = {nullptr, nullptr};   // the coarsest inverses of both
     std::vector<cudaStream_t> s_rho;   // the levels' Arnoldi estimates (RhoEstimate)
     bool use_graphs = true;
     // device-driven solve: the whole nested solve as one CUDA graph whose
@@ -1916,36 +1917,34 @@ static void queue_rho(nbp_ctx *c, Hier &H, int l, Krylov<double> &K, double *out
     }
 }
 
-static void queue_rhos(nbp_ctx *c, Hier &H, RhoEstimate &R) {
+// queued as soon as level l's block-diagonal inverse and sliced copies are
+static void queue_rhos(nbp_ctx *c, Hier &H, int l, RhoEstimate &R) {
+    // a coarsest level with a dense inverse is never smoothed
+    if (l == H.nlev - 1 && (long long)H.L[l].M.nbr * H.bs <= kCoarseDenseMax) return;
     R.c = c;
     R.H = &H;
-    const bool dense = (long long)H.L[H.nlev - 1].M.nbr * H.bs <= kCoarseDenseMax;   // then never smoothed
-    for (int l = 0; l < H.nlev; ++l)
-        if ((l < H.nlev - 1 || !dense) && H.L[l].dinv) R.levels.push_back(l);
-    if (R.levels.empty()) return;
-    NBP_CUDA(cudaEventCreateWithFlags(&R.ev, cudaEventDisableTiming));
-    while (c->s_rho.size() < R.levels.size()) {
+    const size_t i = R.levels.size();
+    if (!R.ev) NBP_CUDA(cudaEventCreateWithFlags(&R.ev, cudaEventDisableTiming));
+    if (c->s_rho.size() <= i) {
         cudaStream_t q;
         NBP_CUDA(cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking));
         c->s_rho.push_back(q);
     }
-    for (size_t i = 0; i < R.levels.size(); ++i) R.dev.push_back(dmalloc<double>((size_t)kRhoSteps * kRhoSlot, c->s));
+    R.dev.push_back(dmalloc<double>((size_t)kRhoSteps * kRhoSlot, c->s));
+    R.levels.push_back(l);
     NBP_CUDA(cudaEventRecord(R.ev, c->s));
-    for (size_t i = 0; i < R.levels.size(); ++i) NBP_CUDA(cudaStreamWaitEvent(c->s_rho[i], R.ev, 0));
-    for (size_t i = 0; i < R.levels.size(); ++i) {   // the finest, longest, first
-        OnStream on(c, c->s_rho[i]);
-        R.on.push_back(c->s);
-        const Level &L = H.L[R.levels[i]];
-        Krylov<double> K;
-        try {
-            K.ensure((long long)L.M.nbr * H.bs, kRhoSteps, c->s);
-            queue_rho(c, H, R.levels[i], K, R.dev[i]);
-        } catch (...) {
-            K.release(c->s);
-            throw;
-        }
+    NBP_CUDA(cudaStreamWaitEvent(c->s_rho[i], R.ev, 0));
+    R.on.push_back(c->s_rho[i]);
+    OnStream on(c, c->s_rho[i]);
+    Krylov<double> K;
+    try {
+        K.ensure((long long)H.L[l].M.nbr * H.bs, kRhoSteps, c->s);
+        queue_rho(c, H, l, K, R.dev[i]);
+    } catch (...) {
         K.release(c->s);
+        throw;
     }
+    K.release(c->s);
 }
 
 static void take_rhos(nbp_ctx *c, RhoEstimate &R) {
@@ -2014,6 +2013,8 @@ static void do_setup(nbp_ctx *c, bool numeric = false) {
     // starts after s's work so far, s goes on after s2's.
     if (!c->s2) NBP_CUDA(cudaStreamCreateWithFlags(&c->s2, cudaStreamNonBlocking));
     if (!c->ev2) NBP_CUDA(cudaEventCreateWithFlags(&c->ev2, cudaEventDisableTiming));
+    for (cudaStream_t &q : c->s_inv)
+        if (!q) NBP_CUDA(cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking));
     NBP_CUDA(cudaEventRecord(c->ev2, s));
     NBP_CUDA(cudaStreamWaitEvent(c->s2, c->ev2, 0));
     std::exception_ptr failed_S, failed_A;
@@ -2022,14 +2023,14 @@ static void do_setup(nbp_ctx *c, bool numeric = false) {
             NBP_CUDA(cudaSetDevice(c->dev));
             g_pool = c->pool;
             build_shat(c->A, c->B, c->C, c->D, c->lr, c->N, c->Shat, c->diagA, c->s2);
-            amg_build(c->HS, c->Shat, c->opt, prec, c->s2, numeric);   // keeps the Gershgorin bound (see kRhoSteps)
+            amg_build(c->HS, c->Shat, c->opt, prec, c->s2, numeric, c->s_inv[1]);   // keeps the Gershgorin bound (see kRhoSteps)
         } catch (...) {
             failed_S = std::current_exception();
         }
     });
     try {
         RhoEstimate rhos;
-        amg_build(c->HA, c->A, c->opt, prec, s, numeric, [&] { queue_rhos(c, c->HA, rhos); });
+        amg_build(c->HA, c->A, c->opt, prec, s, numeric, c->s_inv[0], [&](int l) { queue_rhos(c, c->HA, l, rhos); });
         // The products with A read the finest level's copies: every inner
         // iteration streams both, and one copy stays in L2 where two do not
         // (0.56M unknowns: solve 159.3 -> 157.0 ms; 4.34M 734.8 -> 730.4)
@@ -2087,7 +2088,9 @@ static void destroy_ctx(nbp_ctx *c) {
         cudaStreamSynchronize(c->s2);
         cudaStreamDestroy(c->s2);
     }
+    for (cudaStream_t q : c->s_inv) c->s_rho.push_back(q);
     for (cudaStream_t q : c->s_rho) {
+        if (!q) continue;
         cudaStreamSynchronize(q);
         cudaStreamDestroy(q);
     }
