@@ -230,6 +230,12 @@ nbp_status nbp_amg_level_get(nbp_ctx *ctx, int32_t which, int32_t l, int32_t *ro
 int64_t nbp_shat_nnz(nbp_ctx *ctx);
 nbp_status nbp_shat_get(nbp_ctx *ctx, int32_t *rowptr, int32_t *col, double *val);
 
+/* Device memory of the context, in bytes: *used in its buffers, *reserved what
+ * its memory pool holds for them and keeps for the next setup (a quarter of
+ * what is used; the rest goes back to the device).  A call allocates from the
+ * pool of the context that it works on. */
+nbp_status nbp_memory(nbp_ctx *ctx, uint64_t *used, uint64_t *reserved);
+
 /* Per-kernel device-time accounting of the last solve: total milliseconds and
  * algorithmic bytes of the SpMV family and of the Arnoldi (CGS2) kernels,
  * measured with CUDA events on the context stream when `enable` was set by

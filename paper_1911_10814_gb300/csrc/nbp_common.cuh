@@ -232,14 +232,21 @@ struct Hier {
 namespace nbp {
 
 // ------------------------------------------------------ device memory helpers
-// The memory pool of the context this thread works for (set at the start of
-// every call on it; null: the device's default pool)
+// The memory pool of the context this thread works for: set for the extent of
+// a call on that context (PoolScope) and null outside, so that no call takes
+// memory from another context's pool or through the handle of a destroyed one.
 inline thread_local cudaMemPool_t g_pool = nullptr;
+struct PoolScope {
+    cudaMemPool_t keep;
+    explicit PoolScope(cudaMemPool_t pool) : keep(g_pool) { g_pool = pool; }
+    ~PoolScope() { g_pool = keep; }
+    PoolScope(const PoolScope &) = delete;
+    PoolScope &operator=(const PoolScope &) = delete;
+};
 template <typename T> inline T *dmalloc(size_t n, cudaStream_t s) {
     void *p = nullptr;
-    const size_t bytes = (n ? n : 1) * sizeof(T);
-    if (g_pool) NBP_CUDA(cudaMallocFromPoolAsync(&p, bytes, g_pool, s));
-    else NBP_CUDA(cudaMallocAsync(&p, bytes, s));
+    require(g_pool != nullptr, NBP_ERR_STATE, "device memory asked for outside a call on a context");
+    NBP_CUDA(cudaMallocFromPoolAsync(&p, (n ? n : 1) * sizeof(T), g_pool, s));
     return (T *)p;
 }
 inline void dfree(void *p, cudaStream_t s) {

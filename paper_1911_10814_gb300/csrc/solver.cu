@@ -2021,7 +2021,7 @@ static void do_setup(nbp_ctx *c, bool numeric = false) {
     std::thread build_S([&] {
         try {
             NBP_CUDA(cudaSetDevice(c->dev));
-            g_pool = c->pool;
+            PoolScope scope(c->pool);
             build_shat(c->A, c->B, c->C, c->D, c->lr, c->N, c->Shat, c->diagA, c->s2);
             amg_build(c->HS, c->Shat, c->opt, prec, c->s2, numeric, c->s_inv[1]);   // keeps the Gershgorin bound (see kRhoSteps)
         } catch (...) {
@@ -2109,10 +2109,7 @@ static void destroy_ctx(nbp_ctx *c) {
     c->B64.release(s); c->B32.release(s);
     cudaStreamSynchronize(s);
     if (c->hst && !c->is_transposed) cudaFreeHost(c->hst);
-    if (c->pool && !c->is_transposed) {
-        if (g_pool == c->pool) g_pool = nullptr;
-        cudaMemPoolDestroy(c->pool);
-    }
+    if (c->pool && !c->is_transposed) cudaMemPoolDestroy(c->pool);
     delete c;
 }
 
@@ -2227,7 +2224,6 @@ static std::string profile_report(nbp_ctx *c) {
 
 static void begin_call(nbp_ctx *c) {
     NBP_CUDA(cudaSetDevice(c->dev));
-    g_pool = c->pool;
     c->prof.used = 0;
     c->prof.recs.clear();
     c->prof.launches = 0;
@@ -2242,7 +2238,8 @@ using namespace nbp;
 
 #define NBP_API_BEGIN(ctx) \
     if (!(ctx)) return NBP_ERR_INVALID; \
-    try {
+    try {                               \
+        nbp::PoolScope pool_scope((ctx)->pool);
 #define NBP_API_END(ctx)                                  \
     }                                                     \
     catch (const nbp::Error &e) {                         \
@@ -2292,7 +2289,7 @@ nbp_status nbp_create(nbp_ctx **out, const nbp_system *sys, const nbp_options *o
         props.location.type = cudaMemLocationTypeDevice;
         props.location.id = c->dev;
         NBP_CUDA(cudaMemPoolCreate(&c->pool, &props));
-        g_pool = c->pool;
+        PoolScope scope(c->pool);
         nbp_default_options(&c->opt);
         if (opt) c->opt = *opt;
         std::string m;
@@ -2613,6 +2610,15 @@ nbp_status nbp_shat_get(nbp_ctx *c, int32_t *rowptr, int32_t *col, double *val) 
     NBP_API_END(c)
 }
 
+nbp_status nbp_memory(nbp_ctx *c, uint64_t *used, uint64_t *reserved) {
+    NBP_API_BEGIN(c)
+    require(used && reserved, NBP_ERR_INVALID, "nbp_memory: null pointer");
+    NBP_CUDA(cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrUsedMemCurrent, used));
+    NBP_CUDA(cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrReservedMemCurrent, reserved));
+    return NBP_OK;
+    NBP_API_END(c)
+}
+
 nbp_status nbp_profile(nbp_ctx *c, int32_t enable) {
     if (!c) return NBP_ERR_INVALID;
     c->prof.on = enable != 0;
@@ -2741,6 +2747,7 @@ static nbp_status batch_solve_dl(nbp_batch *B, const double *const *b, double *c
             nbp_ctx *c = B->ctx[i];
             require(dl_supported(c), NBP_ERR_INVALID, "nbp_batch_solve: device_loop needs m_A >= nmax_A, m_S >= nmax_S and "
                                                       "variant 0 or 1");
+            PoolScope scope(c->pool);
             dl_prepare(c);                      // buffers, options upload, counters reset (instance stream)
             if (!stale && (B->dl_gen[i] != c->graph_gen || B->dl_key[i] != c->dl_key)) stale = true;
             NBP_CUDA(cudaEventRecord(B->ev[i], c->s));
@@ -2995,7 +3002,8 @@ struct nbp_vms {
 #define VMS_BEGIN(v)                     \
     if (!(v) || !(v)->ctx) return NBP_ERR_INVALID; \
     nbp_ctx *c = (v)->ctx;               \
-    try {
+    try {                                \
+        nbp::PoolScope pool_scope(c->pool);
 #define VMS_END NBP_API_END(c)
 
 namespace nbp {

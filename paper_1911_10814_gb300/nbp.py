@@ -132,6 +132,7 @@ SIGNATURES = {
     "nbp_amg_level_get": (ctypes.c_int, [_vp, _i32, _i32, _vp, _vp, _vp, _vp, ctypes.POINTER(_d)]),
     "nbp_shat_nnz": (_i64, [_vp]),
     "nbp_shat_get": (ctypes.c_int, [_vp, _vp, _vp, _vp]),
+    "nbp_memory": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_uint64), ctypes.POINTER(ctypes.c_uint64)]),
     "nbp_profile": (ctypes.c_int, [_vp, _i32]),
     "nbp_profile_get": (ctypes.c_int, [_vp, ctypes.POINTER(nbp_profile_info)]),
     "nbp_profile_report": (ctypes.c_char_p, [_vp]),
@@ -509,6 +510,12 @@ class Solver:
         """New tangent values (CUDA float64 tensors on the context's pattern,
         9, 3, 3, 1 per entry); call setup() again before solving."""
         self._check(self.lib.nbp_set_values(self.ctx, _ptr(A), _ptr(B), _ptr(C), _ptr(D)))
+
+    def memory(self):
+        """Device bytes of the context: in its buffers, and held by its pool."""
+        used, reserved = ctypes.c_uint64(), ctypes.c_uint64()
+        self._check(self.lib.nbp_memory(self.ctx, ctypes.byref(used), ctypes.byref(reserved)))
+        return {"used": used.value, "reserved": reserved.value}
 
     def profile(self, enable=True):
         self._check(self.lib.nbp_profile(self.ctx, int(enable)))
