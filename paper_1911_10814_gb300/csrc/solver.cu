@@ -162,7 +162,6 @@ struct nbp_ctx {
     std::string report;
     nbp_ctx *tctx = nullptr;      // transposed system (adjoint), built lazily
     bool is_transposed = false;
-    int rows_beside = 0;          // half the rows of the batch this context is one of (0: alone), see fine_threads
     // CUDA graphs of the AMG cycles, keyed by (hierarchy, value precision, Chebyshev degree)
     struct CycleGraph { cudaGraphExec_t exec = nullptr; int cheb = -1; long long kernels = 0; };
     static constexpr int kMaxChebDegree = 8;
@@ -1991,7 +1990,7 @@ struct PoolHold {
 
 // kernel of the products with the operators and the finest levels (DMat::tuned)
 static int fine_kind(const nbp_ctx *c) {
-    const int t = fine_threads(std::max(c->N, c->rows_beside));
+    const int t = fine_threads(c->N);
     return t > 1 ? kSellMT + t : 0;
 }
 
@@ -2703,9 +2702,6 @@ nbp_status nbp_batch_create(nbp_batch **out, int32_t count, const nbp_system *sy
         if (st != NBP_OK) { nbp_batch_destroy(B); return st; }
         B->ctx.push_back(c);
     }
-    long long rows = 0;
-    for (nbp_ctx *c : B->ctx) rows += c->N;
-    for (nbp_ctx *c : B->ctx) c->rows_beside = (int)std::min<long long>(rows / 2, INT32_MAX);
     *out = B;
     return NBP_OK;
 }

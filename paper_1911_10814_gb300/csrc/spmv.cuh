@@ -23,9 +23,11 @@ int choose_group(const DMat &M);
 // 29,760 rows 52.1 / 42.4 / 41.4 / 42.9 ms, 60,625 rows 51.3 / 47.8 / 48.3 /
 // 54.0 ms, 68,921 rows 66.7 / 61.9 / 64.1 / 71.5 ms; 140,481 rows 176.6 / 169.8;
 // 452,393 and 1,085,825 rows are faster with one.
-// Branches of a batch share the GPU: there half the batch's rows count (16
-// cubes of 12-40, 440,000 rows: one thread 131.8-133.9 ms, by their own sizes
-// 140.2; 16 of 8-14: 31.2 and 24.3).
+// By the matrix's own rows alone: the threads set the order of a row's sum, so
+// an instance of a batch gives the bits of its single solve.  Counting half the
+// batch's rows instead (one thread where the branches fill the GPU together)
+// took 117 against 128 ms for 16 cubes of 12-40 in BF16, 149 against 143 in
+// FP32, and made every result depend on the neighbours.
 int fine_threads(int rows);
 
 // Whether y = M x with the K-cycle's inner products fused (k_sell_dot) runs
