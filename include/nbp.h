@@ -236,6 +236,11 @@ nbp_status nbp_shat_get(nbp_ctx *ctx, int32_t *rowptr, int32_t *col, double *val
  * pool of the context that it works on. */
 nbp_status nbp_memory(nbp_ctx *ctx, uint64_t *used, uint64_t *reserved);
 
+/* Coarse-level shapes whose product kernel this process has timed and keeps
+ * the choice of (at most 4096, those used last).  A setup that meets a new
+ * shape times it; one that does not repeats the choices. */
+int64_t nbp_tuned_shapes(void);
+
 /* Per-kernel device-time accounting of the last solve: total milliseconds and
  * algorithmic bytes of the SpMV family and of the Arnoldi (CGS2) kernels,
  * measured with CUDA events on the context stream when `enable` was set by

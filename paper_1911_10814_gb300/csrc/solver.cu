@@ -36,6 +36,7 @@
 #include "spmv.cuh"
 #include "rcr.cuh"
 #include "vms.cuh"
+#include "tune_cache.cuh"
 
 namespace nbp {
 
@@ -882,10 +883,12 @@ static void vcycle_level(nbp_ctx *c, Hier &H, int l, int vsel, const T *b, T *ou
 // (pre-smoothing, residual, post-smoothing), as here.  Starting at the tuned
 // level keeps the finer levels' work, and its run-to-run noise, out of the
 // comparison.  The median of 5 timed cycles decides.  Decisions are cached
-// per (hierarchy, level shape, precision) for the life of the process so that
-// every context meeting the same shapes rounds the same way.
-static std::mutex g_cycle_tune_mutex;
-static std::map<std::tuple<int, int, long long, int, int>, int> g_cycle_tune;
+// per (hierarchy, level shape, precision) so that every context meeting the
+// same shapes rounds the same way.  The shapes are exact, and a full setup on new values brings
+// new ones: it times them, about 9 ms for a cube of 16 and 35 ms for 0.56M
+// unknowns (setups of 16.4 and 54 ms against 7.0 and 19.5 on shapes met before).
+constexpr size_t kTunedShapes = 4096;   // about 100 bytes each
+static TuneCache<std::tuple<int, int, long long, int, int>, int> g_cycle_tune(kTunedShapes);
 
 template <typename T> static void autotune_cycles(nbp_ctx *c) {
     const int vsel = amg_vsel_of(c->opt.precision);
@@ -904,12 +907,10 @@ template <typename T> static void autotune_cycles(nbp_ctx *c) {
             for (int l = 1; l < last; ++l) {
                 Level &L = H.L[l];
                 DMat &M = L.M;
+                // a level that runs a K-cycle is timed with its products and updates
+                const bool kc = H.kcycle && l < H.nlev - 1 && l <= H.kdepth;
                 const auto key = std::make_tuple(h, M.nbr, (long long)M.nnz, M.br, (int)sizeof(T) * 4 + vsel);
-                {
-                    std::lock_guard<std::mutex> lock(g_cycle_tune_mutex);
-                    auto it = g_cycle_tune.find(key);
-                    if (it != g_cycle_tune.end()) { M.tuned = it->second; continue; }
-                }
+                if (g_cycle_tune.find(key, M.tuned)) continue;
                 if (!flush) flush = dmalloc<char>(kFlushBytes, c->s);
                 const long long n = (long long)M.nbr * H.bs;
                 T *b = wvec<T>(L, 0), *x = wvec<T>(L, 1);
@@ -921,8 +922,6 @@ template <typename T> static void autotune_cycles(nbp_ctx *c) {
                 cands.push_back(g0);
                 if (g0 > 4) cands.push_back(g0 / 2);
                 if (g0 < 32) cands.push_back(g0 * 2);
-                // a level that runs a K-cycle is timed with its products and updates
-                const bool kc = H.kcycle && l < H.nlev - 1 && l <= H.kdepth;
                 auto cycle = [&] {
                     if (kc) kcycle_level<T>(c, H, l, vsel, b, x);
                     else vcycle_level<T>(c, H, l, vsel, b, x);
@@ -944,11 +943,7 @@ template <typename T> static void autotune_cycles(nbp_ctx *c) {
                     std::sort(t, t + kSamples);
                     if (t[kSamples / 2] < best) { best = t[kSamples / 2]; arg = cand; }
                 }
-                std::lock_guard<std::mutex> lock(g_cycle_tune_mutex);
-                auto it = g_cycle_tune.find(key);
-                if (it != g_cycle_tune.end()) arg = it->second;
-                else g_cycle_tune[key] = arg;
-                M.tuned = arg;
+                M.tuned = g_cycle_tune.keep(key, arg);
             }
         }
     } catch (...) {
@@ -2630,6 +2625,8 @@ nbp_status nbp_profile_get(nbp_ctx *c, nbp_profile_info *out) {
     *out = c->pinfo;
     return NBP_OK;
 }
+
+int64_t nbp_tuned_shapes(void) { return (int64_t)nbp::g_cycle_tune.size(); }
 
 const char *nbp_profile_report(const nbp_ctx *c) { return c ? c->report.c_str() : "{}"; }
 
