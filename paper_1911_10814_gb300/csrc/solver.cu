@@ -883,12 +883,13 @@ static void vcycle_level(nbp_ctx *c, Hier &H, int l, int vsel, const T *b, T *ou
 // (pre-smoothing, residual, post-smoothing), as here.  Starting at the tuned
 // level keeps the finer levels' work, and its run-to-run noise, out of the
 // comparison.  The median of 5 timed cycles decides.  Decisions are cached
-// per (hierarchy, level shape, precision) so that every context meeting the
-// same shapes rounds the same way.  The shapes are exact, and a full setup on new values brings
+// per (hierarchy, level shape, precision, what is timed: K-cycle or not and
+// the smoothing degree) so that every context meeting the same work rounds
+// the same way.  The shapes are exact, and a full setup on new values brings
 // new ones: it times them, about 9 ms for a cube of 16 and 35 ms for 0.56M
 // unknowns (setups of 16.4 and 54 ms against 7.0 and 19.5 on shapes met before).
 constexpr size_t kTunedShapes = 4096;   // about 100 bytes each
-static TuneCache<std::tuple<int, int, long long, int, int>, int> g_cycle_tune(kTunedShapes);
+static TuneCache<std::tuple<int, int, long long, int, int, int>, int> g_cycle_tune(kTunedShapes);
 
 template <typename T> static void autotune_cycles(nbp_ctx *c) {
     const int vsel = amg_vsel_of(c->opt.precision);
@@ -909,7 +910,8 @@ template <typename T> static void autotune_cycles(nbp_ctx *c) {
                 DMat &M = L.M;
                 // a level that runs a K-cycle is timed with its products and updates
                 const bool kc = H.kcycle && l < H.nlev - 1 && l <= H.kdepth;
-                const auto key = std::make_tuple(h, M.nbr, (long long)M.nnz, M.br, (int)sizeof(T) * 4 + vsel);
+                const auto key = std::make_tuple(h, M.nbr, (long long)M.nnz, M.br, (int)sizeof(T) * 4 + vsel,
+                                                 2 * H.cheb + (kc ? 1 : 0));
                 if (g_cycle_tune.find(key, M.tuned)) continue;
                 if (!flush) flush = dmalloc<char>(kFlushBytes, c->s);
                 const long long n = (long long)M.nbr * H.bs;

@@ -1,0 +1,33 @@
+"""A coarse level's product kernel is chosen for the work that the level does:
+a context with another cycle or smoothing degree times it anew, one with the
+same options and shapes does not."""
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_1911_10814_gb300 import Solver, load  # noqa: E402
+
+
+def test_choices_belong_to_the_cycle_they_were_timed_in():
+    d = synth.generate(synth.MeshSpec(15, 16, 17, Re=300.0, seed=21, R=(1e3,)))
+    counts = [load().nbp_tuned_shapes()]
+    for opts in (dict(amg_cycle=0), dict(amg_cycle=0), dict(amg_cycle=2), dict(amg_cycle=2), dict(amg_cycle=2, cheb_degree=3)):
+        s = Solver(d, precision=1, amg_kdepth=1, **opts)
+        s.setup()
+        levels = [len(s.amg_levels(w)) for w in (0, 1)]
+        s.close()
+        counts.append(load().nbp_tuned_shapes())
+    new = [b - a for a, b in zip(counts, counts[1:])]
+    # tuned: the levels between the finest and the coarsest (dense) one
+    assert all(n >= 3 for n in levels), levels
+    assert new[0] == sum(n - 2 for n in levels)
+    assert new[1] == 0
+    assert new[2] == 2          # level 1 of both hierarchies runs a K-cycle now
+    assert new[3] == 0
+    assert new[4] == levels[0] - 2   # another degree on AMG(A)
