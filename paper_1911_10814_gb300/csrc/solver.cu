@@ -1647,6 +1647,9 @@ static nbp_status dl_collect(nbp_ctx *c) {
     c->info.A_iters += k.A;
     c->info.S_iters += k.S;
     c->info.I_iters += k.I;
+    c->info.n_A_solves += k.nA;
+    c->info.n_S_solves += k.nS;
+    c->info.n_I_solves += k.nI;
     c->info.rel_res_est = o.bnorm > 0 ? o.res / o.bnorm : 0.0;
     c->info.rel_res_true = o.rel_true;
     c->info.status = o.conv ? NBP_OK : NBP_NOT_CONVERGED;
