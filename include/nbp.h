@@ -236,10 +236,12 @@ nbp_status nbp_shat_get(nbp_ctx *ctx, int32_t *rowptr, int32_t *col, double *val
  * pool of the context that it works on. */
 nbp_status nbp_memory(nbp_ctx *ctx, uint64_t *used, uint64_t *reserved);
 
-/* Coarse-level shapes whose product kernel this process has timed and keeps
- * the choice of (at most 4096, those used last).  A setup that meets a new
- * shape times it; one that does not repeats the choices. */
-int64_t nbp_tuned_shapes(void);
+/* Shapes that this process has timed and keeps the choice for (at most 4096 of
+ * each kind, those used last).  which 0: coarse levels, whose product kernel
+ * the first setup that meets them chooses; 1: vector lengths, whose
+ * Gram-Schmidt grids the first solve chooses.  Other contexts that meet a
+ * shape repeat the choice. */
+int64_t nbp_tuned_shapes(int32_t which);
 
 /* Per-kernel device-time accounting of the last solve: total milliseconds and
  * algorithmic bytes of the SpMV family and of the Arnoldi (CGS2) kernels,

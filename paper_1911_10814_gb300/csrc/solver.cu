@@ -435,31 +435,45 @@ template <typename T> static void scale_inv(nbp_ctx *c, T *v, const T *w, const 
     else k_scale_inv<T, false><<<grid, 256, 0, c->s>>>(v, w, sc, n);
 }
 
+constexpr size_t kTunedShapes = 4096;   // bound of each cache of timed choices, about 100 bytes an entry
+
 // Autotuner of the Gram-Schmidt kernels' grids for one vector length: the
 // candidates (one wave, a half and a quarter of it, a quarter block per SM,
 // just enough blocks for eight 16-byte pieces per thread, and kReduceBlocks
 // and half of it, capped at a block per 256 pieces) are timed on a
 // four-column step in the space's own buffers, as the solve meets it: the
 // multi-dot after a write of a buffer larger than L2 (between two steps the
-// preconditioner's sweeps evict the basis), then the subtract + products and
-// subtract + norm passes on the columns it left in L2.  Three batches of
-// five steps; each kernel keeps its own fastest grid.  A short vector leaves
+// preconditioner's sweeps evict the basis), then the passes that follow on the
+// columns it left in L2 and that take K.grid: subtract + products and, in the
+// host-driven loop, subtract + norm (the device-driven one's norm pass has a
+// grid of its own, see arnoldi_dl).  The loop's own kernels are timed; a space
+// whose device-driven steps run in one cluster has no grid to choose.  Three
+// batches of five steps; each kernel keeps its own fastest grid.  A short vector leaves
 // most of a one-wave grid idle in its reductions (what a batch of small
 // instances meets), while a cold pass over a long one needs every block's
-// loads in flight.  The choice is cached per (vector length, type) for the
-// life of the process, so every space of that length sums in the same order.
-static std::mutex g_arnoldi_tune_mutex;
-static std::map<std::pair<long long, int>, std::pair<unsigned, unsigned>> g_arnoldi_tune;
+// loads in flight.  The choice is cached per (vector length, type, loop), so
+// every space of that length sums in the same order.
+static TuneCache<std::tuple<long long, int, bool>, std::pair<unsigned, unsigned>> g_arnoldi_tune(kTunedShapes);
 
-template <typename T> static void tune_arnoldi(nbp_ctx *c, Krylov<T> &K) {
-    if (K.grid || K.m < 4 || c->prof.on) return;
-    const auto key = std::make_pair(K.n, (int)sizeof(T));
-    {
-        std::lock_guard<std::mutex> lock(g_arnoldi_tune_mutex);
-        auto it = g_arnoldi_tune.find(key);
-        if (it != g_arnoldi_tune.end()) { K.grid = it->second.first; K.grid_md = it->second.second; return; }
+template <typename T> static bool gs_vec(const Krylov<T> &K) {
+    return al16(K.V) && al16(K.w) && (K.ld * (long long)sizeof(T)) % 16 == 0;
+}
+// the device-driven loop's whole step in one cluster: a short vector
+template <typename T> static bool gs_in_cluster(const Krylov<T> &K) {
+    return gs_vec(K) && K.n <= gs_cluster_max<T>() && K.m <= kGsCols;
+}
+
+// dl: for the device-driven loop
+template <typename T> static void tune_arnoldi(nbp_ctx *c, Krylov<T> &K, bool dl) {
+    if (K.grid || K.m < 4 || c->prof.on || (dl && gs_in_cluster(K))) return;
+    const auto key = std::make_tuple(K.n, (int)sizeof(T), dl);
+    std::pair<unsigned, unsigned> grids;
+    if (g_arnoldi_tune.find(key, grids)) {
+        K.grid = grids.first;
+        K.grid_md = grids.second;
+        return;
     }
-    const bool vec = al16(K.V) && al16(K.w) && (K.ld * (long long)sizeof(T)) % 16 == 0;
+    const bool vec = gs_vec(K);
     const ArnoldiGrids<T> &ag = arnoldi_grids<T>();
     static const unsigned w4v = one_wave(k_maxpy_dot<T, 4, true>), w4s = one_wave(k_maxpy_dot<T, 4, false>);
     unsigned gmax = vec ? std::min({ag.mdot_v, ag.mdot_dl_v, ag.mpd_dl_v, w4v})
@@ -481,6 +495,26 @@ template <typename T> static void tune_arnoldi(nbp_ctx *c, Krylov<T> &K) {
     fill<T>(K.V, T(1), (long long)K.ld * 4, c->s);
     fill<T>(K.w, T(1), K.n, c->s);
     NBP_CUDA(cudaMemsetAsync(K.h1, 0, sizeof(double) * 4, c->s));
+    int *jp = dmalloc<int>(1, c->s);   // the loop's column: four columns
+    k_fill<int><<<1, 32, 0, c->s>>>(jp, 3, 1);
+    NBP_LAUNCHED();
+    auto products = [&] {
+        if (!dl) mdot<T>(c, K, K.V, K.ld, 4, K.w, K.h2);
+        else if (vec) k_mdot_dl<T, 8, true><<<K.grid_md, 256, 0, c->s>>>(K.V, K.ld, jp, 1, K.w, K.n, K.partial, K.h2, K.ticket, GivensArgs());
+        else k_mdot_dl<T, 8, false><<<K.grid_md, 256, 0, c->s>>>(K.V, K.ld, jp, 1, K.w, K.n, K.partial, K.h2, K.ticket, GivensArgs());
+        NBP_LAUNCHED();
+    };
+    auto rest = [&] {
+        if (!dl) {
+            maxpy_dot<T>(c, K, K.V, K.ld, 4, K.h1, K.w, 0, K.h2);
+            maxpy_dot<T>(c, K, K.V, K.ld, 4, K.h1, K.w, 1, K.nrm);
+        } else if (vec) {
+            k_maxpy_dot_dl<T, kFusedCols, true><<<K.grid, 256, 0, c->s>>>(K.V, K.ld, jp, 1, K.h1, K.w, K.n, K.partial, K.h2, K.ticket);
+        } else {
+            k_maxpy_dot_dl<T, kFusedCols, false><<<K.grid, 256, 0, c->s>>>(K.V, K.ld, jp, 1, K.h1, K.w, K.n, K.partial, K.h2, K.ticket);
+        }
+        NBP_LAUNCHED();
+    };
     cudaEvent_t ev[3];
     for (cudaEvent_t &e : ev) NBP_CUDA(cudaEventCreate(&e));
     float best = 1e30f, best_md = 1e30f;
@@ -495,10 +529,9 @@ template <typename T> static void tune_arnoldi(nbp_ctx *c, Krylov<T> &K) {
             for (int q = 0; q < 5; ++q) {
                 NBP_CUDA(cudaMemsetAsync(flush, (r * 5 + q) & 0xff, kFlush, c->s));
                 NBP_CUDA(cudaEventRecord(ev[0], c->s));
-                mdot<T>(c, K, K.V, K.ld, 4, K.w, K.h2);
+                products();
                 NBP_CUDA(cudaEventRecord(ev[1], c->s));
-                maxpy_dot<T>(c, K, K.V, K.ld, 4, K.h1, K.w, 0, K.h2);
-                maxpy_dot<T>(c, K, K.V, K.ld, 4, K.h1, K.w, 1, K.nrm);
+                rest();
                 NBP_CUDA(cudaEventRecord(ev[2], c->s));
                 NBP_CUDA(cudaEventSynchronize(ev[2]));
                 float a = 0.f, b = 0.f;
@@ -509,6 +542,7 @@ template <typename T> static void tune_arnoldi(nbp_ctx *c, Krylov<T> &K) {
             }
             tb = std::min(tb, t);
             tb_md = std::min(tb_md, t_md);
+            if (t > 1.3f * best && t_md > 1.3f * best_md) break;   // out of the running
         }
         if (tb < best) { best = tb; arg = g; }
         if (tb_md < best_md) { best_md = tb_md; arg_md = g; }
@@ -516,12 +550,10 @@ template <typename T> static void tune_arnoldi(nbp_ctx *c, Krylov<T> &K) {
     c->prof.launches = launches;
     for (cudaEvent_t &e : ev) cudaEventDestroy(e);
     dfree(flush, c->s);
-    std::lock_guard<std::mutex> lock(g_arnoldi_tune_mutex);
-    auto it = g_arnoldi_tune.find(key);
-    if (it != g_arnoldi_tune.end()) { arg = it->second.first; arg_md = it->second.second; }
-    else g_arnoldi_tune[key] = std::make_pair(arg, arg_md);
-    K.grid = arg;
-    K.grid_md = arg_md;
+    dfree(jp, c->s);
+    grids = g_arnoldi_tune.keep(key, std::make_pair(arg, arg_md));
+    K.grid = grids.first;
+    K.grid_md = grids.second;
 }
 
 // ----------------------------------------------------------------- GMRES
@@ -545,7 +577,7 @@ static GmResult gmres(nbp_ctx *c, Krylov<T> &K, long long n, Op op, Pc pc, const
     GmResult R;
     m = std::max(1, std::min(m, std::max(nmax, 1)));
     K.ensure(n, m, s);
-    tune_arnoldi<T>(c, K);
+    tune_arnoldi<T>(c, K, false);
     fill<T>(x, T(0), n, s);
     mdot<T>(c, K, b, n, 1, b, K.nrm);
     c->prof.launches++;
@@ -888,7 +920,6 @@ static void vcycle_level(nbp_ctx *c, Hier &H, int l, int vsel, const T *b, T *ou
 // the same way.  The shapes are exact, and a full setup on new values brings
 // new ones: it times them, about 9 ms for a cube of 16 and 35 ms for 0.56M
 // unknowns (setups of 16.4 and 54 ms against 7.0 and 19.5 on shapes met before).
-constexpr size_t kTunedShapes = 4096;   // about 100 bytes each
 static TuneCache<std::tuple<int, int, long long, int, int, int>, int> g_cycle_tune(kTunedShapes);
 
 template <typename T> static void autotune_cycles(nbp_ctx *c) {
@@ -1287,13 +1318,13 @@ template <class F> static long long emit_while(nbp_ctx *c, cudaGraphConditionalH
 // condition h.  The new basis vector w / ||w|| is made by the first kernel of
 // the next iteration (k_start_col, k_start_cheb).
 template <typename T> static void arnoldi_dl(nbp_ctx *c, Krylov<T> &K, GmDev *st, cudaGraphConditionalHandle h) {
-    const bool vec = al16(K.V) && al16(K.w) && (K.ld * (long long)sizeof(T)) % 16 == 0;
+    const bool vec = gs_vec(K);
     const int *jp = &st->j;
     GivensArgs gv = K.givens(0);
     gv.dl = st;
     gv.h = h;
     if (c->gs_one_pass) gv.h2 = nullptr;
-    if (vec && K.n <= gs_cluster_max<T>() && K.m <= kGsCols) {   // a short vector: the whole step in one cluster
+    if (gs_in_cluster(K)) {
         klaunch(k_gs_cluster<T>, kGsCluster, (unsigned)kGsThreads, c->s, K.V, K.ld, jp, K.w, K.n, c->gs_one_pass ? 1 : 2, K.h1, K.h2, gv);
         NBP_LAUNCHED();
         return;
@@ -1301,6 +1332,9 @@ template <typename T> static void arnoldi_dl(nbp_ctx *c, Krylov<T> &K, GmDev *st
     // one pass: the multi-dot, then subtract + norm + Givens update
     const double *coef = c->gs_one_pass ? K.h1 : K.h2;
     // the norm pass: a block per 256 pieces up to the partials' kReduceBlocks
+    // (solves with 608 blocks at most / 304 / 152: 4.34M unknowns 648 / 654 /
+    // 671 ms, 0.56M 173.2 / 174.6 / 175.3, 19x23x61 43.1 / 43.3 / 43.3; a block
+    // per 128 or 512 pieces within 0.5 % on both sides)
     const long long pieces = (K.n + Vec16<T>::W - 1) / Vec16<T>::W;
     const unsigned gn = (unsigned)std::max<long long>(1, std::min<long long>(kReduceBlocks, (pieces + 255) / 256));
     if (vec) {
@@ -1546,17 +1580,17 @@ static void dl_prepare(nbp_ctx *c) {
     const nbp_options &o = c->opt;
     auto cl = [](int m, int nmax) { return std::max(1, std::min(m, std::max(nmax, 1))); };
     c->Kout.ensure(n, cl(o.m, o.nmax), s);
-    tune_arnoldi<double>(c, c->Kout);
+    tune_arnoldi<double>(c, c->Kout, true);
     if (o.precision == 0) {
         c->KA64.ensure(3 * N, cl(o.m_A, o.nmax_A), s);
         c->KS64.ensure(N, cl(o.m_S, o.nmax_S), s);
-        tune_arnoldi<double>(c, c->KA64);
-        tune_arnoldi<double>(c, c->KS64);
+        tune_arnoldi<double>(c, c->KA64, true);
+        tune_arnoldi<double>(c, c->KS64, true);
     } else {
         c->KA32.ensure(3 * N, cl(o.m_A, o.nmax_A), s);
         c->KS32.ensure(N, cl(o.m_S, o.nmax_S), s);
-        tune_arnoldi<float>(c, c->KA32);
-        tune_arnoldi<float>(c, c->KS32);
+        tune_arnoldi<float>(c, c->KA32, true);
+        tune_arnoldi<float>(c, c->KS32, true);
     }
     // the graph bakes in these buffers and option switches (the operators'
     // value copies too: a refresh of the values reallocates them)
@@ -2631,7 +2665,9 @@ nbp_status nbp_profile_get(nbp_ctx *c, nbp_profile_info *out) {
     return NBP_OK;
 }
 
-int64_t nbp_tuned_shapes(void) { return (int64_t)nbp::g_cycle_tune.size(); }
+int64_t nbp_tuned_shapes(int32_t which) {
+    return (int64_t)(which ? nbp::g_arnoldi_tune.size() : nbp::g_cycle_tune.size());
+}
 
 const char *nbp_profile_report(const nbp_ctx *c) { return c ? c->report.c_str() : "{}"; }
 

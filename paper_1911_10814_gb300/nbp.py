@@ -133,7 +133,7 @@ SIGNATURES = {
     "nbp_shat_nnz": (_i64, [_vp]),
     "nbp_shat_get": (ctypes.c_int, [_vp, _vp, _vp, _vp]),
     "nbp_memory": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_uint64), ctypes.POINTER(ctypes.c_uint64)]),
-    "nbp_tuned_shapes": (_i64, []),
+    "nbp_tuned_shapes": (_i64, [_i32]),
     "nbp_profile": (ctypes.c_int, [_vp, _i32]),
     "nbp_profile_get": (ctypes.c_int, [_vp, ctypes.POINTER(nbp_profile_info)]),
     "nbp_profile_report": (ctypes.c_char_p, [_vp]),
