@@ -1440,8 +1440,8 @@ void amg_build(Hier &H, const DMat &fine, const nbp_options &o, int precision, c
             L.w64[q] = reinterpret_cast<double *>(L.work + q * v64);
             L.w32[q] = reinterpret_cast<float *>(L.work + Level::kWork * v64 + q * v32);
         }
-        L.kdots = dmalloc<double>(8 + 3 * kKdotBlocks, s);
-        NBP_CUDA(cudaMemsetAsync(L.kdots, 0, sizeof(double) * (8 + 3 * kKdotBlocks), s));
+        L.kdots = dmalloc<double>(8 + 4 * kKdotBlocks, s);
+        NBP_CUDA(cudaMemsetAsync(L.kdots, 0, sizeof(double) * (8 + 4 * kKdotBlocks), s));
         {   // every level, the coarsest included (it is smoothed when too large for a dense solve)
             L.dinv = dmalloc<double>(nv * bs, s);
             k_block_dinv<<<grid_exact(n), 256, 0, s>>>(n, bs, L.M.rp, L.M.ci, L.M.v, L.dinv, singular);
@@ -1460,7 +1460,7 @@ void amg_build(Hier &H, const DMat &fine, const nbp_options &o, int precision, c
             if (k + 1 < H.nlev) make_ap(L, H.L[k + 1].M.nbr, precision, s);
             if (L.M.sl_ci) {   // grids of the sliced kernels, up to 8 threads per row
                 L.kpart_blocks = ((long long)L.M.nslice * L.M.sl_c * 8 + 255) / 256;
-                L.kpart = dmalloc<double>(3 * L.kpart_blocks, s);
+                L.kpart = dmalloc<double>(4 * L.kpart_blocks, s);
             }
             if (level_ready) level_ready(k);
         }

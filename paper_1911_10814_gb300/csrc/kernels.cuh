@@ -788,9 +788,12 @@ __device__ __forceinline__ V fold_warp(V (&v)[NQ], int ln, Add add, Xor xr) {
 // block's threads into partial[(col0 + q) * gridDim.x + blockIdx.x].  FP64
 // kernels: FP64 warp trees, then the warps' sums in order; FP32 kernels: the
 // same in float-float (the partial stored as a float2).  256 threads; columns
-// in folded groups of up to 8 (fold_warp).
-template <typename T, int NQ>
-__device__ __forceinline__ void block_partials(const T (&acc)[NQ], int nq, double *partial, int col0) {
+// in folded groups of up to 8 (fold_warp).  FP32 kernels give the thread's
+// sums as floats or as float-float pairs.
+__device__ __forceinline__ FF as_ff(float v) { return FF{v, 0.f}; }
+__device__ __forceinline__ FF as_ff(FF v) { return v; }
+template <typename T, int NQ, typename A>
+__device__ __forceinline__ void block_partials(const A (&acc)[NQ], int nq, double *partial, int col0) {
     const int warp = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
     constexpr int F = NQ < 8 ? NQ : 8;   // values folded together
     static_assert(NQ % F == 0 && (F & (F - 1)) == 0, "fold size");
@@ -806,12 +809,12 @@ __device__ __forceinline__ void block_partials(const T (&acc)[NQ], int nq, doubl
         for (int q0 = 0; q0 < NQ; q0 += F)
             if (q0 < nq) {   // uniform over the block
                 if (nq - q0 == 1) {   // one column left: a plain warp sum
-                    const FF v = ff_warp_sum(FF{acc[q0], 0.f});
+                    const FF v = ff_warp_sum(as_ff(acc[q0]));
                     if (ln == 0) redf[q0][warp] = v;
                 } else {
                     FF v[F];
 #pragma unroll
-                    for (int q = 0; q < F; ++q) v[q] = FF{acc[q0 + q], 0.f};
+                    for (int q = 0; q < F; ++q) v[q] = as_ff(acc[q0 + q]);
                     const FF r = fold_warp<FF, F>(v, ln, add, xr);
                     if (lead) redf[q0 + q_of][warp] = r;
                 }
@@ -850,18 +853,94 @@ __device__ __forceinline__ void block_partials(const T (&acc)[NQ], int nq, doubl
     }
 }
 
+// The inner products of one step of a K-cycle (x = a1 z1 + a2 (z2 - beta z1),
+// w1 = M z1, w2 = M z2, r the residual after the first step) by the launch that
+// makes w1 or w2.  First step: w1.w1 and w1.b.  Second step, the direction
+// made orthogonal to the first: beta = (w2.w1)/(w1.w1), w2' = w2 - beta w1,
+// a2 = (w2'.r)/(w2'.w2').  The products of w2 itself give both,
+//   w2'.w2' = w2.w2 - beta w2.w1,   w2'.r = w2.r - beta w1.r,
+// without a pass that forms w2' and z2' (2 launches and 10 vector passes fewer
+// per K-cycle than updating, reducing and then combining).  Where w2 is close
+// to w1 the differences cancel: 3.6e-5 of w2.w2 was left at the least and 0.98
+// of it at the median (S_hat levels of four boxes, residuals of 5 cycles).  So
+// FP32 sums exact products (two-product) in float-float, and FP64, whose pipe
+// is too narrow for more digits, sums over w2' itself where less than a half
+// is left, in the last block (1 to 7 cycles in a hundred).
+// Largest relative error of a2 on those levels: FP32 1e-11 (1.3e-6 with w2'
+// formed first and rounded products, 1.7e-4 from rounded products and w1.r
+// taken as zero), FP64 1.7e-15 (1.7e-15 and 4e-12).
+template <typename T> struct GsSum { using type = double; };
+template <> struct GsSum<float> { using type = FF; };
+__device__ __forceinline__ FF gs_add(FF a, FF b) { return ff_add(a, b); }
+__device__ __forceinline__ double gs_add(double a, double b) { return a + b; }
+// a b without rounding (the product and its error by a fused multiply-add)
+__device__ __forceinline__ FF gs_mul(float a, float b) {
+    const float p = __fmul_rn(a, b);
+    return FF{p, __fmaf_rn(a, b, -p)};
+}
+__device__ __forceinline__ double gs_mul(double a, double b) { return a * b; }
+__device__ __forceinline__ void gs_set(FF &s, float v) { s = FF{v, 0.f}; }
+__device__ __forceinline__ void gs_set(double &s, double v) { s = v; }
+
+// By the last block of the launch (256 threads), s = {w.w, w.da, w.db, da.db},
+// w11 = kd[0] and a1 = kd[2] as loaded beside the partials:
+// the first step (da = b): kd[0] = w1.w1, kd[1] = w1.b; the second (da = w1,
+// db = r): the cycle's coefficients kd[3] of z1 and kd[4] of z2.  Where nothing
+// but rounding is left of w2' the second direction is dropped.
+template <typename T>
+__device__ __forceinline__ void kc_finish(const double (&s)[4], double w11, double a1, const T *w2, const T *w1, const T *r,
+                                          long long n, double *kd) {
+    if (!r) {
+        if (threadIdx.x == 0) {
+            kd[0] = s[0];
+            kd[1] = s[1];
+        }
+        return;
+    }
+    const double beta = w11 > 0.0 ? s[1] / w11 : 0.0;
+    double ww = s[0] - beta * s[1], wr = s[2] - beta * s[3];
+    if constexpr (sizeof(T) == 8) {
+        if (ww < 0.5 * s[0]) {   // the same in every thread
+            __shared__ double red[2][8];
+            double p0 = 0.0, p1 = 0.0;
+#pragma unroll 4
+            for (long long i = threadIdx.x; i < n; i += 256) {
+                const double v = __ldcg(w2 + i) - beta * w1[i];   // w2: written by this launch
+                p0 += v * v;
+                p1 += v * r[i];
+            }
+            p0 = warp_sum(p0);
+            p1 = warp_sum(p1);
+            if ((threadIdx.x & 31) == 0) {
+                red[0][threadIdx.x >> 5] = p0;
+                red[1][threadIdx.x >> 5] = p1;
+            }
+            __syncthreads();
+            ww = wr = 0.0;
+            for (int k = 0; k < 8; ++k) {
+                ww += red[0][k];
+                wr += red[1][k];
+            }
+        }
+    }
+    if (threadIdx.x == 0) {
+        const double a2 = ww <= (sizeof(T) == 4 ? 1e-10 : 1e-20) * s[0] ? 0.0 : wr / ww;   // NaN passes through
+        kd[3] = a1 - a2 * beta;
+        kd[4] = a2;
+    }
+}
+
 // Scalar-block (Ŝ level) sliced-ELL product y = M x fused with the inner
-// products the K-cycle takes of it: y . y, y . da and, when db is set, y . db.
-// T threads per row as in k_sellm (T = 1: one thread per row); each row's sum
+// products the K-cycle takes of it (see kc_finish).  T threads per row as in
+// k_sellm (T = 1: one thread per row); each row's sum
 // is the same as the unfused kernels'.  The row products are summed per block
 // (block_partials) into part, and the last block to finish (ticket kd[7])
 // adds the block partials in a fixed order -- one launch instead of a product
 // and a reduction, the same result whatever the order the blocks run in.
 struct DotArgs {
-    const void *da, *db;   // vectors the product is dotted with (same type as y); db may be null
-    double *part;          // 3 x gridDim.x block partials
-    double *kd;            // results; kd[7] is the ticket
-    int oy, oa, ob;        // kd[oy] = y . y, kd[oa] = y . da, kd[ob] = y . db
+    const void *da, *db;   // vectors the product is dotted with (same type as y); db null in the first step
+    double *part;          // 4 x gridDim.x block partials
+    double *kd;            // results (kc_finish); kd[7] is the ticket
 };
 template <typename VT, typename XT, int C, int T>
 __global__ void __launch_bounds__(256) k_sell_dot(SpmvArgs a, DotArgs q) {
@@ -894,26 +973,31 @@ __global__ void __launch_bounds__(256) k_sell_dot(SpmvArgs a, DotArgs q) {
     }
 #pragma unroll
     for (int o = T / 2; o > 0; o >>= 1) acc0 += __shfl_xor_sync(0xffffffffu, acc0, o);
-    AT pp[4] = {0, 0, 0, 0};
+    typename GsSum<AT>::type pp[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) gs_set(pp[k], AT(0));
+    const XT *da = (const XT *)q.da, *db = (const XT *)q.db;
     if (h == 0 && live && row < a.nbr) {
         ((XT *)a.y)[row] = acc0;
-        pp[0] = acc0 * acc0;
-        pp[1] = acc0 * ((const XT *)q.da)[row];
-        if (q.db) pp[2] = acc0 * ((const XT *)q.db)[row];
+        const XT u = da[row];
+        pp[0] = gs_mul(acc0, acc0);
+        pp[1] = gs_mul(acc0, u);
+        if (db) {
+            const XT v = db[row];
+            pp[2] = gs_mul(acc0, v);
+            pp[3] = gs_mul(u, v);
+        }
     }
-    const int nq = q.db ? 3 : 2;
-    block_partials<AT, 4>(pp, nq, q.part, 0);
+    const int nq = db ? 4 : 2;
+    block_partials<AT>(pp, nq, q.part, 0);
     unsigned *ticket = (unsigned *)(q.kd + 7);
     if (!grid_last_block(ticket)) return;
-    __shared__ double out[3];
+    __shared__ double out[4];
+    const double w11 = q.kd[0], a1 = q.kd[2];
     reduce_partials<AT>(q.part, gridDim.x, nq, out);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        q.kd[q.oy] = out[0];
-        q.kd[q.oa] = out[1];
-        if (q.db) q.kd[q.ob] = out[2];
-        *ticket = 0;
-    }
+    kc_finish<XT>(out, w11, a1, (const XT *)a.y, da, db, a.nbr, q.kd);
+    if (threadIdx.x == 0) *ticket = 0;
 }
 
 // ================================================ Givens / least squares
@@ -1380,16 +1464,10 @@ constexpr int kGsCluster = 8, kGsThreads = 512, kGsPieces = 4, kGsCols = 256, kG
 template <typename T> __host__ __device__ constexpr long long gs_cluster_max() {
     return (long long)kGsCluster * kGsThreads * kGsPieces * Vec16<T>::W;
 }
-template <typename T> struct GsSum { using type = double; };
-template <> struct GsSum<float> { using type = FF; };
-__device__ __forceinline__ FF gs_add(FF a, FF b) { return ff_add(a, b); }
-__device__ __forceinline__ double gs_add(double a, double b) { return a + b; }
 __device__ __forceinline__ FF gs_xor(FF a, int o) {
     return FF{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
 }
 __device__ __forceinline__ double gs_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
-__device__ __forceinline__ void gs_set(FF &s, float v) { s = FF{v, 0.f}; }
-__device__ __forceinline__ void gs_set(double &s, double v) { s = v; }
 __device__ __forceinline__ double gs_double(FF a) { return ff_to_double(a); }
 __device__ __forceinline__ double gs_double(double a) { return a; }
 template <typename T>
@@ -1976,39 +2054,40 @@ __global__ void __launch_bounds__(kGemvThreads) k_dense_gemv_rows(const T *__res
 }
 
 // ============================================================== K-cycle
-// The inner products of a K-cycle step where the level's product is the flat
-// kernel or its blocks are 3x3: kd[oy] = y . y, kd[oa] = y . a and, when b is
-// set, kd[ob] = y . b.  Each block reduces a fixed contiguous chunk into
-// kd[8 + blk], kd[8 + nb + blk], ..., and the last block to finish (ticket in
-// kd[7]) sums the block partials in a fixed order: one launch, same result
-// whatever order the blocks run in.
+// The inner products of a K-cycle step (see kc_finish; b null in the first)
+// where the level's product is the flat kernel or its blocks are 3x3.  Each
+// block reduces a fixed contiguous chunk into kd[8 + blk], kd[8 + nb + blk],
+// ..., and the last block to finish (ticket in kd[7]) sums the block partials
+// in a fixed order: one launch, same result whatever order the blocks run in.
 constexpr int kKdotBlocks = 96;
 template <typename T>
-__global__ void __launch_bounds__(256) k_kdots(const T *y, const T *a, const T *b, long long n, double *kd, int oy, int oa,
-                                               int ob) {
+__global__ void __launch_bounds__(256) k_kdots(const T *y, const T *a, const T *b, long long n, double *kd) {
     pdl_wait();
     const long long chunk = (n + gridDim.x - 1) / gridDim.x;
     const long long lo = (long long)blockIdx.x * chunk, hi = min(n, lo + chunk);
-    T pp[4] = {0, 0, 0, 0};   // per-thread sums in the vector type
+    typename GsSum<T>::type pp[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) gs_set(pp[k], T(0));
     for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        const T u = y[i];
-        pp[0] += u * u;
-        pp[1] += u * a[i];
-        if (b) pp[2] += u * b[i];
+        const T u = y[i], p = a[i];
+        pp[0] = gs_add(pp[0], gs_mul(u, u));
+        pp[1] = gs_add(pp[1], gs_mul(u, p));
+        if (b) {
+            const T v = b[i];
+            pp[2] = gs_add(pp[2], gs_mul(u, v));
+            pp[3] = gs_add(pp[3], gs_mul(p, v));
+        }
     }
-    const int nq = b ? 3 : 2;
-    block_partials<T, 4>(pp, nq, kd + 8, 0);
+    const int nq = b ? 4 : 2;
+    block_partials<T>(pp, nq, kd + 8, 0);
     unsigned *ticket = (unsigned *)(kd + 7);
     if (!grid_last_block(ticket)) return;
-    __shared__ double out[3];
+    __shared__ double out[4];
+    const double w11 = kd[0], a1 = kd[2];
     reduce_partials<T>(kd + 8, gridDim.x, nq, out);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        kd[oy] = out[0];
-        kd[oa] = out[1];
-        if (b) kd[ob] = out[2];
-        *ticket = 0;
-    }
+    kc_finish<T>(out, w11, a1, y, a, b, n, kd);
+    if (threadIdx.x == 0) *ticket = 0;
 }
 // r -= a1 w1 with a1 = (w1.r)/(w1.w1) = kd[1]/kd[0], saved in kd[2]; then, where
 // the second cycle starts with a smoothing step from zero (dinv set), that
@@ -2048,25 +2127,10 @@ __global__ void k_kupd1(T *r, const T *w1, double *kd, int nbr, int bs, const T 
             }
     }
 }
-// x = a1 z1 + a2 (z2 - beta z1), the second search direction made orthogonal
-// to the first: beta = (w2.w1)/(w1.w1) = kd[3]/kd[0], w2' = w2 - beta w1, and
-// a2 = (w2'.r)/(w2'.w2') = kd[5] / (kd[4] - beta kd[3]) since w1.r = 0 after
-// the first step: the inner products of w2 itself give it, without a pass
-// that forms w2' and z2' (2 launches and 10 vector passes fewer per K-cycle
-// than updating, reducing and then combining).  Where w2 is parallel to w1 to
-// rounding the second direction is dropped.
+// x = a1 z1 + a2 (z2 - beta z1), the coefficients of z1 and z2 from kc_finish
 template <typename T> __global__ void k_kupd2(T *x, const T *z1, const T *z2, const double *kd, long long n) {
-    __shared__ T c1s, c2s;
     pdl_wait();
-    if (threadIdx.x == 0) {
-        const double beta = kd[0] > 0.0 ? kd[3] / kd[0] : 0.0;
-        const double ww = kd[4] - beta * kd[3];
-        const double a2 = ww > (sizeof(T) == 4 ? 1e-6 : 1e-12) * kd[4] ? kd[5] / ww : 0.0;
-        c1s = (T)(kd[2] - a2 * beta);
-        c2s = (T)a2;
-    }
-    __syncthreads();
-    const T c1 = c1s, c2 = c2s;
+    const T c1 = (T)kd[3], c2 = (T)kd[4];
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         x[i] = c1 * z1[i] + c2 * z2[i];
 }

@@ -753,17 +753,16 @@ static void vcycle_level(nbp_ctx *c, Hier &H, int l, int vsel, const T *b, T *ou
 // coefficient stays on the device, so the whole cycle can be replayed from a
 // CUDA graph.  x = a1 z1 + a2 (z2 - beta z1) with a1 = (w1.b)/(w1.w1), r = b -
 // a1 w1, beta = (w2.w1)/(w1.w1), a2 = (w2'.r)/(w2'.w2'), w2' = w2 - beta w1.
-// w = L.M z with kd[oy] = w . w, kd[oa] = w . da and (db set) kd[ob] = w . db:
-// one fused launch (k_sell_dot) where the level's tuned kernel is a scalar
-// sliced one, else the product and k_kdots
+// w = L.M z with the step's inner products and what follows from them
+// (kc_finish): one fused launch (k_sell_dot) where the level's tuned kernel is
+// a scalar sliced one, else the product and k_kdots
 template <typename T>
-static void kc_product_dots(nbp_ctx *c, Level &L, int vsel, const T *z, T *w, const T *da, const T *db, int oy, int oa,
-                            int ob) {
+static void kc_product_dots(nbp_ctx *c, Level &L, int vsel, const T *z, T *w, const T *da, const T *db) {
     const long long n = (long long)L.M.nbr * L.M.br;
     if (L.kpart && spmv_dot_ok(L.M, vsel, (int)sizeof(T), L.kpart_blocks)) {
         cudaEvent_t e0;
         prof_begin(c, e0);
-        DotArgs q{da, db, L.kpart, L.kdots, oy, oa, ob};
+        DotArgs q{da, db, L.kpart, L.kdots};
         const double bytes = spmv_dot<T>(L.M, vsel, sargs(z, w), q, c->s);
         std::string tag;
         if (c->prof.on) {
@@ -775,7 +774,7 @@ static void kc_product_dots(nbp_ctx *c, Level &L, int vsel, const T *z, T *w, co
     }
     do_spmv<T>(c, L.M, vsel, sargs(z, w), EPI_SET, false);
     timed(c, "kcycle/dots", (db ? 3.0 : 2.0) * (double)n * sizeof(T),
-          [&] { klaunch(k_kdots<T>, (unsigned)kKdotBlocks, 256u, c->s, w, da, db, n, L.kdots, oy, oa, ob); });
+          [&] { klaunch(k_kdots<T>, (unsigned)kKdotBlocks, 256u, c->s, w, da, db, n, L.kdots); });
 }
 
 template <typename T>
@@ -786,7 +785,7 @@ static void kcycle_level(nbp_ctx *c, Hier &H, int cl, int vsel, const T *b, T *x
     const double vn = (double)n * sizeof(T);   // bytes of one level vector
     if (!first_done) copy<T>(r, b, n, c->s);   // else the restriction wrote r
     vcycle_level<T>(c, H, cl, vsel, b, z1, first_done);
-    kc_product_dots<T>(c, L, vsel, z1, w1, r, (const T *)nullptr, 0, 1, 1);   // kd[0] = w1.w1, kd[1] = w1.r
+    kc_product_dots<T>(c, L, vsel, z1, w1, r, (const T *)nullptr);
     // r -= a1 w1 and, with smoothing on this level, the second cycle's first
     // step; algorithmic bytes: each distinct vector read or written, once
     const bool first = H.cheb > 0 && cl < H.nlev - 1;
@@ -797,7 +796,7 @@ static void kcycle_level(nbp_ctx *c, Hier &H, int cl, int vsel, const T *b, T *x
                 first && H.cheb > 1 ? wvec<T>(L, 4) : (T *)nullptr, wvec<T>(L, 2));
     });
     vcycle_level<T>(c, H, cl, vsel, r, z2, first);
-    kc_product_dots<T>(c, L, vsel, z2, w2, w1, r, 4, 3, 5);   // kd[4] = w2.w2, kd[3] = w2.w1, kd[5] = w2.r
+    kc_product_dots<T>(c, L, vsel, z2, w2, w1, r);
     timed(c, "kcycle/update", 3.0 * vn, [&] { klaunch(k_kupd2<T>, grid_for(n), 256u, c->s, x, z1, z2, L.kdots, n); });
 }
 
