@@ -354,12 +354,58 @@ __device__ __forceinline__ double lr_term(const SpmvArgs &a, int e0, int e1, int
     return t;
 }
 
+// A row of the paired BF16 layout by one thread, summed as k_sellm's V threads
+// per row sum it: pair p into chain p % V, an odd width's last slot into the
+// chain whose turn comes next, then the chains in the order of the lanes' tree.
+// The same bits from fewer threads: for the instances of a batch that together
+// fill the GPU, where V threads per row only add work, and whose results must
+// not depend on their neighbours.  48, 57 and 75 registers for V = 2, 4 and 8.
+template <int BS, int C, int K, int V>
+__device__ __forceinline__ void sell_chains(const SpmvArgs &a, long long base, int w, int t, float &acc0, float &acc1,
+                                            float &acc2) {
+    static_assert(V % K == 0, "whole steps of loads");
+    const int np = w / 2;
+    float s0[V] = {}, s1[V] = {}, s2[V] = {};
+    PairBatch<BS, C, K> pb;
+    sell_pairs_load(pb, a, base / 2, np, t, 0, 1);
+    pdl_wait();
+    const float *x = (const float *)a.x + col_off(a, a.x_ld);
+    for (int p = 0; p < np; p += V) {
+#pragma unroll
+        for (int h = 0; h < V; h += K) {
+            if (p + h >= np) break;
+            if (p + h > 0) sell_pairs_load(pb, a, base / 2, np, t, p + h, 1);
+#pragma unroll
+            for (int u = 0; u < K; ++u)
+                if (p + h + u < np) pair_fma<BS>(pb.c[u], pb.m[u], x, s0[h + u], s1[h + u], s2[h + u]);
+        }
+    }
+    if (w & 1) {
+        const int last = np % V;
+#pragma unroll
+        for (int h = 0; h < V; ++h)
+            if (h == last) sell_single<BS, C>(a, base + (long long)C * (w - 1), t, x, s0[h], s1[h], s2[h]);
+    }
+#pragma unroll
+    for (int o = V / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int h = 0; h < o; ++h) {
+            s0[h] += s0[h + o];
+            s1[h] += s1[h + o];
+            s2[h] += s2[h + o];
+        }
+    acc0 = s0[0];
+    acc1 = s1[0];
+    acc2 = s2[0];
+}
+
 // Sliced-ELL product for square BS x BS blocks: one thread per block row, C
 // rows per slice (C = 32: a warp per slice; C = 8 for matrices whose row
 // lengths vary, to cut padding).  Every load of values and columns by the C
 // threads of a slice is one contiguous segment (C x value bytes).  Same
-// epilogues as k_bspmv (a.rp unused; a.sl_* describe the slices).
-template <int BS, typename VT, typename XT, int EPI, bool LR, int C, int K = C == 32 ? 2 : 1>
+// epilogues as k_bspmv (a.rp unused; a.sl_* describe the slices).  V > 1: the
+// sums in the order of k_sellm's V threads per row (sell_chains; BF16 values).
+template <int BS, typename VT, typename XT, int EPI, bool LR, int C, int K = C == 32 ? 2 : 1, int V = 1>
 __global__ void __launch_bounds__(256) k_sell(SpmvArgs a) {
     using AT = XT;
     constexpr int BB = BS * BS;
@@ -373,7 +419,9 @@ __global__ void __launch_bounds__(256) k_sell(SpmvArgs a) {
     const VT *__restrict__ val = (const VT *)a.val;
     const int *__restrict__ ci = a.sl_ci;
     AT acc0 = 0, acc1 = 0, acc2 = 0;
-    if constexpr (std::is_same<VT, __nv_bfloat16>::value) {   // paired layout: w / 2 pairs, then one slot if w is odd
+    if constexpr (V > 1) {
+        sell_chains<BS, C, K, V>(a, base, w, t, acc0, acc1, acc2);
+    } else if constexpr (std::is_same<VT, __nv_bfloat16>::value) {   // paired layout: w / 2 pairs, then one slot if w is odd
         PairBatch<BS, C, K> pb;
         sell_pairs_load(pb, a, base / 2, w / 2, t, 0, 1);
         pdl_wait();

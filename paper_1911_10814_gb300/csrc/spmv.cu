@@ -129,9 +129,31 @@ static void launch_sellm_t(const SpmvArgs &a, int epi, bool lr, cudaStream_t s, 
     else launch_sellm_epi<BS, VT, XT, C, 2>(a, epi, lr, s);
 }
 
+// one thread per row in the sums of V (BF16 values); false: no such form
+template <int BS, int C, int V> static bool launch_chains_v(const SpmvArgs &a, int epi, bool lr, cudaStream_t s) {
+    using B = __nv_bfloat16;
+    constexpr int K = C == 32 ? 2 : 1;
+    const unsigned grid = grid_exact((long long)a.nslice * C);
+    if (epi == EPI_RES) klaunch(k_sell<BS, B, float, EPI_RES, false, C, K, V>, grid, 256u, s, a);
+    else if (epi == EPI_CHEB) klaunch(k_sell<BS, B, float, EPI_CHEB, false, C, K, V>, grid, 256u, s, a);
+    else if (epi != EPI_SET || BS != 3) return false;
+    else if (lr) klaunch(k_sell<3, B, float, EPI_SET, true, C, K, V>, grid, 256u, s, a);
+    else klaunch(k_sell<3, B, float, EPI_SET, false, C, K, V>, grid, 256u, s, a);
+    NBP_LAUNCHED();
+    return true;
+}
+template <int BS, int C> static bool launch_chains(const SpmvArgs &a, int epi, bool lr, cudaStream_t s, int V) {
+    if (V == 8) return launch_chains_v<BS, C, 8>(a, epi, lr, s);
+    if (V == 4) return launch_chains_v<BS, C, 4>(a, epi, lr, s);
+    return V == 2 && launch_chains_v<BS, C, 2>(a, epi, lr, s);
+}
+
 // T threads per row (T = 1: the one-thread kernel)
 template <int BS, typename VT, typename XT>
 static void launch_sell_c(const DMat &M, const SpmvArgs &a, int epi, bool lr, cudaStream_t s, int T) {
+    if constexpr (std::is_same<VT, __nv_bfloat16>::value)
+        if (M.crowded && (M.sl_c == 8 ? launch_chains<BS, 8>(a, epi, lr, s, T) : launch_chains<BS, 32>(a, epi, lr, s, T)))
+            return;
     if (T > 1) {
         if (M.sl_c == 8) launch_sellm_t<BS, VT, XT, 8>(a, epi, lr, s, T);
         else launch_sellm_t<BS, VT, XT, 32>(a, epi, lr, s, T);

@@ -24,10 +24,13 @@ int choose_group(const DMat &M);
 // 54.0 ms, 68,921 rows 66.7 / 61.9 / 64.1 / 71.5 ms; 140,481 rows 176.6 / 169.8;
 // 452,393 and 1,085,825 rows are faster with one.
 // By the matrix's own rows alone: the threads set the order of a row's sum, so
-// an instance of a batch gives the bits of its single solve.  Counting half the
-// batch's rows instead (one thread where the branches fill the GPU together)
-// took 117 against 128 ms for 16 cubes of 12-40 in BF16, 149 against 143 in
-// FP32, and made every result depend on the neighbours.
+// an instance of a batch gives the bits of its single solve.  Where half of a
+// batch's rows would have two threads or one and the instance's own more, its
+// products with BF16 values run one thread per row in the same sums
+// (DMat::crowded, sell_chains).  Mode 4, ms: own threads / so / one thread and
+// its order everywhere: 48 cubes of 12-40 303 / 279 / 262, 24 of 36-40 294 /
+// 274 / 267, 32 of 22-32 200 / 186 / 166, 48 of 12-20 114 / 103 / 94; FP32
+// values gain nothing (16 of 12-40: 143 / 149 / 149).
 int fine_threads(int rows);
 
 // Whether y = M x with the K-cycle's inner products fused (k_sell_dot) runs

@@ -20,7 +20,8 @@ def _t(a):
     return torch.as_tensor(np.ascontiguousarray(a), device="cuda:0")
 
 
-@pytest.mark.parametrize("count,smin,smax,edge", [(4, 18, 20, 12000), (4, 28, 30, 45000), (8, 38, 40, 200000)])
+@pytest.mark.parametrize("count,smin,smax,edge", [(4, 18, 20, 12000), (12, 18, 20, 45000), (4, 28, 30, 45000),
+                                                  (8, 38, 40, 200000)])
 @pytest.mark.parametrize("prec", [0, 4])
 def test_bits_do_not_depend_on_the_neighbours(count, smin, smax, edge, prec):
     systems = [synth.generate(sp) for sp in synth.batch(count=count, seed=5, smin=smin, smax=smax)]
