@@ -235,8 +235,8 @@ template <int BS, int C, int K = C == 32 ? 2 : 1> struct PairBatch {
     __nv_bfloat162 m[K][BS * BS];
 };
 template <int BS, int C, int K>
-__device__ __forceinline__ void sell_pairs_load(PairBatch<BS, C, K> &B, const SpmvArgs &a, long long base2, int np, int t, int p,
-                                                int step) {
+__device__ __forceinline__ void sell_pairs_load(PairBatch<BS, C, K> &B, const SpmvArgs &a, long long base2, int np, int t,
+                                                int p, int step) {
     constexpr int BB = BS * BS;
     const __nv_bfloat162 *__restrict__ val = (const __nv_bfloat162 *)a.val;
     const int2 *__restrict__ ci = (const int2 *)a.sl_ci;

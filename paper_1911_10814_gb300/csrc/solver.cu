@@ -501,8 +501,12 @@ template <typename T> static void tune_arnoldi(nbp_ctx *c, Krylov<T> &K, bool dl
     NBP_LAUNCHED();
     auto products = [&] {
         if (!dl) mdot<T>(c, K, K.V, K.ld, 4, K.w, K.h2);
-        else if (vec) k_mdot_dl<T, 8, true><<<K.grid_md, 256, 0, c->s>>>(K.V, K.ld, jp, 1, K.w, K.n, K.partial, K.h2, K.ticket, GivensArgs());
-        else k_mdot_dl<T, 8, false><<<K.grid_md, 256, 0, c->s>>>(K.V, K.ld, jp, 1, K.w, K.n, K.partial, K.h2, K.ticket, GivensArgs());
+        else if (vec)
+            k_mdot_dl<T, 8, true><<<K.grid_md, 256, 0, c->s>>>(K.V, K.ld, jp, 1, K.w, K.n, K.partial, K.h2, K.ticket,
+                                                               GivensArgs());
+        else
+            k_mdot_dl<T, 8, false><<<K.grid_md, 256, 0, c->s>>>(K.V, K.ld, jp, 1, K.w, K.n, K.partial, K.h2, K.ticket,
+                                                                GivensArgs());
         NBP_LAUNCHED();
     };
     auto rest = [&] {
@@ -510,9 +514,11 @@ template <typename T> static void tune_arnoldi(nbp_ctx *c, Krylov<T> &K, bool dl
             maxpy_dot<T>(c, K, K.V, K.ld, 4, K.h1, K.w, 0, K.h2);
             maxpy_dot<T>(c, K, K.V, K.ld, 4, K.h1, K.w, 1, K.nrm);
         } else if (vec) {
-            k_maxpy_dot_dl<T, kFusedCols, true><<<K.grid, 256, 0, c->s>>>(K.V, K.ld, jp, 1, K.h1, K.w, K.n, K.partial, K.h2, K.ticket);
+            k_maxpy_dot_dl<T, kFusedCols, true><<<K.grid, 256, 0, c->s>>>(K.V, K.ld, jp, 1, K.h1, K.w, K.n, K.partial, K.h2,
+                                                                          K.ticket);
         } else {
-            k_maxpy_dot_dl<T, kFusedCols, false><<<K.grid, 256, 0, c->s>>>(K.V, K.ld, jp, 1, K.h1, K.w, K.n, K.partial, K.h2, K.ticket);
+            k_maxpy_dot_dl<T, kFusedCols, false><<<K.grid, 256, 0, c->s>>>(K.V, K.ld, jp, 1, K.h1, K.w, K.n, K.partial, K.h2,
+                                                                           K.ticket);
         }
         NBP_LAUNCHED();
     };
@@ -817,9 +823,11 @@ static void vcycle_level(nbp_ctx *c, Hier &H, int l, int vsel, const T *b, T *ou
                       const T *ci = cinv_of<T>(H);
                       if constexpr (std::is_same<T, float>::value) {
                           if (H.nc % 4 == 0 && al16(ci) && al16(b))
-                              klaunch(k_dense_gemv_rows<float, true>, (unsigned)H.nc, (unsigned)kGemvThreads, c->s, ci, H.nc, b, out);
+                              klaunch(k_dense_gemv_rows<float, true>, (unsigned)H.nc, (unsigned)kGemvThreads, c->s, ci, H.nc, b,
+                                      out);
                           else
-                              klaunch(k_dense_gemv_rows<float, false>, (unsigned)H.nc, (unsigned)kGemvThreads, c->s, ci, H.nc, b, out);
+                              klaunch(k_dense_gemv_rows<float, false>, (unsigned)H.nc, (unsigned)kGemvThreads, c->s, ci, H.nc,
+                                      b, out);
                       } else {
                           klaunch(k_dense_gemv<T>, grid_exact((long long)H.nc * 32), (unsigned)256, c->s, ci, H.nc, b, out);
                       }
@@ -857,14 +865,13 @@ static void vcycle_level(nbp_ctx *c, Hier &H, int l, int vsel, const T *b, T *ou
         // + the coarse block-diagonal inverse read, d (degree > 1) and x written (+ the copy)
         const double fbytes = rbytes + (double)Lc.M.nbr * bs * bs * sizeof(T) + (k > 1 ? 2.0 : 1.0) * ncv + (kc ? ncv : 0.0);
         timed(c, "amg/restrict+first", fbytes, [&] {
-            klaunch(k_restrict_first<T>, grid_exact((long long)Lc.M.nbr * 8), (unsigned)256, c->s, 
-                L.mptr, L.mem, Lc.M.nbr, bs, r, bc, dinv_of<T>(Lc), (T)(1.0 / chc.theta), k > 1 ? wvec<T>(Lc, 4) : (T *)nullptr,
-                wvec<T>(Lc, 2),
-                kc ? wvec<T>(Lc, 5) : (T *)nullptr);
+            klaunch(k_restrict_first<T>, grid_exact((long long)Lc.M.nbr * 8), 256u, c->s, L.mptr, L.mem, Lc.M.nbr, bs, r, bc,
+                    dinv_of<T>(Lc), (T)(1.0 / chc.theta), k > 1 ? wvec<T>(Lc, 4) : (T *)nullptr, wvec<T>(Lc, 2),
+                    kc ? wvec<T>(Lc, 5) : (T *)nullptr);
         });
     } else {
         timed(c, "amg/restrict", rbytes,
-              [&] { klaunch(k_restrict<T>, grid_exact((long long)Lc.M.nbr * 8), (unsigned)256, c->s, L.mptr, L.mem, Lc.M.nbr, bs, r, bc); });
+              [&] { klaunch(k_restrict<T>, grid_exact((long long)Lc.M.nbr * 8), 256u, c->s, L.mptr, L.mem, Lc.M.nbr, bs, r, bc); });
     }
     // (a prolongation fused into the coarse level's last kernel, as a scatter
     // over each aggregate's members, was slower: uncoalesced fine updates)
@@ -1325,7 +1332,8 @@ template <typename T> static void arnoldi_dl(nbp_ctx *c, Krylov<T> &K, GmDev *st
     gv.h = h;
     if (c->gs_one_pass) gv.h2 = nullptr;
     if (gs_in_cluster(K)) {
-        klaunch(k_gs_cluster<T>, kGsCluster, (unsigned)kGsThreads, c->s, K.V, K.ld, jp, K.w, K.n, c->gs_one_pass ? 1 : 2, K.h1, K.h2, gv);
+        klaunch(k_gs_cluster<T>, kGsCluster, (unsigned)kGsThreads, c->s, K.V, K.ld, jp, K.w, K.n, c->gs_one_pass ? 1 : 2, K.h1,
+                K.h2, gv);
         NBP_LAUNCHED();
         return;
     }
@@ -1340,21 +1348,21 @@ template <typename T> static void arnoldi_dl(nbp_ctx *c, Krylov<T> &K, GmDev *st
     if (vec) {
         const unsigned g1 = K.grid_md ? K.grid_md : arnoldi_grids<T>().mdot_dl_v;
         const unsigned g2 = K.grid ? K.grid : arnoldi_grids<T>().mpd_dl_v;
-        klaunch(k_mdot_dl<T, 8, true>, g1, (unsigned)256, c->s, K.V, K.ld, jp, 1, K.w, K.n, K.partial, K.h1, K.ticket, GivensArgs());
+        klaunch(k_mdot_dl<T, 8, true>, g1, 256u, c->s, K.V, K.ld, jp, 1, K.w, K.n, K.partial, K.h1, K.ticket, GivensArgs());
         if (!c->gs_one_pass)
-            klaunch(k_maxpy_dot_dl<T, kFusedCols, true>, g2, (unsigned)256, c->s, K.V, K.ld, jp, 1, K.h1, K.w, K.n, K.partial,
+            klaunch(k_maxpy_dot_dl<T, kFusedCols, true>, g2, 256u, c->s, K.V, K.ld, jp, 1, K.h1, K.w, K.n, K.partial,
                     K.h2, K.ticket);
         klaunch(k_maxpy_norm_dl<T, true>, gn, 256u, c->s, K.V, K.ld, jp, coef, K.m + 1, K.w, K.n, K.partial, K.nrm, K.ticket,
                 gv);
     } else {
         const unsigned g1 = K.grid_md ? K.grid_md : arnoldi_grids<T>().mdot_dl_s;
         const unsigned g2 = K.grid ? K.grid : arnoldi_grids<T>().mpd_dl_s;
-        klaunch(k_mdot_dl<T, 8, false>, g1, (unsigned)256, c->s, K.V, K.ld, jp, 1, K.w, K.n, K.partial, K.h1, K.ticket, GivensArgs());
+        klaunch(k_mdot_dl<T, 8, false>, g1, 256u, c->s, K.V, K.ld, jp, 1, K.w, K.n, K.partial, K.h1, K.ticket, GivensArgs());
         if (!c->gs_one_pass)
-            klaunch(k_maxpy_dot_dl<T, kFusedCols, false>, g2, (unsigned)256, c->s, K.V, K.ld, jp, 1, K.h1, K.w, K.n, K.partial,
+            klaunch(k_maxpy_dot_dl<T, kFusedCols, false>, g2, 256u, c->s, K.V, K.ld, jp, 1, K.h1, K.w, K.n, K.partial,
                     K.h2, K.ticket);
-        klaunch(k_maxpy_norm_dl<T, false>, gn, 256u, c->s, K.V, K.ld, jp, coef, K.m + 1, K.w, K.n, K.partial, K.nrm, K.ticket,
-                gv);
+        klaunch(k_maxpy_norm_dl<T, false>, gn, 256u, c->s, K.V, K.ld, jp, coef, K.m + 1, K.w, K.n, K.partial, K.nrm,
+                K.ticket, gv);
     }
     NBP_LAUNCHED();
 }
@@ -1424,9 +1432,8 @@ template <typename T> static const T *cycle_from_col(nbp_ctx *c, Hier &H, Krylov
     T *gb = wvec<T>(L0, 0), *gx = wvec<T>(L0, 1);
     if (H.cheb > 0 && H.nlev > 1) {
         const Cheb ch = cheb_of(L0);
-        klaunch(k_start_cheb<T>, grid_exact(n), (unsigned)256, c->s, L0.M.nbr, H.bs, dinv_of<T>(L0), K.V, K.ld, &st->j, b, K.w, K.st,
-                                                         (T)(1.0 / ch.theta), H.cheb > 1 ? wvec<T>(L0, 4) : (T *)nullptr,
-                                                         wvec<T>(L0, 2));
+        klaunch(k_start_cheb<T>, grid_exact(n), 256u, c->s, L0.M.nbr, H.bs, dinv_of<T>(L0), K.V, K.ld, &st->j, b, K.w, K.st,
+                (T)(1.0 / ch.theta), H.cheb > 1 ? wvec<T>(L0, 4) : (T *)nullptr, wvec<T>(L0, 2));
         NBP_LAUNCHED();
         c->col = nbp_ctx::ColIO{&L0, K.V, K.Z, K.ld, &st->j};
         try {
@@ -2056,7 +2063,8 @@ static void do_setup(nbp_ctx *c, bool numeric = false) {
             NBP_CUDA(cudaSetDevice(c->dev));
             PoolScope scope(c->pool);
             build_shat(c->A, c->B, c->C, c->D, c->lr, c->N, c->Shat, c->diagA, c->s2);
-            amg_build(c->HS, c->Shat, c->opt, prec, c->s2, numeric, c->s_inv[1]);   // keeps the Gershgorin bound (see kRhoSteps)
+            // keeps the Gershgorin bound (see kRhoSteps)
+            amg_build(c->HS, c->Shat, c->opt, prec, c->s2, numeric, c->s_inv[1]);
         } catch (...) {
             failed_S = std::current_exception();
         }

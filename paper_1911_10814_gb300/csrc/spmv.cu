@@ -318,14 +318,14 @@ double spmv(const DMat &M, int vsel, SpmvArgs a, int epi, bool lr, cudaStream_t 
     return product_bytes(M, vsel, xs, epi, false);
 }
 
-// Threads per row and pairs loaded at once of the post-smoothing product (rows
-// of A P hold 6-8 blocks, those of S_hat P 10-20 scalars): one thread streams
-// long levels, its epilogue's operands loaded after the products (4.34M unknowns:
-// 745 ms a solve; 752 with them loaded first; 806 against 780 with two threads), two with two pairs fill the GPU on shorter ones (0.56M: 171.8 ms
-// against 178.0 with one pair each and 174.9 with one thread and four; 171.0
-// against 176.6 with four threads on its 20,000-row level), four where a row's
-// chain of loads is all there is (cube of 16: 20.6 ms against 21.2; unpaired
-// values, 29,760 rows: 40.1 against 41.0).
+// Threads per row of the post-smoothing product (rows of A P hold 6-8 blocks,
+// those of S_hat P 10-20 scalars): one streams long levels, its epilogue's
+// operands loaded after the products; two with two pairs at once fill the GPU on
+// shorter ones; four where a row's chain of loads is all there is.  Solves with
+// one / two / four threads on the levels of each range, ms: from 400,000 rows on
+// 4.34M unknowns 648 / 675; between 654 / 648 / 653, 0.56M 156.5 / 155.6 / 159.1,
+// 24x24x96 FP64 77.4 / 74.2 / 76.3; below (two / four) cube of 16 17.3 / 17.0,
+// 19x23x61 FP32 43.3 / 42.1, 24x24x96 FP64 76.1 / 74.2.
 static int post_threads(const DMat &AP, bool paired) {
     if (AP.nbr < (paired ? 8000 : 40000)) return 4;
     return AP.nbr < 400000 ? 2 : 1;

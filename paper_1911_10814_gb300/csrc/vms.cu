@@ -481,7 +481,8 @@ __global__ void k_tan_tet(int E, const double *X, const int *tets, const double 
 // dual numbers, and since the corrector stops after a few inexact steps that
 // moved the accepted ydot by up to 3e-8 (k_tan_tet keeps FP32 as it was).
 __global__ void __launch_bounds__(128) k_tan_tet64(int E, const double *X, const int *tets, const double *vd,
-                                                 const double *v, const double *p, const double *vt, VmsConst k, double *Ke) {
+                                                   const double *v, const double *p, const double *vt, VmsConst k,
+                                                   double *Ke) {
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const bool live = tid < 4LL * E;
     const int e = live ? (int)(tid >> 2) : E - 1, b = (int)(tid & 3);
@@ -629,7 +630,7 @@ __global__ void __launch_bounds__(128) k_tan_tet64(int E, const double *X, const
         Sg += ga;
         Scn += cn;
         Sed += ed;
-                E4[q] = ed;
+        E4[q] = ed;
         F4[q] = cn;
         H4[q] = be;
         K4[q] = ga;
