@@ -527,13 +527,24 @@ template <typename T> static void tune_arnoldi(nbp_ctx *c, Krylov<T> &K, bool dl
     float best = 1e30f, best_md = 1e30f;
     unsigned arg = gmax, arg_md = gmax;
     const long long launches = c->prof.launches;
+    // the largest first: a small grid's step on a long vector takes several times
+    // the best one's, and leaves after one step then.  On a vector that fills 608
+    // blocks a smaller grid has to be 5 % faster: bases longer than the four
+    // columns favour the larger one (4.34M unknowns, tied here: FP64 1396 ms with
+    // 608 blocks in the multi-dot, 1412 with 304; mode 4 347 with 608 in both, 351
+    // with 152 in the second).  On a shorter one the smaller grid is taken at a
+    // tie: a batch's branches share the SMs (48 cubes of 12-40 281 ms; 286 with
+    // the margin everywhere)
+    const float margin = pieces >= 256LL * kReduceBlocks ? 0.95f : 1.f;
+    std::reverse(cands.begin(), cands.end());
     for (unsigned g : cands) {
         if (g == 0) continue;
         K.grid = K.grid_md = g;
         float tb = 1e30f, tb_md = 1e30f;
-        for (int r = 0; r < 3; ++r) {
+        bool out = false;
+        for (int r = 0; r < 3 && !out; ++r) {
             float t = 0.f, t_md = 0.f;
-            for (int q = 0; q < 5; ++q) {
+            for (int q = 0; q < 5 && !out; ++q) {
                 NBP_CUDA(cudaMemsetAsync(flush, (r * 5 + q) & 0xff, kFlush, c->s));
                 NBP_CUDA(cudaEventRecord(ev[0], c->s));
                 products();
@@ -546,13 +557,15 @@ template <typename T> static void tune_arnoldi(nbp_ctx *c, Krylov<T> &K, bool dl
                 NBP_CUDA(cudaEventElapsedTime(&b, ev[1], ev[2]));
                 t_md += a;
                 t += b;
+                out = 5 * a > 2 * best_md && 5 * b > 2 * best;
             }
+            if (out) break;
             tb = std::min(tb, t);
             tb_md = std::min(tb_md, t_md);
-            if (t > 1.3f * best && t_md > 1.3f * best_md) break;   // out of the running
+            out = t > 1.3f * best && t_md > 1.3f * best_md;
         }
-        if (tb < best) { best = tb; arg = g; }
-        if (tb_md < best_md) { best_md = tb_md; arg_md = g; }
+        if (tb <= margin * best) { best = tb; arg = g; }
+        if (tb_md <= margin * best_md) { best_md = tb_md; arg_md = g; }
     }
     c->prof.launches = launches;
     for (cudaEvent_t &e : ev) cudaEventDestroy(e);
