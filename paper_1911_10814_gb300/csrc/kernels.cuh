@@ -912,8 +912,8 @@ __device__ __forceinline__ void block_partials(const A (&acc)[NQ], int nq, doubl
 // to w1 the differences cancel: 3.6e-5 of w2.w2 was left at the least and 0.98
 // of it at the median (S_hat levels of four boxes, residuals of 5 cycles).  So
 // FP32 sums exact products (two-product) in float-float, and FP64, whose pipe
-// is too narrow for more digits, sums over w2' itself where less than a half
-// is left, in the last block (1 to 7 cycles in a hundred).
+// is too narrow for more digits, sums over w2' itself where less than a quarter
+// is left, in the last block (0 to 6 cycles in a hundred).
 // Largest relative error of a2 on those levels: FP32 1e-11 (1.3e-6 with w2'
 // formed first and rounded products, 1.7e-4 from rounded products and w1.r
 // taken as zero), FP64 1.7e-15 (1.7e-15 and 4e-12).
@@ -945,15 +945,27 @@ __device__ __forceinline__ void kc_finish(const double (&s)[4], double w11, doub
         }
         return;
     }
-    const double beta = w11 > 0.0 ? s[1] / w11 : 0.0;
-    double ww = s[0] - beta * s[1], wr = s[2] - beta * s[3];
+    // by one thread: a warp's FP64 operation holds the pipe for 16 clocks
+    double beta = 0.0, ww = 0.0, wr = 0.0;
+    if (threadIdx.x == 0) {
+        beta = w11 > 0.0 ? s[1] / w11 : 0.0;
+        ww = s[0] - beta * s[1];
+        wr = s[2] - beta * s[3];
+    }
     if constexpr (sizeof(T) == 8) {
-        if (ww < 0.5 * s[0]) {   // the same in every thread
-            __shared__ double red[2][8];
+        __shared__ double sbeta, red[2][8];
+        __shared__ int direct;
+        if (threadIdx.x == 0) {
+            sbeta = beta;
+            direct = ww < 0.25 * s[0];
+        }
+        __syncthreads();
+        if (direct) {
+            const double bt = sbeta;
             double p0 = 0.0, p1 = 0.0;
 #pragma unroll 4
             for (long long i = threadIdx.x; i < n; i += 256) {
-                const double v = __ldcg(w2 + i) - beta * w1[i];   // w2: written by this launch
+                const double v = __ldcg(w2 + i) - bt * w1[i];   // w2: written by this launch
                 p0 += v * v;
                 p1 += v * r[i];
             }
@@ -964,10 +976,12 @@ __device__ __forceinline__ void kc_finish(const double (&s)[4], double w11, doub
                 red[1][threadIdx.x >> 5] = p1;
             }
             __syncthreads();
-            ww = wr = 0.0;
-            for (int k = 0; k < 8; ++k) {
-                ww += red[0][k];
-                wr += red[1][k];
+            if (threadIdx.x == 0) {
+                ww = wr = 0.0;
+                for (int k = 0; k < 8; ++k) {
+                    ww += red[0][k];
+                    wr += red[1][k];
+                }
             }
         }
     }

@@ -7,7 +7,7 @@ a2 = (w2'.r)/(w2'.w2'), w2' = w2 - beta w1.  FP32 vectors: their products are
 exact in float-float and 64 roundoffs of 2^-43 bound a tree of such adds, so
 w2'.w2' is off by at most 64 2^-43 of the magnitudes that cancel in it, w2'.r
 likewise.  FP64: the same with 2^-53 where the sums do not cancel (more than a
-half is left), else with the magnitudes of w2' itself, whose elements carry a
+quarter is left), else with the magnitudes of w2' itself, whose elements carry a
 roundoff of |w2| + |beta w1|."""
 import ctypes
 import os
@@ -103,7 +103,7 @@ def test_coefficients_of_close_directions(lib, form, dtype):
                 assert k[4] == 0.0 and k[3] == 0.25
                 continue
             mag = abs(L2) + abs(beta * L1)
-            if dtype is np.float64 and ww < 0.5 * s22:
+            if dtype is np.float64 and ww < 0.25 * s22:
                 dww, dwr = 64 * u * np.sum(abs(V) * mag), 64 * u * np.sum(mag * abs(R))
             else:
                 dww, dwr = 64 * u * 2 * s22, 64 * u * np.sum(mag * abs(R))
