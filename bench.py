@@ -728,7 +728,8 @@ def main():
     tr = _traffic_record(a.precision)
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": (achieved / peak) if achieved else None,
-                "traffic": tr.get(key) if tr else None,
+                # the A product's record is the mean over that mode's FP32 and BF16 launches
+                "traffic": tr.get(key) if tr and (key != "a0" or tr.get("precision") == a.precision) else None,
                 "kernel": kname, "algorithmic_bytes_per_launch": bytes_per, "avg_launch_us": avg_ms * 1e3,
                 "share_of_spmv_time": prof[key + "_ms"] / prof["spmv_ms"] if prof["spmv_ms"] else None,
                 "peak_kind": peak_kind,
