@@ -578,10 +578,11 @@ __global__ void __launch_bounds__(256) k_sellr(SpmvArgs a) {
 // Sliced-ELL product with T threads per block row (T = 2, 4, 8: thread h
 // takes slots h, h + T, ..., then an xor-shuffle tree over the T lanes), for
 // levels whose rows are few, so that one thread per row leaves the SMs with
-// little memory parallelism.
+// little memory parallelism.  V > T: T threads in the sums of V, the same bits
+// (see sell_chains, which is the form for one thread and BF16 values).
 constexpr int kSellMT = 1000;   // DMat::tuned code kSellMT + T selects this kernel with T threads per row
 __host__ __device__ inline bool is_sellm(int g) { return g == kSellMT + 2 || g == kSellMT + 4 || g == kSellMT + 8; }
-template <int BS, typename VT, typename XT, int EPI, int C, int T, bool LR = false, int K = C == 32 ? 2 : 1>
+template <int BS, typename VT, typename XT, int EPI, int C, int T, bool LR = false, int K = C == 32 ? 2 : 1, int V = T>
 __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
     using AT = XT;
     constexpr int BB = BS * BS;
@@ -636,7 +637,50 @@ __global__ void __launch_bounds__(256) k_sellm(SpmvArgs a) {
         }
     }
     AT acc0 = 0, acc1 = 0, acc2 = 0;
-    if constexpr (PAIRED) {
+    if constexpr (V > T) {
+        // this thread's chains h, h + T, ... of V, added as the V lanes' tree adds them
+        constexpr int Q = V / T;
+        const int np = PAIRED ? w / 2 : w;
+        AT s0[Q] = {}, s1[Q] = {}, s2[Q] = {};
+        if constexpr (PAIRED) {
+            for (int p = h; p < np; p += V) {
+#pragma unroll
+                for (int q = 0; q < Q; q += K) {
+                    if (p + q * T >= np) break;
+                    if (p + q * T != h) sell_pairs_load(pb, a, base / 2, np, t, p + q * T, T);
+#pragma unroll
+                    for (int u = 0; u < K; ++u)
+                        if (p + (q + u) * T < np) pair_fma<BS>(pb.c[u], pb.m[u], x, s0[q + u], s1[q + u], s2[q + u]);
+                }
+            }
+            if ((w & 1) && np % T == h) {
+                const int last = np % V / T;
+#pragma unroll
+                for (int q = 0; q < Q; ++q)
+                    if (q == last) sell_single<BS, C>(a, base + (long long)C * (w - 1), t, x, s0[q], s1[q], s2[q]);
+            }
+        } else {
+            for (int k = h; k < w; k += V) {
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    if (k + q * T >= w) break;
+                    if (k + q * T != h) slot_load<BB, C>(sb, val, ci, base, t, k + q * T);
+                    slot_fma<BS, VT, AT>(sb, x, s0[q], s1[q], s2[q]);
+                }
+            }
+        }
+#pragma unroll
+        for (int o = Q / 2; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < o; ++q) {
+                s0[q] += s0[q + o];
+                s1[q] += s1[q + o];
+                s2[q] += s2[q + o];
+            }
+        acc0 = s0[0];
+        acc1 = s1[0];
+        acc2 = s2[0];
+    } else if constexpr (PAIRED) {
         sell_pairs(pb, a, base / 2, w / 2, t, h, T, x, acc0, acc1, acc2);
         // an odd width's last slot goes to the thread whose turn comes next
         if ((w & 1) && h == (w / 2) % T) sell_single<BS, C>(a, base + (long long)C * (w - 1), t, x, acc0, acc1, acc2);

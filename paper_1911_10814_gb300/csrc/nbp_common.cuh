@@ -171,7 +171,7 @@ struct DMat {
     long long *sl2_ptr = nullptr;
     int *sl2_ci = nullptr;
     __nv_bfloat16 *sl_v16 = nullptr;
-    bool crowded = false;            // BF16 products: one thread per row in the sums of the tuned kernel's (fine_threads)
+    int beside = 0;                  // in a batch: threads per row that run, in the sums of the tuned kernel's (fine_threads)
     bool sl_lent = false;            // the sl_* arrays belong to another matrix (lend_sell)
     int tuned = -1;                  // autotuned kernel: -1 untuned, 0 sliced ELL, 1000 + T sliced ELL with T threads per row, other > 0 flat with that many lanes per row
     int bb() const { return br * bc; }

@@ -163,7 +163,7 @@ struct nbp_ctx {
     std::string report;
     nbp_ctx *tctx = nullptr;      // transposed system (adjoint), built lazily
     bool is_transposed = false;
-    bool crowded = false;         // an instance of a batch that fills the GPU (see fine_threads)
+    int beside = 0;               // an instance of a batch: threads per row that half the batch's rows ask for (fine_threads)
     // CUDA graphs of the AMG cycles, keyed by (hierarchy, value precision, Chebyshev degree)
     struct CycleGraph { cudaGraphExec_t exec = nullptr; int cheb = -1; long long kernels = 0; };
     static constexpr int kMaxChebDegree = 8;
@@ -2122,7 +2122,7 @@ static void do_setup(nbp_ctx *c, bool numeric = false) {
     const int fine = fine_kind(c);
     for (DMat *M : {&c->A, &c->B, &c->C, &c->D}) M->tuned = M->sl_ci ? fine : -1;
     for (Hier *H : {&c->HA, &c->HS}) H->L[0].M.tuned = H->L[0].M.sl_ci ? fine : -1;
-    c->A.crowded = c->HA.L[0].M.crowded = c->HS.L[0].M.crowded = c->crowded;
+    c->A.beside = c->HA.L[0].M.beside = c->HS.L[0].M.beside = c->beside;
     if (prec >= 1) autotune_cycles<float>(c);
     else autotune_cycles<double>(c);
     NBP_CUDA(cudaStreamSynchronize(s));
@@ -2765,7 +2765,7 @@ nbp_status nbp_batch_create(nbp_batch **out, int32_t count, const nbp_system *sy
     long long rows = 0;
     for (nbp_ctx *c : B->ctx) rows += c->N;
     const int t = nbp::fine_threads((int)std::min<long long>(rows / 2, INT32_MAX));
-    for (nbp_ctx *c : B->ctx) c->crowded = t <= 2 && t < nbp::fine_threads(c->N);
+    for (nbp_ctx *c : B->ctx) c->beside = t;
     *out = B;
     return NBP_OK;
 }

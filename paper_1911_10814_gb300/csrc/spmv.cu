@@ -148,11 +148,39 @@ template <int BS, int C> static bool launch_chains(const SpmvArgs &a, int epi, b
     return V == 2 && launch_chains_v<BS, C, 2>(a, epi, lr, s);
 }
 
+// P threads per row in the sums of V; false: no such form
+template <int BS, typename VT, int C, int P, int V>
+static bool launch_few_v(const SpmvArgs &a, int epi, bool lr, cudaStream_t s) {
+    constexpr int K = C == 32 && std::is_same<VT, __nv_bfloat16>::value ? 2 : 1;
+    const unsigned grid = grid_exact((long long)a.nslice * C * P);
+    if (epi == EPI_RES) klaunch(k_sellm<BS, VT, float, EPI_RES, C, P, false, K, V>, grid, 256u, s, a);
+    else if (epi == EPI_CHEB) klaunch(k_sellm<BS, VT, float, EPI_CHEB, C, P, false, K, V>, grid, 256u, s, a);
+    else if (epi != EPI_SET || BS != 3) return false;
+    else if (lr) klaunch(k_sellm<3, VT, float, EPI_SET, C, P, true, K, V>, grid, 256u, s, a);
+    else klaunch(k_sellm<3, VT, float, EPI_SET, C, P, false, K, V>, grid, 256u, s, a);
+    NBP_LAUNCHED();
+    return true;
+}
+// as few threads per row as a batch's rows leave room for, in the sums of V
+template <int BS, typename VT, int C>
+static bool launch_beside(const SpmvArgs &a, int epi, bool lr, cudaStream_t s, int P, int V) {
+    if (P == 2 && V == 8) return launch_few_v<BS, VT, C, 2, 8>(a, epi, lr, s);
+    if (P == 2 && V == 4) return launch_few_v<BS, VT, C, 2, 4>(a, epi, lr, s);
+    if (P == 4 && V == 8) return launch_few_v<BS, VT, C, 4, 8>(a, epi, lr, s);
+    if (P != 1) return false;
+    if constexpr (std::is_same<VT, __nv_bfloat16>::value) return launch_chains<BS, C>(a, epi, lr, s, V);
+    else if (V == 8) return launch_few_v<BS, VT, C, 1, 8>(a, epi, lr, s);
+    else if (V == 4) return launch_few_v<BS, VT, C, 1, 4>(a, epi, lr, s);
+    else return V == 2 && launch_few_v<BS, VT, C, 1, 2>(a, epi, lr, s);
+}
+
 // T threads per row (T = 1: the one-thread kernel)
 template <int BS, typename VT, typename XT>
 static void launch_sell_c(const DMat &M, const SpmvArgs &a, int epi, bool lr, cudaStream_t s, int T) {
-    if constexpr (std::is_same<VT, __nv_bfloat16>::value)
-        if (M.crowded && (M.sl_c == 8 ? launch_chains<BS, 8>(a, epi, lr, s, T) : launch_chains<BS, 32>(a, epi, lr, s, T)))
+    if constexpr (std::is_same<VT, __nv_bfloat16>::value || (std::is_same<VT, float>::value && BS == 3))
+        if (M.beside && M.beside < T &&
+            (M.sl_c == 8 ? launch_beside<BS, VT, 8>(a, epi, lr, s, M.beside, T)
+                         : launch_beside<BS, VT, 32>(a, epi, lr, s, M.beside, T)))
             return;
     if (T > 1) {
         if (M.sl_c == 8) launch_sellm_t<BS, VT, XT, 8>(a, epi, lr, s, T);

@@ -24,13 +24,14 @@ int choose_group(const DMat &M);
 // 54.0 ms, 68,921 rows 66.7 / 61.9 / 64.1 / 71.5 ms; 140,481 rows 176.6 / 169.8;
 // 452,393 and 1,085,825 rows are faster with one.
 // By the matrix's own rows alone: the threads set the order of a row's sum, so
-// an instance of a batch gives the bits of its single solve.  Where half of a
-// batch's rows would have two threads or one and the instance's own more, its
-// products with BF16 values run one thread per row in the same sums
-// (DMat::crowded, sell_chains).  Mode 4, ms: own threads / so / one thread and
-// its order everywhere: 48 cubes of 12-40 303 / 279 / 262, 24 of 36-40 294 /
-// 274 / 267, 32 of 22-32 200 / 186 / 166, 48 of 12-20 114 / 103 / 94; FP32
-// values gain nothing (16 of 12-40: 143 / 149 / 149).
+// an instance of a batch gives the bits of its single solve.  Where half of the
+// batch's rows ask for fewer threads, its products with A and the finest levels
+// run with those (DMat::beside), each keeping the partial sums of several of
+// the own threads apart: the same bits.  48 cubes of 12-40 in mode 4, ms: own
+// threads / so / those threads and their own order everywhere 303 / 279 / 262; 30
+// batches of 3-16 cubes of 8-36, speed against the last: own threads 0.968 / 0.955
+// / 0.962 (modes 1, 3, 4), so 0.981 / 0.993 / 1.007, with the coupling products
+// and S_hat's FP32 ones in the same way 0.968 / 0.972 / 0.987.
 int fine_threads(int rows);
 
 // Whether y = M x with the K-cycle's inner products fused (k_sell_dot) runs

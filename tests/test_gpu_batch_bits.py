@@ -1,7 +1,7 @@
 """An instance's result does not depend on its neighbours: batches whose total
 rows lie in another range of threads per row (12,000 / 45,000 / 200,000 rows
 of the finest level) than each instance's own give the bits of the instances'
-single solves, in both precisions of the products."""
+single solves, in FP64, FP32 and mixed precision."""
 import numpy as np
 import pytest
 
@@ -22,7 +22,7 @@ def _t(a):
 
 @pytest.mark.parametrize("count,smin,smax,edge", [(4, 18, 20, 12000), (12, 18, 20, 45000), (4, 28, 30, 45000),
                                                   (8, 38, 40, 200000)])
-@pytest.mark.parametrize("prec", [0, 4])
+@pytest.mark.parametrize("prec", [0, 1, 4])
 def test_bits_do_not_depend_on_the_neighbours(count, smin, smax, edge, prec):
     systems = [synth.generate(sp) for sp in synth.batch(count=count, seed=5, smin=smin, smax=smax)]
     assert max(d["n_nodes"] for d in systems) < edge <= sum(d["n_nodes"] for d in systems) / 2

@@ -1,7 +1,7 @@
-"""One thread per row in the sums of V threads (k_sell with V > 1, BF16 values)
-against k_sellm with V threads: the same bits for every row width from none to
-past two rounds of the chains, both slice heights and block sizes, every
-epilogue that a batch runs so."""
+"""Few threads per row in the sums of V threads (k_sell with V > 1: one, BF16
+values; k_sellm with V > T) against k_sellm with V threads: the same bits for
+every row width from none to past two rounds of the chains, both slice heights
+and block sizes, every epilogue that a batch runs so, BF16 and FP32 values."""
 import ctypes
 import subprocess
 
@@ -20,28 +20,33 @@ SRC = r"""
 #include "kernels.cuh"
 using namespace nbp;
 using B = __nv_bfloat16;
-template <int BS, int EPI, int C, int V> static void run(const SpmvArgs &a, int one) {
-    if (one) k_sell<BS, B, float, EPI, false, C, C == 32 ? 2 : 1, V><<<grid_exact((long long)a.nslice * C), 256>>>(a);
-    else k_sellm<BS, B, float, EPI, C, V><<<grid_exact((long long)a.nslice * C * V), 256>>>(a);
+// P threads in the sums of V (P == V: as it is); f32: FP32 values, unpaired
+template <int BS, typename VT, int EPI, int C, int P, int V> static void run(const SpmvArgs &a) {
+    constexpr bool B16 = std::is_same<VT, B>::value;
+    constexpr int K = C == 32 && B16 ? 2 : 1;
+    const unsigned grid = grid_exact((long long)a.nslice * C * P);
+    if constexpr (P == 1 && B16) k_sell<BS, B, float, EPI, false, C, K, V><<<grid, 256>>>(a);
+    else k_sellm<BS, VT, float, EPI, C, P, false, K, V><<<grid, 256>>>(a);
 }
-template <int BS, int EPI, int C> static void by_v(const SpmvArgs &a, int V, int one) {
-    if (V == 2) run<BS, EPI, C, 2>(a, one);
-    else if (V == 4) run<BS, EPI, C, 4>(a, one);
-    else run<BS, EPI, C, 8>(a, one);
+template <int BS, typename VT, int EPI, int C> static void by_v(const SpmvArgs &a, int V, int P) {
+    if (V == 2) P == 2 ? run<BS, VT, EPI, C, 2, 2>(a) : run<BS, VT, EPI, C, 1, 2>(a);
+    else if (V == 4) P == 4 ? run<BS, VT, EPI, C, 4, 4>(a) : P == 2 ? run<BS, VT, EPI, C, 2, 4>(a) : run<BS, VT, EPI, C, 1, 4>(a);
+    else P == 8 ? run<BS, VT, EPI, C, 8, 8>(a) : P == 4 ? run<BS, VT, EPI, C, 4, 8>(a) : P == 2 ? run<BS, VT, EPI, C, 2, 8>(a) : run<BS, VT, EPI, C, 1, 8>(a);
 }
-template <int BS, int C> static void by_epi(const SpmvArgs &a, int epi, int V, int one) {
-    if (epi == EPI_RES) by_v<BS, EPI_RES, C>(a, V, one);
-    else if (epi == EPI_CHEB) by_v<BS, EPI_CHEB, C>(a, V, one);
-    else by_v<BS, EPI_SET, C>(a, V, one);
+template <int BS, typename VT, int C> static void by_epi(const SpmvArgs &a, int epi, int V, int P) {
+    if (epi == EPI_RES) by_v<BS, VT, EPI_RES, C>(a, V, P);
+    else if (epi == EPI_CHEB) by_v<BS, VT, EPI_CHEB, C>(a, V, P);
+    else by_v<BS, VT, EPI_SET, C>(a, V, P);
 }
-extern "C" int product(int bs, int C, int V, int epi, int one, int n, const long long *ptr, const int *ci, const void *val,
+extern "C" int product(int bs, int C, int V, int epi, int P, int f32, int n, const long long *ptr, const int *ci, const void *val,
                        const void *x, const void *b, const void *dinv, void *d, void *y, int more) {
     SpmvArgs a = {};
     a.nbr = n; a.nslice = (n + C - 1) / C; a.sl_ptr = ptr; a.sl_ci = ci; a.val = val; a.x = x; a.b = b; a.dinv = dinv; a.d = d;
     a.y = a.xout = y; a.c1f = 0.3f; a.c2f = 0.7f; a.d_read = a.d_write = more;
     a.lr_rev = -1;
-    if (bs == 3) C == 32 ? by_epi<3, 32>(a, epi, V, one) : by_epi<3, 8>(a, epi, V, one);
-    else C == 32 ? by_epi<1, 32>(a, epi, V, one) : by_epi<1, 8>(a, epi, V, one);
+    if (f32) C == 32 ? by_epi<3, float, 32>(a, epi, V, P) : by_epi<3, float, 8>(a, epi, V, P);
+    else if (bs == 3) C == 32 ? by_epi<3, B, 32>(a, epi, V, P) : by_epi<3, B, 8>(a, epi, V, P);
+    else C == 32 ? by_epi<1, B, 32>(a, epi, V, P) : by_epi<1, B, 8>(a, epi, V, P);
     return (int)cudaDeviceSynchronize();
 }
 """
@@ -61,9 +66,9 @@ def _p(t):
     return ctypes.c_void_p(t.data_ptr())
 
 
-@pytest.mark.parametrize("bs", [1, 3])
+@pytest.mark.parametrize("bs,f32", [(1, 0), (3, 0), (3, 1)])
 @pytest.mark.parametrize("C", [8, 32])
-def test_the_same_bits(lib, bs, C):
+def test_the_same_bits(lib, bs, f32, C):
     dev = "cuda:0"
     g = torch.Generator(device=dev).manual_seed(10 * bs + C)
     rnd = lambda *n: torch.randn(*n, device=dev, generator=g)  # noqa: E731
@@ -72,7 +77,7 @@ def test_the_same_bits(lib, bs, C):
     ptr = torch.as_tensor(np.concatenate([[0], np.cumsum(C * widths)]), dtype=torch.int64, device=dev)
     slots = int(ptr[-1])
     ci = torch.randint(0, n, (slots,), dtype=torch.int32, device=dev, generator=g)
-    val = rnd(slots * bs * bs).to(torch.bfloat16)
+    val = rnd(slots * bs * bs).to(torch.float32 if f32 else torch.bfloat16)
     x, b, d0 = rnd(n * bs), rnd(n * bs), rnd(n * bs)
     dinv = rnd(n * bs * bs)
     for V in (2, 4, 8):
@@ -80,9 +85,10 @@ def test_the_same_bits(lib, bs, C):
             if bs == 1 and epi == 0:
                 continue
             got = []
-            for one in (0, 1):
+            for P in (V, *(p for p in (1, 2, 4) if p < V)):
                 y, d = torch.full_like(x, float("nan")), d0.clone()
-                assert lib.product(bs, C, V, epi, one, n, _p(ptr), _p(ci), _p(val), _p(x), _p(b), _p(dinv), _p(d), _p(y), more) == 0
+                assert lib.product(bs, C, V, epi, P, f32, n, _p(ptr), _p(ci), _p(val), _p(x), _p(b), _p(dinv), _p(d), _p(y), more) == 0
                 got.append((y, d))
             assert torch.isfinite(got[0][0]).all()
-            assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1]), (V, epi, more)
+            for y, d in got[1:]:
+                assert torch.equal(got[0][0], y) and torch.equal(got[0][1], d), (V, epi, more)
